@@ -10,6 +10,7 @@
 // Per class a lane reads the cell's four corner logits and interpolates vertically, then horizontally, with one
 // fused multiply-add per step.  No pixel is shared between cells, so blocks are independent.
 #include "st_internal.h"
+#include "miou.cuh"
 
 namespace st {
 
@@ -21,6 +22,7 @@ constexpr int SM_WARPS = 4;                                              // cell
 #endif
 constexpr int SM_SPLIT = ST_MASK_SPLIT, SM_RW = 4 / SM_SPLIT;           // warps per cell row, frame rows per warp
 constexpr int SM_THREADS = SM_WARPS * SM_SPLIT * 32;
+static_assert(SM_THREADS == 256, "the mean IoU is taken by blocks of 256 threads");
 constexpr int SM_TH = SM_WARPS + 1, SM_TW = 40, SM_T = SM_TH * SM_TW;   // tile: 5 node rows x 40 columns (34 used, start at a multiple of 4)
 constexpr int kMaxChunk = 32;                                            // classes held in shared memory at a time
 
@@ -40,6 +42,8 @@ student_mask_kernel(StudentMaskArgs a, int chunk)
     extern __shared__ __align__(16) float zs[];                   // [chunk][SM_TH][SM_TW]
     unsigned int* hist = reinterpret_cast<unsigned int*>(zs + chunk * SM_T);   // [C][C] (CONF)
     __shared__ bool is_last;
+    __shared__ double iou[SM_THREADS];
+    __shared__ int present[SM_THREADS];
     const int C = a.C, h = a.h, w = a.w, H = h * kUp, W = w * kUp;
     const int64_t p = (int64_t)h * w;
     const int tid = threadIdx.x, wi = tid / (32 * SM_SPLIT), l = tid & 31;   // wi: cell row inside the block
@@ -153,40 +157,15 @@ student_mask_kernel(StudentMaskArgs a, int chunk)
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    double* iou = reinterpret_cast<double*>(zs);                  // [C] then present [C] (the tile is no longer needed)
-    int* present = reinterpret_cast<int*>(iou + C);
-    // the matrix goes to shared memory in one coalesced pass if it fits behind them (the tile region is free now)
-    unsigned long long* cm = reinterpret_cast<unsigned long long*>(present + C + (C & 1));
-    const bool staged = (size_t)C * (sizeof(double) + sizeof(int)) + 8 + (size_t)C * C * 8 <= (size_t)chunk * SM_T * sizeof(float);
-    if (staged) {
-        for (int e = tid; e < C * C; e += SM_THREADS) cm[e] = __ldcg(&a.conf[e]);
-        __syncthreads();
-    }
-    for (int c = tid; c < C; c += SM_THREADS) {
-        unsigned long long row = 0, col = 0;
-        for (int q = 0; q < C; ++q) {
-            row += staged ? cm[c * C + q] : __ldcg(&a.conf[c * C + q]);
-            col += staged ? cm[q * C + c] : __ldcg(&a.conf[q * C + c]);
-        }
-        double v = 0.0; int pr = 0;
-        if (row > 0) {
-            const unsigned long long inter = staged ? cm[c * C + c] : __ldcg(&a.conf[c * C + c]);
-            v = (double)inter / (double)(row + col - inter);
-            pr = 1;
-        }
-        iou[c] = v; present[c] = pr;
-    }
-    __syncthreads();
+    const double m = block_miou(a.conf, C, iou, present);
     if (a.conf_out) {                                             // deliver the matrix, leave the counters at zero
         for (int e = tid; e < C * C; e += SM_THREADS) {
-            a.conf_out[e] = staged ? cm[e] : __ldcg(&a.conf[e]);
+            a.conf_out[e] = __ldcg(&a.conf[e]);
             a.conf[e] = 0;
         }
     }
     if (tid == 0) {
-        double sum = 0.0; int cnt = 0;
-        for (int k = 0; k < C; ++k) { sum += iou[k]; cnt += present[k]; }
-        *a.miou = cnt ? sum / cnt : 0.0;
+        *a.miou = m;
         *a.ticket = 0;                                            // ready for the next launch
     }
 }
@@ -194,12 +173,7 @@ student_mask_kernel(StudentMaskArgs a, int chunk)
 size_t mask_smem(int C, bool conf, int* chunk)
 {
     *chunk = C < kMaxChunk ? C : kMaxChunk;
-    size_t tile = (size_t)*chunk * SM_T * sizeof(float);
-    const size_t tail = conf ? (size_t)C * C * sizeof(unsigned int) : 0;
-    // the tile region is reused for C doubles + C ints by the last block
-    const size_t need = (size_t)C * (sizeof(double) + sizeof(int));
-    if (conf && tile < need) tile = (need + 15) / 16 * 16;
-    return tile + tail;
+    return (size_t)*chunk * SM_T * sizeof(float) + (conf ? (size_t)C * C * sizeof(unsigned int) : 0);
 }
 
 }  // namespace

@@ -36,6 +36,7 @@
 #include "st_internal.h"
 #include "tc_common.cuh"
 #include "fused_tile.cuh"
+#include "cell_softmax.cuh"
 
 #include <string.h>
 
@@ -50,44 +51,12 @@ constexpr int TZ_H = RN_Y + 2;
 // (32 used, starting at a multiple of 4 so that rows are whole 16-byte vectors), 32 when the block computes its logits
 // itself (kTwFused).
 constexpr int kTwLoad = 36, kTwFused = fused::kTileCols;
-constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
 // Classes per iteration of the two fast-path class sweeps.  The sweeps are rolled loops: unrolled over all classes
 // they were ~70 KB of straight-line code that every warp ran through once, and instruction fetch was the main stall.
 #ifndef ST_K3_CLASS_UNROLL
 #define ST_K3_CLASS_UNROLL 3
 #endif
 constexpr int kClassUnroll = ST_K3_CLASS_UNROLL;
-// Largest change of a class's logit between two corners of a cell (in log2 units) for which the cell stays on the
-// fast path.  All 16 products of the progressions are exponentials of the cell's own pixels (at most 1 after the
-// shift), the step factors stay below 2^20, and the relative error of a product grows with the size of the exponent
-// arguments: about 5e-6 at this limit, below the tolerance of the logit gradient.
-#ifndef ST_K3_FAST_RANGE
-#define ST_K3_FAST_RANGE 40.0f
-#endif
-constexpr float kFastRange = ST_K3_FAST_RANGE;
-
-__device__ __forceinline__ float ex2_approx(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// Byte k: (row eighths) x (column eighths of pixel k toward the left node column: 7, 5, 3, 1; toward the right one:
-// 1, 3, 5, 7) -- the integer adjoint weights (units of 1/64) of a row's four pixels for one corner node.
-__host__ __device__ constexpr uint32_t corner_weights(int row_eighths, bool right)
-{
-    return right ? (uint32_t)(row_eighths * 1) | (uint32_t)(row_eighths * 3) << 8 | (uint32_t)(row_eighths * 5) << 16 | (uint32_t)(row_eighths * 7) << 24
-                 : (uint32_t)(row_eighths * 7) | (uint32_t)(row_eighths * 5) << 8 | (uint32_t)(row_eighths * 3) << 16 | (uint32_t)(row_eighths * 1) << 24;
-}
-
 // A lane reads its cell's corner logits at clamped tile coordinates, so the clamped borders (node row -1 is row 0, node
 // column w is column w-1, ...) need no copies in the tile.
 struct RowCtx {
@@ -129,57 +98,6 @@ __device__ __forceinline__ void pass1(const RowCtx& rc, const float (&sk)[4], fl
             Zs[k] += ex2_approx(u[k]);
         }
     }
-}
-
-// The 16 exponentials exp2(u(r,k) - M) of one class inside the lane's cell, u bilinear between the four
-// corner logits (own column: the two node rows from shared memory, dq elements apart; right column from the next lane).
-// With ly_r = (2r+1)/8 and fr_k = (2k+1)/8:  u(r,k) = A + B k + G r + D k r, so the values are geometric
-// progressions along k and r: 4 exp2 and 12 multiplications (8 of them packed: X01[k] = (E(0,k), E(1,k)),
-// X23[k] = (E(2,k), E(3,k))).  Returns the largest corner difference
-// in the logits' own units (the caller leaves the fast path if a class changes by more than kFastRange log2-units across
-// the cell: the progressions would lose their small terms).  q points at raw logits; M is in log2 units.
-// The four quantities everything else is a product of: X01[0] = (E(0,0), E(1,0)), X23[0] = (E(2,0), E(3,0)) and the
-// per-row ratios between neighbouring pixels q01 = (q_0, q_1), q23 = (q_2, q_3), E(r,k) = E(r,0) q_r^k.
-__device__ __forceinline__ float cell_bases(const float* q, int dq, float M, float2& x01, float2& x23, float2& q01, float2& q23)
-{
-    const float a = q[0], b = q[dq];
-    const float ar = __shfl_down_sync(0xffffffffu, a, 1), br = __shfl_down_sync(0xffffffffu, b, 1);
-    const float p = b - a, qq = br - ar, e0 = ar - a;
-    const float qp = qq - p;
-    const float wv = fmaf(qp, 0.125f, e0);
-    const float A = fmaf(wv, 0.125f, fmaf(p, 0.125f, a));
-    const float E00 = ex2_approx(fmaf(A, kLog2e, -M)), QB = ex2_approx((0.25f * kLog2e) * wv),
-                TG = ex2_approx(fmaf(qp, 0.03125f * kLog2e, (0.25f * kLog2e) * p)), SD = ex2_approx((0.0625f * kLog2e) * qp);
-    const float TG2 = TG * TG, SD2 = SD * SD;
-    q01 = make_float2(QB, QB * SD);
-    q23 = __fmul2_rn(q01, make_float2(SD2, SD2));
-    x01 = make_float2(E00, E00 * TG);
-    x23 = __fmul2_rn(x01, make_float2(TG2, TG2));
-    return fmaxf(fabsf(p), fmaxf(fabsf(qq), fabsf(e0)));
-}
-
-__device__ __forceinline__ float cell_exponentials(const float* q, int dq, float M, float2 (&X01)[4], float2 (&X23)[4])
-{
-    const float a = q[0], b = q[dq];
-    const float ar = __shfl_down_sync(0xffffffffu, a, 1), br = __shfl_down_sync(0xffffffffu, b, 1);
-    const float p = b - a, qq = br - ar, e0 = ar - a;
-    const float qp = qq - p;
-    const float wv = fmaf(qp, 0.125f, e0);
-    const float A = fmaf(wv, 0.125f, fmaf(p, 0.125f, a));
-    const float E00 = ex2_approx(fmaf(A, kLog2e, -M)), QB = ex2_approx((0.25f * kLog2e) * wv),
-                TG = ex2_approx(fmaf(qp, 0.03125f * kLog2e, (0.25f * kLog2e) * p)), SD = ex2_approx((0.0625f * kLog2e) * qp);
-    // rows (0, 1) and (2, 3) ride in the two halves of packed fp32x2 registers: one multiply advances two rows
-    const float TG2 = TG * TG, SD2 = SD * SD;
-    const float2 q01 = make_float2(QB, QB * SD);
-    const float2 q23 = __fmul2_rn(q01, make_float2(SD2, SD2));
-    X01[0] = make_float2(E00, E00 * TG);
-    X23[0] = __fmul2_rn(X01[0], make_float2(TG2, TG2));
-#pragma unroll
-    for (int k = 1; k < 4; ++k) {
-        X01[k] = __fmul2_rn(X01[k - 1], q01);
-        X23[k] = __fmul2_rn(X23[k - 1], q23);
-    }
-    return fmaxf(fabsf(p), fmaxf(fabsf(qq), fabsf(e0)));
 }
 
 // pass 2 of one row on the slow path: the exponentials are formed again, multiplied by the adjoint interpolation
@@ -491,7 +409,7 @@ upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_
 #pragma unroll kClassUnroll
         for (int c = 0; c < CB; ++c) {
             float2 X01[4], X23[4];
-            wmax = fmaxf(wmax, cell_exponentials(rc.za + c * TZ, rc.dq, rc.M, X01, X23));
+            wmax = fmaxf(wmax, cell_exponentials(rc.za[c * TZ], rc.za[c * TZ + rc.dq], rc.M, X01, X23));
 #pragma unroll
             for (int k = 0; k < 4; ++k) { Z01[k] = __fadd2_rn(Z01[k], X01[k]); Z23[k] = __fadd2_rn(Z23[k], X23[k]); }
             if (CONF) {
@@ -594,18 +512,10 @@ upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_
             const float2 bw01 = make_float2(bw[0], bw[1]), bw23 = make_float2(bw[2], bw[3]);
 #pragma unroll kClassUnroll
             for (int c = 0; c < CB; ++c) {
-                // a row's four exponentials are E(r,0) q_r^k, so the row's weighted sum is E(r,0) times a cubic in q_r
-                // with the pixel weights as coefficients: Horner's rule, the progression itself is not formed again
-                float2 x01, x23, q01, q23;
-                cell_bases(rc.za + c * TZ, rc.dq, rc.M, x01, x23, q01, q23);
-                float2 aL01 = WL01[3], aL23 = WL23[3], aR01 = WR01[3], aR23 = WR23[3];
-#pragma unroll
-                for (int k = 2; k >= 0; --k) {
-                    aL01 = __ffma2_rn(aL01, q01, WL01[k]); aL23 = __ffma2_rn(aL23, q23, WL23[k]);
-                    aR01 = __ffma2_rn(aR01, q01, WR01[k]); aR23 = __ffma2_rn(aR23, q23, WR23[k]);
-                }
-                aL01 = __fmul2_rn(aL01, x01); aL23 = __fmul2_rn(aL23, x23);
-                aR01 = __fmul2_rn(aR01, x01); aR23 = __fmul2_rn(aR23, x23);
+                float2 x01, x23, q01, q23, aL01, aL23, aR01, aR23;
+                cell_bases(rc.za[c * TZ], rc.za[c * TZ + rc.dq], rc.M, x01, x23, q01, q23);
+                cell_row_sums(x01, x23, q01, q23, WL01, WL23, aL01, aL23);
+                cell_row_sums(x01, x23, q01, q23, WR01, WR23, aR01, aR23);
                 // own cell's left part + left cell's right part, per row
                 const float2 hs01 = __fadd2_rn(aL01, make_float2(__shfl_up_sync(0xffffffffu, aR01.x, 1), __shfl_up_sync(0xffffffffu, aR01.y, 1)));
                 const float2 hs23 = __fadd2_rn(aL23, make_float2(__shfl_up_sync(0xffffffffu, aR23.x, 1), __shfl_up_sync(0xffffffffu, aR23.y, 1)));
@@ -680,10 +590,10 @@ upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_
     }
     if (node_ok) {
         if (a.dz) {
-            float* dzp = a.dz + (int64_t)s * C * p + (int64_t)y * w + n;
+            float* dzp = a.dz + (int64_t)s * C * a.dz_plane + (int64_t)y * a.dz_pitch + n;
 #pragma unroll
             for (int c = 0; c < CB; ++c)
-                if (c < C) dzp[(int64_t)c * p] = v[c];
+                if (c < C) dzp[(int64_t)c * a.dz_plane] = v[c];
         }
         if (a.dz_bf16) {
             bf16* dzb = a.dz_bf16 + (int64_t)s * kClassPad * a.dz_bf16_pitch + (int64_t)y * w + n;

@@ -41,21 +41,35 @@ __device__ __forceinline__ double block_miou(const unsigned long long* conf_g, i
         __syncthreads();
         conf = staged;
     }
-    const int c = threadIdx.x;
-    double v = 0.0; int pr = 0;
-    if (c < C) {
-        unsigned long long row = 0, col = 0;
-        for (int q = 0; q < C; ++q) { row += conf == staged ? conf[c * C + q] : __ldcg(conf + c * C + q); col += conf == staged ? conf[q * C + c] : __ldcg(conf + q * C + c); }
-        if (row > 0) {
-            const unsigned long long inter = conf == staged ? conf[c * C + c] : __ldcg(conf + c * C + c);
-            v = (double)inter / (double)(row + col - inter);
-            pr = 1;
+    if (conf == staged) {
+        const int c = threadIdx.x;
+        double v = 0.0; int pr = 0;
+        if (c < C) {
+            unsigned long long row = 0, col = 0;
+            for (int q = 0; q < C; ++q) { row += conf[c * C + q]; col += conf[q * C + c]; }
+            if (row > 0) { const unsigned long long inter = conf[c * C + c]; v = (double)inter / (double)(row + col - inter); pr = 1; }
+        }
+        iou[c] = v; present[c] = pr;
+    } else {
+        // larger matrices stay in global memory: a warp per class, its lanes along the row and the column (81 classes: 162
+        // dependent-latency loads per thread otherwise)
+        const int lane = threadIdx.x & 31;
+        for (int c = threadIdx.x >> 5; c < C; c += blockDim.x >> 5) {
+            unsigned long long row = 0, col = 0;
+#pragma unroll 4
+            for (int q = lane; q < C; q += 32) { row += __ldcg(conf + c * C + q); col += __ldcg(conf + q * C + c); }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) { row += __shfl_xor_sync(0xffffffffu, row, o); col += __shfl_xor_sync(0xffffffffu, col, o); }
+            if (lane == 0) {
+                const unsigned long long inter = __ldcg(conf + c * C + c);
+                iou[c] = row > 0 ? (double)inter / (double)(row + col - inter) : 0.0;
+                present[c] = row > 0;
+            }
         }
     }
-    iou[c] = v; present[c] = pr;
     __syncthreads();
     double m = 0.0;
-    if (c == 0) {
+    if (threadIdx.x == 0) {
         double sum = 0.0; int n = 0;
         for (int k = 0; k < C; ++k) { sum += iou[k]; n += present[k]; }
         m = n ? sum / n : 0.0;

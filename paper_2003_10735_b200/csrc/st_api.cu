@@ -208,21 +208,25 @@ UpdateArgs make_update_args(st_ctx* c, int slot, const int* skip = nullptr, int6
         ly.w_off = c->layout.w_off[L]; ly.b_off = c->layout.b_off[L];
         ly.cout = c->layout.cout[L]; ly.cin = c->layout.cin[L]; ly.taps = c->layout.taps[L];
         const bool last = (L == n_all - 1);
-        if (last) { ly.b_partials = c->db_part; ly.n_bpart = c->n_k3_blocks; }
+        if (last) {
+            ly.b_partials = c->db_part; ly.n_bpart = c->n_k3_blocks;
+            ly.w_partials = c->w2_partials; ly.n_split = c->n_split2;
+            ly.w_split_stride = (int64_t)(c->bf16_mode ? kClassPad : ly.cout) * ly.cin;
+            ly.w_stream_stride = ly.w_split_stride * c->n_split2;
+        } else {
+            const st_ctx::Block& k = c->blk[L];
+            ly.w_partials = k.w_partials; ly.n_split = c->n_split1;
+            ly.w_split_stride = (int64_t)9 * ly.cout * ly.cin;
+            ly.w_stream_stride = ly.w_split_stride * c->n_split1;
+            ly.b_partials = k.b_partials; ly.n_bpart = k.n_bpart;
+        }
         if (c->bf16_mode) {
             if (last) {
-                ly.w_partials = c->w2_partials; ly.n_split = c->n_split2;
-                ly.w_split_stride = (int64_t)kClassPad * ly.cin;
-                ly.w_stream_stride = ly.w_split_stride * c->n_split2;
                 ly.shadow = c->w2_shadow; ly.shadow_stream_stride = (int64_t)kClassPad * ly.cin;
             } else {
                 const st_ctx::Block& k = c->blk[L];
-                ly.w_partials = k.w_partials; ly.n_split = c->n_split1;
-                ly.w_split_stride = (int64_t)9 * ly.cout * ly.cin;
-                ly.w_stream_stride = ly.w_split_stride * c->n_split1;
                 ly.shadow = k.w; ly.shadow_stream_stride = (int64_t)9 * ly.cout * ly.cin;
                 ly.shadow_t = k.w_t; ly.shadow_t_stream_stride = (int64_t)9 * k.c_prev * ly.cout; ly.c_take = k.c_prev;
-                ly.b_partials = k.b_partials; ly.n_bpart = k.n_bpart;
             }
         }
     }
@@ -262,18 +266,15 @@ st_status enqueue_forward(st_ctx* c, StageTimer* t = nullptr, const int* skip = 
         c->launches += tc_forward(c->plan, s, t, skip, skip_stride, after_update, c->first_trained < c->n_blocks ? c->first_trained : c->n_blocks);
     } else if (c->Ch == 0) {
         ST_REPEAT(t) launch_conv_fwd_f32(c->x_f32, c->Cin, c->h, c->w, c->theta + c->layout.w_off[0], c->theta + c->layout.b_off[0],
-                            c->C, 1, false, c->z, c->S, (int64_t)c->Cin * c->p, c->n_params, c->n_params,
-                            (int64_t)c->C * c->p, s);
+                                         c->C, 1, false, c->z, false, c->S, c->n_params, s);
         if (t) t->mark("conv1x1_fwd_f32", s, st_repeats(t));
         c->launches += st_repeats(t);
     } else {
         ST_REPEAT(t) launch_conv_fwd_f32(c->x_f32, c->Cin, c->h, c->w, c->theta + c->layout.w_off[0], c->theta + c->layout.b_off[0],
-                            c->Ch, 3, true, c->hid_f32, c->S, (int64_t)c->Cin * c->p, c->n_params, c->n_params,
-                            (int64_t)c->Ch * c->p, s);
+                                         c->Ch, 3, true, c->hid_f32, true, c->S, c->n_params, s);
         if (t) t->mark("conv3x3_fwd_f32", s, st_repeats(t));
         ST_REPEAT(t) launch_conv_fwd_f32(c->hid_f32, c->Ch, c->h, c->w, c->theta + c->layout.w_off[1], c->theta + c->layout.b_off[1],
-                            c->C, 1, false, c->z, c->S, (int64_t)c->Ch * c->p, c->n_params, c->n_params,
-                            (int64_t)c->C * c->p, s);
+                                         c->C, 1, false, c->z, false, c->S, c->n_params, s);
         if (t) t->mark("conv1x1_fwd_f32", s, st_repeats(t));
         c->launches += 2 * st_repeats(t);
     }
@@ -299,7 +300,9 @@ UpsampleCeArgs k3_args(st_ctx* c, bool fp32_grad, bool bf16_grad, unsigned long 
     UpsampleCeArgs k3;
     k3.z = c->z; k3.labels = c->heavy_w > 1 ? c->labels_tagged : c->labels;
     k3.heavy_w = c->heavy_w;
-    k3.dz = fp32_grad ? c->dz : nullptr;
+    const PadF32 pad(c->h, c->w);              // the fp32 convolutions read it as a padded plane
+    k3.dz = !fp32_grad ? nullptr : c->bf16_mode ? c->dz : c->dz + pad.origin;
+    k3.dz_pitch = c->bf16_mode ? c->w : pad.pitch; k3.dz_plane = c->bf16_mode ? c->p : pad.plane;
     k3.dz_bf16 = bf16_grad ? c->dz_bf16 : nullptr;
     k3.dz_bf16_pitch = c->dz_pitch;
     k3.loss_part = c->loss_part; k3.db_part = c->db_part;
@@ -342,21 +345,18 @@ st_status enqueue_backward(st_ctx* c, StageTimer* t = nullptr, const int* skip =
     if (c->bf16_mode) {
         c->launches += tc_backward(c->plan, s, t, skip, skip_stride, ctl);
     } else if (c->Ch == 0) {
-        ST_REPEAT(t) launch_conv_wgrad_f32(c->x_f32, c->dz, c->Cin, c->C, c->h, c->w, 1, c->grad + c->layout.w_off[0], c->S,
-                              (int64_t)c->Cin * c->p, (int64_t)c->C * c->p, c->n_params, s);
+        ST_REPEAT(t) launch_conv_wgrad_f32(c->x_f32, c->dz, c->Cin, c->C, c->h, c->w, 1, c->w2_partials, nullptr, c->S, s);
         if (t) t->mark("conv1x1_wgrad_f32", s, st_repeats(t));
         c->launches += st_repeats(t);
     } else {
-        const int64_t hs = (int64_t)c->Ch * c->p;
-        launch_conv_wgrad_f32(c->hid_f32, c->dz, c->Ch, c->C, c->h, c->w, 1, c->grad + c->layout.w_off[1], c->S,
-                              hs, (int64_t)c->C * c->p, c->n_params, s);
-        launch_conv1x1_dgrad_relu_f32(c->theta + c->layout.w_off[1], c->dz, c->hid_f32, c->C, c->Ch, c->p,
-                                      c->dhid_f32, c->S, c->n_params, (int64_t)c->C * c->p, hs, s);
-        launch_conv_wgrad_f32(c->x_f32, c->dhid_f32, c->Cin, c->Ch, c->h, c->w, 3, c->grad + c->layout.w_off[0], c->S,
-                              (int64_t)c->Cin * c->p, hs, c->n_params, s);
-        launch_bias_grad_f32(c->dhid_f32, c->Ch, c->p, c->grad + c->layout.b_off[0], c->S, hs, c->n_params, s);
-        if (t) t->mark("backward_f32", s, 4);
-        c->launches += 4;
+        ST_REPEAT(t) launch_conv_wgrad_f32(c->hid_f32, c->dz, c->Ch, c->C, c->h, c->w, 1, c->w2_partials, nullptr, c->S, s);
+        if (t) t->mark("conv1x1_wgrad_f32", s, st_repeats(t));
+        ST_REPEAT(t) launch_conv1x1_dgrad_relu_f32(c->theta + c->layout.w_off[1], c->dz, c->hid_f32, c->C, c->Ch, c->h, c->w,
+                                                   c->dhid_f32, c->S, c->n_params, s);
+        if (t) t->mark("conv1x1_dgrad_f32", s, st_repeats(t));
+        ST_REPEAT(t) launch_conv_wgrad_f32(c->x_f32, c->dhid_f32, c->Cin, c->Ch, c->h, c->w, 3, c->blk[0].w_partials, c->blk[0].b_partials, c->S, s);
+        if (t) t->mark("conv3x3_wgrad_f32", s, st_repeats(t));
+        c->launches += 3 * st_repeats(t);
     }
     return check_launch(c, "head backward");
 }
@@ -606,7 +606,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     if (c->adam) ALLOC(vel2, S * c->n_params);
     ALLOC(labels, S * c->P);
     if (c->heavy_w > 1) ALLOC(labels_tagged, S * c->P);
-    ALLOC(z, S * c->C * c->p); ALLOC(dz, S * c->C * c->p);
+    ALLOC(z, S * c->C * c->p); ALLOC(dz, S * c->C * (c->bf16_mode ? c->p : PadF32(c->h, c->w).plane));
     ALLOC(loss_part, S * c->n_k3_blocks); ALLOC(db_part, (size_t)S * c->n_k3_blocks * c->C);
     ALLOC(loss_buf, S * kMaxSteps);
     ALLOC(miou_tmp, 4); ALLOC(mask_tmp, c->P); ALLOC(mask_tmp2, c->P); ALLOC(conf_tmp, 2 * c->C * c->C + 1);   // counters (zero between calls), the block counter, the delivered matrix
@@ -638,13 +638,22 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             }
         }
     } else {
-        ALLOC(x_f32, S * c->Cin * c->p);
-        if (c->Ch) { ALLOC(hid_f32, S * c->Ch * c->p); ALLOC(dhid_f32, S * c->Ch * c->p); }
+        const int64_t plane = PadF32(c->h, c->w).plane;
+        ALLOC(x_f32, S * c->Cin * plane);
+        c->n_split2 = conv_wgrad_f32_splits(c_last, c->C, c->h, c->w, 1, S);
+        ALLOC(w2_partials, (size_t)S * c->n_split2 * c->C * c_last);
+        if (c->Ch) {
+            ALLOC(hid_f32, S * c->Ch * plane); ALLOC(dhid_f32, S * c->Ch * plane);
+            c->n_split1 = c->blk[0].n_bpart = conv_wgrad_f32_splits(c->Cin, c->Ch, c->h, c->w, 3, S);
+            ALLOC(blk[0].w_partials, (size_t)S * c->n_split1 * 9 * c->Ch * c->Cin);
+            ALLOC(blk[0].b_partials, (size_t)S * c->n_split1 * c->Ch);
+        }
     }
 #undef ALLOC
     if (e == cudaSuccess) e = prepare_upsample_ce(c->C);
     if (e == cudaSuccess) c->k3_has_map = make_logit_tile_map(&c->k3_map, c->z, S, c->C, c->h, c->w) ? 1 : 0;
     if (e == cudaSuccess) e = prepare_student_mask(c->C);
+    if (e == cudaSuccess && !c->bf16_mode) e = prepare_conv_f32();
     if (e != cudaSuccess) {
         st_status code = fail(nullptr, e == cudaErrorMemoryAllocation ? ST_ERR_OOM : ST_ERR_CUDA,
                               "st_init_head: device allocation failed: %s", cudaGetErrorString(e));
@@ -716,17 +725,16 @@ st_status st_set_frozen_features(st_ctx* ctx, int32_t stream, const float* feat_
     if (st != ST_OK) return st;
     if (!feat_chw) return fail(ctx, ST_ERR_INVALID_ARG, "st_set_frozen_features: NULL features");
     const size_t bytes = (size_t)ctx->Cin * ctx->p * sizeof(float);
-    if (ctx->bf16_mode) {
-        const void* src = nullptr;
-        st = to_device(ctx, feat_chw, bytes, &src);
-        if (st != ST_OK) return st;
+    const void* src = nullptr;
+    st = to_device(ctx, feat_chw, bytes, &src);
+    if (st != ST_OK) return st;
+    if (ctx->bf16_mode)
         launch_feat_to_bf16_nhwc((const float*)src, ctx->Cin, ctx->p, ctx->x_bf16 + (int64_t)stream * ctx->p * ctx->Cin, ctx->stream);
-        ctx->launches += 1;
-        st = check_launch(ctx, "feature cache");
-        if (st != ST_OK) return st;
-    } else {
-        ST_CUDA(ctx, cudaMemcpyAsync(ctx->x_f32 + (int64_t)stream * ctx->Cin * ctx->p, feat_chw, bytes, cudaMemcpyDefault, ctx->stream));
-    }
+    else
+        launch_pad_planes((const float*)src, ctx->x_f32 + (int64_t)stream * ctx->Cin * PadF32(ctx->h, ctx->w).plane, ctx->Cin, ctx->h, ctx->w, ctx->stream);
+    ctx->launches += 1;
+    st = check_launch(ctx, "feature cache");
+    if (st != ST_OK) return st;
     ctx->has_feat[stream] = 1;
     ctx->z_current = false;
     ctx->prefix_current = false;
@@ -1260,6 +1268,10 @@ st_status st_read_tensor(st_ctx* ctx, int32_t stream, st_tensor which, float* ds
     }
     const float* src = nullptr;
     const int64_t s = stream;
+    auto unpad = [&](const float* padded, int channels) {         // fp32 mode: the tensor without its zero border
+        launch_unpad_planes(padded + s * channels * PadF32(ctx->h, ctx->w).plane, ctx->read_tmp, channels, ctx->h, ctx->w, ctx->stream);
+        return (const float*)ctx->read_tmp;
+    };
     if ((which == ST_TENSOR_LOGITS || which == ST_TENSOR_LOGIT_GRAD) && ctx->z_unkept) {
         st = student_forward(ctx, stream, "st_read_tensor");     // the forward of the student the last call left behind
         if (st != ST_OK) return st;
@@ -1271,17 +1283,17 @@ st_status st_read_tensor(st_ctx* ctx, int32_t stream, st_tensor which, float* ds
                 launch_upsample_ce(k3_args(ctx, true, false, nullptr), &ctx->k3_map, ctx->stream);
                 ctx->launches += 1;
             }
-            src = ctx->dz + s * ctx->C * ctx->p;
+            src = ctx->bf16_mode ? ctx->dz + s * ctx->C * ctx->p : unpad(ctx->dz, ctx->C);
             break;
         case ST_TENSOR_PARAM_GRAD: launch_pack(ctx->grad + s * ctx->n_params, ctx->read_tmp, ctx->layout, 0, ctx->n_params, 1, ctx->stream); src = ctx->read_tmp; break;
         case ST_TENSOR_MOMENTUM: launch_pack(ctx->vel + s * ctx->n_params, ctx->read_tmp, ctx->layout, 0, ctx->n_params, 1, ctx->stream); src = ctx->read_tmp; break;
         case ST_TENSOR_HIDDEN:
             if (ctx->bf16_mode) { launch_nhwc_bf16_to_chw(ctx->blk[ctx->n_blocks - 1].out + s * ctx->p * ctx->Ch, ctx->Ch, ctx->p, ctx->read_tmp, ctx->stream); src = ctx->read_tmp; }
-            else src = ctx->hid_f32 + s * ctx->Ch * ctx->p;
+            else src = unpad(ctx->hid_f32, ctx->Ch);
             break;
         case ST_TENSOR_HIDDEN_GRAD:
             if (ctx->bf16_mode) { launch_nhwc_bf16_to_chw(ctx->blk[ctx->n_blocks - 1].dout + s * ctx->p * ctx->Ch, ctx->Ch, ctx->p, ctx->read_tmp, ctx->stream); src = ctx->read_tmp; }
-            else src = ctx->dhid_f32 + s * ctx->Ch * ctx->p;
+            else src = unpad(ctx->dhid_f32, ctx->Ch);
             break;
         case ST_TENSOR_HIDDEN_FIRST:
             launch_nhwc_bf16_to_chw(ctx->blk[0].out + s * ctx->p * ctx->blk[0].c_out, ctx->blk[0].c_out, ctx->p, ctx->read_tmp, ctx->stream);
@@ -1293,7 +1305,7 @@ st_status st_read_tensor(st_ctx* ctx, int32_t stream, st_tensor which, float* ds
             break;
         case ST_TENSOR_FEATURES:
             if (ctx->bf16_mode) { launch_nhwc_bf16_to_chw(ctx->x_bf16 + s * ctx->p * ctx->Cin, ctx->Cin, ctx->p, ctx->read_tmp, ctx->stream); src = ctx->read_tmp; }
-            else src = ctx->x_f32 + s * ctx->Cin * ctx->p;
+            else src = unpad(ctx->x_f32, ctx->Cin);
             break;
     }
     st = check_launch(ctx, "read tensor");

@@ -89,7 +89,9 @@ void launch_object_weight_tags(const uint8_t* labels, int H, int W, int backgrou
 struct UpsampleCeArgs {
     const float* z;          // [S][C][h][w]
     const uint8_t* labels;   // [S][H][W]
-    float* dz;               // [S][C][h][w]     gradient of the mean loss, or nullptr (only the bf16 copy is wanted)
+    float* dz;               // pixel (0, 0) of the gradient of the mean loss, or nullptr (only the bf16 copy is wanted); rows
+    int dz_pitch;            //   dz_pitch and channels dz_plane floats apart, streams C channels
+    int64_t dz_plane;
     bf16* dz_bf16;           // [S][kClassPad][dz_bf16_pitch] or nullptr (rows >= C untouched)
     int64_t dz_bf16_pitch;
     float* loss_part;        // [S][n_blocks]    per-block partial sums of per-pixel losses
@@ -164,19 +166,30 @@ bool student_mask_fused_supported(int C);   // confusion counters fit shared mem
 cudaError_t prepare_student_mask(int C);    // once per device and class count, outside any stream capture
 void launch_student_mask(const StudentMaskArgs& a, cudaStream_t s);
 
-// ---- fp32 CUDA-core convolutions (gemm_precision 0), planar [C][h][w] -------------------------
-void launch_conv_fwd_f32(const float* in, int Cin, int h, int w, const float* Wt, const float* b,
-                         int Cout, int ks, bool relu, float* out, int S, int64_t in_stride,
-                         int64_t w_stride, int64_t b_stride, int64_t out_stride, cudaStream_t s);
-void launch_conv_wgrad_f32(const float* in, const float* dout, int Cin, int Cout, int h, int w, int ks,
-                           float* dW, int S, int64_t in_stride, int64_t dout_stride,
-                           int64_t dw_stride, cudaStream_t s);
-void launch_conv1x1_dgrad_relu_f32(const float* W2, const float* dz, const float* Hact, int C, int Ch,
-                                   int64_t p, float* dH, int S, int64_t w_stride, int64_t dz_stride,
-                                   int64_t h_stride, cudaStream_t s);
-// db[c] = sum_p d[c][p] (one block per channel, fixed-order reduction)
-void launch_bias_grad_f32(const float* d, int C, int64_t p, float* db, int S, int64_t d_stride,
-                          int64_t db_stride, cudaStream_t s);
+// ---- fp32 CUDA-core convolutions (gemm_precision 0) -------------------------------------------
+// Planes [C][rows][pitch] with the map at row kPadTop, column kPadLeft and zeros around it (allocated zero; every writer
+// touches the interior only).  Rows start on 16-byte boundaries at any width and reach past the last 32 x 4 pixel tile.
+constexpr int kPadTop = 1, kPadLeft = 4;
+struct PadF32 {
+    int pitch, rows;
+    int64_t plane, origin;      // floats per channel; index of pixel (0, 0)
+    __host__ __device__ PadF32(int h, int w)
+        : pitch((w + 31) / 32 * 32 + 2 * kPadLeft), rows((h + 3) / 4 * 4 + 2 * kPadTop), plane((int64_t)pitch * rows), origin(kPadTop * pitch + kPadLeft) {}
+};
+void launch_pad_planes(const float* plain, float* padded, int C, int h, int w, cudaStream_t s);
+void launch_unpad_planes(const float* padded, float* plain, int C, int h, int w, cudaStream_t s);
+// Inputs and gradients are padded planes of S streams back to back; the output is one too if out_padded, else [Cout][h][w].
+// Weight, bias and (w_stride floats per stream) parameters as in PackLayout.
+void launch_conv_fwd_f32(const float* in, int Cin, int h, int w, const float* Wt, const float* b, int Cout, int ks, bool relu,
+                         float* out, bool out_padded, int S, int64_t w_stride, cudaStream_t s);
+// Weight gradient as n_split = conv_wgrad_f32_splits(...) partial results [S][n_split][tap][Cout][Cin], which the parameter
+// update adds; with b_partials also the bias gradient's, [S][n_split][Cout]
+int conv_wgrad_f32_splits(int Cin, int Cout, int h, int w, int ks, int S);
+void launch_conv_wgrad_f32(const float* in, const float* dout, int Cin, int Cout, int h, int w, int ks, float* partials,
+                           float* b_partials, int S, cudaStream_t s);
+void launch_conv1x1_dgrad_relu_f32(const float* W2, const float* dz, const float* Hact, int C, int Ch, int h, int w, float* dH, int S,
+                                   int64_t w_stride, cudaStream_t s);
+cudaError_t prepare_conv_f32();   // once per device, outside any stream capture
 
 // ---- control of Algorithm 1 (Train): assessed once per prediction, per stream, by the update kernel that follows the
 // prediction (metric of the prediction, best_student, the break) ----------------------------------------------
