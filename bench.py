@@ -456,7 +456,7 @@ def run_ours(args, cfg):
                                 lambda i: key_frame(i, feats_d, logits_d, packed_d), between=reset_parameters)
         if clocks:
             clocks.end()
-        launches = (st.st_launch_count(ctx) - launches0 - n_blocks * S * (2 if cfg.gemm_precision == 1 else 1)) // n_blocks
+        launches = (st.st_launch_count(ctx) - launches0 - n_blocks * S) // n_blocks
         last_miou_dev = float(miou_d[0].item())
         block_ms = [max_over_ranks(m, dist, "cuda") for m in block_ms]
         ms_total = statistics.median(block_ms)

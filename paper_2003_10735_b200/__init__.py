@@ -146,6 +146,7 @@ def load_library() -> ctypes.CDLL:
 
 # ---------------------------------------------------------------------------- marshalling
 _NP_OF = {"float32": np.float32, "float64": np.float64, "uint8": np.uint8, "int32": np.int32, "int64": np.int64}
+_NAME_OF = {}        # torch dtype object -> its name here, filled as they are met (a look-up per call instead of a string)
 
 
 def _ptr(buf, dtype: str, min_elems: int, what: str) -> Optional[int]:
@@ -158,13 +159,18 @@ def _ptr(buf, dtype: str, min_elems: int, what: str) -> Optional[int]:
         if buf.size < min_elems:
             raise ValueError(f"{what}: {buf.size} elements, need {min_elems}")
         return buf.ctypes.data
-    if hasattr(buf, "data_ptr"):
-        if str(buf.dtype) != "torch." + dtype or not buf.is_contiguous():
-            raise TypeError(f"{what}: need a contiguous {dtype} tensor, got {buf.dtype}")
-        if buf.numel() < min_elems:
-            raise ValueError(f"{what}: {buf.numel()} elements, need {min_elems}")
-        return buf.data_ptr()
-    raise TypeError(f"{what}: expected a torch tensor or numpy array")
+    try:
+        kind, address = buf.dtype, buf.data_ptr
+    except AttributeError:
+        raise TypeError(f"{what}: expected a torch tensor or numpy array") from None
+    name = _NAME_OF.get(kind)
+    if name is None:
+        name = _NAME_OF[kind] = str(kind).removeprefix("torch.")
+    if name != dtype or not buf.is_contiguous():
+        raise TypeError(f"{what}: need a contiguous {dtype} tensor, got {buf.dtype}")
+    if buf.numel() < min_elems:
+        raise ValueError(f"{what}: {buf.numel()} elements, need {min_elems}")
+    return address()
 
 
 class _Ctx:
@@ -176,6 +182,7 @@ class _Ctx:
         self.S, self.C = desc.n_streams, desc.n_classes
         self.p = desc.feat_h * desc.feat_w
         self.P = self.p * desc.up * desc.up
+        self.c_in = desc.c_in
         # n_params: the values UpdatedPart carries (the trained layers); n_params_all: every layer of the back part
         self.n_params_all, self.n_params = st_head_param_counts(desc)
 
@@ -233,8 +240,7 @@ def st_init_head(*, n_streams: int = 1, c_in: int, c_hidden: int = 0, n_classes:
 
 
 def st_set_frozen_features(ctx: _Ctx, stream: int, feat_chw) -> None:
-    n = ctx.desc.c_in * ctx.p
-    _check(load_library().st_set_frozen_features(ctx.handle, stream, _ptr(feat_chw, "float32", n, "feat_chw")), ctx)
+    _check(load_library().st_set_frozen_features(ctx.handle, stream, _ptr(feat_chw, "float32", ctx.c_in * ctx.p, "feat_chw")), ctx)
 
 
 def st_set_skip_features(ctx: _Ctx, stream: int, block: int, feat_chw) -> None:
@@ -285,9 +291,8 @@ def st_pack_updated_params(ctx: _Ctx, stream: int, dst, dst_capacity: Optional[i
     if dst is None:
         cap, addr = 0, None
     else:
-        nelem = dst.size if isinstance(dst, np.ndarray) else dst.numel()
-        cap = nelem * 4 if dst_capacity is None else dst_capacity
         addr = _ptr(dst, "float32", 0, "dst")
+        cap = (dst.size if isinstance(dst, np.ndarray) else dst.numel()) * 4 if dst_capacity is None else dst_capacity
     nbytes = ctypes.c_size_t(0)
     _check(load_library().st_pack_updated_params(ctx.handle, stream, addr, cap, ctypes.byref(nbytes)), ctx)
     return int(nbytes.value)

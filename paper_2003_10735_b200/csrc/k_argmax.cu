@@ -10,18 +10,19 @@
 
 namespace st {
 
+template <int U>
 __global__ void __launch_bounds__(256)
-argmax_u8_vec4_kernel(const float4* __restrict__ T, int C, int64_t n_quads, uint32_t* __restrict__ out)
+argmax_u8_vec4_kernel(const float4* __restrict__ T, int C, int64_t n_quads, uint32_t* __restrict__ out, uint32_t* __restrict__ copy)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n_quads) return;
     const float4* p = T + q;
     float4 best = __ldcs(p);
     uint32_t ix = 0, iy = 0, iz = 0, iw = 0;
-    // Two planes per iteration: each thread then has two 16-byte loads in flight and the GPU as a whole reads few
-    // streams at once.  Measured at 720p, C = 21 (78 MB): 16.1 us with one plane per iteration, 14.0 us with two,
-    // 17.6 us and more with three, four, seven or all (many concurrent streams spread the DRAM accesses too thin).
-#pragma unroll 2
+    // U planes per iteration: each thread has U 16-byte loads in flight.
+#pragma unroll U
     for (int c = 1; c < C; ++c) {
         float4 v = __ldcs(p + (int64_t)c * n_quads);
         if (v.x > best.x) { best.x = v.x; ix = c; }
@@ -29,13 +30,17 @@ argmax_u8_vec4_kernel(const float4* __restrict__ T, int C, int64_t n_quads, uint
         if (v.z > best.z) { best.z = v.z; iz = c; }
         if (v.w > best.w) { best.w = v.w; iw = c; }
     }
-    out[q] = ix | (iy << 8) | (iz << 16) | (iw << 24);
+    const uint32_t four = ix | (iy << 8) | (iz << 16) | (iw << 24);
+    out[q] = four;
+    if (copy) copy[q] = four;
 }
 
 // Fallback for pixel counts or pointers that do not allow 16-byte vectors.
 __global__ void __launch_bounds__(256)
-argmax_u8_scalar_kernel(const float* __restrict__ T, int C, int64_t P, uint8_t* __restrict__ out)
+argmax_u8_scalar_kernel(const float* __restrict__ T, int C, int64_t P, uint8_t* __restrict__ out, uint8_t* __restrict__ copy)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P) return;
     float best = __ldcs(T + i);
@@ -45,19 +50,24 @@ argmax_u8_scalar_kernel(const float* __restrict__ T, int C, int64_t P, uint8_t* 
         if (v > best) { best = v; idx = c; }
     }
     out[i] = (uint8_t)idx;
+    if (copy) copy[i] = (uint8_t)idx;
 }
 
-void launch_argmax_u8(const float* logits, int C, int64_t P, uint8_t* labels, cudaStream_t s)
+void launch_argmax_u8(const float* logits, int C, int64_t P, uint8_t* labels, uint8_t* copy, cudaStream_t s)
 {
     if (P <= 0) return;
-    bool vec = (P % 4 == 0) && ((uintptr_t)logits % 16 == 0) && ((uintptr_t)labels % 4 == 0);
+    bool vec = (P % 4 == 0) && ((uintptr_t)logits % 16 == 0) && ((uintptr_t)labels % 4 == 0) && ((uintptr_t)copy % 4 == 0);
     if (vec) {
         int64_t nq = P / 4;
         unsigned blocks = (unsigned)((nq + 255) / 256);
-        argmax_u8_vec4_kernel<<<blocks, 256, 0, s>>>((const float4*)logits, C, nq, (uint32_t*)labels);
+        // Measured at 720p, C = 21 (78 MB): 16.1 us with one plane per iteration, 14.0 us with two, 17.6 us and more with
+        // three, four, seven or all (many concurrent streams spread the DRAM accesses too thin).  A frame that leaves
+        // the SMs half empty has too few bytes in flight with two: 360p, C = 21 (19 MB), 6.2 us with two, 5.1 us with eight.
+        launch_early(pdl_enabled(), nq <= 148 * 1024 ? argmax_u8_vec4_kernel<8> : argmax_u8_vec4_kernel<2>, dim3(blocks), dim3(256), 0, s,
+                     (const float4*)logits, C, nq, (uint32_t*)labels, (uint32_t*)copy);
     } else {
         unsigned blocks = (unsigned)((P + 255) / 256);
-        argmax_u8_scalar_kernel<<<blocks, 256, 0, s>>>(logits, C, P, labels);
+        launch_early(pdl_enabled(), argmax_u8_scalar_kernel, dim3(blocks), dim3(256), 0, s, logits, C, P, labels, copy);
     }
 }
 

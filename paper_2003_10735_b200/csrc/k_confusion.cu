@@ -39,6 +39,8 @@ confusion_kernel(const uint8_t* __restrict__ label, const uint8_t* __restrict__ 
     const int CC = C * C;
     const int copies = MODE == 0 ? kConfWarps : (MODE == 1 ? 1 : 0);
     for (int i = threadIdx.x; i < CC * copies; i += kConfThreads) hist_all[i] = 0;
+    pdl_wait();                  // the masks, and the counters that the kernel before this one may still be clearing
+    pdl_launch_dependents();
     __syncthreads();
     unsigned int* hist = hist_all + (MODE == 0 ? (threadIdx.x >> 5) * CC : 0);
     unsigned int n_bad = 0;
@@ -161,11 +163,11 @@ void launch_confusion(const uint8_t* label, const uint8_t* pred, int64_t P, int 
     // the 48 KB a block gets without opting in
     constexpr size_t kDynLimit = 36 * 1024;
     if (one * kConfWarps <= kDynLimit)
-        confusion_kernel<0><<<blocks, kConfThreads, one * kConfWarps, s>>>(label, pred, P, C, conf, bad, fin);
+        launch_early(pdl_enabled(), confusion_kernel<0>, dim3(blocks), dim3(kConfThreads), one * kConfWarps, s, label, pred, P, C, conf, bad, fin);
     else if (one <= kDynLimit)
-        confusion_kernel<1><<<blocks, kConfThreads, one, s>>>(label, pred, P, C, conf, bad, fin);
+        launch_early(pdl_enabled(), confusion_kernel<1>, dim3(blocks), dim3(kConfThreads), one, s, label, pred, P, C, conf, bad, fin);
     else
-        confusion_kernel<2><<<blocks, kConfThreads, 0, s>>>(label, pred, P, C, conf, bad, fin);
+        launch_early(pdl_enabled(), confusion_kernel<2>, dim3(blocks), dim3(kConfThreads), 0, s, label, pred, P, C, conf, bad, fin);
 }
 
 }  // namespace st

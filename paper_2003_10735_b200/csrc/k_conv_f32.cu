@@ -78,6 +78,7 @@ conv_fwd_f32_kernel(ConvF32 a, int tiles_x)
     const int cs = warp % kCiSplit, g = warp / kCiSplit;
     const int x0 = (blockIdx.x % tiles_x) * kTileX, y0 = (blockIdx.x / tiles_x) * kFwdRows, co0 = blockIdx.y * COB;
     const PadF32 pad(a.h, a.w);
+    pdl_wait();
     // first row and vector of the tile in the padded planes
     const float* in = a.in + s * a.in_stride + (int64_t)(y0 + (KS == 3 ? 0 : kPadTop)) * pad.pitch + x0 + (KS == 3 ? 0 : kPadLeft);
     const float* Wt = a.Wt + s * a.w_stride;
@@ -146,6 +147,7 @@ conv_fwd_f32_kernel(ConvF32 a, int tiles_x)
         }
         __syncthreads();
     }
+    pdl_launch_dependents();     // late: blocks of the next kernel launched earlier crowd the SMs that finish first
     // the four quarters of the input channels, added in order: [quarter][group][row][channel][lane]
     float* red = smem_f;
 #pragma unroll
@@ -172,7 +174,7 @@ conv_fwd_f32_kernel(ConvF32 a, int tiles_x)
 }
 
 template <int KS, int CO>
-void launch_fwd(const ConvF32& a, int S, cudaStream_t s)
+void launch_fwd(const ConvF32& a, int S, bool early, cudaStream_t s)
 {
     const int tiles_x = (a.w + kTileX - 1) / kTileX, tiles_y = (a.h + kFwdRows - 1) / kFwdRows;
     const int tiles = tiles_x * tiles_y, groups = (a.Cout + CO - 1) / CO;
@@ -186,7 +188,7 @@ void launch_fwd(const ConvF32& a, int S, cudaStream_t s)
         const int64_t busiest = ((int64_t)tiles * y * S + 147) / 148 * n;
         if (busiest < least) { least = busiest; ng = n; ny = y; }
     }
-    conv_fwd_f32_kernel<KS, CO><<<dim3((unsigned)tiles, (unsigned)ny, (unsigned)S), 32 * kCiSplit * ng, fwd_smem<KS, CO>(ng), s>>>(a, tiles_x);
+    launch_chain(early, conv_fwd_f32_kernel<KS, CO>, dim3((unsigned)tiles, (unsigned)ny, (unsigned)S), dim3(32 * kCiSplit * ng), fwd_smem<KS, CO>(ng), s, a, tiles_x);
 }
 
 }  // namespace
@@ -234,6 +236,7 @@ conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
     const int g = warp / RW, rw = warp % RW;
     const int split = blockIdx.x, ci0 = (blockIdx.y % ci_tiles) * 32, co0 = (blockIdx.y / ci_tiles) * COB;
     const PadF32 pad(a.h, a.w);
+    pdl_wait();
     const float* in = a.in + s * a.in_stride + (KS == 3 ? 0 : kPadTop * pad.pitch + kPadLeft);
     const float* dout = a.dout + s * a.dout_stride + kPadTop * pad.pitch + kPadLeft;
     const int c_begin = (int)((int64_t)n_chunks * split / a.n_split), c_end = (int)((int64_t)n_chunks * (split + 1) / a.n_split);
@@ -312,6 +315,7 @@ conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
             for (int i = 0; i < RW * kTileX; ++i) bias += ds[i * pitch + lane];
         __syncthreads();
     }
+    pdl_launch_dependents();
     if (a.b_partials && ci0 == 0 && rw == 0 && lane < CO && co0 + g * CO + lane < a.Cout)
         a.b_partials[((int64_t)s * a.n_split + split) * a.Cout + co0 + g * CO + lane] = bias;
     // the rows' sums, added in order: [row warp - 1][group][channel pair, tap][lane]
@@ -375,10 +379,10 @@ WgradShape wgrad_shape_of(int Cin, int Cout, int h, int w, int ks, int S)
 }
 
 template <int KS, int CO>
-void launch_wgrad(const WgradF32& a, const WgradShape& q, int S, cudaStream_t s)
+void launch_wgrad(const WgradF32& a, const WgradShape& q, int S, bool early, cudaStream_t s)
 {
     const dim3 grid((unsigned)q.n_split, (unsigned)(q.ci_tiles * q.co_tiles), (unsigned)S);
-    conv_wgrad_f32_kernel<KS, CO><<<grid, 32 * wg_rows<KS>() * q.ng, wg_smem<KS, CO>(q.ng), s>>>(a, q.tiles_x, q.n_chunks, q.ci_tiles);
+    launch_chain(early, conv_wgrad_f32_kernel<KS, CO>, grid, dim3(32 * wg_rows<KS>() * q.ng), wg_smem<KS, CO>(q.ng), s, a, q.tiles_x, q.n_chunks, q.ci_tiles);
 }
 
 }  // namespace
@@ -395,49 +399,51 @@ cudaError_t prepare_conv_f32()
     return e;
 }
 
-static void launch_fwd_any(const ConvF32& a, int ks, int S, cudaStream_t s)
+static void launch_fwd_any(const ConvF32& a, int ks, int S, bool early, cudaStream_t s)
 {
-    if (ks == 3) launch_fwd<3, 8>(a, S, s);
-    else if (narrow(a.Cout)) launch_fwd<1, 4>(a, S, s);
-    else launch_fwd<1, 8>(a, S, s);
+    if (ks == 3) launch_fwd<3, 8>(a, S, early, s);
+    else if (narrow(a.Cout)) launch_fwd<1, 4>(a, S, early, s);
+    else launch_fwd<1, 8>(a, S, early, s);
 }
 
 void launch_conv_fwd_f32(const float* in, int Cin, int h, int w, const float* Wt, const float* b, int Cout, int ks, bool relu,
-                         float* out, bool out_padded, int S, int64_t w_stride, cudaStream_t s)
+                         float* out, bool out_padded, int S, int64_t w_stride, bool early, cudaStream_t s)
 {
     const PadF32 pad(h, w);
     const ConvF32 a = {in, Wt, b, nullptr, out_padded ? out + pad.origin : out, Cin, Cout, h, w, relu ? 1 : 0, 0,
                        out_padded ? pad.pitch : w, out_padded ? pad.plane : (int64_t)h * w,
                        Cin * pad.plane, w_stride, w_stride, Cout * (out_padded ? pad.plane : (int64_t)h * w)};
-    launch_fwd_any(a, ks, S, s);
+    launch_fwd_any(a, ks, S, early, s);
 }
 
 void launch_conv1x1_dgrad_relu_f32(const float* W2, const float* dz, const float* Hact, int C, int Ch, int h, int w, float* dH, int S,
-                                   int64_t w_stride, cudaStream_t s)
+                                   int64_t w_stride, bool early, cudaStream_t s)
 {
     const PadF32 pad(h, w);
     const ConvF32 a = {dz, W2, nullptr, Hact + pad.origin, dH + pad.origin, C, Ch, h, w, 0, 1, pad.pitch, pad.plane,
                        C * pad.plane, w_stride, 0, Ch * pad.plane};
-    launch_fwd_any(a, 1, S, s);
+    launch_fwd_any(a, 1, S, early, s);
 }
 
 int conv_wgrad_f32_splits(int Cin, int Cout, int h, int w, int ks, int S) { return wgrad_shape_of(Cin, Cout, h, w, ks, S).n_split; }
 
 void launch_conv_wgrad_f32(const float* in, const float* dout, int Cin, int Cout, int h, int w, int ks, float* partials,
-                           float* b_partials, int S, cudaStream_t s)
+                           float* b_partials, int S, bool early, cudaStream_t s)
 {
     const WgradShape q = wgrad_shape_of(Cin, Cout, h, w, ks, S);
     const PadF32 pad(h, w);
     const WgradF32 a = {in, dout, partials, b_partials, Cin, Cout, h, w, q.n_split, Cin * pad.plane, Cout * pad.plane};
-    if (ks == 3) launch_wgrad<3, 8>(a, q, S, s);
-    else if (narrow(Cout)) launch_wgrad<1, 4>(a, q, S, s);
-    else launch_wgrad<1, 16>(a, q, S, s);
+    if (ks == 3) launch_wgrad<3, 8>(a, q, S, early, s);
+    else if (narrow(Cout)) launch_wgrad<1, 4>(a, q, S, early, s);
+    else launch_wgrad<1, 16>(a, q, S, early, s);
 }
 
 // between plain planes [C][h][w] and padded ones (interior only)
 __global__ void __launch_bounds__(256)
 pad_planes_kernel(const float* __restrict__ src, float* __restrict__ dst, int h, int w, int64_t src_plane, int src_pitch, int64_t dst_plane, int dst_pitch)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     const int x = blockIdx.x * 32 + (threadIdx.x & 31), c = blockIdx.z;
     for (int y = blockIdx.y * 32 + (threadIdx.x >> 5), n = 0; n < 4 && y < h; ++n, y += 8)
         if (x < w) dst[c * dst_plane + (int64_t)y * dst_pitch + x] = __ldg(src + c * src_plane + (int64_t)y * src_pitch + x);
@@ -446,14 +452,14 @@ pad_planes_kernel(const float* __restrict__ src, float* __restrict__ dst, int h,
 void launch_pad_planes(const float* plain, float* padded, int C, int h, int w, cudaStream_t s)
 {
     const PadF32 pad(h, w);
-    pad_planes_kernel<<<dim3((unsigned)((w + 31) / 32), (unsigned)((h + 31) / 32), (unsigned)C), 256, 0, s>>>(
+    launch_early(pdl_enabled(), pad_planes_kernel, dim3((unsigned)((w + 31) / 32), (unsigned)((h + 31) / 32), (unsigned)C), dim3(256), 0, s,
         plain, padded + pad.origin, h, w, (int64_t)h * w, w, pad.plane, pad.pitch);
 }
 
 void launch_unpad_planes(const float* padded, float* plain, int C, int h, int w, cudaStream_t s)
 {
     const PadF32 pad(h, w);
-    pad_planes_kernel<<<dim3((unsigned)((w + 31) / 32), (unsigned)((h + 31) / 32), (unsigned)C), 256, 0, s>>>(
+    launch_early(pdl_enabled(), pad_planes_kernel, dim3((unsigned)((w + 31) / 32), (unsigned)((h + 31) / 32), (unsigned)C), dim3(256), 0, s,
         padded + pad.origin, plain, h, w, pad.plane, pad.pitch, (int64_t)h * w, w);
 }
 

@@ -18,6 +18,8 @@ constexpr int kFeatGroup = 16;
 __global__ void __launch_bounds__(256)
 feat_to_bf16_nhwc_kernel(const float* __restrict__ in, int Cin, int64_t p, bf16* __restrict__ out)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     const int64_t pix = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int c0 = blockIdx.y * kFeatGroup;
     if (pix >= p) return;
@@ -41,7 +43,7 @@ feat_to_bf16_nhwc_kernel(const float* __restrict__ in, int Cin, int64_t p, bf16*
 void launch_feat_to_bf16_nhwc(const float* feat_chw, int Cin, int64_t p, bf16* out, cudaStream_t s)
 {
     dim3 grid((unsigned)((p + 255) / 256), (unsigned)((Cin + kFeatGroup - 1) / kFeatGroup));
-    feat_to_bf16_nhwc_kernel<<<grid, 256, 0, s>>>(feat_chw, Cin, p, out);
+    launch_early(pdl_enabled(), feat_to_bf16_nhwc_kernel, grid, dim3(256), 0, s, feat_chw, Cin, p, out);
 }
 
 // Verification helper: bf16 [p][C] -> fp32 [C][p].  Not on the hot path.

@@ -50,6 +50,7 @@ student_eval_kernel(StudentMaskArgs a, const __grid_constant__ CUtensorMap x_map
     const int ry_top = min(max(i, 0), h - 1) - (y0 - 1), ry_bot = min(max(i + 1, 0), h - 1) - (y0 - 1);
     const int rx_l = min(max(n, 0), w - 1) - (x0 - 1), rx_r = min(max(n + 1, 0), w - 1) - (x0 - 1);
 
+    if (!a.settled) pdl_wait();                            // a kernel that may still be running writes the features or the labels
     uint32_t labw[4] = {0, 0, 0, 0};                       // labels of the lane's 16 pixels (two aligned 16-bit loads per row)
     if (CONF) {
 #pragma unroll
@@ -65,7 +66,7 @@ student_eval_kernel(StudentMaskArgs a, const __grid_constant__ CUtensorMap x_map
     }
 
     fused::Args fa;
-    fa.kblocks = a.kblocks; fa.x_early = 1;                // nothing that can still be running writes the features
+    fa.kblocks = a.kblocks; fa.x_early = 1;                // features and labels are there, or have just been waited for
     fa.skip = nullptr; fa.err = a.err; fa.bias = a.bias; fa.z_out = nullptr;
     fa.C = C; fa.h = h; fa.w = w;
     fa.spin_limit = tc::kSpinLimit; fa.stall_bytes = 0;
@@ -73,6 +74,7 @@ student_eval_kernel(StudentMaskArgs a, const __grid_constant__ CUtensorMap x_map
         if (CONF) for (int e = tid; e < C * C; e += kThreads) hist[e] = 0;
     };
     const fused::Tile tile = fused::logit_tile<CB>(fa, &x_map, &w_map, fsh, zt, a.stream, x0, y0, after_mma);
+    pdl_launch_dependents();
     if (!tile.ok) return;
     const uint32_t tmem = tile.tmem;
 
@@ -176,9 +178,9 @@ cudaError_t launch_cb(const StudentMaskArgs& a, cudaStream_t s)
     const dim3 grid((unsigned)((a.w + kOwnCols - 1) / kOwnCols), (unsigned)((a.h + kOwnRows - 1) / kOwnRows));
     const size_t smem = eval_smem_bytes<CB>(a.C);
     const bool conf = a.labels != nullptr;
-    if (!conf) student_eval_kernel<CB, true, false><<<grid, kThreads, smem, s>>>(a, *a.x_map, *a.w_map);
-    else if (a.mask) student_eval_kernel<CB, true, true><<<grid, kThreads, smem, s>>>(a, *a.x_map, *a.w_map);
-    else student_eval_kernel<CB, false, true><<<grid, kThreads, smem, s>>>(a, *a.x_map, *a.w_map);
+    if (!conf) launch_early(pdl_enabled(), student_eval_kernel<CB, true, false>, grid, dim3(kThreads), smem, s, a, *a.x_map, *a.w_map);
+    else if (a.mask) launch_early(pdl_enabled(), student_eval_kernel<CB, true, true>, grid, dim3(kThreads), smem, s, a, *a.x_map, *a.w_map);
+    else launch_early(pdl_enabled(), student_eval_kernel<CB, false, true>, grid, dim3(kThreads), smem, s, a, *a.x_map, *a.w_map);
     return cudaGetLastError();
 }
 

@@ -55,6 +55,8 @@ student_mask_kernel(StudentMaskArgs a, int chunk)
     const bool v01 = cell_ok && X0 >= 0 && X0 + 1 < W, v23 = cell_ok && X0 + 2 >= 0 && X0 + 3 < W;
 
     if (CONF) for (int e = tid; e < C * C; e += SM_THREADS) hist[e] = 0;
+    pdl_wait();
+    pdl_launch_dependents();
     // labels of the lane's 16 pixels, fetched before the sweep over the classes (two aligned 16-bit loads per row)
     uint32_t labw[SM_RW] = {};
     if (CONF) {
@@ -202,9 +204,9 @@ void launch_student_mask(const StudentMaskArgs& a, cudaStream_t s)
     const bool conf = a.labels != nullptr;
     const size_t smem = mask_smem(a.C, conf, &chunk);
     dim3 grid((unsigned)((a.w + 1 + 31) / 32), (unsigned)((a.h + 1 + SM_WARPS - 1) / SM_WARPS));
-    if (!conf) student_mask_kernel<true, false><<<grid, SM_THREADS, smem, s>>>(a, chunk);
-    else if (a.mask) student_mask_kernel<true, true><<<grid, SM_THREADS, smem, s>>>(a, chunk);
-    else student_mask_kernel<false, true><<<grid, SM_THREADS, smem, s>>>(a, chunk);
+    if (!conf) launch_early(pdl_enabled(), student_mask_kernel<true, false>, grid, dim3(SM_THREADS), smem, s, a, chunk);
+    else if (a.mask) launch_early(pdl_enabled(), student_mask_kernel<true, true>, grid, dim3(SM_THREADS), smem, s, a, chunk);
+    else launch_early(pdl_enabled(), student_mask_kernel<false, true>, grid, dim3(SM_THREADS), smem, s, a, chunk);
 }
 
 }  // namespace st

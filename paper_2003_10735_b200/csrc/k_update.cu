@@ -245,8 +245,11 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int64_t range_begin)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (lane == 0) {
-            if (a.loss_slot >= 0 && a.loss_slot < kMaxSteps)
-                a.loss_buf[(int64_t)s * kMaxSteps + a.loss_slot] = (float)(t * a.inv_P);
+            if (a.loss_slot >= 0 && a.loss_slot < kMaxSteps) {
+                const float mean = (float)(t * a.inv_P);
+                a.loss_buf[(int64_t)s * kMaxSteps + a.loss_slot] = mean;
+                if (a.loss_out) a.loss_out[(int64_t)s * a.loss_pitch + a.loss_slot] = mean;
+            }
         }
     }
 }
@@ -350,33 +353,18 @@ int launch_sgd_update(const UpdateArgs& a, cudaStream_t s)
     return a.adam ? launch_sgd_update_t<true>(a, s) : launch_sgd_update_t<false>(a, s);
 }
 
-__global__ void step_tick_kernel(long long* step_base, int S, int add, const int* add_per_stream)
+__global__ void step_tick_kernel(long long* step_base, int S, int add)
 {
     const int s = threadIdx.x;
-    if (s < S) step_base[s] += add_per_stream ? add_per_stream[s] : add;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (s < S) step_base[s] += add;
 }
 
-void launch_step_tick(long long* step_base, int S, int add, const int* add_per_stream, cudaStream_t s)
+void launch_step_tick(long long* step_base, int S, int add, cudaStream_t s)
 {
     for (int s0 = 0; s0 < S; s0 += 256)
-        step_tick_kernel<<<1, 256, 0, s>>>(step_base + s0, S - s0 < 256 ? S - s0 : 256, add, add_per_stream ? add_per_stream + s0 : nullptr);
-}
-
-__global__ void refresh_shadow_kernel(UpdateArgs a)
-{
-    const int s = blockIdx.y;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n_params) return;
-    for (int L = 0; L < a.n_layers; ++L) {
-        const LayerUpdate& ly = a.layer[L];
-        const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
-        if (i >= ly.w_off && i < ly.w_off + nw) write_shadows(ly, s, i - ly.w_off, a.theta[(int64_t)s * a.n_params + i]);
-    }
-}
-
-void launch_refresh_shadow(const UpdateArgs& a, cudaStream_t s)
-{
-    refresh_shadow_kernel<<<dim3((unsigned)((a.n_params + 255) / 256), (unsigned)a.S), 256, 0, s>>>(a);
+        launch_early(pdl_enabled(), step_tick_kernel, dim3(1), dim3(256), 0, s, step_base + s0, S - s0 < 256 ? S - s0 : 256, add);
 }
 
 __global__ void __launch_bounds__(256) miou_kernel(const unsigned long long* __restrict__ conf, int C, double* out)
@@ -387,18 +375,24 @@ __global__ void __launch_bounds__(256) miou_kernel(const unsigned long long* __r
     if (threadIdx.x == 0) *out = m;
 }
 
-// ---- Algorithm 1, the lines after "metric <- ComputeMetric(prediction, label)" ------------------------
-// One launch per prediction; blockIdx.y = stream.  Every block computes the stream's mean IoU from the confusion
-// matrix of the prediction (same arithmetic as miou_kernel), all blocks together copy the parameters into
-// best_student if the metric is a new best, and block 0 records the decisions:
-//   prediction 0 (the incoming student):  best_metric <- metric; the loop is entered iff best_metric < THRESHOLD
-//   prediction i > 0 (after i updates):   if metric > best_metric: best_metric, best_student <- metric, student;
-//                                         if metric > THRESHOLD: break;  the loop also ends at i = MAX_UPDATES.
-__global__ void __launch_bounds__(256) train_commit_kernel(const float* __restrict__ best_theta, float* __restrict__ theta, int64_t n_params,
-                                                           int64_t begin)
+// End of Train (Algorithm 1): student <- best_student for the trained parameters, with the bf16 copies the GEMMs read; Adam's
+// step count moves on by the steps taken.
+__global__ void __launch_bounds__(256) train_commit_kernel(UpdateArgs a, const float* __restrict__ best_theta, const int* __restrict__ n_updates)
 {
-    const int64_t base = (int64_t)blockIdx.y * n_params;
-    for (int64_t e = begin + (int64_t)blockIdx.x * 256 + threadIdx.x; e < n_params; e += (int64_t)gridDim.x * 256) theta[base + e] = best_theta[base + e];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int s = blockIdx.y;
+    const int64_t base = (int64_t)s * a.n_params;
+    for (int64_t i = a.param_begin + (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.n_params; i += (int64_t)gridDim.x * 256) {
+        const float t = best_theta[base + i];
+        a.theta[base + i] = t;
+        for (int L = 0; L < a.n_layers; ++L) {
+            const LayerUpdate& ly = a.layer[L];
+            const int64_t e = i - ly.w_off;
+            if (e >= 0 && e < (int64_t)ly.cout * ly.cin * ly.taps) write_shadows(ly, s, e, t);
+        }
+    }
+    if (a.adam && blockIdx.x == 0 && threadIdx.x == 0) a.step_base[s] += n_updates[s];
 }
 
 void launch_miou(const unsigned long long* conf, int C, double* out, cudaStream_t s)
@@ -412,44 +406,96 @@ static unsigned copy_blocks(int64_t n_params)
     return (unsigned)(b < 1 ? 1 : (b > 592 ? 592 : b));
 }
 
-void launch_train_commit(const TrainCtl& t, float* theta, cudaStream_t s)
+void launch_train_commit(const UpdateArgs& a, const float* best_theta, const int* n_updates, cudaStream_t s)
 {
-    train_commit_kernel<<<dim3(copy_blocks(t.n_params - t.param_begin), (unsigned)t.S), 256, 0, s>>>(t.best_theta, theta, t.n_params, t.param_begin);
+    launch_early(pdl_enabled(), train_commit_kernel, dim3(copy_blocks(a.n_params - a.param_begin), (unsigned)a.S), dim3(256), 0, s, a, best_theta, n_updates);
+}
+
+__global__ void train_results_kernel(TrainCtl t, const float* __restrict__ loss_buf, TrainResults out)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    const int s = blockIdx.x, i = threadIdx.x, n = t.max_updates + 1;
+    if (i == 0 && out.n_updates) out.n_updates[s] = t.n_updates[s];
+    if (i == 0 && out.best) out.best[s] = t.best[(int64_t)s * kCtlPitch + n];
+    if (i < n && out.metric) out.metric[(int64_t)s * n + i] = t.metric[(int64_t)s * kCtlPitch + i];
+    if (i < n && out.loss) out.loss[(int64_t)s * n + i] = loss_buf[(int64_t)s * kMaxSteps + i];
+}
+
+void launch_train_results(const TrainCtl& t, const float* loss_buf, const TrainResults& out, cudaStream_t s)
+{
+    launch_early(pdl_enabled(), train_results_kernel, dim3((unsigned)t.S), dim3(kMaxSteps), 0, s, t, loss_buf, out);
 }
 
 // ---- pack / unpack ---------------------------------------------------------------------------------
+// A block moves 256 (output, input) channel pairs of a layer with all their taps: the packed side, [pair][tap], is one contiguous
+// piece, the internal side one piece per tap; a 3x3 layer's values change places in shared memory.  (A thread per packed
+// value reads or writes with a stride of a whole tap plane: 11 us for 2.4 MB at 256 -> 256 channels, 4 us this way.)  The last block
+// of a buffer takes the biases.  Unpacking also writes the bf16 copies that the GEMMs read.
+// The packed buffer may be pinned host memory: it is then read or written over the bus by the kernel itself.
+constexpr int kPackPairs = 256;
 template <bool TO_PACKED>
-__global__ void pack_kernel(const float* __restrict__ src, float* __restrict__ dst, PackLayout L, int64_t begin, int64_t count)
+__global__ void __launch_bounds__(kPackPairs)
+pack_kernel(const float* __restrict__ src, float* __restrict__ dst, PackLayout L, int first, int64_t begin, int64_t count, UpdateArgs u, int s0)
 {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // index in the packed buffer
-    if (q >= count) return;
-    const int64_t i = begin + q;                                         // the parameter's index in packed order
-    const int64_t base = (int64_t)blockIdx.y * L.n_params;
-    int64_t j = i;                                                       // its index in internal order
-    for (int k = 0; k < L.n_layers; ++k) {
-        const int64_t nw = (int64_t)L.cout[k] * L.cin[k] * L.taps[k];
-        if (i >= L.w_off[k] && i < L.w_off[k] + nw) {
-            const int64_t e = i - L.w_off[k];
-            const int tap = (int)(e % L.taps[k]);
-            const int64_t r = e / L.taps[k];
-            const int ci = (int)(r % L.cin[k]), co = (int)(r / L.cin[k]);
-            j = L.w_off[k] + ((int64_t)tap * L.cout[k] + co) * L.cin[k] + ci;
+    __shared__ float sh[kPackPairs * 9];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int s = blockIdx.y, tid = threadIdx.x;
+    const float* from = src + (int64_t)s * (TO_PACKED ? L.n_params : count);
+    float* to = dst + (int64_t)s * (TO_PACKED ? count : L.n_params);
+    int blk = blockIdx.x;
+    for (int k = first; k < L.n_layers; ++k) {
+        const int64_t pairs = (int64_t)L.cout[k] * L.cin[k];
+        const int blocks = (int)((pairs + kPackPairs - 1) / kPackPairs), taps = L.taps[k];
+        if (blk >= blocks) { blk -= blocks; continue; }
+        const int64_t p0 = (int64_t)blk * kPackPairs, w = L.w_off[k], packed = w - begin + p0 * taps;
+        const int n = (int)(pairs - p0 < kPackPairs ? pairs - p0 : kPackPairs);
+        if (TO_PACKED) {
+            if (tid < n)
+                for (int t = 0; t < taps; ++t) sh[tid * taps + t] = from[w + t * pairs + p0 + tid];
+            __syncthreads();
+            for (int e = tid; e < n * taps; e += kPackPairs) to[packed + e] = sh[e];
+        } else {
+            for (int e = tid; e < n * taps; e += kPackPairs) sh[e] = from[packed + e];
+            __syncthreads();
+            if (tid < n)
+                for (int t = 0; t < taps; ++t) {
+                    const int64_t e = t * pairs + p0 + tid;
+                    const float v = sh[tid * taps + t];
+                    to[w + e] = v;
+                    if (u.n_layers) write_shadows(u.layer[k - first], s0 + s, e, v);
+                }
         }
+        return;
     }
-    if (TO_PACKED) dst[(int64_t)blockIdx.y * count + q] = src[base + j];
-    else dst[base + j] = src[(int64_t)blockIdx.y * count + q];
+    for (int k = first; k < L.n_layers; ++k)
+        for (int i = tid; i < L.cout[k]; i += kPackPairs) {
+            const int64_t b = L.b_off[k] + i;
+            if (TO_PACKED) to[b - begin] = from[b];
+            else to[b] = from[b - begin];
+        }
 }
 
-void launch_pack(const float* internal, float* packed, const PackLayout& L, int64_t begin, int64_t count, int n_bufs, cudaStream_t s)
+static dim3 pack_grid(const PackLayout& L, int first, int n_bufs)
 {
-    if (count <= 0) return;
-    pack_kernel<true><<<dim3((unsigned)((count + 255) / 256), (unsigned)n_bufs), 256, 0, s>>>(internal, packed, L, begin, count);
+    int64_t blocks = 1;
+    for (int k = first; k < L.n_layers; ++k) blocks += ((int64_t)L.cout[k] * L.cin[k] + kPackPairs - 1) / kPackPairs;
+    return dim3((unsigned)blocks, (unsigned)n_bufs);
 }
 
-void launch_unpack(const float* packed, float* internal, const PackLayout& L, int64_t begin, int64_t count, int n_bufs, cudaStream_t s)
+void launch_pack(const float* internal, float* packed, const PackLayout& L, int first, int n_bufs, cudaStream_t s)
 {
-    if (count <= 0) return;
-    pack_kernel<false><<<dim3((unsigned)((count + 255) / 256), (unsigned)n_bufs), 256, 0, s>>>(packed, internal, L, begin, count);
+    const int64_t begin = L.w_off[first];
+    UpdateArgs none;
+    none.n_layers = 0;
+    launch_early(pdl_enabled(), pack_kernel<true>, pack_grid(L, first, n_bufs), dim3(kPackPairs), 0, s, internal, packed, L, first, begin, L.n_params - begin, none, 0);
+}
+
+void launch_unpack(const float* packed, float* internal, const PackLayout& L, int first, int n_bufs, const UpdateArgs& u, int s0, cudaStream_t s)
+{
+    const int64_t begin = L.w_off[first];
+    launch_early(pdl_enabled(), pack_kernel<false>, pack_grid(L, first, n_bufs), dim3(kPackPairs), 0, s, packed, internal, L, first, begin, L.n_params - begin, u, s0);
 }
 
 }  // namespace st

@@ -75,7 +75,6 @@ upsample_ce_many_kernel(UpsampleCeArgs a)
     const uint8_t* labels = a.labels + (int64_t)s * H * W;
     const int tid = threadIdx.x, l = tid & 31, warp = tid >> 5, wi = warp % NR, g = warp / NR;
     pdl_wait();
-    pdl_launch_dependents();
     if (a.skip && a.skip[(int64_t)s * a.skip_stride]) return;     // this stream's training loop has ended (block-uniform)
 
     const int i = y0 - 1 + wi, n = x0 - 1 + l;                    // cell row, node column
@@ -369,6 +368,7 @@ upsample_ce_many_kernel(UpsampleCeArgs a)
         }
         __syncthreads();
     }
+    pdl_launch_dependents();
     for (int c = tid; c < C; c += NT) {
         float t = 0.f;
         for (int k = 1; k < NR; ++k) t += bsum[c * NR + k];

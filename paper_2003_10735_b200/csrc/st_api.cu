@@ -12,6 +12,7 @@
 #include <tuple>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using namespace st;
@@ -23,8 +24,10 @@ thread_local std::string g_init_error;
 // threshold whose bit pattern is `thr` (train = true).
 struct GraphKey {
     int n_steps; bool conf; bool train; uint64_t thr;
-    bool operator<(const GraphKey& o) const { return std::tie(n_steps, conf, train, thr) < std::tie(o.n_steps, o.conf, o.train, o.thr); }
+    float* loss;       // nullptr, or the caller's device buffer that the updates write the losses to as well
+    bool operator<(const GraphKey& o) const { return std::tie(n_steps, conf, train, thr, loss) < std::tie(o.n_steps, o.conf, o.train, o.thr, o.loss); }
 };
+constexpr size_t kMaxGraphs = 32;       // replayable graphs kept per context
 }  // namespace
 
 struct st_ctx {
@@ -74,6 +77,8 @@ struct st_ctx {
     int fused_fwd = 0;          //   (one-layer head with bf16 GEMMs; ST_FUSED_FORWARD=0 switches it off)
     int test_stall_fused = 0;   // test of the give-up path inside that kernel (environment ST_TEST_STALL_FUSED=1 at context creation)
     float* loss_buf = nullptr;              // [S][kMaxSteps]
+    float* loss_seen = nullptr;             // the device buffer that the last st_distill_step delivered its losses to
+    float* loss_direct = nullptr; int loss_pitch = 0;   // during a call: where the updates write the losses as well
     unsigned long long* conf_buf = nullptr; // [S][kMaxSteps][C][C], allocated on first use
     // Train (Algorithm 1), allocated on first use
     float* best_theta = nullptr;            // [S][n_params] best_student
@@ -98,6 +103,7 @@ struct st_ctx {
     struct Prefetch { float* feat = nullptr; float* logits = nullptr; cudaEvent_t copied = nullptr, consumed = nullptr; bool pending = false, used_once = false; };
     std::vector<Prefetch> prefetch;
     bool z_current = false;                 // z holds the forward of the current parameters and features of every stream
+    bool settled = false;                   // a step loop has run since the features and labels were last written: nothing in flight writes them
     bool z_unkept = false;                  // the last call multiplied its logits inside the loss kernel and kept none of them
     TcPlan* plan = nullptr;
     struct StepGraph { cudaGraphExec_t exec; int64_t n_launches; };
@@ -147,12 +153,19 @@ cudaError_t dev_alloc(st_ctx* ctx, T** ptr, size_t count, bool zero = true)
     return cudaSuccess;
 }
 
-bool is_device_ptr(const void* q)
+// What a caller's pointer is: device memory, pinned host memory that kernels can reach (`dev` is its device address), or
+// ordinary host memory.
+enum class Where { device, pinned, host };
+Where locate(const void* q, const void** dev = nullptr)
 {
     cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, q) != cudaSuccess) { cudaGetLastError(); return false; }
-    return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+    if (dev) *dev = q;
+    if (cudaPointerGetAttributes(&at, q) != cudaSuccess) { cudaGetLastError(); return Where::host; }
+    if (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) return Where::device;
+    if (at.type == cudaMemoryTypeHost && at.devicePointer) { if (dev) *dev = at.devicePointer; return Where::pinned; }
+    return Where::host;
 }
+bool is_device_ptr(const void* q) { return locate(q) == Where::device; }
 
 st_status ensure_staging(st_ctx* ctx, size_t bytes)
 {
@@ -176,6 +189,14 @@ st_status to_device(st_ctx* ctx, const void* src, size_t bytes, const void** dev
     ST_CUDA(ctx, cudaMemcpyAsync(ctx->staging, src, bytes, cudaMemcpyHostToDevice, ctx->stream));
     *dev = ctx->staging;
     return ST_OK;
+}
+
+// The same for a buffer of a student's size: pinned host memory is read by the kernel itself (21 KB over the bus inside an
+// unpacking kernel: predict at 720p 46 -> 38 us; the copy engine's start and its hand-over to the kernel cost more than the bytes).
+st_status small_to_device(st_ctx* ctx, const void* src, size_t bytes, const void** dev)
+{
+    if (locate(src, dev) != Where::host) return ST_OK;
+    return to_device(ctx, src, bytes, dev);
 }
 
 st_status check_stream_index(st_ctx* ctx, int32_t s)
@@ -232,6 +253,7 @@ UpdateArgs make_update_args(st_ctx* c, int slot, const int* skip = nullptr, int6
     }
     u.loss_part = c->loss_part; u.n_loss_part = c->n_k3_blocks;
     u.loss_buf = c->loss_buf; u.loss_slot = slot;
+    u.loss_out = c->loss_direct; u.loss_pitch = c->loss_pitch;
     u.inv_P = 1.0 / (double)c->P;
     u.skip = skip; u.skip_stride = skip_stride;
     u.adam = c->adam ? 1 : 0; u.vel2 = c->vel2; u.step_base = c->step_base;
@@ -266,15 +288,15 @@ st_status enqueue_forward(st_ctx* c, StageTimer* t = nullptr, const int* skip = 
         c->launches += tc_forward(c->plan, s, t, skip, skip_stride, after_update, c->first_trained < c->n_blocks ? c->first_trained : c->n_blocks);
     } else if (c->Ch == 0) {
         ST_REPEAT(t) launch_conv_fwd_f32(c->x_f32, c->Cin, c->h, c->w, c->theta + c->layout.w_off[0], c->theta + c->layout.b_off[0],
-                                         c->C, 1, false, c->z, false, c->S, c->n_params, s);
+                                         c->C, 1, false, c->z, false, c->S, c->n_params, c->chain_early, s);
         if (t) t->mark("conv1x1_fwd_f32", s, st_repeats(t));
         c->launches += st_repeats(t);
     } else {
         ST_REPEAT(t) launch_conv_fwd_f32(c->x_f32, c->Cin, c->h, c->w, c->theta + c->layout.w_off[0], c->theta + c->layout.b_off[0],
-                                         c->Ch, 3, true, c->hid_f32, true, c->S, c->n_params, s);
+                                         c->Ch, 3, true, c->hid_f32, true, c->S, c->n_params, c->chain_early, s);
         if (t) t->mark("conv3x3_fwd_f32", s, st_repeats(t));
         ST_REPEAT(t) launch_conv_fwd_f32(c->hid_f32, c->Ch, c->h, c->w, c->theta + c->layout.w_off[1], c->theta + c->layout.b_off[1],
-                                         c->C, 1, false, c->z, false, c->S, c->n_params, s);
+                                         c->C, 1, false, c->z, false, c->S, c->n_params, c->chain_early, s);
         if (t) t->mark("conv1x1_fwd_f32", s, st_repeats(t));
         c->launches += 2 * st_repeats(t);
     }
@@ -331,6 +353,8 @@ st_status enqueue_loss(st_ctx* c, unsigned long long* conf, StageTimer* t = null
         k3.theta = c->theta; k3.n_params = c->n_params; k3.b_off = c->layout.b_off[c->layout.n_layers - 1];
         k3.z_out = keep_logits ? c->z : nullptr;         // logits that the next iteration overwrites unread stay on the chip
         k3.test_stall = c->test_stall_fused;
+        // the first iteration's predecessor may have written the labels and the features, which are fetched before the wait
+        if (!after_update) k3.chain_early = 0;
     }
     ST_REPEAT(t) launch_upsample_ce(k3, &c->k3_map, s, &c->fx_map, &c->fw_map);
     if (t) t->mark(k3.fused ? "fwd1x1_upsample_ce" : "upsample_ce", s, st_repeats(t));
@@ -345,16 +369,16 @@ st_status enqueue_backward(st_ctx* c, StageTimer* t = nullptr, const int* skip =
     if (c->bf16_mode) {
         c->launches += tc_backward(c->plan, s, t, skip, skip_stride, ctl);
     } else if (c->Ch == 0) {
-        ST_REPEAT(t) launch_conv_wgrad_f32(c->x_f32, c->dz, c->Cin, c->C, c->h, c->w, 1, c->w2_partials, nullptr, c->S, s);
+        ST_REPEAT(t) launch_conv_wgrad_f32(c->x_f32, c->dz, c->Cin, c->C, c->h, c->w, 1, c->w2_partials, nullptr, c->S, c->chain_early, s);
         if (t) t->mark("conv1x1_wgrad_f32", s, st_repeats(t));
         c->launches += st_repeats(t);
     } else {
-        ST_REPEAT(t) launch_conv_wgrad_f32(c->hid_f32, c->dz, c->Ch, c->C, c->h, c->w, 1, c->w2_partials, nullptr, c->S, s);
+        ST_REPEAT(t) launch_conv_wgrad_f32(c->hid_f32, c->dz, c->Ch, c->C, c->h, c->w, 1, c->w2_partials, nullptr, c->S, c->chain_early, s);
         if (t) t->mark("conv1x1_wgrad_f32", s, st_repeats(t));
         ST_REPEAT(t) launch_conv1x1_dgrad_relu_f32(c->theta + c->layout.w_off[1], c->dz, c->hid_f32, c->C, c->Ch, c->h, c->w,
-                                                   c->dhid_f32, c->S, c->n_params, s);
+                                                   c->dhid_f32, c->S, c->n_params, c->chain_early, s);
         if (t) t->mark("conv1x1_dgrad_f32", s, st_repeats(t));
-        ST_REPEAT(t) launch_conv_wgrad_f32(c->x_f32, c->dhid_f32, c->Cin, c->Ch, c->h, c->w, 3, c->blk[0].w_partials, c->blk[0].b_partials, c->S, s);
+        ST_REPEAT(t) launch_conv_wgrad_f32(c->x_f32, c->dhid_f32, c->Cin, c->Ch, c->h, c->w, 3, c->blk[0].w_partials, c->blk[0].b_partials, c->S, c->chain_early, s);
         if (t) t->mark("conv3x3_wgrad_f32", s, st_repeats(t));
         c->launches += 3 * st_repeats(t);
     }
@@ -571,7 +595,8 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     if (const char* e = getenv("ST_NO_GRAPH")) if (e[0] == '1') c->use_graphs = false;
     // Programmatic dependent launch along the step's chain: with the one-layer head every kernel has something to do
     // before its predecessor's results are needed (label fetch, feature tiles) and the step is 2 us shorter; the
-    // two-layer head's kernels fill the SMs to the end and gain nothing (measured: 1 us slower).  ST_PDL=0 / 1 force it.
+    // two-layer head's kernels fill the SMs to the end and gain nothing (measured: 1 us slower; with fp32 convolutions 10 us
+    // slower: waiting blocks crowd the SMs that finish first).  ST_PDL=0 / 1 force it.
     c->chain_early = pdl_enabled() && c->Ch == 0;
     if (const char* e = getenv("ST_PDL")) if (e[0] == '1') c->chain_early = true;
 
@@ -665,7 +690,12 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     // parameters: packed order -> internal order (the momentum buffer serves as scratch, then is zeroed)
     const size_t pbytes = (size_t)S * c->n_params * sizeof(float);
     e = cudaMemcpyAsync(c->vel, init_params, pbytes, cudaMemcpyDefault, c->stream);
-    if (e == cudaSuccess) { launch_unpack(c->vel, c->theta, c->layout, 0, c->n_params, S, c->stream); e = cudaGetLastError(); }
+    if (e == cudaSuccess) {
+        UpdateArgs u = make_update_args(c, -1, nullptr, 0, true);
+        if (!c->bf16_mode) u.n_layers = 0;
+        launch_unpack(c->vel, c->theta, c->layout, 0, S, u, 0, c->stream);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(c->vel, 0, pbytes, c->stream);
     if (e == cudaSuccess && c->bf16_mode) {
         TcBuffers b;
@@ -694,8 +724,6 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             st_destroy(c);
             return code;
         }
-        launch_refresh_shadow(make_update_args(c, -1, nullptr, 0, true), c->stream);
-        e = cudaGetLastError();
         const char* off = getenv("ST_FUSED_FORWARD");
         if (n_blocks == 0 && !(off && off[0] == '0') && fused_forward_supported(c->C, c->h, c->w, c->Cin)) {
             const uint64_t ci = (uint64_t)c->Cin;
@@ -714,7 +742,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
         st_destroy(c);
         return code;
     }
-    c->launches += 2;
+    c->launches += 1;
     *out = c;
     return ST_OK;
 }
@@ -736,6 +764,7 @@ st_status st_set_frozen_features(st_ctx* ctx, int32_t stream, const float* feat_
     st = check_launch(ctx, "feature cache");
     if (st != ST_OK) return st;
     ctx->has_feat[stream] = 1;
+    ctx->settled = false;
     ctx->z_current = false;
     ctx->prefix_current = false;
     return ST_OK;
@@ -771,12 +800,15 @@ st_status st_teacher_labels(st_ctx* ctx, int32_t stream, const float* logits_chw
     st = to_device(ctx, logits_chw, (size_t)ctx->C * ctx->P * sizeof(float), &src);
     if (st != ST_OK) return st;
     uint8_t* dst = ctx->labels + (int64_t)stream * ctx->P;
-    launch_argmax_u8((const float*)src, ctx->C, ctx->P, dst, ctx->stream);
+    // the caller's device map is written by the same kernel; any other destination gets a copy
+    const bool direct = labels_out && ((uintptr_t)labels_out & 3u) == 0 && is_device_ptr(labels_out);
+    launch_argmax_u8((const float*)src, ctx->C, ctx->P, dst, direct ? labels_out : nullptr, ctx->stream);
     ctx->launches += 1;
     st = check_launch(ctx, "teacher argmax");
     if (st != ST_OK) return st;
-    if (labels_out) ST_CUDA(ctx, cudaMemcpyAsync(labels_out, dst, (size_t)ctx->P, cudaMemcpyDefault, ctx->stream));
+    if (labels_out && !direct) ST_CUDA(ctx, cudaMemcpyAsync(labels_out, dst, (size_t)ctx->P, cudaMemcpyDefault, ctx->stream));
     ctx->has_labels[stream] = 1;
+    ctx->settled = false;
     return tag_labels(ctx, stream);
 }
 
@@ -828,6 +860,7 @@ st_status st_set_labels(st_ctx* ctx, int32_t stream, const uint8_t* labels)
     if (!labels) return fail(ctx, ST_ERR_INVALID_ARG, "st_set_labels: NULL labels");
     ST_CUDA(ctx, cudaMemcpyAsync(ctx->labels + (int64_t)stream * ctx->P, labels, (size_t)ctx->P, cudaMemcpyDefault, ctx->stream));
     ctx->has_labels[stream] = 1;
+    ctx->settled = false;
     return tag_labels(ctx, stream);
 }
 
@@ -868,15 +901,26 @@ st_status st_distill_step(st_ctx* ctx, int32_t n_steps, float* loss_out, int64_t
     }
 
     st_status st = ST_OK;
+    // A caller that gives the same device buffer again gets its losses written by the updates themselves (one replayable graph
+    // per buffer); the first time, and for host memory, they are copied out behind the steps.
+    float* given = loss_out && ((uintptr_t)loss_out & 3u) == 0 && is_device_ptr(loss_out) ? loss_out : nullptr;
+    ctx->loss_direct = given && (given == ctx->loss_seen || !ctx->use_graphs) ? given : nullptr;
+    ctx->loss_pitch = n_steps;
+    ctx->loss_seen = given;
     if (ctx->use_graphs) {
-        GraphKey key{n_steps, want_conf, false, 0};
+        GraphKey key{n_steps, want_conf, false, 0, ctx->loss_direct};
+        if (ctx->graphs.size() >= kMaxGraphs && !ctx->graphs.count(key)) {
+            ST_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+            for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.second.exec);
+            ctx->graphs.clear();
+        }
         auto it = ctx->graphs.find(key);
         if (it == ctx->graphs.end()) {
             cudaGraph_t graph = nullptr;
             const int64_t before = ctx->launches;
             ST_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
             for (int k = 0; k < n_steps && st == ST_OK; ++k) st = enqueue_step(ctx, k, want_conf, nullptr, k == n_steps - 1);
-            if (st == ST_OK && ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, n_steps, nullptr, ctx->stream); ctx->launches += 1; }
+            if (st == ST_OK && ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, n_steps, ctx->stream); ctx->launches += 1; }
             cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
             const int64_t n_launches = ctx->launches - before;
             ctx->launches = before;
@@ -895,9 +939,12 @@ st_status st_distill_step(st_ctx* ctx, int32_t n_steps, float* loss_out, int64_t
             st = enqueue_step(ctx, k, want_conf, nullptr, k == n_steps - 1);
             if (st != ST_OK) return st;
         }
-        if (ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, n_steps, nullptr, ctx->stream); ctx->launches += 1; }
+        if (ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, n_steps, ctx->stream); ctx->launches += 1; }
     }
-    if (loss_out)
+    ctx->settled = true;
+    const bool delivered = ctx->loss_direct != nullptr;
+    ctx->loss_direct = nullptr;
+    if (loss_out && !delivered)
         ST_CUDA(ctx, cudaMemcpy2DAsync(loss_out, (size_t)n_steps * sizeof(float), ctx->loss_buf, kMaxSteps * sizeof(float),
                                        (size_t)n_steps * sizeof(float), ctx->S, cudaMemcpyDefault, ctx->stream));
     if (conf_out)
@@ -941,10 +988,8 @@ st_status enqueue_train(st_ctx* c, int max_updates, double threshold)
         if (st == ST_OK) st = enqueue_update(c, i, nullptr, 0, nullptr, &ctl, side ? 2 : 1);
     }
     if (st != ST_OK) return st;
-    launch_train_commit(train_ctl(c, 0, max_updates, threshold), c->theta, c->stream);    // student <- best_student
-    launch_refresh_shadow(make_update_args(c, 0), c->stream);
-    c->launches += 2;
-    if (c->adam) { launch_step_tick(c->step_base, c->S, 0, c->ctl_n_updates, c->stream); c->launches += 1; }   // steps taken
+    launch_train_commit(make_update_args(c, 0), c->best_theta, c->ctl_n_updates, c->stream);    // student <- best_student; Adam: steps taken
+    c->launches += 1;
     return check_launch(c, "train commit");
 }
 }  // namespace
@@ -962,6 +1007,7 @@ st_status st_train_key_frame(st_ctx* ctx, double threshold, int32_t max_updates,
         if (ready != ST_OK) return ready;
     }
     const size_t cc = (size_t)ctx->C * ctx->C;
+    ctx->loss_direct = nullptr;
     ctx->z_current = false;
     ctx->z_unkept = ctx->fused_fwd != 0;    // the loop's logits never leave the loss kernel
     cudaError_t e = cudaSuccess;
@@ -982,7 +1028,7 @@ st_status st_train_key_frame(st_ctx* ctx, double threshold, int32_t max_updates,
     if (ctx->use_graphs) {
         uint64_t thr_bits;
         memcpy(&thr_bits, &threshold, sizeof thr_bits);
-        GraphKey key{max_updates, true, true, thr_bits};
+        GraphKey key{max_updates, true, true, thr_bits, nullptr};
         auto it = ctx->graphs.find(key);
         if (it == ctx->graphs.end()) {
             cudaGraph_t graph = nullptr;
@@ -1006,27 +1052,36 @@ st_status st_train_key_frame(st_ctx* ctx, double threshold, int32_t max_updates,
         st = enqueue_train(ctx, max_updates, threshold);
         if (st != ST_OK) return st;
     }
+    ctx->settled = true;
     const int n_pred = max_updates + 1;
     bool host_out = false;
-    if (n_updates_out) {
-        ST_CUDA(ctx, cudaMemcpyAsync(n_updates_out, ctx->ctl_n_updates, (size_t)ctx->S * sizeof(int), cudaMemcpyDefault, ctx->stream));
-        host_out |= !is_device_ptr(n_updates_out);
+    // device and pinned host destinations are written by one kernel, others are copied to
+    TrainResults out{};
+    auto reach = [&](void* q, size_t align, auto** slot) {
+        if (!q) return true;
+        const void* dev = nullptr;
+        const Where where = locate(q, &dev);
+        host_out |= where != Where::device;
+        if (where == Where::host || ((uintptr_t)dev & (align - 1))) return false;
+        *slot = reinterpret_cast<std::remove_reference_t<decltype(**slot)>*>(const_cast<void*>(dev));
+        return true;
+    };
+    const bool r_n = reach(n_updates_out, 4, &out.n_updates), r_best = reach(best_metric_out, 8, &out.best), r_metric = reach(metric_out, 8, &out.metric),
+               r_loss = reach(loss_out, 4, &out.loss);
+    if (out.n_updates || out.best || out.metric || out.loss) {
+        launch_train_results(train_ctl(ctx, 0, max_updates, threshold), ctx->loss_buf, out, ctx->stream);
+        ctx->launches += 1;
     }
-    if (best_metric_out) {     // best_metric after the last prediction was assessed
+    if (!r_n) ST_CUDA(ctx, cudaMemcpyAsync(n_updates_out, ctx->ctl_n_updates, (size_t)ctx->S * sizeof(int), cudaMemcpyDefault, ctx->stream));
+    if (!r_best)               // best_metric after the last prediction was assessed
         ST_CUDA(ctx, cudaMemcpy2DAsync(best_metric_out, sizeof(double), ctx->ctl_best + n_pred, kCtlPitch * sizeof(double),
                                        sizeof(double), ctx->S, cudaMemcpyDefault, ctx->stream));
-        host_out |= !is_device_ptr(best_metric_out);
-    }
-    if (metric_out) {
+    if (!r_metric)
         ST_CUDA(ctx, cudaMemcpy2DAsync(metric_out, (size_t)n_pred * sizeof(double), ctx->ctl_metric, kCtlPitch * sizeof(double),
                                        (size_t)n_pred * sizeof(double), ctx->S, cudaMemcpyDefault, ctx->stream));
-        host_out |= !is_device_ptr(metric_out);
-    }
-    if (loss_out) {
+    if (!r_loss)
         ST_CUDA(ctx, cudaMemcpy2DAsync(loss_out, (size_t)n_pred * sizeof(float), ctx->loss_buf, kMaxSteps * sizeof(float),
                                        (size_t)n_pred * sizeof(float), ctx->S, cudaMemcpyDefault, ctx->stream));
-        host_out |= !is_device_ptr(loss_out);
-    }
     if (conf_out) {
         ST_CUDA(ctx, cudaMemcpy2DAsync(conf_out, (size_t)n_pred * cc * 8, ctx->conf_buf, (size_t)kMaxSteps * cc * 8,
                                        (size_t)n_pred * cc * 8, ctx->S, cudaMemcpyDefault, ctx->stream));
@@ -1057,7 +1112,7 @@ st_status st_profile_step(st_ctx* ctx, int32_t n_steps, int32_t* n_stages, float
         cudaEventRecord(t.ev[0], ctx->stream);
         st = enqueue_step(ctx, 0, false, &t);
         if (st != ST_OK) break;
-        if (ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, 1, nullptr, ctx->stream); ctx->launches += 1; }
+        if (ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, 1, ctx->stream); ctx->launches += 1; }
         if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) { st = fail(ctx, ST_ERR_CUDA, "st_profile_step: synchronize failed"); break; }
         n = t.n;
         for (int i = 0; i < n; ++i) {
@@ -1083,15 +1138,20 @@ st_status st_pack_updated_params(st_ctx* ctx, int32_t stream, void* dst, size_t 
     if (dst_capacity < need)
         return fail(ctx, ST_ERR_BUFFER_TOO_SMALL, "st_pack_updated_params: capacity %zu < %zu bytes", dst_capacity, need);
     const float* src = ctx->theta + (int64_t)stream * ctx->n_params;
-    if (is_device_ptr(dst)) {
-        launch_pack(src, (float*)dst, ctx->layout, ctx->trained_begin, ctx->n_trained, 1, ctx->stream);
+    const int first = ctx->bf16_mode ? ctx->first_trained : 0;
+    const void* to = nullptr;
+    const Where where = locate(dst, &to);
+    if (where != Where::host) {             // device memory, or pinned host memory written by the kernel itself
+        launch_pack(src, (float*)const_cast<void*>(to), ctx->layout, first, 1, ctx->stream);
         ctx->launches += 1;
-        return check_launch(ctx, "pack");
+        st = check_launch(ctx, "pack");
+        if (st == ST_OK && where == Where::pinned) ST_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        return st;
     }
-    // host destination: pack into the staging buffer, then copy out
+    // other host memory: pack into the staging buffer, then copy out
     st = ensure_staging(ctx, need);
     if (st != ST_OK) return st;
-    launch_pack(src, (float*)ctx->staging, ctx->layout, ctx->trained_begin, ctx->n_trained, 1, ctx->stream);
+    launch_pack(src, (float*)ctx->staging, ctx->layout, first, 1, ctx->stream);
     ctx->launches += 1;
     st = check_launch(ctx, "pack");
     if (st != ST_OK) return st;
@@ -1108,12 +1168,13 @@ st_status st_apply_update(st_ctx* ctx, int32_t stream, const void* src, size_t n
     if (!src) return fail(ctx, ST_ERR_INVALID_ARG, "st_apply_update: NULL source");
     if (nbytes != need) return fail(ctx, ST_ERR_INVALID_ARG, "st_apply_update: %zu bytes given, the updated part has %zu", nbytes, need);
     const void* dev = nullptr;
-    st = to_device(ctx, src, need, &dev);
+    st = small_to_device(ctx, src, need, &dev);
     if (st != ST_OK) return st;
     ctx->z_current = false;
-    launch_unpack((const float*)dev, ctx->theta + (int64_t)stream * ctx->n_params, ctx->layout, ctx->trained_begin, ctx->n_trained, 1, ctx->stream);
+    UpdateArgs u = make_update_args(ctx, -1);
+    if (!ctx->bf16_mode) u.n_layers = 0;
+    launch_unpack((const float*)dev, ctx->theta + (int64_t)stream * ctx->n_params, ctx->layout, ctx->bf16_mode ? ctx->first_trained : 0, 1, u, stream, ctx->stream);
     ctx->launches += 1;
-    if (ctx->bf16_mode) { launch_refresh_shadow(make_update_args(ctx, -1), ctx->stream); ctx->launches += 1; }
     return check_launch(ctx, "apply update");
 }
 
@@ -1138,7 +1199,7 @@ StudentMaskArgs mask_args(st_ctx* ctx, int32_t stream, uint8_t* mask)
     a.C = ctx->C; a.h = ctx->h; a.w = ctx->w;
     a.mask = mask;
     if (ctx->fused_fwd) {               // the mask kernel multiplies the logits itself: no forward before it, `z` is not read
-        a.fused = 1; a.kblocks = ctx->Cin / 64; a.stream = stream;
+        a.fused = 1; a.kblocks = ctx->Cin / 64; a.stream = stream; a.settled = ctx->settled ? 1 : 0;
         a.bias = ctx->theta + (int64_t)stream * ctx->n_params + ctx->layout.b_off[ctx->layout.n_layers - 1];
         a.err = ctx->bad + 2;
         a.x_map = &ctx->fx_map; a.w_map = &ctx->fw_map;
@@ -1198,6 +1259,7 @@ st_status st_agreement(st_ctx* ctx, int32_t stream, const uint8_t* pred, const u
         st = ctx->fused_fwd ? ready_to_run(ctx, "st_agreement", false) : student_forward(ctx, stream, "st_agreement");
         if (st != ST_OK) return st;
         StudentMaskArgs a = mask_args(ctx, stream, nullptr);
+        if (label) a.settled = 0;           // the caller's own map may come from a kernel that is still running
         a.labels = d_label; a.conf = ctx->conf_tmp; a.bad = ctx->bad + 1; a.miou = miou_res;
         a.ticket = reinterpret_cast<unsigned int*>(ctx->conf_tmp + cc);
         a.conf_out = conf_res;
@@ -1285,8 +1347,8 @@ st_status st_read_tensor(st_ctx* ctx, int32_t stream, st_tensor which, float* ds
             }
             src = ctx->bf16_mode ? ctx->dz + s * ctx->C * ctx->p : unpad(ctx->dz, ctx->C);
             break;
-        case ST_TENSOR_PARAM_GRAD: launch_pack(ctx->grad + s * ctx->n_params, ctx->read_tmp, ctx->layout, 0, ctx->n_params, 1, ctx->stream); src = ctx->read_tmp; break;
-        case ST_TENSOR_MOMENTUM: launch_pack(ctx->vel + s * ctx->n_params, ctx->read_tmp, ctx->layout, 0, ctx->n_params, 1, ctx->stream); src = ctx->read_tmp; break;
+        case ST_TENSOR_PARAM_GRAD: launch_pack(ctx->grad + s * ctx->n_params, ctx->read_tmp, ctx->layout, 0, 1, ctx->stream); src = ctx->read_tmp; break;
+        case ST_TENSOR_MOMENTUM: launch_pack(ctx->vel + s * ctx->n_params, ctx->read_tmp, ctx->layout, 0, 1, ctx->stream); src = ctx->read_tmp; break;
         case ST_TENSOR_HIDDEN:
             if (ctx->bf16_mode) { launch_nhwc_bf16_to_chw(ctx->blk[ctx->n_blocks - 1].out + s * ctx->p * ctx->Ch, ctx->Ch, ctx->p, ctx->read_tmp, ctx->stream); src = ctx->read_tmp; }
             else src = unpad(ctx->hid_f32, ctx->Ch);

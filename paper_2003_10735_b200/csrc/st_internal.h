@@ -64,7 +64,8 @@ constexpr int kMaxBlocks = 2;     // student blocks in front of the classifier (
 constexpr int kMaxLayers = kMaxBlocks + 1;
 
 // ---- K1: teacher logits -> uint8 labels -------------------------------------------------------
-void launch_argmax_u8(const float* logits, int C, int64_t P, uint8_t* labels, cudaStream_t s);
+// `copy`: nullptr, or a second device map that receives the same labels
+void launch_argmax_u8(const float* logits, int C, int64_t P, uint8_t* labels, uint8_t* copy, cudaStream_t s);
 
 // ---- K6: confusion matrix of two uint8 masks ---------------------------------------------------
 // conf: int64 [C][C], accumulated into (caller zeroes it); bad: count of pixels with l or q >= C.
@@ -154,6 +155,7 @@ struct StudentMaskArgs {
     unsigned long long* conf_out;  // with `miou`: the last block writes the finished matrix here and clears `conf`
     // One-layer head with bf16 features: the kernel multiplies the logits itself (k_student_eval.cu) and `z` is not read
     int fused;                 // 0, or 1: the fields below are set
+    int settled;               // the features and the labels were complete before the kernel launched just before this one began
     int kblocks, stream;       // 64-channel slices of the features; the stream (a coordinate of the tile maps)
     const float* bias;         // the classifier's bias of that stream (fp32 master parameters)
     unsigned int* err;         // device word: first wait that gave up
@@ -179,16 +181,16 @@ struct PadF32 {
 void launch_pad_planes(const float* plain, float* padded, int C, int h, int w, cudaStream_t s);
 void launch_unpad_planes(const float* padded, float* plain, int C, int h, int w, cudaStream_t s);
 // Inputs and gradients are padded planes of S streams back to back; the output is one too if out_padded, else [Cout][h][w].
-// Weight, bias and (w_stride floats per stream) parameters as in PackLayout.
+// Weight, bias and (w_stride floats per stream) parameters as in PackLayout.  `early`: see launch_chain.
 void launch_conv_fwd_f32(const float* in, int Cin, int h, int w, const float* Wt, const float* b, int Cout, int ks, bool relu,
-                         float* out, bool out_padded, int S, int64_t w_stride, cudaStream_t s);
+                         float* out, bool out_padded, int S, int64_t w_stride, bool early, cudaStream_t s);
 // Weight gradient as n_split = conv_wgrad_f32_splits(...) partial results [S][n_split][tap][Cout][Cin], which the parameter
 // update adds; with b_partials also the bias gradient's, [S][n_split][Cout]
 int conv_wgrad_f32_splits(int Cin, int Cout, int h, int w, int ks, int S);
 void launch_conv_wgrad_f32(const float* in, const float* dout, int Cin, int Cout, int h, int w, int ks, float* partials,
-                           float* b_partials, int S, cudaStream_t s);
+                           float* b_partials, int S, bool early, cudaStream_t s);
 void launch_conv1x1_dgrad_relu_f32(const float* W2, const float* dz, const float* Hact, int C, int Ch, int h, int w, float* dH, int S,
-                                   int64_t w_stride, cudaStream_t s);
+                                   int64_t w_stride, bool early, cudaStream_t s);
 cudaError_t prepare_conv_f32();   // once per device, outside any stream capture
 
 // ---- control of Algorithm 1 (Train): assessed once per prediction, per stream, by the update kernel that follows the
@@ -248,6 +250,8 @@ struct UpdateArgs {
     int n_loss_part;
     float* loss_buf;         // [S][kMaxSteps]
     int loss_slot;           // slot of loss_buf written by this step
+    float* loss_out;         // nullptr, or the caller's losses [S][loss_pitch], written as well
+    int loss_pitch;
     double inv_P;
     const int* skip;         // nullptr, or one flag per stream (skip[s * skip_stride]): non-zero = leave the stream's
     int64_t skip_stride;     //   parameters and momentum untouched (the loss is still finalised)
@@ -255,7 +259,7 @@ struct UpdateArgs {
     int adam;
     float* vel2;             // [S][n_params]
     double b1, b2, eps, ln_b1, ln_b2;
-    const long long* step_base;   // [S] optimisation steps taken before this call
+    long long* step_base;   // [S] optimisation steps taken before this call
     int chain_early;         // launch so that the kernel may start while its predecessor on the stream drains
     // Train (Algorithm 1): the update also assesses the prediction it follows.  Every block works the metric out from the
     // prediction's confusion matrix (same counts, same arithmetic, same answer), keeps the old value of its parameters
@@ -264,24 +268,26 @@ struct UpdateArgs {
     int has_ctl;             // 0; 1: this kernel assesses the prediction; 2: the backward before it has (see tc_backward), read the outcome
     TrainCtl ctl;
 };
-// step_base[s] += add (add_per_stream == nullptr) or += add_per_stream[s]
-void launch_step_tick(long long* step_base, int S, int add, const int* add_per_stream, cudaStream_t s);
+void launch_step_tick(long long* step_base, int S, int add, cudaStream_t s);   // step_base[s] += add
 int launch_sgd_update(const UpdateArgs& a, cudaStream_t s);   // returns the number of kernels launched
-// refresh the bf16 shadows from the fp32 master parameters (after init)
-void launch_refresh_shadow(const UpdateArgs& a, cudaStream_t s);
 // mean IoU (Section 3.2) from an int64 confusion matrix, in double, one block
 void launch_miou(const unsigned long long* conf, int C, double* out, cudaStream_t s);
-// student <- best_student for the trained parameters (the caller refreshes the bf16 copies afterwards)
-void launch_train_commit(const TrainCtl& t, float* theta, cudaStream_t s);
+// student <- best_student for the trained parameters (the layers of `a`) and their bf16 copies; Adam: step count += n_updates[s]
+void launch_train_commit(const UpdateArgs& a, const float* best_theta, const int* n_updates, cudaStream_t s);
 
+// Train's results to the caller (each optional, device or pinned host memory): updates taken [S], best metric [S], metrics and
+// losses [S][max_updates + 1]
+struct TrainResults { int* n_updates; double *best, *metric; float* loss; };
+void launch_train_results(const TrainCtl& t, const float* loss_buf, const TrainResults& out, cudaStream_t s);
 
 // ---- K7: packed parameter buffer <-> internal order ---------------------------------------------
 // packed: per layer weight [cout][cin][kh][kw] then bias; internal: weight [tap][cout][cin] then bias.
-// `begin`, `count`: the range of one stream's parameters that the packed buffer carries (all of them at initialisation;
-// the trained layers, which come last, in UpdatedPart); packed buffers of consecutive streams lie `count` floats apart.
+// The packed buffer carries the layers from `first` on (all of them at initialisation; the trained layers, which come last, in
+// UpdatedPart); packed buffers of consecutive streams lie back to back.  It may be device or pinned host memory.
+// Unpacking writes the bf16 copies too where `u` lists the layers' (u.layer[k - first], streams s0, s0 + 1, ...).
 struct PackLayout { int n_layers; int64_t w_off[kMaxLayers], b_off[kMaxLayers]; int cout[kMaxLayers], cin[kMaxLayers], taps[kMaxLayers]; int64_t n_params; };
-void launch_pack(const float* internal, float* packed, const PackLayout& L, int64_t begin, int64_t count, int n_bufs, cudaStream_t s);
-void launch_unpack(const float* packed, float* internal, const PackLayout& L, int64_t begin, int64_t count, int n_bufs, cudaStream_t s);
+void launch_pack(const float* internal, float* packed, const PackLayout& L, int first, int n_bufs, cudaStream_t s);
+void launch_unpack(const float* packed, float* internal, const PackLayout& L, int first, int n_bufs, const UpdateArgs& u, int s0, cudaStream_t s);
 
 // ---- bf16 tensor-core GEMMs (gemm_precision 1) -------------------------------------------------
 struct TcPlan;   // tensor maps and launch geometry; built once per context
