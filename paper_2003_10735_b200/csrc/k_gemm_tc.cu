@@ -471,8 +471,8 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
     pdl_wait();                  // inputs come from the previous kernel of the step
     bool ok = true;
 
-    if (tid == 0) {
-        // ---- producer: the ring index runs on across tiles
+    if (warp == 0) {
+        // ---- producer (the whole warp walks the loop, its first lane issues): the ring index runs on across tiles
         int g = 0;
         for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
             const Item im = item_of(wi);
@@ -486,6 +486,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
                 const int st = g % STAGES;                                                                                \
                 if (g >= STAGES) ok = mbar_wait(smem_u32(&empty[st]), ((g / STAGES) - 1) & 1, err, kWaitEmpty);          \
                 if (!ok) break;                                                                                           \
+                if (lane == 0) {                                                                                          \
                 const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;                                   \
                 mbar_expect_tx(bar, a_bytes + (uint32_t)im.chn * 128);                                                    \
                 tma_load_4d(sa, &(src), bar, (a_coord), x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);                          \
@@ -493,6 +494,8 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
                 else                                                                                                      \
                     for (int j = 0; j < im.chn / 64; ++j)        /* 64 weight rows per copy, laid out like the single copy */ \
                         tma_load_3d(sa + a_bytes + j * (64 * 128), &tmBq, bar, kb * kBlockK, tap * Ch + im.ch0 + j * 64, s); \
+                }                                                                                                         \
+                __syncwarp();                                                                                             \
                 ++g;                                                                                                      \
             }
             for (int tap = 0; tap < 9 && ok; ++tap) {
@@ -503,7 +506,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
 #undef ST_FWD3_STAGE
         }
         pdl_launch_dependents();     // every load is issued: the next kernel of the step may set itself up
-    } else if (tid == 32) {
+    } else if (warp == 1) {
         // ---- MMA issuer
         int g = 0, j = 0;
         for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
@@ -520,13 +523,16 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
                 ok = mbar_wait(smem_u32(&full[st]), (g / STAGES) & 1, err, kWaitFull);
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t sa = base + st * stage_bytes, sb = sa + a_bytes;
+                if (lane == 0) {
+                    const uint64_t da = smem_desc(base + st * stage_bytes, 16, 1024), db = da + (a_bytes >> 4);
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    umma(acc, smem_desc(sa + k * 32, 16, 1024), smem_desc(sb + k * 32, 16, 1024), idesc, (it | k) != 0);
-                umma_commit(smem_u32(&empty[st]));
+                    for (int k = 0; k < 4; ++k) umma(acc, da + 2 * k, db + 2 * k, idesc, (it | k) != 0);
+                    umma_commit(smem_u32(&empty[st]));
+                }
+                __syncwarp();
             }
-            if (ok) umma_commit(smem_u32(&acc_full[buf]));
+            if (ok && lane == 0) umma_commit(smem_u32(&acc_full[buf]));
+            __syncwarp();
             ++j;                                                       // j counts the tiles this block works on
         }
     } else if (warp >= 2) {

@@ -66,23 +66,25 @@ __device__ __forceinline__ ParamState load_state(const UpdateArgs& a, int64_t gi
 }
 
 template <bool ADAM>
-__device__ __forceinline__ float apply_update(const UpdateArgs& a, int64_t gi, float g, const AdamCorr& k, const ParamState& p)
+__device__ __forceinline__ float updated(const UpdateArgs& a, float g, const AdamCorr& k, const ParamState& p, float& vel, float& vel2)
 {
-    a.grad[gi] = g;
     if (ADAM) {
         const double gd = (double)g;
         const double m = a.b1 * (double)p.vel + (1.0 - a.b1) * gd;
         const double v = a.b2 * (double)p.vel2 + (1.0 - a.b2) * gd * gd;
-        a.vel[gi] = (float)m;
-        a.vel2[gi] = (float)v;
-        const float t = (float)((double)p.theta - (double)a.lr * (m / k.c1) / (sqrt(v / k.c2) + a.eps));
-        a.theta[gi] = t;
-        return t;
+        vel = (float)m; vel2 = (float)v;
+        return (float)((double)p.theta - (double)a.lr * (m / k.c1) / (sqrt(v / k.c2) + a.eps));
     }
-    float v = fmaf(a.mu, p.vel, g);
-    a.vel[gi] = v;
-    const float t = fmaf(-a.lr, v, p.theta);
-    a.theta[gi] = t;
+    vel = fmaf(a.mu, p.vel, g); vel2 = 0.f;
+    return fmaf(-a.lr, vel, p.theta);
+}
+template <bool ADAM>
+__device__ __forceinline__ float apply_update(const UpdateArgs& a, int64_t gi, float g, const AdamCorr& k, const ParamState& p)
+{
+    float vel, vel2;
+    const float t = updated<ADAM>(a, g, k, p, vel, vel2);
+    a.grad[gi] = g; a.vel[gi] = vel; a.theta[gi] = t;
+    if (ADAM) a.vel2[gi] = vel2;
     return t;
 }
 template <bool ADAM>
@@ -91,40 +93,133 @@ __device__ __forceinline__ float apply_update(const UpdateArgs& a, int64_t gi, f
     return apply_update<ADAM>(a, gi, g, k, load_state<ADAM>(a, gi));
 }
 
+// A large weight tensor with a moderate number of split-K partials (a 3x3 layer): a pure stream.  Each thread owns VEC
+// consecutive weights and reads them from every partial with all loads in flight.
+template <int VEC, bool ADAM>
+__device__ __forceinline__ void update_stream(const UpdateArgs& a, const LayerUpdate& ly, int s, int block)
+{
+    bool skip = a.skip && a.skip[(int64_t)s * a.skip_stride], better = false;
+    if (a.has_ctl) {                                                   // the grouped part's first block writes the history
+        const TrainHistory hist = train_history(a.ctl, s);
+        if (a.has_ctl == 1) { const MiouFetch f = train_fetch(a.ctl, s, hist); train_decision(a.ctl, s, false, hist, &f, skip, better); }
+        else if (hist.ended) skip = true;
+        else train_outcome(a.ctl, s, skip, better);
+    }
+    if (skip && !better) return;
+    const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
+    const int64_t e = ((int64_t)block * kUpdThreads + threadIdx.x) * VEC;
+    if (e >= nw) return;
+    const float* src = ly.w_partials + (int64_t)s * ly.w_stream_stride + e;
+    const int64_t gi = (int64_t)s * a.n_params + ly.w_off + e;
+    const bool vec = VEC == 4 && (gi & 3) == 0;                        // the parameters as whole vectors too
+    ParamState state[VEC];
+    if (vec) {
+        const float4 t = *reinterpret_cast<const float4*>(a.theta + gi), v = *reinterpret_cast<const float4*>(a.vel + gi);
+        const float4 v2 = ADAM ? *reinterpret_cast<const float4*>(a.vel2 + gi) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float tt[4] = {t.x, t.y, t.z, t.w}, vv[4] = {v.x, v.y, v.z, v.w}, ww[4] = {v2.x, v2.y, v2.z, v2.w};
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) { state[j].theta = tt[j % 4]; state[j].vel = vv[j % 4]; state[j].vel2 = ww[j % 4]; }
+    } else {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) state[j] = load_state<ADAM>(a, gi + j);
+    }
+    float g[VEC];
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) g[j] = 0.f;
+    for (int k0 = 0; k0 < ly.n_split; k0 += 8) {
+        if (VEC == 4) {
+            float4 t[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                t[j] = k0 + j < ly.n_split ? __ldg(reinterpret_cast<const float4*>(src + (int64_t)(k0 + j) * ly.w_split_stride))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { g[0] += t[j].x; g[1 % VEC] += t[j].y; g[2 % VEC] += t[j].z; g[3 % VEC] += t[j].w; }
+        } else {
+            float t[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) t[j] = k0 + j < ly.n_split ? __ldg(src + (int64_t)(k0 + j) * ly.w_split_stride) : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) g[0] += t[j];
+        }
+    }
+    const AdamCorr corr = adam_corrections<ADAM>(a, s);
+    if (!vec || skip) {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) {
+            if (better) a.ctl.best_theta[gi + j] = state[j].theta;
+            if (!skip) write_shadows(ly, s, e + j, apply_update<ADAM>(a, gi + j, g[j], corr, state[j]));
+        }
+        return;
+    }
+    if (better) *reinterpret_cast<float4*>(a.ctl.best_theta + gi) = make_float4(state[0].theta, state[1 % VEC].theta, state[2 % VEC].theta, state[3 % VEC].theta);
+    float t[4], v[4], v2[4];
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) t[j % 4] = updated<ADAM>(a, g[j], corr, state[j], v[j % 4], v2[j % 4]);
+    *reinterpret_cast<float4*>(a.theta + gi) = make_float4(t[0], t[1], t[2], t[3]);
+    *reinterpret_cast<float4*>(a.vel + gi) = make_float4(v[0], v[1], v[2], v[3]);
+    if (ADAM) *reinterpret_cast<float4*>(a.vel2 + gi) = make_float4(v2[0], v2[1], v2[2], v2[3]);
+    *reinterpret_cast<float4*>(a.grad + gi) = make_float4(g[0], g[1 % VEC], g[2 % VEC], g[3 % VEC]);
+    if (ly.shadow && !ly.shadow_t) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(t[0], t[1]), hi = __floats2bfloat162_rn(t[2], t[3]);
+        *reinterpret_cast<uint2*>(ly.shadow + (int64_t)s * ly.shadow_stream_stride + e) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+    } else {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) write_shadows(ly, s, e + j, t[j % 4]);
+    }
+}
+
 // Parameter blocks: a block covers kUpdThreads / G consecutive parameters; the G thread groups of a
 // block each sum every G-th split-K partial of "their" parameter (coalesced along the parameters),
 // the group sums are added in group order through shared memory, and group 0 applies the update.
 template <int G, int E, bool ADAM>
 __global__ void __launch_bounds__(kUpdThreads)
-sgd_update_kernel(UpdateArgs a, int n_param_blocks, int64_t range_begin)
+sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
 {
     constexpr int kRow = kUpdThreads / G;      // consecutive parameters covered by one thread group
     constexpr int kPer = kRow * E;             // parameters per block
     __shared__ float part[G][kPer];
     const int s = blockIdx.y;
     const int64_t base = (int64_t)s * a.n_params;
+    if ((int)blockIdx.x >= n_grouped) {                  // the streamed layers' blocks lie behind the grouped ones
+        pdl_wait();
+        pdl_launch_dependents();
+        int block = (int)blockIdx.x - n_grouped;
+        for (int L = 0; L < a.n_layers; ++L) {
+            const LayerUpdate& ly = a.layer[L];
+            if (!ly.streamed) continue;
+            const int per = kUpdThreads * (ly.streamed == 4 ? 4 : 1);
+            const int blocks = (int)(((int64_t)ly.cout * ly.cin * ly.taps + per - 1) / per);
+            if (block >= blocks) { block -= blocks; continue; }
+            if (ly.streamed == 4) update_stream<4, ADAM>(a, ly, s, block);
+            else update_stream<1, ADAM>(a, ly, s, block);
+            return;
+        }
+        return;
+    }
     const bool param_block = (int)blockIdx.x < n_param_blocks;
     const int col = threadIdx.x % kRow, g = threadIdx.x / kRow;
     int layer[E];
-    bool is_weight[E], has_partials[E];
+    int64_t param[E];                          // index in one stream's parameters
     ParamState state[E];
-    // which parameters this thread looks after, and (first thread group) their current state: none of it comes from the
-    // kernels just before this one, so it is done before their completion is waited for
+    // which parameters this thread looks after (weights of the layers that are not streamed, one layer behind the other), and
+    // (first thread group) their current state: none of it comes from the kernels just before this one, so it is done before
+    // their completion is waited for
     if (param_block) {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const int64_t i = range_begin + (int64_t)blockIdx.x * kPer + e * kRow + col;
-            layer[e] = -1; is_weight[e] = false; has_partials[e] = false;
+            int64_t i = (int64_t)blockIdx.x * kPer + e * kRow + col;
+            layer[e] = -1; param[e] = 0;
             state[e].theta = state[e].vel = state[e].vel2 = 0.f;
-            if (i < a.n_params) {
-                for (int L = 0; L < a.n_layers; ++L) {
-                    const LayerUpdate& ly = a.layer[L];
-                    const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
-                    if (i >= ly.w_off && i < ly.w_off + nw && !ly.streamed) { layer[e] = L; is_weight[e] = true; }
-                    if (i >= ly.b_off && i < ly.b_off + ly.cout) { layer[e] = L; is_weight[e] = false; }
-                }
+            for (int L = 0; L < a.n_layers && layer[e] < 0; ++L) {
+                const LayerUpdate& ly = a.layer[L];
+                if (ly.streamed) continue;
+                const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
+                if (i < nw) { layer[e] = L; param[e] = ly.w_off + i; }
+                else i -= nw;
             }
-            if (g == 0 && layer[e] >= 0 && (is_weight[e] || !a.layer[layer[e]].b_partials)) state[e] = load_state<ADAM>(a, base + i);
+            if (g == 0 && layer[e] >= 0) state[e] = load_state<ADAM>(a, base + param[e]);
         }
     }
     TrainHistory hist{};
@@ -149,12 +244,10 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int64_t range_begin)
         // E parameters per thread, all of their split-K loads issued before any is consumed
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const int64_t i = range_begin + (int64_t)blockIdx.x * kPer + e * kRow + col;
             sum[e] = 0.f;
-            if (layer[e] >= 0 && is_weight[e] && a.layer[layer[e]].w_partials) {
+            if (layer[e] >= 0) {
                 const LayerUpdate& ly = a.layer[layer[e]];
-                has_partials[e] = true;
-                const float* src = ly.w_partials + (int64_t)s * ly.w_stream_stride + (i - ly.w_off);
+                const float* src = ly.w_partials + (int64_t)s * ly.w_stream_stride + (param[e] - ly.w_off);
                 // batches of 8 predicated loads: all in flight together, no one-at-a-time remainder loop
                 float t = 0.f;
                 for (int k0 = g; k0 < ly.n_split; k0 += 8 * G) {
@@ -178,23 +271,13 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int64_t range_begin)
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             if (layer[e] < 0) continue;
-            const int64_t i = range_begin + (int64_t)blockIdx.x * kPer + e * kRow + col;
+            const int64_t i = param[e];
             const LayerUpdate& ly = a.layer[layer[e]];
-            if (is_weight[e]) {
-                float gr;
-                if (has_partials[e]) {
-                    gr = 0.f;
+            float gr = 0.f;
 #pragma unroll
-                    for (int k = 0; k < G; ++k) gr += part[k][e * kRow + col];
-                } else {
-                    gr = a.grad[base + i];
-                }
-                if (better) best_theta[base + i] = state[e].theta;
-                if (!skip) write_shadows(ly, s, i - ly.w_off, apply_update<ADAM>(a, base + i, gr, corr, state[e]));
-            } else if (!ly.b_partials) {
-                if (better) best_theta[base + i] = state[e].theta;
-                if (!skip) apply_update<ADAM>(a, base + i, a.grad[base + i], corr, state[e]);
-            }   // biases with partial sums are finished by the reduction warps below
+            for (int k = 0; k < G; ++k) gr += part[k][e * kRow + col];
+            if (better) best_theta[base + i] = state[e].theta;
+            if (!skip) write_shadows(ly, s, i - ly.w_off, apply_update<ADAM>(a, base + i, gr, corr, state[e]));
         }
         return;
     }
@@ -206,7 +289,6 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int64_t range_begin)
     int item = warp;
     for (int L = 0; L < a.n_layers; ++L) {
         const LayerUpdate& ly = a.layer[L];
-        if (!ly.b_partials) continue;
         if (item < ly.cout) {
             const float* src = ly.b_partials + (int64_t)s * ly.n_bpart * ly.cout + item;
             float g = 0.f;
@@ -254,98 +336,44 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int64_t range_begin)
     }
 }
 
-// A large weight tensor with a moderate number of split-K partials (the 3x3 layer): a pure stream.
-// Each thread owns VEC consecutive weights and reads them from every partial with all loads in flight.
-template <int VEC, bool ADAM>
-__global__ void __launch_bounds__(256)
-sgd_update_stream_kernel(UpdateArgs a, int L)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    const LayerUpdate& ly = a.layer[L];
-    const int s = blockIdx.y;
-    bool skip = a.skip && a.skip[(int64_t)s * a.skip_stride], better = false;
-    if (a.has_ctl) {                                                   // the grouped kernel's block 0 writes the history
-        const TrainHistory hist = train_history(a.ctl, s);
-        if (a.has_ctl == 1) { const MiouFetch f = train_fetch(a.ctl, s, hist); train_decision(a.ctl, s, false, hist, &f, skip, better); }
-        else if (hist.ended) skip = true;
-        else train_outcome(a.ctl, s, skip, better);
-    }
-    if (skip && !better) return;
-    const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
-    const int64_t e = ((int64_t)blockIdx.x * 256 + threadIdx.x) * VEC;
-    if (e >= nw) return;
-    const float* src = ly.w_partials + (int64_t)s * ly.w_stream_stride + e;
-    float g[VEC];
-#pragma unroll
-    for (int j = 0; j < VEC; ++j) g[j] = 0.f;
-    for (int k0 = 0; k0 < ly.n_split; k0 += 8) {
-        if (VEC == 4) {
-            float4 t[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                t[j] = k0 + j < ly.n_split ? __ldg(reinterpret_cast<const float4*>(src + (int64_t)(k0 + j) * ly.w_split_stride))
-                                           : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) { g[0] += t[j].x; g[1] += t[j].y; g[2] += t[j].z; g[3] += t[j].w; }
-        } else {
-            float t[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) t[j] = k0 + j < ly.n_split ? __ldg(src + (int64_t)(k0 + j) * ly.w_split_stride) : 0.f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) g[0] += t[j];
-        }
-    }
-    const int64_t gi = (int64_t)s * a.n_params + ly.w_off + e;
-    const AdamCorr corr = adam_corrections<ADAM>(a, s);
-#pragma unroll
-    for (int j = 0; j < VEC; ++j) {
-        if (better) a.ctl.best_theta[gi + j] = a.theta[gi + j];
-        if (!skip) write_shadows(ly, s, e + j, apply_update<ADAM>(a, gi + j, g[j], corr));
-    }
-}
-
 template <bool ADAM>
 static int launch_sgd_update_t(const UpdateArgs& a, cudaStream_t s)
 {
-    int n_launches = 1;
-    // large layers with partial sums go through the streaming kernel; everything else (small layers, biases,
-    // loss) through the grouped kernel, which then starts after the streamed range
-    int64_t range_begin = a.param_begin;
-    UpdateArgs g = a;                    // what the grouped kernel gets: streamed layers lose their partial sums there
+    // Large layers are streamed, everything else (small layers, biases, loss) goes through the grouped part.  One launch: the grouped part is all latency and hides behind the stream
+    // (256 -> 256 channels, 3x3: 19.9 us as two launches, 14.3 us as one, launch gap included).
+    UpdateArgs g = a;
+    int64_t stream_blocks = 0, n_rest = 0;
     for (int L = 0; L < a.n_layers; ++L) {
         const LayerUpdate& ly = a.layer[L];
         const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
-        if (ly.w_partials && nw >= 65536) {
+        if (nw >= 65536) {
             const bool vec = nw % 4 == 0 && ly.w_split_stride % 4 == 0 && ly.w_stream_stride % 4 == 0 &&
                              ((uintptr_t)ly.w_partials % 16 == 0);
-            if (vec) launch_chain(a.chain_early != 0, sgd_update_stream_kernel<4, ADAM>, dim3((unsigned)((nw / 4 + 255) / 256), (unsigned)a.S), dim3(256), 0, s, a, L);
-            else launch_chain(a.chain_early != 0, sgd_update_stream_kernel<1, ADAM>, dim3((unsigned)((nw + 255) / 256), (unsigned)a.S), dim3(256), 0, s, a, L);
-            if (ly.w_off == range_begin) range_begin = ly.w_off + nw;     // the grouped kernel starts behind leading streamed layers
-            g.layer[L].streamed = 1;                                       // ... and leaves the weights of later ones alone
-            ++n_launches;
-        }
+            g.layer[L].streamed = vec ? 4 : 1;
+            const int per = kUpdThreads * (vec ? 4 : 1);
+            stream_blocks += (nw + per - 1) / per;
+        } else n_rest += nw;
     }
     int items = 1, max_split = 1;
     for (int L = 0; L < a.n_layers; ++L) {
-        if (a.layer[L].b_partials) items += a.layer[L].cout;
-        if (a.layer[L].w_partials && !g.layer[L].streamed && a.layer[L].n_split > max_split) max_split = a.layer[L].n_split;
+        items += a.layer[L].cout;
+        if (!g.layer[L].streamed && a.layer[L].n_split > max_split) max_split = a.layer[L].n_split;
     }
     const int n_red_blocks = (items + kUpdThreads / 32 - 1) / (kUpdThreads / 32);
-    const int64_t n_rest = a.n_params - range_begin;
     const bool big = n_rest > 65536;
     // many partial sums per parameter: 16 thread groups, so that a group's share fits one batch of loads
     const int G = max_split <= 1 ? 1 : (max_split > 64 && !big ? 16 : 8), E = big ? 4 : 1;
     const int per = kUpdThreads / G * E;
     const int n_param_blocks = (int)((n_rest + per - 1) / per);
-    const dim3 grid((unsigned)(n_param_blocks + n_red_blocks), (unsigned)a.S);
+    const int n_grouped = n_param_blocks + n_red_blocks;
+    const dim3 grid((unsigned)(n_grouped + stream_blocks), (unsigned)a.S);
     const dim3 blk(kUpdThreads);
-    if (G == 1 && E == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<1, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, range_begin);
-    else if (G == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<1, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, range_begin);
-    else if (G == 16) launch_chain(a.chain_early != 0, sgd_update_kernel<16, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, range_begin);
-    else if (E == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<8, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, range_begin);
-    else launch_chain(a.chain_early != 0, sgd_update_kernel<8, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, range_begin);
-    return n_launches;
+    if (G == 1 && E == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<1, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    else if (G == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<1, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    else if (G == 16) launch_chain(a.chain_early != 0, sgd_update_kernel<16, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    else if (E == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<8, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    else launch_chain(a.chain_early != 0, sgd_update_kernel<8, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    return 1;
 }
 
 int launch_sgd_update(const UpdateArgs& a, cudaStream_t s)

@@ -223,18 +223,18 @@ struct TrainCtl {
 struct LayerUpdate {
     int64_t w_off, b_off;      // offsets (floats) of weight / bias in one stream's parameter buffer
     int cout, cin, taps;       // weight in internal order [tap][cout][cin]
-    const float* w_partials;   // nullptr: grad buffer already holds dW; else split-K partial sums whose
-    int n_split;               //   element index equals the internal weight index
+    const float* w_partials;   // split-K partial sums whose element index equals the internal weight index
+    int n_split;
     int64_t w_split_stride;    // floats between splits
     int64_t w_stream_stride;   // floats between streams
-    const float* b_partials;   // nullptr: grad buffer already holds db; else [S][n_bpart][cout]
+    const float* b_partials;   // [S][n_bpart][cout]
     int n_bpart;
     bf16* shadow;              // nullptr or the bf16 copy of the weight read by the GEMMs (same linear index)
     int64_t shadow_stream_stride;
     bf16* shadow_t;            // nullptr, or a second bf16 copy [9][c_take][cout] with the taps mirrored and the channels
     int64_t shadow_t_stream_stride;   // transposed, for the first c_take input channels: what the gradient passed back
     int c_take;                //   through this 3x3 layer multiplies
-    int streamed;              // set by the launcher: the streaming kernel updates this layer's weights, the grouped one skips them
+    int streamed;              // set by the launcher: 0, or the layer's weights are updated by streaming blocks, 4 or 1 per thread
 };
 struct UpdateArgs {
     float* theta;      // [S][n_params]   internal order
