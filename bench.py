@@ -265,8 +265,8 @@ def kernel_table(st, ctx, cfg, peaks, arith, n_profile_steps):
             k.update(bound="tensor", achieved=block_flop(1 if name.endswith("#2") else 0) / ms / 1e9, peak=tensor_peak, unit="TFLOP/s")
         elif name == "tc_dgrad3x3":     # through block 1 into block 0's output channels
             k.update(bound="tensor", achieved=2.0 * S * p * blocks[0][0] * 9 * blocks[1][0] / ms / 1e9, peak=tensor_peak, unit="TFLOP/s")
-        elif name == "tc_dgrad":
-            k.update(bound="hbm", achieved=S * (2 * p * c_last * 2 + C * p * 4) / ms / 1e6, peak=hbm, unit="GB/s")
+        elif name == "tc_back1x1":      # hidden activation in, its gradient out, both products of the 1x1 layer
+            k.update(bound="hbm", achieved=S * (2 * p * c_last * 2 + C * p * 2) / ms / 1e6, peak=hbm, unit="GB/s")
         else:
             k.update(bound="latency")
         kernels[name] = k

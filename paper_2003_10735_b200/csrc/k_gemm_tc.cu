@@ -6,7 +6,7 @@
 //   fwd 1x1   z[c][pix]       = b[c] + sum_k A[pix][k] W[c][k]                 A = features or hidden
 //   fwd 3x3   Hd[pix][co]     = ReLU(b1[co] + sum_{tap,ci} X[pix+tap][ci] W1[tap][co][ci])
 //   wgrad 1x1 dW[c][k]        = sum_pix dz[c][pix] A[pix][k]                   split over pixel ranges
-//   dgrad     dHd[pix][k]     = [Hd[pix][k] > 0] sum_c dz[c][pix] W2[c][k]     (bf16 out)
+//   dgrad     dHd[pix][k]     = [Hd[pix][k] > 0] sum_c dz[c][pix] W2[c][k]     (bf16 out; one kernel with wgrad 1x1)
 //   wgrad 3x3 dW1[tap][co][ci]= sum_pix dHd[pix][co] X[pix+tap][ci]            split over pixel ranges
 //
 // Pixel-major activations [pix][channel] are K-major operands when the GEMM reduces over channels
@@ -744,134 +744,199 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
 }
 
 // ------------------------------------------------------------------------------------------------
-// dgrad through the 1x1 output layer with the ReLU mask of the hidden activation:
-//   dHd[pix][k] = [Hd[pix][k] > 0] * sum_c dz[c][pix] * W2[c][k]
-// One 128-pixel tile per block, N = Ch, K = 32 class rows (rows >= C are zero in both operands).
-// dz rows [c][pix] and weight rows [c][k] are both contiguous along the non-reduced index, so both are
-// MN-major operands.  The epilogue applies the mask, writes bf16 (a GEMM operand next) and emits the
-// block's sums over pixels of the unrounded result: the bias gradient of the 3x3 layer.
+// Both backward products of the 1x1 output layer behind a trained hidden layer, in one pass over the logit gradient and the
+// hidden activation:
+//   dHd[pix][k] = [Hd[pix][k] > 0] * sum_c dz[c][pix] * W2[c][k]        (bf16, and its unrounded sums over pixels: the bias
+//                                                                         gradient of the 3x3 layer)
+//   dW2[c][k]  += dz[c][pix] * Hd[pix][k]
+// A block owns 128 hidden channels (an odd 64 at the end of the layer arrives zero-filled) and a range of 128-pixel tiles.  dz
+// rows [c][pix] are the MN-major A operand of the first product and the K-major B operand of the second, from one copy;
+// weight rows [c][k] and activation rows [pix][k] are MN-major.  A ring of stages (producer warp), one warp that issues both
+// products, two sets of four warps that drain the two accumulators of the first in turn; the second accumulates over the
+// whole range, which leaves one partial sum per block, like the bias gradient.
+// Bound by L2: at 720p and 256 channels 29 MB of activations come in and as much gradient goes out, 16.8 us (4 TB/s).  As two
+// kernels (gradient: a block per 128 pixels and half of the channels; weight gradient: a pass of its own) 18.8 + 9.7 us;
+// at 1080p 33.3 + 15.1 us, now 33.0.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreadsTc)
-tc_dgrad_kernel(const __grid_constant__ CUtensorMap tmA,   // dz  {p, 32, S}  box {64, 32, 1}
-                const __grid_constant__ CUtensorMap tmB,   // W2  {Ch, 32, S} box {64, 32, 1}
-                const uint32_t* __restrict__ relu_bits,     // [S][p][Ch/32]
-                bf16* __restrict__ dhidden,                 // [S][p][Ch]
-                float* __restrict__ b1_partials,            // [S][n_blocks][Ch]
-                int Ch, int p, int tmem_cols, unsigned int* err, const int* __restrict__ skip, int64_t skip_stride)
+constexpr int kBackStages = 4, kBackThreads = 320, kBackCols = 128;
+constexpr uint32_t kBackActBytes = kTileM * 128 * 2, kBackDzBytes = 2 * kClassPad * 128, kBackStageBytes = kBackActBytes + kBackDzBytes, kBackWBytes = 2 * kClassPad * 128;
+
+__global__ void __launch_bounds__(kBackThreads, 1)
+tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  box {64, 128, 1}
+                  const __grid_constant__ CUtensorMap tmD,   // dz {p, 32, S}  box {64, 32, 1}
+                  const __grid_constant__ CUtensorMap tmW,   // W2 {Ch, 32, S} box {64, 32, 1}
+                  const uint32_t* __restrict__ relu_bits,     // [S][p][Ch/32]
+                  bf16* __restrict__ dhidden,                 // [S][p][Ch]
+                  float* __restrict__ b_partials,             // [S][n_split][Ch]
+                  float* __restrict__ w_partials,             // [S][n_split][32][Ch]
+                  int Ch, int p, int n_tiles, int per, int n_groups, unsigned int* err, const int* __restrict__ skip, int64_t skip_stride,
+                  int has_ctl, const TrainCtl ctl)
 {
+    const int s = blockIdx.y;
+    if (has_ctl && blockIdx.x == gridDim.x - 1) {            // Train: one more block assesses the prediction meanwhile
+        const TrainHistory hist = train_history(ctl, s);
+        pdl_wait();
+        bool stop, better;
+        train_decision(ctl, s, true, hist, nullptr, stop, better);
+        pdl_launch_dependents();
+        return;
+    }
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_smem(smem_raw);
-    const uint32_t a_base = smem_u32(smem);
-    const uint32_t blk_bytes = kClassPad * 128;                 // 32 class rows x 64 elements
-    const uint32_t b_base = a_base + 2 * blk_bytes;
-    // gridDim.z blocks share a pixel tile, each with its own range of Ch / gridDim.z hidden channels (more and
-    // shorter blocks: the kernel's time is the latency of one block's epilogue)
-    const int Chb = Ch / (int)gridDim.z, ch0 = (int)blockIdx.z * Chb;
-    const int b_blocks = Chb / kBlockK;
-    __shared__ float part[4 * 256];                             // per-warp channel sums
-    __shared__ __align__(8) uint64_t full, done;
+    const uint32_t base = smem_u32(smem), w_base = base + kBackStages * kBackStageBytes;
+    __shared__ __align__(8) uint64_t full[kBackStages], empty[kBackStages], w_full, acc_full[2], acc_empty[2], done;
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int s = blockIdx.y, pix0 = blockIdx.x * kTileM;
+    __shared__ float part[8 * kBackCols];                        // per-warp channel sums
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n_split = ((int)gridDim.x - (has_ctl ? 1 : 0)) / n_groups, split = (int)blockIdx.x / n_groups, ch0 = (int)blockIdx.x % n_groups * kBackCols;
+    const int t_begin = split * per, t_end = min(n_tiles, t_begin + per), width = min(kBackCols, Ch - ch0);
 
-    if (warp == 0) tmem_alloc(smem_u32(&tmem_slot), tmem_cols);
+    if (warp == 0) tmem_alloc(smem_u32(&tmem_slot), 512);
     if (tid == 0) {
-        mbar_init(smem_u32(&full), 1); mbar_init(smem_u32(&done), 1);
+        for (int i = 0; i < kBackStages; ++i) { mbar_init(smem_u32(&full[i]), 1); mbar_init(smem_u32(&empty[i]), 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&acc_full[i]), 1); mbar_init(smem_u32(&acc_empty[i]), 4); }
+        mbar_init(smem_u32(&w_full), 1); mbar_init(smem_u32(&done), 1);
         fence_barrier_init();
     }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = tmem_slot, acc_w = tmem + 2 * kBackCols;       // two accumulators of the first product, then the second's
     pdl_wait();                  // inputs come from the previous kernel of the step
-    if (skip && skip[(int64_t)blockIdx.y * skip_stride]) {     // this stream's training loop has ended (block-uniform; the flag
-        tc_fence_before_sync();                                 // comes from an earlier kernel, so it is read after the wait)
+    if (skip && skip[(int64_t)s * skip_stride]) {            // this stream's training loop has ended (block-uniform)
+        tc_fence_before_sync();
         __syncthreads();
-        if (warp == 0) tmem_dealloc(tmem, tmem_cols);
+        if (warp == 0) tmem_dealloc(tmem, 512);
         return;
     }
     bool ok = true;
-
-    if (tid == 0) {
-        const uint32_t bar = smem_u32(&full);
-        mbar_expect_tx(bar, (2 + b_blocks) * blk_bytes);
-        tma_load_3d(a_base, &tmA, bar, pix0, 0, s);
-        tma_load_3d(a_base + blk_bytes, &tmA, bar, pix0 + 64, 0, s);
-        for (int cb = 0; cb < b_blocks; ++cb) tma_load_3d(b_base + cb * blk_bytes, &tmB, bar, ch0 + cb * kBlockK, 0, s);
-    } else if (tid == 32) {
-        const uint32_t idesc = instr_desc(kTileM, Chb, 1, 1);
-        ok = mbar_wait(smem_u32(&full), 0, err, kWaitFull);
-        if (ok) {
-            tc_fence_after_sync();
-#pragma unroll
-            for (int j = 0; j < kClassPad / 16; ++j)
-                umma(tmem, smem_desc(a_base + j * (16 * 128), blk_bytes, 1024), smem_desc(b_base + j * (16 * 128), blk_bytes, 1024),
-                     idesc, j != 0);
+    if (warp == 0) {
+        // ---- producer (the whole warp walks the loop, its first lane issues)
+        if (lane == 0) {
+            mbar_expect_tx(smem_u32(&w_full), kBackWBytes);
+            tma_load_3d(w_base, &tmW, smem_u32(&w_full), ch0, 0, s);
+            tma_load_3d(w_base + kClassPad * 128, &tmW, smem_u32(&w_full), ch0 + kBlockK, 0, s);
         }
-        umma_commit(smem_u32(&done));
+        for (int i = t_begin; i < t_end; ++i) {
+            const int it = i - t_begin, st = it % kBackStages;
+            if (it >= kBackStages) ok = mbar_wait(smem_u32(&empty[st]), ((it / kBackStages) - 1) & 1, err, kWaitEmpty);
+            if (!ok) break;
+            if (lane == 0) {
+                const uint32_t bar = smem_u32(&full[st]), sa = base + st * kBackStageBytes;
+                mbar_expect_tx(bar, kBackStageBytes);
+                tma_load_3d(sa + kBackActBytes, &tmD, bar, i * kTileM, 0, s);
+                tma_load_3d(sa + kBackActBytes + kClassPad * 128, &tmD, bar, i * kTileM + 64, 0, s);
+                tma_load_3d(sa, &tmH, bar, ch0, i * kTileM, s);
+                tma_load_3d(sa + kTileM * 128, &tmH, bar, ch0 + kBlockK, i * kTileM, s);
+            }
+            __syncwarp();
+        }
+    } else if (warp == 1) {
+        // ---- both products
+        ok = mbar_wait(smem_u32(&w_full), 0, err, kWaitFull);
+        const uint64_t w_mn = smem_desc(w_base, kClassPad * 128, 1024);
+        const uint32_t id1 = instr_desc(kTileM, width, 1, 1);
+        constexpr uint32_t id2 = instr_desc(kTileM, kClassPad, 1, 0);
+        for (int i = t_begin; i < t_end && ok; ++i) {
+            const int it = i - t_begin, st = it % kBackStages, buf = it & 1;
+            ok = mbar_wait(smem_u32(&full[st]), (it / kBackStages) & 1, err, kWaitFull);
+            if (ok && it >= 2) ok = mbar_wait(smem_u32(&acc_empty[buf]), ((it >> 1) - 1) & 1, err, kWaitEmpty);
+            if (!ok) break;
+            tc_fence_after_sync();
+            if (lane == 0) {
+                const uint32_t sa = base + st * kBackStageBytes, sd = sa + kBackActBytes;
+                const uint64_t dz_mn = smem_desc(sd, kClassPad * 128, 1024), dz_k = smem_desc(sd, 16, 1024), h_mn = smem_desc(sa, kTileM * 128, 1024);
+#pragma unroll
+                for (int j = 0; j < kClassPad / 16; ++j)
+                    umma(tmem + buf * kBackCols, dz_mn + j * ((16 * 128) >> 4), w_mn + j * ((16 * 128) >> 4), id1, j != 0);
+                umma_commit(smem_u32(&acc_full[buf]));
+#pragma unroll
+                for (int j = 0; j < kTileM / 16; ++j)
+                    umma(acc_w, h_mn + j * ((16 * 128) >> 4), dz_k + (j >> 2) * ((kClassPad * 128) >> 4) + (j & 3) * 2, id2, (it | j) != 0);
+                umma_commit(smem_u32(&empty[st]));
+            }
+            __syncwarp();
+        }
+        if (lane == 0) umma_commit(smem_u32(&done));
+    } else {
+        // ---- epilogue: set e takes every other tile; TMEM lanes 32*(warp % 4) .. +31 = pixels
+        const int e = (warp - 2) >> 2, q = warp & 3, groups = width / 32;
+        float sums[4] = {0.f, 0.f, 0.f, 0.f};                // lane c: sum over the warp's pixels so far of channel ch0 + 32 g + c
+        for (int i = t_begin + e; i < t_end && ok; i += 2) {
+            const int pix = i * kTileM + q * 32 + lane;
+            const bool in = pix < p;
+            uint32_t bits[4] = {0, 0, 0, 0};                 // ReLU mask of this thread's pixel, fetched while the products run
+            if (in) {
+                const uint32_t* mp = relu_bits + ((int64_t)s * p + pix) * (Ch / 32) + ch0 / 32;
+#pragma unroll
+                for (int g = 0; g < 4; ++g) if (g < groups) bits[g] = __ldg(mp + g);
+            }
+            ok = mbar_wait(smem_u32(&acc_full[e]), ((i - t_begin) >> 1) & 1, err, kWaitDone);
+            if (!ok) break;
+            tc_fence_after_sync();
+            bf16* dst = dhidden + ((int64_t)s * p + (in ? pix : 0)) * Ch + ch0;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                if (g >= groups) break;
+                float v[32];
+                tmem_ld_32x32(tmem + ((uint32_t)(q * 32) << 16) + e * kBackCols + g * 32, v);
+                uint32_t o[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {               // the mask of a pixel outside the frame is empty
+                    if (!((bits[g] >> (2 * k)) & 1u)) v[2 * k] = 0.f;
+                    if (!((bits[g] >> (2 * k + 1)) & 1u)) v[2 * k + 1] = 0.f;
+                    const __nv_bfloat162 two = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+                    o[k] = *reinterpret_cast<const uint32_t*>(&two);
+                }
+                if (in) { store_256(dst + g * 32, o); store_256(dst + g * 32 + 16, o + 8); }
+                // sums over the warp's 32 pixels, fixed order: a reduce-scatter over the lanes (lanes whose bit is set keep the
+                // upper half of the channels), after which lane c holds the sum of channel c of the group
+#pragma unroll
+                for (int half = 16; half >= 1; half >>= 1) {
+                    const bool up = (lane & half) != 0;
+#pragma unroll
+                    for (int k = 0; k < half; ++k) {
+                        const float keep = up ? v[k + half] : v[k];
+                        const float send = up ? v[k] : v[k + half];
+                        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+                    }
+                }
+                sums[g] += v[0];
+            }
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[e]));
+        }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) part[(warp - 2) * kBackCols + g * 32 + lane] = sums[g];
     }
     __syncwarp();
-    // the ReLU mask of this thread's pixel (one bit per hidden channel), fetched while the MMAs run
-    const int pix = pix0 + tid;
-    const bool in = pix < p;
-    uint32_t mbits[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (in) {
-        const uint32_t* mp = relu_bits + ((int64_t)s * p + pix) * (Ch / 32);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) if (j < Chb / 32) mbits[j] = __ldg(mp + ch0 / 32 + j);
-    }
-    ok = mbar_wait(smem_u32(&done), 0, err, kWaitDone);
-    pdl_launch_dependents();             // only the epilogue is left
+    if (!mbar_wait(smem_u32(&done), 0, err, kWaitDone)) ok = false;
+    pdl_launch_dependents();     // only the partial sums are left
     tc_fence_after_sync();
-    ok = __syncthreads_and(ok);          // the epilogue below synchronises the block: all or none
+    ok = __syncthreads_and(ok);
     if (ok) {
-        const int64_t row = ((int64_t)s * p + (in ? pix : 0)) * Ch;
-        for (int n0 = 0; n0 < Chb; n0 += 32) {
+        const int64_t row = (int64_t)s * n_split + split;
+        if (warp >= 6) {                                     // the second product: lanes = channels, columns = classes
+            const int k = (warp & 3) * 32 + lane;
             float v[32];
-            tmem_ld_32x32(tmem + ((uint32_t)(warp * 32) << 16) + n0, v);
-            if (in) {
-                uint4 out[4];
-                __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(out);
-                uint32_t bits = 0;
+            tmem_ld_32x32(acc_w + ((uint32_t)((warp & 3) * 32) << 16), v);
+            float* dst = w_partials + row * kClassPad * Ch + ch0 + k;
+            if (k < width)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) if (j == n0 / 32) bits = mbits[j];
+                for (int c = 0; c < kClassPad; ++c) dst[(int64_t)c * Ch] = v[c];
+        } else if (tid < width) {
+            float t = 0.f;
 #pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    if (!((bits >> (2 * k)) & 1u)) v[2 * k] = 0.f;
-                    if (!((bits >> (2 * k + 1)) & 1u)) v[2 * k + 1] = 0.f;
-                    o2[k] = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
-                }
-                store_256(dhidden + row + ch0 + n0, reinterpret_cast<const uint32_t*>(out));
-                store_256(dhidden + row + ch0 + n0 + 16, reinterpret_cast<const uint32_t*>(out) + 8);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 32; ++k) v[k] = 0.f;
-            }
-            // sums over the warp's 32 pixels, fixed order: a reduce-scatter over the lanes (lanes whose bit
-            // is set keep the upper half of the channels), after which lane c holds the sum of channel n0 + c
-            const int lane = tid & 31;
-#pragma unroll
-            for (int half = 16; half >= 1; half >>= 1) {
-                const bool up = (lane & half) != 0;
-#pragma unroll
-                for (int k = 0; k < half; ++k) {
-                    const float keep = up ? v[k + half] : v[k];
-                    const float send = up ? v[k] : v[k + half];
-                    v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-                }
-            }
-            part[warp * 256 + n0 + lane] = v[0];
+            for (int x = 0; x < 8; ++x) t += part[x * kBackCols + tid];
+            b_partials[row * Ch + ch0 + tid] = t;
         }
-        __syncthreads();
-        for (int k = tid; k < Chb; k += kThreadsTc)
-            b1_partials[((int64_t)s * gridDim.x + blockIdx.x) * Ch + ch0 + k] =
-                (part[k] + part[256 + k]) + (part[512 + k] + part[768 + k]);
     } else {
         drain_after_error();
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, tmem_cols);
+    if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
 // ---- host side -------------------------------------------------------------------------------------
@@ -959,8 +1024,9 @@ struct TcPlan {
     CUtensorMap dz_map;      // {p, 32, S} box {64, 32, 1}
     TcBlockPlan blk[kMaxBlocks];
     int split2, chunks2, per2, cols2, msplit2;
+    int tiles_b, per_b, split_b, groups_b;   // backward of the 1x1 layer behind a trained block: pixel tiles, tiles per range, ranges, channel groups
     int split1, chunks1, per1;          // pixel chunks of the 3x3 weight gradients (the same for every block)
-    size_t smem_fwd1, smem_fwd1p, smem_wg1, smem_dgrad;
+    size_t smem_fwd1, smem_fwd1p, smem_wg1, smem_back1;
     bool fwd1_persistent;
     int n_sms;
     bool test_stall;         // test of the give-up path (environment ST_TEST_STALL_FWD1X1=1 when the plan is made)
@@ -982,7 +1048,13 @@ int tc_wgrad_splits(int layer, int c_last, int h, int w)
     return n;
 }
 
-int tc_b1_partials(int h, int w) { return (int)(((int64_t)h * w + kTileM - 1) / kTileM); }
+// pixel ranges of the 1x1 layer's backward behind a trained hidden layer: with the groups of 128 channels about one block per SM
+int tc_back_splits(int c_last, int h, int w)
+{
+    int per, n;
+    split_geometry((int)(((int64_t)h * w + kTileM - 1) / kTileM), 148 / ((c_last + kBackCols - 1) / kBackCols), &per, &n);
+    return n;
+}
 
 int tc_tile3_count(int h, int w) { return ((w + kTileW - 1) / kTileW) * ((h + kTileH - 1) / kTileH); }
 
@@ -1099,9 +1171,12 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
     if (nb) {
         P->chunks1 = ((b.w + kChunkW - 1) / kChunkW) * ((b.h + kChunkH - 1) / kChunkH);
         split_geometry(P->chunks1, 148 / 9, &P->per1, &P->split1);
-        P->smem_dgrad = (size_t)(2 + P->c_last / kBlockK) * kClassPad * 128 + kSmemAlign;
+        P->tiles_b = (P->p + kTileM - 1) / kTileM;
+        P->groups_b = (P->c_last + kBackCols - 1) / kBackCols;
+        split_geometry(P->tiles_b, 148 / P->groups_b, &P->per_b, &P->split_b);
+        P->smem_back1 = (size_t)kBackStages * kBackStageBytes + kBackWBytes + kSmemAlign;
     }
-    if (P->c_last / kBlockK > kMaxKBlocks || (!P->fwd1_persistent && P->smem_fwd1 > lim) || P->smem_wg1 > lim || P->smem_dgrad > lim) {
+    if (P->c_last / kBlockK > kMaxKBlocks || (!P->fwd1_persistent && P->smem_fwd1 > lim) || P->smem_wg1 > lim) {
         snprintf(err, err_len, "shared memory per block exceeds 227 KB for these channel counts");
         delete P; return nullptr;
     }
@@ -1124,7 +1199,7 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         if (e == cudaSuccess && b.blk[i].pass_back) e = allow((const void*)fwd3_kernel<1>(q.stages_back), q.smem_back);
         if (e == cudaSuccess) e = allow((const void*)wgrad3_kernel(q.stages_wg), q.smem_wg);
     }
-    if (nb && e == cudaSuccess) e = allow((const void*)tc_dgrad_kernel, P->smem_dgrad);
+    if (nb && e == cudaSuccess) e = allow((const void*)tc_back1x1_kernel, P->smem_back1);
     if (e != cudaSuccess) { snprintf(err, err_len, "shared-memory attribute: %s", cudaGetErrorString(e)); delete P; return nullptr; }
     return P;
 }
@@ -1200,24 +1275,24 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
 {
     const TcBuffers& b = P->b;
     int n = 0;
-    // one-layer head: the activations are the frozen features, which no kernel of the loop writes
-    const int a_early = (!b.n_blocks && !skip && !t && b.chain_early) ? 1 : 0;
     TrainCtl no_ctl;
     memset(&no_ctl, 0, sizeof no_ctl);
-    ST_REPEAT(t) launch_chain(b.chain_early != 0, tc_wgrad1x1_kernel<kWg1Stages>, dim3(P->split2 * P->msplit2 + (ctl ? 1 : 0), b.S), dim3(kThreadsTc),
-        P->smem_wg1, s, P->act_wg, P->dz_map, b.w2_partials, P->c_last, P->chunks2, P->per2, P->msplit2, P->cols2, b.err, skip, skip_stride,
-        a_early, ctl ? 1 : 0, ctl ? *ctl : no_ctl);
-    if (t) t->mark("tc_wgrad1x1", s, st_repeats(t));
-    n += st_repeats(t);
     const int nb = b.n_blocks;
-    if (!nb || !b.blk[nb - 1].trained) return n;          // nothing is passed back into a frozen block (Section 4.2)
+    if (!nb || !b.blk[nb - 1].trained) {                  // nothing is passed back into a frozen block (Section 4.2)
+        // one-layer head: the activations are the frozen features, which no kernel of the loop writes
+        const int a_early = (!nb && !skip && !t && b.chain_early) ? 1 : 0;
+        ST_REPEAT(t) launch_chain(b.chain_early != 0, tc_wgrad1x1_kernel<kWg1Stages>, dim3(P->split2 * P->msplit2 + (ctl ? 1 : 0), b.S), dim3(kThreadsTc),
+            P->smem_wg1, s, P->act_wg, P->dz_map, b.w2_partials, P->c_last, P->chunks2, P->per2, P->msplit2, P->cols2, b.err, skip, skip_stride,
+            a_early, ctl ? 1 : 0, ctl ? *ctl : no_ctl);
+        if (t) t->mark("tc_wgrad1x1", s, st_repeats(t));
+        return n + st_repeats(t);
+    }
     {
         const TcBlock& k = b.blk[nb - 1];
-        const int blocks = tc_b1_partials(b.h, b.w);
-        const int n_ch_split = (k.c_out % 128 == 0) ? 2 : 1;      // each block: a multiple of 64 channels (four ways measured no better)
-        ST_REPEAT(t) launch_chain(b.chain_early != 0, tc_dgrad_kernel, dim3(blocks, b.S, n_ch_split), dim3(kThreadsTc), P->smem_dgrad, s,
-            P->dz_map, P->w2_map, k.relu_bits, k.dout, k.b_partials, k.c_out, P->p, pow2_cols(k.c_out / n_ch_split), b.err, skip, skip_stride);
-        if (t) t->mark("tc_dgrad", s, st_repeats(t));
+        ST_REPEAT(t) launch_chain(b.chain_early != 0, tc_back1x1_kernel, dim3(P->split_b * P->groups_b + (ctl ? 1 : 0), b.S), dim3(kBackThreads),
+            P->smem_back1, s, P->act_fwd, P->dz_map, P->w2_map, k.relu_bits, k.dout, k.b_partials, b.w2_partials, k.c_out, P->p, P->tiles_b,
+            P->per_b, P->groups_b, b.err, skip, skip_stride, ctl ? 1 : 0, ctl ? *ctl : no_ctl);
+        if (t) t->mark("tc_back1x1", s, st_repeats(t));
         n += st_repeats(t);
     }
     const int total = tc_tile3_count(b.h, b.w) * b.S;

@@ -339,8 +339,8 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
 template <bool ADAM>
 static int launch_sgd_update_t(const UpdateArgs& a, cudaStream_t s)
 {
-    // Large layers are streamed, everything else (small layers, biases, loss) goes through the grouped part.  One launch: the grouped part is all latency and hides behind the stream
-    // (256 -> 256 channels, 3x3: 19.9 us as two launches, 14.3 us as one, launch gap included).
+    // Large layers are streamed, everything else (small layers, biases, loss) goes through the grouped part.  One launch: the
+    // grouped part is all latency and hides behind the stream (256 -> 256 channels, 3x3: 19.9 us as two launches, 14.3 us as one, launch gap included).
     UpdateArgs g = a;
     int64_t stream_blocks = 0, n_rest = 0;
     for (int L = 0; L < a.n_layers; ++L) {

@@ -641,7 +641,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
         c->dz_pitch = tc_dz_pitch(c->h, c->w);
         ALLOC(dz_bf16, (size_t)S * kClassPad * c->dz_pitch);
         ALLOC(w2_shadow, (size_t)S * kClassPad * c_last);
-        c->n_split2 = tc_wgrad_splits(2, c_last, c->h, c->w);
+        c->n_split2 = n_blocks > first_trained ? tc_back_splits(c_last, c->h, c->w) : tc_wgrad_splits(2, c_last, c->h, c->w);
         ALLOC(w2_partials, (size_t)S * c->n_split2 * kClassPad * c_last);
         c->n_split1 = n_blocks ? tc_wgrad_splits(1, 0, c->h, c->w) : 0;
         for (int i = 0; i < n_blocks; ++i) {
@@ -655,9 +655,9 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             if (trained) {
                 ALLOC(blk[i].dout, S * c->p * k.c_out);
                 ALLOC(blk[i].w_partials, (size_t)S * c->n_split1 * 9 * k.c_out * tot);
-                // the block in front of the classifier gets its gradient from the 128-pixel tiles of the 1x1 layer's
-                // kernel, the others from the 4 x 32 tiles of the 3x3 tile walk
-                k.n_bpart = i == n_blocks - 1 ? tc_b1_partials(c->h, c->w) : tc_tile3_count(c->h, c->w);
+                // the block in front of the classifier gets its gradient from the 1x1 layer's backward kernel, the others from
+                // the 4 x 32 tiles of the 3x3 tile walk
+                k.n_bpart = i == n_blocks - 1 ? c->n_split2 : tc_tile3_count(c->h, c->w);
                 ALLOC(blk[i].b_partials, (size_t)S * k.n_bpart * k.c_out);
                 if (i > first_trained) ALLOC(blk[i].w_t, (size_t)S * 9 * k.c_prev * k.c_out);
             }
