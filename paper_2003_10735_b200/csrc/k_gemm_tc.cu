@@ -754,19 +754,21 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
 // weight rows [c][k] and activation rows [pix][k] are MN-major.  A ring of stages (producer warp), one warp that issues both
 // products, two sets of four warps that drain the two accumulators of the first in turn; the second accumulates over the
 // whole range, which leaves one partial sum per block, like the bias gradient.
-// Bound by L2: at 720p and 256 channels 29 MB of activations come in and as much gradient goes out, 16.8 us (4 TB/s).  As two
-// kernels (gradient: a block per 128 pixels and half of the channels; weight gradient: a pass of its own) 18.8 + 9.7 us;
-// at 1080p 33.3 + 15.1 us, now 33.0.
+// Bound by L2: at 720p and 256 channels 29 MB of activations come in and as much gradient goes out, 12.9 us (5 TB/s); 16.8 us
+// with 32-byte stores straight from the accumulator rows, which go out through shared memory and TMA instead.  As two kernels
+// (gradient: a block per 128 pixels and half of the channels; weight gradient: a pass of its own) 18.8 + 9.7 us; at 1080p
+// 33.3 + 15.1 us, now 28.1.  Bias sums kept in registers over the tiles cost the narrow layers 2 us and gained nothing.
 // ------------------------------------------------------------------------------------------------
-constexpr int kBackStages = 4, kBackThreads = 320, kBackCols = 128;
-constexpr uint32_t kBackActBytes = kTileM * 128 * 2, kBackDzBytes = 2 * kClassPad * 128, kBackStageBytes = kBackActBytes + kBackDzBytes, kBackWBytes = 2 * kClassPad * 128;
+constexpr int kBackStages = 3, kBackThreads = 320, kBackCols = 128;
+constexpr uint32_t kBackActBytes = kTileM * 128 * 2, kBackDzBytes = 2 * kClassPad * 128, kBackStageBytes = kBackActBytes + kBackDzBytes, kBackWBytes = 2 * kClassPad * 128,
+                   kBackOutBytes = 8 * 32 * kBackCols * 2;   // a 32 x 128 piece of the gradient for each epilogue warp
 
 __global__ void __launch_bounds__(kBackThreads, 1)
 tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  box {64, 128, 1}
                   const __grid_constant__ CUtensorMap tmD,   // dz {p, 32, S}  box {64, 32, 1}
                   const __grid_constant__ CUtensorMap tmW,   // W2 {Ch, 32, S} box {64, 32, 1}
+                  const __grid_constant__ CUtensorMap tmO,   // dHd {Ch, p, S} box {64, 32, 1}
                   const uint32_t* __restrict__ relu_bits,     // [S][p][Ch/32]
-                  bf16* __restrict__ dhidden,                 // [S][p][Ch]
                   float* __restrict__ b_partials,             // [S][n_split][Ch]
                   float* __restrict__ w_partials,             // [S][n_split][32][Ch]
                   int Ch, int p, int n_tiles, int per, int n_groups, unsigned int* err, const int* __restrict__ skip, int64_t skip_stride,
@@ -861,6 +863,7 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
     } else {
         // ---- epilogue: set e takes every other tile; TMEM lanes 32*(warp % 4) .. +31 = pixels
         const int e = (warp - 2) >> 2, q = warp & 3, groups = width / 32;
+        const uint32_t out_base = w_base + kBackWBytes + (warp - 2) * (32 * kBackCols * 2);
         float sums[4] = {0.f, 0.f, 0.f, 0.f};                // lane c: sum over the warp's pixels so far of channel ch0 + 32 g + c
         for (int i = t_begin + e; i < t_end && ok; i += 2) {
             const int pix = i * kTileM + q * 32 + lane;
@@ -874,7 +877,8 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
             ok = mbar_wait(smem_u32(&acc_full[e]), ((i - t_begin) >> 1) & 1, err, kWaitDone);
             if (!ok) break;
             tc_fence_after_sync();
-            bf16* dst = dhidden + ((int64_t)s * p + (in ? pix : 0)) * Ch + ch0;
+            if (lane == 0) tma_store_wait_read<0>();         // this warp's piece of the tile before last has been read
+            __syncwarp();
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 if (g >= groups) break;
@@ -888,7 +892,14 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
                     const __nv_bfloat162 two = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
                     o[k] = *reinterpret_cast<const uint32_t*>(&two);
                 }
-                if (in) { store_256(dst + g * 32, o); store_256(dst + g * 32 + 16, o + 8); }
+                const uint32_t orow = out_base + (g >> 1) * 4096 + lane * 128;      // 128-byte swizzle: 16-byte chunks ^ (row % 8)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) st_shared_128(orow + ((((g & 1) * 4 + k) ^ (lane & 7)) << 4), o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+                if (g & 1) {                                  // widths are multiples of 64
+                    fence_async_shared();
+                    __syncwarp();
+                    if (lane == 0 && pix < p) { tma_store_3d(&tmO, out_base + (g >> 1) * 4096, ch0 + (g >> 1) * 64, pix, s); tma_store_commit(); }
+                }
                 // sums over the warp's 32 pixels, fixed order: a reduce-scatter over the lanes (lanes whose bit is set keep the
                 // upper half of the channels), after which lane c holds the sum of channel c of the group
 #pragma unroll
@@ -907,6 +918,7 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&acc_empty[e]));
         }
+        if (lane == 0) tma_store_wait();
 #pragma unroll
         for (int g = 0; g < 4; ++g) part[(warp - 2) * kBackCols + g * 32 + lane] = sums[g];
     }
@@ -1022,6 +1034,7 @@ struct TcPlan {
     CUtensorMap act_wg;      // same tensor, box {64, 64, 1}
     CUtensorMap w2_map;      // {c_last, 32, S} box {64, 32, 1}
     CUtensorMap dz_map;      // {p, 32, S} box {64, 32, 1}
+    CUtensorMap dout_map;    // gradient of the last-layer input, where it is formed: {c_last, p, S} box {64, 32, 1}
     TcBlockPlan blk[kMaxBlocks];
     int split2, chunks2, per2, cols2, msplit2;
     int tiles_b, per_b, split_b, groups_b;   // backward of the 1x1 layer behind a trained block: pixel tiles, tiles per range, ranges, channel groups
@@ -1081,6 +1094,9 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         uint32_t box_f[3] = {64, 128, 1}, box_w[3] = {64, 64, 1};
         ok = ok && make_map(&P->act_fwd, act, 3, dims, str, box_f, err, err_len, "last-layer input (forward)");
         ok = ok && make_map(&P->act_wg, act, 3, dims, str, box_w, err, err_len, "last-layer input (wgrad)");
+        uint32_t box_o[3] = {64, 32, 1};
+        if (nb && b.blk[nb - 1].trained)
+            ok = ok && make_map(&P->dout_map, b.blk[nb - 1].dout, 3, dims, str, box_o, err, err_len, "last-layer input gradient");
     }
     if (ok) {
         uint64_t dims[3] = {cl, (uint64_t)kClassPad, S}, str[2] = {cl * 2, (uint64_t)kClassPad * cl * 2};
@@ -1174,7 +1190,7 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         P->tiles_b = (P->p + kTileM - 1) / kTileM;
         P->groups_b = (P->c_last + kBackCols - 1) / kBackCols;
         split_geometry(P->tiles_b, 148 / P->groups_b, &P->per_b, &P->split_b);
-        P->smem_back1 = (size_t)kBackStages * kBackStageBytes + kBackWBytes + kSmemAlign;
+        P->smem_back1 = (size_t)kBackStages * kBackStageBytes + kBackWBytes + kBackOutBytes + kSmemAlign;
     }
     if (P->c_last / kBlockK > kMaxKBlocks || (!P->fwd1_persistent && P->smem_fwd1 > lim) || P->smem_wg1 > lim) {
         snprintf(err, err_len, "shared memory per block exceeds 227 KB for these channel counts");
@@ -1290,7 +1306,7 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
     {
         const TcBlock& k = b.blk[nb - 1];
         ST_REPEAT(t) launch_chain(b.chain_early != 0, tc_back1x1_kernel, dim3(P->split_b * P->groups_b + (ctl ? 1 : 0), b.S), dim3(kBackThreads),
-            P->smem_back1, s, P->act_fwd, P->dz_map, P->w2_map, k.relu_bits, k.dout, k.b_partials, b.w2_partials, k.c_out, P->p, P->tiles_b,
+            P->smem_back1, s, P->act_fwd, P->dz_map, P->w2_map, P->dout_map, k.relu_bits, k.b_partials, b.w2_partials, k.c_out, P->p, P->tiles_b,
             P->per_b, P->groups_b, b.err, skip, skip_stride, ctl ? 1 : 0, ctl ? *ctl : no_ctl);
         if (t) t->mark("tc_back1x1", s, st_repeats(t));
         n += st_repeats(t);
