@@ -310,9 +310,9 @@ st_status enqueue_forward(st_ctx* c, StageTimer* t = nullptr, const int* skip = 
 st_status tag_labels(st_ctx* c, int32_t stream)
 {
     if (c->heavy_w <= 1) return ST_OK;
-    launch_object_weight_tags(c->labels + (int64_t)stream * c->P, c->H, c->W, c->background, c->heavy_radius, c->mask_tmp,
+    launch_object_weight_tags(c->labels + (int64_t)stream * c->P, c->H, c->W, c->background, c->heavy_radius,
                               c->labels_tagged + (int64_t)stream * c->P, c->stream);
-    c->launches += 2;
+    c->launches += 1;
     return check_launch(c, "object weights");
 }
 

@@ -82,9 +82,8 @@ void launch_feat_to_bf16_nhwc(const float* feat_chw, int Cin, int64_t p, bf16* o
 void launch_nhwc_bf16_to_chw(const bf16* in, int C, int64_t p, float* out, cudaStream_t s);
 
 // ---- loss weighting near objects: labels [H][W] of one stream -> labels with bit 7 set where the pixel is within
-// `radius` of a non-background pixel; tmp is a scratch map of H*W bytes
-void launch_object_weight_tags(const uint8_t* labels, int H, int W, int background, int radius, uint8_t* tmp, uint8_t* tagged,
-                               cudaStream_t s);
+// `radius` (at most 64) of a non-background pixel; W is a multiple of 4
+void launch_object_weight_tags(const uint8_t* labels, int H, int W, int background, int radius, uint8_t* tagged, cudaStream_t s);
 
 // ---- K3: upsample x4 + softmax cross-entropy + gradient w.r.t. the low-res logits ---------------
 struct UpsampleCeArgs {
