@@ -419,6 +419,10 @@ tc_fwd1x1p_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {
 // The K loop runs over 9 taps x (kblocks1 + kblocks2) channel blocks: the first kblocks1 come from tmA (the previous
 // block's output, or the frozen part's), the others from tmA2 (the block's skip input): the concatenation of
 // Section 5.2 is never materialised.
+// Bound by the tensor pipe at 256 channels (0.9 of the measured peak inside a round of tiles; 53.8 us at 720p), by the issue
+// of copies and MMAs at 64 and 128 (29.4, 33.3 us).  With the issuing lane picked by number instead of elect_one 57.5, 39.7
+// and 42.5 us.  One slab of pixels per horizontal shift for the three taps above each other halves the activation traffic
+// but adds waits to the chain: 68, 50, 54 us, not kept.
 template <int STAGES, int MODE>
 __global__ void __launch_bounds__(kFwd3Threads)
 tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}     box {64, 32, 4, 1}
@@ -442,7 +446,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_slot;
     __shared__ float part[MODE == 1 ? 4 * 256 : 1];             // MODE 1: per-warp channel sums of the tile
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int tiles_x = (w + kTileW - 1) / kTileW, tiles_y = (h + kTileH - 1) / kTileH;
     const int tiles_per_stream = tiles_x * tiles_y;
     const int kblocks = kblocks1 + kblocks2, n_iter = 9 * kblocks;
@@ -486,7 +490,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
                 const int st = g % STAGES;                                                                                \
                 if (g >= STAGES) ok = mbar_wait(smem_u32(&empty[st]), ((g / STAGES) - 1) & 1, err, kWaitEmpty);          \
                 if (!ok) break;                                                                                           \
-                if (lane == 0) {                                                                                          \
+                if (elect_one()) {                                                                                        \
                 const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;                                   \
                 mbar_expect_tx(bar, a_bytes + (uint32_t)im.chn * 128);                                                    \
                 tma_load_4d(sa, &(src), bar, (a_coord), x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);                          \
@@ -523,7 +527,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
                 ok = mbar_wait(smem_u32(&full[st]), (g / STAGES) & 1, err, kWaitFull);
                 if (!ok) break;
                 tc_fence_after_sync();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint64_t da = smem_desc(base + st * stage_bytes, 16, 1024), db = da + (a_bytes >> 4);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) umma(acc, da + 2 * k, db + 2 * k, idesc, (it | k) != 0);
@@ -531,7 +535,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
                 }
                 __syncwarp();
             }
-            if (ok && lane == 0) umma_commit(smem_u32(&acc_full[buf]));
+            if (ok && elect_one()) umma_commit(smem_u32(&acc_full[buf]));
             __syncwarp();
             ++j;                                                       // j counts the tiles this block works on
         }
@@ -634,7 +638,9 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
 // wgrad 3x3: for one tap, D[ci][co] += sum over this block's pixel chunks of X[pix+tap][ci] * dHd[pix][co].
 // Both operands are MN-major (pixel-major activations, reduction over pixels).  A block keeps
 // ceil(Cin/128) accumulators of Ch columns (all input channels of one tap) so that the dHd tile of a
-// stage is shared by all of them.
+// stage is shared by all of them.  Bound by the issue of copies and MMAs, like the forward: with producer and issuer as single
+// threads 51.4 us at 720p and 256 channels, 37 and 41 us in a stack of 64 and 128; as whole warps with elect_one 47.5, 29.4
+// and 32.5 us.
 // ------------------------------------------------------------------------------------------------
 template <int STAGES>
 __global__ void __launch_bounds__(kThreadsTc)
@@ -656,7 +662,7 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     const uint32_t a_bytes = a_blocks * blk_bytes, stage_bytes = a_bytes + b_blocks * blk_bytes;
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int tap = blockIdx.x % 9, split = blockIdx.x / 9, s = blockIdx.y;
     const int chunks_x = (w + kChunkW - 1) / kChunkW;
     const int c_begin = split * chunks_per_block, c_end = min(n_chunks, c_begin + chunks_per_block);
@@ -680,43 +686,46 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     }
     bool ok = true;
 
-    if (tid == 0) {
+    if (warp == 0) {             // producer and issuer walk their loops as whole warps, one lane issues
         for (int i = c_begin; i < c_end; ++i) {
             const int it = i - c_begin, st = it % STAGES;
             if (it >= STAGES) ok = mbar_wait(smem_u32(&empty[st]), ((it / STAGES) - 1) & 1, err, kWaitEmpty);
             if (!ok) break;
             const int x0 = (i % chunks_x) * kChunkW, y0 = (i / chunks_x) * kChunkH;
-            const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;
-            mbar_expect_tx(bar, stage_bytes);
-            // blocks past the last channel arrive as zeros (out-of-range fill); two loops, each with its own tensor map
-            // (a map chosen at run time costs every copy a slow look-up)
-            const int n_first = blocks1 * kBlockK == Cin ? a_blocks : blocks1;
-            int cb = 0;
-            for (; cb < n_first; ++cb)
-                tma_load_4d(sa + cb * blk_bytes, &tmA, bar, cb * kBlockK, x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);
-            for (; cb < a_blocks; ++cb)
-                tma_load_4d(sa + cb * blk_bytes, &tmA2, bar, (cb - blocks1) * kBlockK, x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);
-            for (int cb = 0; cb < b_blocks; ++cb)
-                tma_load_4d(sa + a_bytes + cb * blk_bytes, &tmB, bar, cb * kBlockK, x0, y0, s);
+            if (elect_one()) {
+                const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;
+                mbar_expect_tx(bar, stage_bytes);
+                // blocks past the last channel arrive as zeros (out-of-range fill); two loops, each with its own tensor map
+                // (a map chosen at run time costs every copy a slow look-up)
+                const int n_first = blocks1 * kBlockK == Cin ? a_blocks : blocks1;
+                int cb = 0;
+                for (; cb < n_first; ++cb)
+                    tma_load_4d(sa + cb * blk_bytes, &tmA, bar, cb * kBlockK, x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);
+                for (; cb < a_blocks; ++cb)
+                    tma_load_4d(sa + cb * blk_bytes, &tmA2, bar, (cb - blocks1) * kBlockK, x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);
+                for (int cb = 0; cb < b_blocks; ++cb)
+                    tma_load_4d(sa + a_bytes + cb * blk_bytes, &tmB, bar, cb * kBlockK, x0, y0, s);
+            }
+            __syncwarp();
         }
-    } else if (tid == 32) {
+    } else if (warp == 1) {
         const uint32_t idesc = instr_desc(kTileM, Ch, 1, 1);
         for (int i = c_begin; i < c_end; ++i) {
             const int it = i - c_begin, st = it % STAGES;
             ok = mbar_wait(smem_u32(&full[st]), (it / STAGES) & 1, err, kWaitFull);
             if (!ok) break;
             tc_fence_after_sync();
-            const uint32_t sa = base + st * stage_bytes, sb = sa + a_bytes;
-            for (int m = 0; m < m_tiles; ++m)
+            if (elect_one()) {
+                const uint64_t da = smem_desc(base + st * stage_bytes, blk_bytes, 1024), db = da + (a_bytes >> 4);
+                for (int m = 0; m < m_tiles; ++m)
 #pragma unroll
-                for (int j = 0; j < kChunkPix / 16; ++j) {
-                    const uint64_t da = smem_desc(sa + (2 * m) * blk_bytes + j * (16 * 128), blk_bytes, 1024);
-                    const uint64_t db = smem_desc(sb + j * (16 * 128), blk_bytes, 1024);
-                    umma(tmem + m * Ch, da, db, idesc, (it | j) != 0);
-                }
-            umma_commit(smem_u32(&empty[st]));
+                    for (int j = 0; j < kChunkPix / 16; ++j)
+                        umma(tmem + m * Ch, da + ((2 * m * blk_bytes + j * (16 * 128)) >> 4), db + j * ((16 * 128) >> 4), idesc, (it | j) != 0);
+                umma_commit(smem_u32(&empty[st]));
+            }
+            __syncwarp();
         }
-        umma_commit(smem_u32(&done));
+        if (elect_one()) umma_commit(smem_u32(&done));
     }
     __syncwarp();
     ok = mbar_wait(smem_u32(&done), 0, err, kWaitDone);
@@ -789,7 +798,7 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
     __shared__ __align__(8) uint64_t full[kBackStages], empty[kBackStages], w_full, acc_full[2], acc_empty[2], done;
     __shared__ uint32_t tmem_slot;
     __shared__ float part[8 * kBackCols];                        // per-warp channel sums
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int n_split = ((int)gridDim.x - (has_ctl ? 1 : 0)) / n_groups, split = (int)blockIdx.x / n_groups, ch0 = (int)blockIdx.x % n_groups * kBackCols;
     const int t_begin = split * per, t_end = min(n_tiles, t_begin + per), width = min(kBackCols, Ch - ch0);
 
@@ -814,7 +823,7 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
     bool ok = true;
     if (warp == 0) {
         // ---- producer (the whole warp walks the loop, its first lane issues)
-        if (lane == 0) {
+        if (elect_one()) {
             mbar_expect_tx(smem_u32(&w_full), kBackWBytes);
             tma_load_3d(w_base, &tmW, smem_u32(&w_full), ch0, 0, s);
             tma_load_3d(w_base + kClassPad * 128, &tmW, smem_u32(&w_full), ch0 + kBlockK, 0, s);
@@ -823,7 +832,7 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
             const int it = i - t_begin, st = it % kBackStages;
             if (it >= kBackStages) ok = mbar_wait(smem_u32(&empty[st]), ((it / kBackStages) - 1) & 1, err, kWaitEmpty);
             if (!ok) break;
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t bar = smem_u32(&full[st]), sa = base + st * kBackStageBytes;
                 mbar_expect_tx(bar, kBackStageBytes);
                 tma_load_3d(sa + kBackActBytes, &tmD, bar, i * kTileM, 0, s);
@@ -845,7 +854,7 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
             if (ok && it >= 2) ok = mbar_wait(smem_u32(&acc_empty[buf]), ((it >> 1) - 1) & 1, err, kWaitEmpty);
             if (!ok) break;
             tc_fence_after_sync();
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t sa = base + st * kBackStageBytes, sd = sa + kBackActBytes;
                 const uint64_t dz_mn = smem_desc(sd, kClassPad * 128, 1024), dz_k = smem_desc(sd, 16, 1024), h_mn = smem_desc(sa, kTileM * 128, 1024);
 #pragma unroll
@@ -859,7 +868,7 @@ tc_back1x1_kernel(const __grid_constant__ CUtensorMap tmH,   // Hd {Ch, p, S}  b
             }
             __syncwarp();
         }
-        if (lane == 0) umma_commit(smem_u32(&done));
+        if (elect_one()) umma_commit(smem_u32(&done));
     } else {
         // ---- epilogue: set e takes every other tile; TMEM lanes 32*(warp % 4) .. +31 = pixels
         const int e = (warp - 2) >> 2, q = warp & 3, groups = width / 32;

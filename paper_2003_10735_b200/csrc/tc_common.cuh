@@ -39,6 +39,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// One lane of a converged warp, chosen so that the compiler knows it to be one: the operands of copies and MMAs then stay in
+// uniform registers.  Behind `lane == 0` the issue of four MMAs and a commit took 300 cycles, and the rings of the 3x3
+// kernels turned at 583 cycles per stage whatever the layer's width.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    return one != 0;
+}
 // Bounded wait; on give-up writes `code` (tagged with the block) into *err and returns false.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned int* err, unsigned int code,
                                           uint32_t limit = kSpinLimit)
