@@ -62,7 +62,7 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
     float m_loc = -INFINITY;
     uint32_t tmem;
     constexpr int TW = kTileCols, TZ = kTile, RN_Y = kOwnRows, RN_X = kOwnCols;
-    const int tid = threadIdx.x, wi = tid >> 5, l = tid & 31;
+    const int tid = threadIdx.x, wi = __shfl_sync(0xffffffffu, tid >> 5, 0), l = tid & 31;
     const int C = a.C, h = a.h, w = a.w;
     const int64_t p = (int64_t)h * w;
     const uint32_t ring = tc::smem_u32(zt), w_base = ring + kStages * kStageBytes;
@@ -82,14 +82,14 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
     tmem = sh.tmem_slot;
     const int kblocks = a.kblocks;
     const int n_pre = a.x_early ? min(kStages, kblocks) : 0;
-    if (tid == 0)
+    if (wi == 0 && tc::elect_one())
         for (int kb = 0; kb < n_pre; ++kb) {
             tc::mbar_expect_tx(full_bar(kb), kStageBytes + (kb == 0 ? a.stall_bytes : 0u));
             tc::tma_load_4d(ring + kb * kStageBytes, x_map, full_bar(kb), kb * 64, x0 - 1, y0 - 1, s);
         }
     pdl_wait();                                        // the weights come from the previous kernel of the stream
     if (a.skip && *a.skip) {                           // this stream's training loop has ended (block-uniform)
-        if (tid == 0)                                   // copies already on their way land before shared memory is given back
+        if (wi == 0)                                    // copies already on their way land before shared memory is given back
             for (int kb = 0; kb < n_pre; ++kb) tc::mbar_wait(full_bar(kb), 0, a.err, tc::kWaitFull);
         tc::tc_fence_before_sync();
         __syncthreads();
@@ -98,18 +98,22 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
     }
     if (tid < kClassPad) sh.bias[tid] = tid < C ? a.bias[tid] : 0.f;
     bool ok = true;
-    if (tid == 0) {
-        tc::mbar_expect_tx(w_bar, (uint32_t)kblocks * kWeightBytes);
-        for (int kb = 0; kb < kblocks; ++kb) tc::tma_load_3d(w_base + kb * kWeightBytes, w_map, w_bar, kb * 64, 0, s);
+    if (wi == 0) {               // producer and issuer walk their loops as whole warps, one lane issues
+        if (tc::elect_one()) {
+            tc::mbar_expect_tx(w_bar, (uint32_t)kblocks * kWeightBytes);
+            for (int kb = 0; kb < kblocks; ++kb) tc::tma_load_3d(w_base + kb * kWeightBytes, w_map, w_bar, kb * 64, 0, s);
+        }
+        __syncwarp();
         for (int kb = n_pre; kb < kblocks && ok; ++kb) {
             const int st = kb % kStages;
             if (kb >= kStages) ok = tc::mbar_wait(empty_bar(st), ((kb / kStages) - 1) & 1, a.err, tc::kWaitEmpty);
-            if (ok) {
+            if (ok && tc::elect_one()) {
                 tc::mbar_expect_tx(full_bar(st), kStageBytes + (kb == 0 ? a.stall_bytes : 0u));
                 tc::tma_load_4d(ring + st * kStageBytes, x_map, full_bar(st), kb * 64, x0 - 1, y0 - 1, s);
             }
+            __syncwarp();
         }
-    } else if (tid == 32) {
+    } else if (wi == 1) {
         constexpr uint32_t idesc = tc::instr_desc(128, kClassPad, 0, 0);
         ok = tc::mbar_wait(w_bar, 0, a.err, tc::kWaitFull);
         for (int kb = 0; kb < kblocks && ok; ++kb) {
@@ -117,16 +121,18 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
             ok = tc::mbar_wait(full_bar(st), (kb / kStages) & 1, a.err, tc::kWaitFull, a.spin_limit);
             if (!ok) break;
             tc::tc_fence_after_sync();
+            if (tc::elect_one()) {
+                const uint64_t dx = tc::smem_desc(ring + st * kStageBytes, 16, 1024), dw = tc::smem_desc(w_base + kb * kWeightBytes, 16, 1024);
 #pragma unroll
-            for (int m = 0; m < 3; ++m)
+                for (int m = 0; m < 3; ++m)
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    tc::umma(tmem + m * kClassPad, tc::smem_desc(ring + st * kStageBytes + m * (128 * 128) + k * 32, 16, 1024),
-                             tc::smem_desc(w_base + kb * kWeightBytes + k * 32, 16, 1024), idesc, (kb | k) != 0);
-            tc::umma_commit(empty_bar(st));
+                    for (int k = 0; k < 4; ++k) tc::umma(tmem + m * kClassPad, dx + ((m * (128 * 128)) >> 4) + 2 * k, dw + 2 * k, idesc, (kb | k) != 0);
+                tc::umma_commit(empty_bar(st));
+            }
+            __syncwarp();
         }
         if (!ok) sh.gave_up = 1;
-        tc::umma_commit(done_bar);
+        if (tc::elect_one()) tc::umma_commit(done_bar);
     }
     __syncwarp();
     ok = tc::mbar_wait(done_bar, 0, a.err, tc::kWaitDone);

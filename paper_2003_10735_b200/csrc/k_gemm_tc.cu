@@ -66,7 +66,7 @@ tc_fwd1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {6
     const uint32_t b_base = a_base + kblocks * (kTileM * 128);
     __shared__ __align__(8) uint64_t bars[kMaxKBlocks + 1];
     __shared__ uint32_t tmem_slot, gave_up;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int s = blockIdx.y, pix0 = blockIdx.x * kTileM;
 
     if (warp == 0) tmem_alloc(smem_u32(&tmem_slot), 32);
@@ -82,7 +82,7 @@ tc_fwd1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {6
     // a_early: the kernel before this one on the stream (the previous iteration's parameter update) writes the weights
     // but not the activations, and this kernel was launched to start while that one still runs: the activation tile
     // is fetched now, the weights after the wait.  Each barrier expects both parts.
-    if (a_early && tid == 0) {
+    if (a_early && warp == 0 && elect_one()) {
         for (int kb = 0; kb < kblocks; ++kb) {
             const uint32_t bar = smem_u32(&bars[kb]);
             mbar_expect_tx(bar, kTileM * 128 + kClassPad * 128 + (kb == 0 ? stall_bytes : 0u));
@@ -99,7 +99,8 @@ tc_fwd1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {6
     const uint32_t done_bar = smem_u32(&bars[kblocks]);
     bool ok = true;
 
-    if (tid == 0) {
+    if (warp == 0) {
+        if (elect_one())
         for (int kb = 0; kb < kblocks; ++kb) {
             const uint32_t bar = smem_u32(&bars[kb]);
             if (!a_early) {
@@ -108,20 +109,20 @@ tc_fwd1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {6
             }
             tma_load_3d(b_base + kb * (kClassPad * 128), &tmB, bar, kb * kBlockK, 0, s);
         }
-    } else if (tid == 32) {
+    } else if (warp == 1) {
         constexpr uint32_t idesc = instr_desc(kTileM, kClassPad, 0, 0);
         for (int kb = 0; kb < kblocks; ++kb) {
             ok = mbar_wait(smem_u32(&bars[kb]), 0, err, kWaitFull, spin_limit);
             if (!ok) { gave_up = 1; break; }
             tc_fence_after_sync();
+            if (elect_one()) {
+                const uint64_t da = smem_desc(a_base + kb * (kTileM * 128), 16, 1024), db = smem_desc(b_base + kb * (kClassPad * 128), 16, 1024);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint64_t da = smem_desc(a_base + kb * (kTileM * 128) + k * 32, 16, 1024);
-                const uint64_t db = smem_desc(b_base + kb * (kClassPad * 128) + k * 32, 16, 1024);
-                umma(tmem, da, db, idesc, (kb | k) != 0);
+                for (int k = 0; k < 4; ++k) umma(tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
             }
+            __syncwarp();
         }
-        umma_commit(done_bar);
+        if (elect_one()) umma_commit(done_bar);
     }
     __syncwarp();
     ok = mbar_wait(done_bar, 0, err, kWaitDone);
@@ -185,7 +186,7 @@ tc_wgrad1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}      
     const uint32_t base = smem_u32(smem);
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int s = blockIdx.y, split = (int)blockIdx.x / m_split, n_split = n_blocks_x / m_split;
     const int c_begin = split * chunks_per_block;
     const int c_end = min(n_chunks, c_begin + chunks_per_block);
@@ -204,7 +205,7 @@ tc_wgrad1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}      
     // launched while its predecessor (which produces the logit gradient) is still running: the activation part of the
     // first stages is fetched now, the gradient part after the wait.  Each barrier expects both parts.
     const int n_pre = a_early ? min(STAGES, c_end - c_begin) : 0;
-    if (tid == 0)
+    if (warp == 0 && elect_one())
         for (int it = 0; it < n_pre; ++it) {
             const uint32_t bar = smem_u32(&full[it]), sa = base + it * stage_bytes;
             mbar_expect_tx(bar, stage_bytes);
@@ -220,38 +221,40 @@ tc_wgrad1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}      
     }
     bool ok = true;
 
-    if (tid == 0) {
+    if (warp == 0) {
         for (int i = c_begin; i < c_end; ++i) {
             const int it = i - c_begin, st = it % STAGES;
             if (it >= STAGES) ok = mbar_wait(smem_u32(&empty[st]), ((it / STAGES) - 1) & 1, err, kWaitEmpty);
             if (!ok) break;
-            const uint32_t bar = smem_u32(&full[st]);
-            const uint32_t sa = base + st * stage_bytes;
-            if (it >= n_pre) {
-                mbar_expect_tx(bar, stage_bytes);
-                for (int cb = 0; cb < a_blocks; ++cb)
-                    tma_load_3d(sa + cb * (kChunkPix * 128), &tmA, bar, (2 * m0 + cb) * kBlockK, i * kChunkPix, s);
+            if (elect_one()) {
+                const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;
+                if (it >= n_pre) {
+                    mbar_expect_tx(bar, stage_bytes);
+                    for (int cb = 0; cb < a_blocks; ++cb)
+                        tma_load_3d(sa + cb * (kChunkPix * 128), &tmA, bar, (2 * m0 + cb) * kBlockK, i * kChunkPix, s);
+                }
+                tma_load_3d(sa + a_stage_bytes, &tmB, bar, i * kChunkPix, 0, s);
             }
-            tma_load_3d(sa + a_stage_bytes, &tmB, bar, i * kChunkPix, 0, s);
+            __syncwarp();
         }
-    } else if (tid == 32) {
+    } else if (warp == 1) {
         constexpr uint32_t idesc = instr_desc(kTileM, kClassPad, 1, 0);
         for (int i = c_begin; i < c_end; ++i) {
             const int it = i - c_begin, st = it % STAGES;
             ok = mbar_wait(smem_u32(&full[st]), (it / STAGES) & 1, err, kWaitFull);
             if (!ok) break;
             tc_fence_after_sync();
-            const uint32_t sa = base + st * stage_bytes, sb = sa + a_stage_bytes;
-            for (int m = 0; m < m_tiles; ++m)
+            if (elect_one()) {
+                const uint64_t da = smem_desc(base + st * stage_bytes, kChunkPix * 128, 1024), db = smem_desc(base + st * stage_bytes + a_stage_bytes, 16, 1024);
+                for (int m = 0; m < m_tiles; ++m)
 #pragma unroll
-                for (int j = 0; j < kChunkPix / 16; ++j) {
-                    const uint64_t da = smem_desc(sa + (2 * m) * (kChunkPix * 128) + j * (16 * 128), kChunkPix * 128, 1024);
-                    const uint64_t db = smem_desc(sb + j * 32, 16, 1024);
-                    umma(tmem + m * kClassPad, da, db, idesc, (it | j) != 0);
-                }
-            umma_commit(smem_u32(&empty[st]));
+                    for (int j = 0; j < kChunkPix / 16; ++j)
+                        umma(tmem + m * kClassPad, da + ((2 * m * (kChunkPix * 128) + j * (16 * 128)) >> 4), db + 2 * j, idesc, (it | j) != 0);
+                umma_commit(smem_u32(&empty[st]));
+            }
+            __syncwarp();
         }
-        umma_commit(smem_u32(&done));
+        if (elect_one()) umma_commit(smem_u32(&done));
     }
     __syncwarp();
     ok = mbar_wait(smem_u32(&done), 0, err, kWaitDone);
@@ -316,7 +319,7 @@ tc_fwd1x1p_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {
     const uint32_t b_base = a_base + kF1Stages * kF1StageBytes;
     __shared__ __align__(8) uint64_t full[kF1Stages], empty[kF1Stages], b_full, acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int s = blockIdx.y;
     const int n_items = (p + kTileM - 1) / kTileM;
 
@@ -340,24 +343,30 @@ tc_fwd1x1p_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {
     }
     bool ok = true;
 
-    if (tid == 0) {
-        // ---- producer
-        const uint32_t bb = smem_u32(&b_full);
-        mbar_expect_tx(bb, (uint32_t)kblocks * kClassPad * 128);
-        for (int kb = 0; kb < kblocks; ++kb) tma_load_3d(b_base + kb * (kClassPad * 128), &tmB, bb, kb * kBlockK, 0, s);
+    if (warp == 0) {
+        // ---- producer (it and the issuer walk their loops as whole warps, one lane issues)
+        if (elect_one()) {
+            const uint32_t bb = smem_u32(&b_full);
+            mbar_expect_tx(bb, (uint32_t)kblocks * kClassPad * 128);
+            for (int kb = 0; kb < kblocks; ++kb) tma_load_3d(b_base + kb * (kClassPad * 128), &tmB, bb, kb * kBlockK, 0, s);
+        }
+        __syncwarp();
         int g = 0;
         for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
             for (int kb = 0; kb < kblocks; ++kb, ++g) {
                 const int st = g % kF1Stages;
                 if (g >= kF1Stages) ok = mbar_wait(smem_u32(&empty[st]), ((g / kF1Stages) - 1) & 1, err, kWaitEmpty);
                 if (!ok) break;
-                const uint32_t bar = smem_u32(&full[st]);
-                mbar_expect_tx(bar, kF1StageBytes);
-                tma_load_3d(a_base + st * kF1StageBytes, &tmA, bar, kb * kBlockK, it * kTileM, s);
+                if (elect_one()) {
+                    const uint32_t bar = smem_u32(&full[st]);
+                    mbar_expect_tx(bar, kF1StageBytes);
+                    tma_load_3d(a_base + st * kF1StageBytes, &tmA, bar, kb * kBlockK, it * kTileM, s);
+                }
+                __syncwarp();
             }
         }
         pdl_launch_dependents();     // every load is issued: the next kernel of the step may set itself up
-    } else if (tid == 32) {
+    } else if (warp == 1) {
         // ---- MMA issuer
         constexpr uint32_t idesc = instr_desc(kTileM, kClassPad, 0, 0);
         ok = mbar_wait(smem_u32(&b_full), 0, err, kWaitFull);
@@ -373,13 +382,16 @@ tc_fwd1x1p_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {
                 ok = mbar_wait(smem_u32(&full[st]), (g / kF1Stages) & 1, err, kWaitFull);
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t sa = a_base + st * kF1StageBytes, sb = b_base + kb * (kClassPad * 128);
+                if (elect_one()) {
+                    const uint64_t da = smem_desc(a_base + st * kF1StageBytes, 16, 1024), db = smem_desc(b_base + kb * (kClassPad * 128), 16, 1024);
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    umma(acc, smem_desc(sa + k * 32, 16, 1024), smem_desc(sb + k * 32, 16, 1024), idesc, (kb | k) != 0);
-                umma_commit(smem_u32(&empty[st]));
+                    for (int k = 0; k < 4; ++k) umma(acc, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+                    umma_commit(smem_u32(&empty[st]));
+                }
+                __syncwarp();
             }
-            if (ok) umma_commit(smem_u32(&acc_full[buf]));
+            if (ok && elect_one()) umma_commit(smem_u32(&acc_full[buf]));
+            __syncwarp();
         }
     } else if (warp >= 2) {
         // ---- epilogue warps: TMEM lanes 32*(warp % 4) .. +31 = pixels of the tile

@@ -48,12 +48,13 @@ __device__ __forceinline__ bool elect_one()
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
     return one != 0;
 }
-// Bounded wait; on give-up writes `code` (tagged with the block) into *err and returns false.
+// Bounded wait of a converged warp, with one outcome for all its lanes; on give-up writes `code` (tagged with the block) into
+// *err and returns false.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned int* err, unsigned int code,
                                           uint32_t limit = kSpinLimit)
 {
     for (uint32_t it = 0; it < limit; ++it)
-        if (mbar_try_wait(bar, parity)) return true;
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     atomicCAS(err, 0u, code | (blockIdx.x << 8));
     return false;
 }
