@@ -101,14 +101,14 @@ tc_fwd1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {6
 
     if (warp == 0) {
         if (elect_one())
-        for (int kb = 0; kb < kblocks; ++kb) {
-            const uint32_t bar = smem_u32(&bars[kb]);
-            if (!a_early) {
-                mbar_expect_tx(bar, kTileM * 128 + kClassPad * 128 + (kb == 0 ? stall_bytes : 0u));
-                tma_load_3d(a_base + kb * (kTileM * 128), &tmA, bar, kb * kBlockK, pix0, s);
+            for (int kb = 0; kb < kblocks; ++kb) {
+                const uint32_t bar = smem_u32(&bars[kb]);
+                if (!a_early) {
+                    mbar_expect_tx(bar, kTileM * 128 + kClassPad * 128 + (kb == 0 ? stall_bytes : 0u));
+                    tma_load_3d(a_base + kb * (kTileM * 128), &tmA, bar, kb * kBlockK, pix0, s);
+                }
+                tma_load_3d(b_base + kb * (kClassPad * 128), &tmB, bar, kb * kBlockK, 0, s);
             }
-            tma_load_3d(b_base + kb * (kClassPad * 128), &tmB, bar, kb * kBlockK, 0, s);
-        }
     } else if (warp == 1) {
         constexpr uint32_t idesc = instr_desc(kTileM, kClassPad, 0, 0);
         for (int kb = 0; kb < kblocks; ++kb) {
@@ -304,6 +304,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 #define ST_F1_STAGES 8
 #endif
 constexpr int kF1Threads = 192, kF1Stages = ST_F1_STAGES;
+constexpr uint32_t kOutPieceBytes = 32 * 128;     // 3x3 tile walk: 32 pixels x 64 channels of an epilogue warp on their way out
 constexpr uint32_t kF1StageBytes = kTileM * 128;
 
 __global__ void __launch_bounds__(kF1Threads)
@@ -431,10 +432,12 @@ tc_fwd1x1p_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {
 // The K loop runs over 9 taps x (kblocks1 + kblocks2) channel blocks: the first kblocks1 come from tmA (the previous
 // block's output, or the frozen part's), the others from tmA2 (the block's skip input): the concatenation of
 // Section 5.2 is never materialised.
-// Bound by the tensor pipe at 256 channels (0.9 of the measured peak inside a round of tiles; 53.8 us at 720p), by the issue
-// of copies and MMAs at 64 and 128 (29.4, 33.3 us).  With the issuing lane picked by number instead of elect_one 57.5, 39.7
-// and 42.5 us.  One slab of pixels per horizontal shift for the three taps above each other halves the activation traffic
-// but adds waits to the chain: 68, 50, 54 us, not kept.
+// Bound by the tensor pipe at 256 channels inside a tile (512 cycles per stage), by start, tile changes and the issue of copies
+// and MMAs at 64 and 128.  720p: 256 channels 50.2 us, 192 -> 64 31.6, 128 -> 64 29.1, gradient 64 -> 64 passed back 18.7.  With
+// 32-byte stores of every lane's own pixel row instead of pieces laid down in shared memory and stored by TMA 53.8, 33.6, 31.0
+// and 21.0 (the epilogue of a tile took 16000 to 24000 cycles, its multiplications 18400); with the issuing lane picked by
+// number 57.5, 42.5, 39.7, 24.1.  Not kept: one slab of pixels per horizontal shift for the three taps above each other (39, 35
+// us in the narrow layers), two units per stage (34, 29, 23), the next tile's pixels prefetched into L2 (55 us).
 template <int STAGES, int MODE>
 __global__ void __launch_bounds__(kFwd3Threads)
 tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}     box {64, 32, 4, 1}
@@ -445,7 +448,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
                  int tail_split,                             // the tiles of the last, partly filled round are cut into this many
                                                              // ranges of output channels (1, 2 or 4), one work item each
                  const float* __restrict__ theta, int64_t n_params, int64_t b_off,   // MODE 0: bias
-                 bf16* __restrict__ out,                     // [S][p][Ch]
+                 const __grid_constant__ CUtensorMap tmO,   // output {Ch, w, h, S} box {64, 32, 1, 1}
                  uint32_t* __restrict__ relu_bits,           // [S][p][Ch/32]: bit k of word j = out[32j + k] > 0 (MODE 0: written;
                                                              //   MODE 1: the receiving block's bits, read)
                  float* __restrict__ b_partials,             // MODE 1: [S][tiles per stream][Ch] channel sums of each tile
@@ -457,11 +460,11 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
     const uint32_t a_bytes = kTileM * 128, b_bytes = (uint32_t)Ch * 128, stage_bytes = a_bytes + b_bytes;
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_slot;
-    __shared__ float part[MODE == 1 ? 4 * 256 : 1];             // MODE 1: per-warp channel sums of the tile
+    __shared__ __align__(16) float part[4 * 256];               // per epilogue warp: MODE 0 the bias, MODE 1 channel sums of the tile
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int tiles_x = (w + kTileW - 1) / kTileW, tiles_y = (h + kTileH - 1) / kTileH;
     const int tiles_per_stream = tiles_x * tiles_y;
-    const int kblocks = kblocks1 + kblocks2, n_iter = 9 * kblocks;
+    const int kblocks = kblocks1 + kblocks2, n_stages = 9 * kblocks;
     // Work items: whole tiles while every block has one, then the remaining tiles in tail_split pieces each, so that
     // the last round is short instead of leaving most blocks idle for a full tile's time.
     const int n_full = tail_split > 1 ? (n_tiles_total / (int)gridDim.x) * (int)gridDim.x : n_tiles_total;
@@ -488,43 +491,47 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
     bool ok = true;
 
     if (warp == 0) {
-        // ---- producer (the whole warp walks the loop, its first lane issues): the ring index runs on across tiles
-        int g = 0;
+        // ---- producer (the whole warp walks the loop, its first lane issues): the ring runs on across tiles
+        int st = 0;
+        uint32_t parity = 1;             // a barrier nobody has arrived at yet counts as one whose phase 1 has ended
         for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
             const Item im = item_of(wi);
             const int s = im.tile / tiles_per_stream, tt = im.tile % tiles_per_stream;
             if (skip && skip[(int64_t)s * skip_stride]) continue;     // all three roles leave out the same items
             const int x0 = (tt % tiles_x) * kTileW, y0 = (tt / tiles_x) * kTileH;
+            const uint32_t item_bytes = a_bytes + (uint32_t)im.chn * 128;
             // One stage: wait for its slot, then the activation block (from `src`, whose tensor map is fixed at each of
             // the two places this is expanded: a map chosen at run time costs every copy a slow look-up) and the weights.
 #define ST_FWD3_STAGE(src, a_coord)                                                                                       \
             {                                                                                                             \
-                const int st = g % STAGES;                                                                                \
-                if (g >= STAGES) ok = mbar_wait(smem_u32(&empty[st]), ((g / STAGES) - 1) & 1, err, kWaitEmpty);          \
+                ok = mbar_wait(smem_u32(&empty[st]), parity, err, kWaitEmpty);                                            \
                 if (!ok) break;                                                                                           \
                 if (elect_one()) {                                                                                        \
-                const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;                                   \
-                mbar_expect_tx(bar, a_bytes + (uint32_t)im.chn * 128);                                                    \
-                tma_load_4d(sa, &(src), bar, (a_coord), x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);                          \
-                if (im.chn == Ch) tma_load_3d(sa + a_bytes, &tmB, bar, kb * kBlockK, tap * Ch, s);                        \
-                else                                                                                                      \
-                    for (int j = 0; j < im.chn / 64; ++j)        /* 64 weight rows per copy, laid out like the single copy */ \
-                        tma_load_3d(sa + a_bytes + j * (64 * 128), &tmBq, bar, kb * kBlockK, tap * Ch + im.ch0 + j * 64, s); \
+                    const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;                               \
+                    mbar_expect_tx(bar, item_bytes);                                                                      \
+                    tma_load_4d(sa, &(src), bar, (a_coord), x, y, s);                                                     \
+                    if (im.chn == Ch) tma_load_3d(sa + a_bytes, &tmB, bar, kb * kBlockK, row, s);                         \
+                    else                                                                                                  \
+                        for (int j = 0; j < im.chn / 64; ++j)    /* 64 weight rows per copy, laid out like the single copy */ \
+                            tma_load_3d(sa + a_bytes + j * (64 * 128), &tmBq, bar, kb * kBlockK, row + im.ch0 + j * 64, s); \
                 }                                                                                                         \
                 __syncwarp();                                                                                             \
-                ++g;                                                                                                      \
+                if (++st == STAGES) { st = 0; parity ^= 1; }                                                              \
             }
-            for (int tap = 0; tap < 9 && ok; ++tap) {
-                int kb = 0;
-                for (; kb < kblocks1; ++kb) ST_FWD3_STAGE(tmA, kb * kBlockK)
-                for (; kb < kblocks && ok; ++kb) ST_FWD3_STAGE(tmA2, (kb - kblocks1) * kBlockK)
-            }
+            int row = 0;
+            for (int y = y0 - 1; y <= y0 + 1 && ok; ++y)
+                for (int x = x0 - 1; x <= x0 + 1 && ok; ++x, row += Ch) {
+                    int kb = 0;
+                    for (; kb < kblocks1; ++kb) ST_FWD3_STAGE(tmA, kb * kBlockK)
+                    for (; kb < kblocks && ok; ++kb) ST_FWD3_STAGE(tmA2, (kb - kblocks1) * kBlockK)
+                }
 #undef ST_FWD3_STAGE
         }
         pdl_launch_dependents();     // every load is issued: the next kernel of the step may set itself up
     } else if (warp == 1) {
         // ---- MMA issuer
-        int g = 0, j = 0;
+        int st = 0, j = 0;
+        uint32_t parity = 0;
         for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
             const Item im = item_of(wi);
             if (skip && skip[(int64_t)(im.tile / tiles_per_stream) * skip_stride]) continue;
@@ -534,9 +541,8 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
             if (!ok) break;
             tc_fence_after_sync();
             const uint32_t acc = tmem + buf * acc_cols;
-            for (int it = 0; it < n_iter; ++it, ++g) {
-                const int st = g % STAGES;
-                ok = mbar_wait(smem_u32(&full[st]), (g / STAGES) & 1, err, kWaitFull);
+            for (int it = 0; it < n_stages; ++it) {
+                ok = mbar_wait(smem_u32(&full[st]), parity, err, kWaitFull);
                 if (!ok) break;
                 tc_fence_after_sync();
                 if (elect_one()) {
@@ -546,6 +552,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
                     umma_commit(smem_u32(&empty[st]));
                 }
                 __syncwarp();
+                if (++st == STAGES) { st = 0; parity ^= 1; }
             }
             if (ok && elect_one()) umma_commit(smem_u32(&acc_full[buf]));
             __syncwarp();
@@ -553,7 +560,9 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
         }
     } else if (warp >= 2) {
         // ---- epilogue warps: TMEM lanes 32*(warp % 4) .. +31 = pixel rows of the tile
+        // (a warp's 32 pixels are one row of the tile)
         const int q = warp & 3, row = q * 32 + lane;
+        const uint32_t piece = base + STAGES * stage_bytes + q * kOutPieceBytes, orow = piece + lane * 128;
         int j = 0;
         for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
             const Item im = item_of(wi);
@@ -561,6 +570,11 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
             if (skip && skip[(int64_t)s * skip_stride]) continue;
             const int buf = j & 1;
             const int x = (tt % tiles_x) * kTileW + row % kTileW, y = (tt / tiles_x) * kTileH + row / kTileW;
+            if (MODE == 0) {
+                const float* bias = theta + (int64_t)s * n_params + b_off + im.ch0;
+                for (int c = lane; c < im.chn; c += 32) part[q * 256 + c] = __ldg(bias + c);
+                __syncwarp();
+            }
             ok = mbar_wait(smem_u32(&acc_full[buf]), (j >> 1) & 1, err, kWaitDone);
             if (MODE == 1) {                                           // the four epilogue warps stay together: they share `part`
                 int all_ok;
@@ -572,59 +586,66 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
             tc_fence_after_sync();
             const bool in = y < h && x < w;
             const int64_t pixel = (int64_t)s * h * w + (int64_t)y * w + x;
-            bf16* dst = out + pixel * Ch + im.ch0;
-            const float* bias = theta + (int64_t)s * n_params + b_off + im.ch0;
-            for (int n0 = 0; n0 < im.chn; n0 += 32) {
-                float v[32];
-                tmem_ld_32x32(tmem + ((uint32_t)(q * 32) << 16) + buf * acc_cols + n0, v);
-                if (MODE == 0) {
-                    if (in) {
-                        uint4 o4[4];
-                        __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(o4);
-                        uint32_t bits = 0;
+            for (int n0 = 0; n0 < im.chn; n0 += 64) {
+                uint32_t words[2] = {0, 0};                            // ReLU bits
+                if (MODE == 1 && in) {
+                    const uint2 b = __ldg(reinterpret_cast<const uint2*>(relu_bits + pixel * (Ch / 32) + (im.ch0 + n0) / 32));
+                    words[0] = b.x; words[1] = b.y;                    // ... none where the tile reaches beyond the frame
+                }
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    float v[32];
+                    tmem_ld_32x32(tmem + ((uint32_t)(q * 32) << 16) + buf * acc_cols + n0 + g * 32, v);
+                    uint32_t o[16];
+                    if (MODE == 0) {
+                        const float4* b4 = reinterpret_cast<const float4*>(part + q * 256 + n0 + g * 32);
 #pragma unroll
                         for (int k = 0; k < 16; ++k) {
-                            const float a = fmaxf(v[2 * k] + __ldg(bias + n0 + 2 * k), 0.f), b = fmaxf(v[2 * k + 1] + __ldg(bias + n0 + 2 * k + 1), 0.f);
-                            o2[k] = __floats2bfloat162_rn(a, b);
+                            const float4 b = b4[k >> 1];
+                            const float x0f = fmaxf(v[2 * k] + ((k & 1) ? b.z : b.x), 0.f), x1f = fmaxf(v[2 * k + 1] + ((k & 1) ? b.w : b.y), 0.f);
+                            const __nv_bfloat162 two = __floats2bfloat162_rn(x0f, x1f);
+                            o[k] = *reinterpret_cast<const uint32_t*>(&two);
                             // the mask is taken on the stored (rounded) activation, the value the next layer sees
-                            bits |= (__low2float(o2[k]) > 0.f ? 1u : 0u) << (2 * k);
-                            bits |= (__high2float(o2[k]) > 0.f ? 1u : 0u) << (2 * k + 1);
+                            words[g] |= (__low2float(two) > 0.f ? 1u : 0u) << (2 * k);
+                            words[g] |= (__high2float(two) > 0.f ? 1u : 0u) << (2 * k + 1);
                         }
-                        store_256(dst + n0, reinterpret_cast<const uint32_t*>(o4));            // 32 channels = 64 bytes
-                        store_256(dst + n0 + 16, reinterpret_cast<const uint32_t*>(o4) + 8);
-                        relu_bits[pixel * (Ch / 32) + (im.ch0 + n0) / 32] = bits;
-                    }
-                } else {
-                    if (in) {
-                        const uint32_t bits = __ldg(relu_bits + pixel * (Ch / 32) + (im.ch0 + n0) / 32);
-                        uint4 o4[4];
-                        __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(o4);
-#pragma unroll
-                        for (int k = 0; k < 16; ++k) {
-                            if (!((bits >> (2 * k)) & 1u)) v[2 * k] = 0.f;
-                            if (!((bits >> (2 * k + 1)) & 1u)) v[2 * k + 1] = 0.f;
-                            o2[k] = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
-                        }
-                        store_256(dst + n0, reinterpret_cast<const uint32_t*>(o4));
-                        store_256(dst + n0 + 16, reinterpret_cast<const uint32_t*>(o4) + 8);
                     } else {
 #pragma unroll
-                        for (int k = 0; k < 32; ++k) v[k] = 0.f;
-                    }
-                    // sums over the warp's 32 pixels in a fixed order: a reduce-scatter over the lanes, after which lane c
-                    // holds the sum of channel n0 + c
-#pragma unroll
-                    for (int half = 16; half >= 1; half >>= 1) {
-                        const bool up = (lane & half) != 0;
-#pragma unroll
-                        for (int k = 0; k < half; ++k) {
-                            const float keep = up ? v[k + half] : v[k];
-                            const float send = up ? v[k] : v[k + half];
-                            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+                        for (int k = 0; k < 16; ++k) {
+                            if (!((words[g] >> (2 * k)) & 1u)) v[2 * k] = 0.f;
+                            if (!((words[g] >> (2 * k + 1)) & 1u)) v[2 * k + 1] = 0.f;
+                            const __nv_bfloat162 two = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+                            o[k] = *reinterpret_cast<const uint32_t*>(&two);
                         }
                     }
-                    part[q * 256 + n0 + lane] = v[0];
+                    if (g == 0) {
+                        if (lane == 0) tma_store_wait_read<0>();       // the piece that was here before has been read
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)                        // 128-byte swizzle: 16-byte chunks ^ (row % 8)
+                        st_shared_128(orow + (((g * 4 + k) ^ (lane & 7)) << 4), o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+                    if (MODE == 1) {
+                        // sums over the warp's 32 pixels in a fixed order: a reduce-scatter over the lanes, after which lane c
+                        // holds the sum of channel c of the group
+#pragma unroll
+                        for (int half = 16; half >= 1; half >>= 1) {
+                            const bool up = (lane & half) != 0;
+#pragma unroll
+                            for (int k = 0; k < half; ++k) {
+                                const float keep = up ? v[k + half] : v[k];
+                                const float send = up ? v[k] : v[k + half];
+                                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+                            }
+                        }
+                        part[q * 256 + n0 + g * 32 + lane] = v[0];
+                    }
                 }
+                if (MODE == 0 && in)
+                    *reinterpret_cast<uint2*>(relu_bits + pixel * (Ch / 32) + (im.ch0 + n0) / 32) = make_uint2(words[0], words[1]);
+                fence_async_shared();
+                __syncwarp();
+                if (lane == 0 && y < h) { tma_store_4d(&tmO, piece, im.ch0 + n0, x, y, s); tma_store_commit(); }
             }
             tc_fence_before_sync();
             __syncwarp();
@@ -639,6 +660,7 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
             }
             ++j;
         }
+        if (lane == 0) tma_store_wait();
     }
     if (!ok) drain_after_error();
     tc_fence_before_sync();
@@ -650,16 +672,17 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
 // wgrad 3x3: for one tap, D[ci][co] += sum over this block's pixel chunks of X[pix+tap][ci] * dHd[pix][co].
 // Both operands are MN-major (pixel-major activations, reduction over pixels).  A block keeps
 // ceil(Cin/128) accumulators of Ch columns (all input channels of one tap) so that the dHd tile of a
-// stage is shared by all of them.  Bound by the issue of copies and MMAs, like the forward: with producer and issuer as single
-// threads 51.4 us at 720p and 256 channels, 37 and 41 us in a stack of 64 and 128; as whole warps with elect_one 47.5, 29.4
-// and 32.5 us.
+// stage is shared by all of them.  Bound by the tensor pipe and
+// 37 MB of partial sums at 256 channels (47.5 us at 720p), by the issue of copies and MMAs in narrow layers.  With producer and
+// issuer as single threads 51.4 us, and 37 / 41 us in a stack of 64 and 128; as whole warps with elect_one 47.5, 30 and 33;
+// with one copy for all channels of a chunk (64 x w x h x blocks of 64) and two chunks per stage 47.4, 22.9 and 30.9.
 // ------------------------------------------------------------------------------------------------
-template <int STAGES>
+template <int STAGES, int G>
 __global__ void __launch_bounds__(kThreadsTc)
-tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output {C1, w, h, S} box {64, 32, 2, 1}
-                   const __grid_constant__ CUtensorMap tmA2,  // skip input      {C2, w, h, S} box {64, 32, 2, 1} (unused if C2 == 0)
+tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output {64, w, h, C1/64, S} box {64, 32, 2, C1/64, 1}
+                   const __grid_constant__ CUtensorMap tmA2,  // skip input      {64, w, h, C2/64, S} box {64, 32, 2, C2/64, 1} (unused if C2 == 0)
                    int blocks1,                                // C1 / 64: input-channel blocks that come from tmA
-                   const __grid_constant__ CUtensorMap tmB,   // dHd {Ch,  w, h, S} box {64, 32, 2, 1}
+                   const __grid_constant__ CUtensorMap tmB,   // dHd {64, w, h, Ch/64, S} box {64, 32, 2, Ch/64, 1}
                    float* __restrict__ partials,              // [S][n_split][9][Ch][Cin]
                    int Cin, int Ch, int h, int w, int n_chunks, int chunks_per_block, int n_split,
                    int tmem_cols, unsigned int* err, const int* __restrict__ skip, int64_t skip_stride)
@@ -669,13 +692,15 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     uint8_t* smem = align_smem(smem_raw);
     const uint32_t base = smem_u32(smem);
     const int m_tiles = (Cin + kTileM - 1) / kTileM;
-    const int a_blocks = m_tiles * 2, b_blocks = Ch / kBlockK;
+    const int a_blocks = Cin / kBlockK, b_blocks = Ch / kBlockK;
     const uint32_t blk_bytes = kChunkPix * 128;
-    const uint32_t a_bytes = a_blocks * blk_bytes, stage_bytes = a_bytes + b_blocks * blk_bytes;
+    // G chunks of pixels per stage.  If the input channels end on an odd 64, the last accumulator's upper half multiplies what
+    // lies behind them in the stage; nobody looks at those rows.
+    const uint32_t a_bytes = a_blocks * blk_bytes, chunk_bytes = a_bytes + b_blocks * blk_bytes, stage_bytes = G * chunk_bytes;
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const int tap = blockIdx.x % 9, split = blockIdx.x / 9, s = blockIdx.y;
+    const int tap = blockIdx.x % 9, dx = tap % 3 - 1, dy = tap / 3 - 1, split = blockIdx.x / 9, s = blockIdx.y;
     const int chunks_x = (w + kChunkW - 1) / kChunkW;
     const int c_begin = split * chunks_per_block, c_end = min(n_chunks, c_begin + chunks_per_block);
 
@@ -699,43 +724,50 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     bool ok = true;
 
     if (warp == 0) {             // producer and issuer walk their loops as whole warps, one lane issues
-        for (int i = c_begin; i < c_end; ++i) {
-            const int it = i - c_begin, st = it % STAGES;
-            if (it >= STAGES) ok = mbar_wait(smem_u32(&empty[st]), ((it / STAGES) - 1) & 1, err, kWaitEmpty);
+        int st = 0;
+        uint32_t parity = 1;
+        for (int i = c_begin; i < c_end && ok; i += G) {
+            ok = mbar_wait(smem_u32(&empty[st]), parity, err, kWaitEmpty);
             if (!ok) break;
-            const int x0 = (i % chunks_x) * kChunkW, y0 = (i / chunks_x) * kChunkH;
             if (elect_one()) {
                 const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;
-                mbar_expect_tx(bar, stage_bytes);
-                // blocks past the last channel arrive as zeros (out-of-range fill); two loops, each with its own tensor map
-                // (a map chosen at run time costs every copy a slow look-up)
-                const int n_first = blocks1 * kBlockK == Cin ? a_blocks : blocks1;
-                int cb = 0;
-                for (; cb < n_first; ++cb)
-                    tma_load_4d(sa + cb * blk_bytes, &tmA, bar, cb * kBlockK, x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);
-                for (; cb < a_blocks; ++cb)
-                    tma_load_4d(sa + cb * blk_bytes, &tmA2, bar, (cb - blocks1) * kBlockK, x0 + tap % 3 - 1, y0 + tap / 3 - 1, s);
-                for (int cb = 0; cb < b_blocks; ++cb)
-                    tma_load_4d(sa + a_bytes + cb * blk_bytes, &tmB, bar, cb * kBlockK, x0, y0, s);
+                mbar_expect_tx(bar, min(G, c_end - i) * chunk_bytes);
+#pragma unroll
+                for (int n = 0; n < G; ++n)
+                    if (n == 0 || i + n < c_end) {
+                        const int x0 = (i + n) % chunks_x * kChunkW, y0 = (i + n) / chunks_x * kChunkH;
+                        const uint32_t to = sa + n * chunk_bytes;
+                        tma_load_5d(to, &tmA, bar, 0, x0 + dx, y0 + dy, 0, s);
+                        if (blocks1 < a_blocks) tma_load_5d(to + blocks1 * blk_bytes, &tmA2, bar, 0, x0 + dx, y0 + dy, 0, s);
+                        tma_load_5d(to + a_bytes, &tmB, bar, 0, x0, y0, 0, s);
+                    }
             }
             __syncwarp();
+            if (++st == STAGES) { st = 0; parity ^= 1; }
         }
     } else if (warp == 1) {
         const uint32_t idesc = instr_desc(kTileM, Ch, 1, 1);
-        for (int i = c_begin; i < c_end; ++i) {
-            const int it = i - c_begin, st = it % STAGES;
-            ok = mbar_wait(smem_u32(&full[st]), (it / STAGES) & 1, err, kWaitFull);
+        int st = 0;
+        uint32_t parity = 0;
+        for (int i = c_begin; i < c_end; i += G) {
+            ok = mbar_wait(smem_u32(&full[st]), parity, err, kWaitFull);
             if (!ok) break;
             tc_fence_after_sync();
             if (elect_one()) {
-                const uint64_t da = smem_desc(base + st * stage_bytes, blk_bytes, 1024), db = da + (a_bytes >> 4);
-                for (int m = 0; m < m_tiles; ++m)
+                const uint64_t d0 = smem_desc(base + st * stage_bytes, blk_bytes, 1024);
 #pragma unroll
-                    for (int j = 0; j < kChunkPix / 16; ++j)
-                        umma(tmem + m * Ch, da + ((2 * m * blk_bytes + j * (16 * 128)) >> 4), db + j * ((16 * 128) >> 4), idesc, (it | j) != 0);
+                for (int n = 0; n < G; ++n)
+                    if (n == 0 || i + n < c_end) {
+                        const uint64_t da = d0 + n * (chunk_bytes >> 4), db = da + (a_bytes >> 4);
+                        for (int m = 0; m < m_tiles; ++m)
+#pragma unroll
+                            for (int j = 0; j < kChunkPix / 16; ++j)
+                                umma(tmem + m * Ch, da + ((2 * m * blk_bytes + j * (16 * 128)) >> 4), db + j * ((16 * 128) >> 4), idesc, i != c_begin || (n | j) != 0);
+                    }
                 umma_commit(smem_u32(&empty[st]));
             }
             __syncwarp();
+            if (++st == STAGES) { st = 0; parity ^= 1; }
         }
         if (elect_one()) umma_commit(smem_u32(&done));
     }
@@ -1025,15 +1057,33 @@ bool encode_tensor_map(CUtensorMap* m, CUtensorMapDataType dtype, CUtensorMapSwi
     return true;
 }
 
-// the instantiation of a 3x3 kernel with a given pipeline depth (all depths share one function type)
+// Pipeline depth of the 3x3 tile walk: as many stages as fit beside the epilogue's pieces (a stage of a narrow layer is small,
+// and with only four of them in flight the copies' latency, not the tensor pipe, sets the pace).
+static int fwd3_stages(int n_out) { return n_out <= 64 ? 8 : (n_out <= 128 ? 6 : 4); }
+static size_t fwd3_bytes(int n_out) { return (size_t)fwd3_stages(n_out) * (kTileM + n_out) * 128 + 4 * kOutPieceBytes + kSmemAlign; }
 template <int MODE>
-static decltype(&tc_fwd3x3_kernel<4, MODE>) fwd3_kernel(int stages)
+static decltype(&tc_fwd3x3_kernel<4, MODE>) fwd3_kernel(int n_out)
 {
-    return stages >= 8 ? tc_fwd3x3_kernel<8, MODE> : (stages >= 6 ? tc_fwd3x3_kernel<6, MODE> : tc_fwd3x3_kernel<4, MODE>);
+    const int n = fwd3_stages(n_out);
+    return n == 8 ? tc_fwd3x3_kernel<8, MODE> : (n == 6 ? tc_fwd3x3_kernel<6, MODE> : tc_fwd3x3_kernel<4, MODE>);
 }
-static decltype(&tc_wgrad3x3_kernel<3>) wgrad3_kernel(int stages)
+// The stages of the weight gradient: two chunks of pixels each if three such stages fit (for the same reason), else one; as
+// many as fit in about 208 KB, five at most.
+struct Wg3Ring { int stages, chunks; size_t bytes; };
+static Wg3Ring wg3_ring(int c_in, int c_out)
 {
-    return stages >= 5 ? tc_wgrad3x3_kernel<5> : (stages >= 4 ? tc_wgrad3x3_kernel<4> : tc_wgrad3x3_kernel<3>);
+    const size_t chunk = (size_t)((c_in + c_out) / kBlockK) * kChunkPix * 128;
+    const int fit = (int)((size_t)208 * 1024 / chunk);
+    Wg3Ring g;
+    g.chunks = fit >= 6 ? 2 : 1;
+    g.stages = g.chunks == 2 ? (fit >= 8 ? 4 : 3) : (fit >= 5 ? 5 : (fit >= 4 ? 4 : 3));
+    g.bytes = (size_t)g.stages * g.chunks * chunk + kSmemAlign;
+    return g;
+}
+static decltype(&tc_wgrad3x3_kernel<3, 1>) wgrad3_kernel(const Wg3Ring& g)
+{
+    if (g.chunks == 2) return g.stages == 4 ? tc_wgrad3x3_kernel<4, 2> : tc_wgrad3x3_kernel<3, 2>;
+    return g.stages == 5 ? tc_wgrad3x3_kernel<5, 1> : (g.stages == 4 ? tc_wgrad3x3_kernel<4, 1> : tc_wgrad3x3_kernel<3, 1>);
 }
 
 struct TcBlockPlan {
@@ -1042,10 +1092,11 @@ struct TcBlockPlan {
     CUtensorMap w_map, w_map_q;      // {c_tot, 9*c_out, S}, boxes {64, c_out, 1} and {64, 64, 1}
     CUtensorMap wt_map, wt_map_q;    // mirrored, transposed weights {c_out, 9*c_prev, S}, boxes {64, c_prev, 1} and {64, 64, 1}
     CUtensorMap dout_fwd;            // the block's output gradient {c_out, w, h, S}, box {64, 32, 4, 1} (A operand when passed back)
+    CUtensorMap out_st, dprev_st;    // the block's output and its first input's gradient {C, w, h, S}, box {64, 32, 1, 1} (stores)
     CUtensorMap dout_wg;             // same tensor, box {64, 32, 2, 1} (B operand of the weight gradient)
     int cols_wg;                     // tensor-memory columns of the weight gradient
-    int stages_fwd, stages_back, stages_wg;   // pipeline depths of the three kernels of this block
-    size_t smem_fwd, smem_back, smem_wg;
+    Wg3Ring wg;
+    size_t smem_fwd, smem_back;
 };
 
 struct TcPlan {
@@ -1135,12 +1186,15 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         TcBlockPlan& q = P->blk[i];
         const uint64_t w = (uint64_t)b.w, h = (uint64_t)b.h, c1 = (uint64_t)k.c_prev, c2 = (uint64_t)k.c_skip, co = (uint64_t)k.c_out,
                        ct = c1 + c2;
-        const uint32_t bf[4] = {64, (uint32_t)kTileW, (uint32_t)kTileH, 1}, bw[4] = {64, (uint32_t)kChunkW, (uint32_t)kChunkH, 1};
+        const uint32_t bf[4] = {64, (uint32_t)kTileW, (uint32_t)kTileH, 1};
         auto act_maps = [&](const bf16* base, uint64_t c, CUtensorMap* fwd, CUtensorMap* wg, const char* what) {
             uint64_t d[4] = {c, w, h, S}, st[3] = {c * 2, w * c * 2, h * w * c * 2};
+            // all channels of a chunk in one copy: one block of 64 behind the other
+            uint64_t d5[5] = {64, w, h, c / 64, S}, st5[4] = {c * 2, w * c * 2, 128, h * w * c * 2};
+            uint32_t bw[5] = {64, (uint32_t)kChunkW, (uint32_t)kChunkH, (uint32_t)(c / 64), 1};
             bool r = true;
             if (fwd) r = r && make_map(fwd, base, 4, d, st, bf, err, err_len, what);
-            if (wg) r = r && make_map(wg, base, 4, d, st, bw, err, err_len, what);
+            if (wg) r = r && make_map(wg, base, 5, d5, st5, bw, err, err_len, what);
             return r;
         };
         ok = ok && act_maps(k.in_prev, c1, &q.in_fwd, &q.in_wg, "block input");
@@ -1153,7 +1207,14 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
             ok = ok && make_map(&q.w_map, k.w, 3, dw, sw, bwt, err, err_len, "3x3 weight");
             ok = ok && make_map(&q.w_map_q, k.w, 3, dw, sw, bwq, err, err_len, "3x3 weight (64 rows)");
         }
+        auto store_map = [&](const bf16* base, uint64_t c, CUtensorMap* m, const char* what) {
+            uint64_t d[4] = {c, w, h, S}, st[3] = {c * 2, w * c * 2, h * w * c * 2};
+            uint32_t bo[4] = {64, (uint32_t)kTileW, 1, 1};
+            return make_map(m, base, 4, d, st, bo, err, err_len, what);
+        };
+        ok = ok && store_map(k.out, co, &q.out_st, "block output (stores)");
         if (ok && k.pass_back) {
+            ok = store_map(b.blk[i - 1].dout, c1, &q.dprev_st, "previous block's output gradient (stores)");
             uint64_t dw[3] = {co, 9 * c1, S}, sw[2] = {co * 2, 9 * c1 * co * 2};
             uint32_t bwt[3] = {64, (uint32_t)c1, 1}, bwq[3] = {64, 64, 1};
             ok = ok && make_map(&q.wt_map, k.w_t, 3, dw, sw, bwt, err, err_len, "3x3 weight, transposed");
@@ -1161,23 +1222,14 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         }
         const int m_in = ((int)ct + kTileM - 1) / kTileM;
         q.cols_wg = pow2_cols(m_in * k.c_out);
-        // pipeline depth: as many stages as fit in about 208 KB (a stage of a narrow layer is small, and with only four
-        // of them in flight the copies' latency, not the tensor pipe, sets the pace)
-        auto pick = [](size_t stage_bytes, int lo, int mid, int hi) {
-            const size_t fit = ((size_t)208 * 1024) / stage_bytes;
-            return fit >= (size_t)hi ? hi : (fit >= (size_t)mid ? mid : lo);
-        };
-        const size_t st_fwd = (size_t)kTileM * 128 + (size_t)k.c_out * 128, st_back = (size_t)kTileM * 128 + (size_t)k.c_prev * 128,
-                     st_wg = (size_t)(m_in * 2 + k.c_out / kBlockK) * kChunkPix * 128;
-        q.stages_fwd = pick(st_fwd, 4, 6, 8); q.stages_back = pick(st_back, 4, 6, 8); q.stages_wg = pick(st_wg, 3, 4, 5);
-        q.smem_fwd = q.stages_fwd * st_fwd + kSmemAlign;
-        q.smem_back = q.stages_back * st_back + kSmemAlign;
-        q.smem_wg = q.stages_wg * st_wg + kSmemAlign;
+        q.wg = wg3_ring((int)ct, k.c_out);
+        q.smem_fwd = fwd3_bytes(k.c_out);
+        q.smem_back = fwd3_bytes(k.c_prev);
         if (ok && q.cols_wg > 512) {
             snprintf(err, err_len, "a block with %d input and %d output channels needs %d TMEM columns (> 512)", (int)ct, k.c_out, q.cols_wg);
             ok = false;
         }
-        if (ok && (q.smem_fwd > lim || q.smem_wg > lim || (k.pass_back && (q.smem_back > lim || k.c_prev > 256)))) {
+        if (ok && (q.smem_fwd > lim || q.wg.bytes > lim || (k.pass_back && (q.smem_back > lim || k.c_prev > 256)))) {
             snprintf(err, err_len, "shared memory per block exceeds 227 KB for these channel counts");
             ok = false;
         }
@@ -1232,9 +1284,9 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
     if (e == cudaSuccess) e = allow((const void*)tc_wgrad1x1_kernel<kWg1Stages>, P->smem_wg1);
     for (int i = 0; i < nb; ++i) {
         const TcBlockPlan& q = P->blk[i];
-        if (e == cudaSuccess) e = allow((const void*)fwd3_kernel<0>(q.stages_fwd), q.smem_fwd);
-        if (e == cudaSuccess && b.blk[i].pass_back) e = allow((const void*)fwd3_kernel<1>(q.stages_back), q.smem_back);
-        if (e == cudaSuccess) e = allow((const void*)wgrad3_kernel(q.stages_wg), q.smem_wg);
+        if (e == cudaSuccess) e = allow((const void*)fwd3_kernel<0>(b.blk[i].c_out), q.smem_fwd);
+        if (e == cudaSuccess && b.blk[i].pass_back) e = allow((const void*)fwd3_kernel<1>(b.blk[i].c_prev), q.smem_back);
+        if (e == cudaSuccess) e = allow((const void*)wgrad3_kernel(q.wg), q.wg.bytes);
     }
     if (nb && e == cudaSuccess) e = allow((const void*)tc_back1x1_kernel, P->smem_back1);
     if (e != cudaSuccess) { snprintf(err, err_len, "shared-memory attribute: %s", cudaGetErrorString(e)); delete P; return nullptr; }
@@ -1276,9 +1328,9 @@ int tc_forward_blocks(const TcPlan* P, int first, int last, cudaStream_t s, Stag
         const TcBlockPlan& q = P->blk[i];
         int grid, tail_split;
         tile_walk(P, total, k.c_out, &grid, &tail_split);
-        ST_REPEAT(t) launch_chain(b.chain_early != 0, fwd3_kernel<0>(q.stages_fwd), dim3(grid), dim3(kFwd3Threads), q.smem_fwd, s,
+        ST_REPEAT(t) launch_chain(b.chain_early != 0, fwd3_kernel<0>(k.c_out), dim3(grid), dim3(kFwd3Threads), q.smem_fwd, s,
             q.in_fwd, q.skip_fwd, k.c_prev / kBlockK, k.c_skip / kBlockK, q.w_map, q.w_map_q, tail_split, b.theta, b.n_params, k.b_off,
-            k.out, k.relu_bits, (float*)nullptr, k.c_out, b.h, b.w, total, pow2_cols(k.c_out), b.err, skip, skip_stride);
+            q.out_st, k.relu_bits, (float*)nullptr, k.c_out, b.h, b.w, total, pow2_cols(k.c_out), b.err, skip, skip_stride);
         if (t) t->mark(kFwd3Names[i], s, st_repeats(t));
         n += st_repeats(t);
     }
@@ -1336,7 +1388,7 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
     for (int i = nb - 1; i >= 0 && b.blk[i].trained; --i) {
         const TcBlock& k = b.blk[i];
         const TcBlockPlan& q = P->blk[i];
-        ST_REPEAT(t) launch_chain(b.chain_early != 0, wgrad3_kernel(q.stages_wg), dim3(9 * P->split1, b.S), dim3(kThreadsTc), q.smem_wg, s,
+        ST_REPEAT(t) launch_chain(b.chain_early != 0, wgrad3_kernel(q.wg), dim3(9 * P->split1, b.S), dim3(kThreadsTc), q.wg.bytes, s,
             q.in_wg, q.skip_wg, k.c_prev / kBlockK, q.dout_wg, k.w_partials, k.c_prev + k.c_skip, k.c_out, b.h, b.w, P->chunks1, P->per1,
             P->split1, q.cols_wg, b.err, skip, skip_stride);
         if (t) t->mark(kWg3Names[i], s, st_repeats(t));
@@ -1347,9 +1399,9 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
             const TcBlock& r = b.blk[i - 1];
             int grid, tail_split;
             tile_walk(P, total, k.c_prev, &grid, &tail_split);
-            ST_REPEAT(t) launch_chain(b.chain_early != 0, fwd3_kernel<1>(q.stages_back), dim3(grid), dim3(kFwd3Threads), q.smem_back, s,
+            ST_REPEAT(t) launch_chain(b.chain_early != 0, fwd3_kernel<1>(k.c_prev), dim3(grid), dim3(kFwd3Threads), q.smem_back, s,
                 q.dout_fwd, q.dout_fwd, k.c_out / kBlockK, 0, q.wt_map, q.wt_map_q, tail_split, (const float*)nullptr, (int64_t)0, (int64_t)0,
-                r.dout, r.relu_bits, r.b_partials, k.c_prev, b.h, b.w, total, pow2_cols(k.c_prev), b.err, skip, skip_stride);
+                q.dprev_st, r.relu_bits, r.b_partials, k.c_prev, b.h, b.w, total, pow2_cols(k.c_prev), b.err, skip, skip_stride);
             if (t) t->mark("tc_dgrad3x3", s, st_repeats(t));
             n += st_repeats(t);
         }
