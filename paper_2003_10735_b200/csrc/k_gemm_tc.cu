@@ -1245,10 +1245,12 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
     P->smem_fwd1p = (size_t)kF1Stages * kF1StageBytes + (size_t)(P->c_last / kBlockK) * kClassPad * 128 + kSmemAlign;
     {
         // The persistent form wins where every block has many tiles to stream (16 streams at 720p: 90 us against
-        // 110 us, 0.93 of the HBM copy bandwidth); with about three tiles per SM (one 720p stream) its partly filled
-        // last round costs more than the one-tile blocks' second wave.  ST_FWD1X1_PERSISTENT=0/1 forces a choice.
+        // 110 us, 0.93 of the HBM copy bandwidth) or more than a ring of stages (one 720p stream of 256 channels, twelve
+        // stages per SM: 8.7 us against 10.6).  With three tiles of 64 channels per SM, or three of 128, its partly filled
+        // last round costs more than the one-tile blocks' second wave (8.6 us against 7.1).  ST_FWD1X1_PERSISTENT=0/1
+        // forces a choice.
         const int64_t tiles = (int64_t)((P->p + kTileM - 1) / kTileM) * b.S;
-        bool use = tiles >= (int64_t)6 * 148;
+        bool use = tiles >= (int64_t)6 * 148 || tiles * (P->c_last / kBlockK) >= (int64_t)9 * 148;
         if (const char* e = getenv("ST_FWD1X1_PERSISTENT")) { if (e[0] == '0') use = false; else if (e[0] == '1') use = true; }
         if (const char* e = getenv("ST_TEST_STALL_FWD1X1")) if (e[0] == '1') { P->test_stall = true; use = false; }
         // the one-tile form keeps the whole channel extent of its tile in shared memory: beyond 704 channels it no
