@@ -594,10 +594,14 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     c->use_graphs = c->stream != nullptr && c->stream != cudaStreamLegacy && c->stream != cudaStreamPerThread;
     if (const char* e = getenv("ST_NO_GRAPH")) if (e[0] == '1') c->use_graphs = false;
     // Programmatic dependent launch along the step's chain: with the one-layer head every kernel has something to do
-    // before its predecessor's results are needed (label fetch, feature tiles) and the step is 2 us shorter; the
-    // two-layer head's kernels fill the SMs to the end and gain nothing (measured: 1 us slower; with fp32 convolutions 10 us
-    // slower: waiting blocks crowd the SMs that finish first).  ST_PDL=0 / 1 force it.
-    c->chain_early = pdl_enabled() && c->Ch == 0;
+    // before its predecessor's results are needed (label fetch, feature tiles) and the step is 2 us shorter.  Blocks of 3x3
+    // layers with at most 128 output channels are many short kernels, whose starts (barriers, tensor memory) hide behind the one
+    // before: 2 % of a call (two blocks of 64 channels, 720p: 1560 -> 1527 us; 128 channels, 101 x 187: 659 -> 645).  Kernels of
+    // 256 channels fill the SMs to the end and waiting blocks crowd those that finish first: 0.6 % slower; with fp32
+    // convolutions 10 us a step slower.  ST_PDL=0 / 1 force it.
+    int widest = 0;
+    for (int i = 0; i < n_blocks; ++i) if (blk_out[i] > widest) widest = blk_out[i];
+    c->chain_early = pdl_enabled() && (c->Ch == 0 || (c->bf16_mode && widest <= 128));
     if (const char* e = getenv("ST_PDL")) if (e[0] == '1') c->chain_early = true;
 
     // layers in forward order: the 3x3 layers (blocks, or the fp32 path's hidden layer), then the classifier
