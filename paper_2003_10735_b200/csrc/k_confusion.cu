@@ -133,8 +133,8 @@ confusion_kernel(const uint8_t* __restrict__ label, const uint8_t* __restrict__ 
 
     // ---- the last block to finish delivers the matrix and its mean IoU and leaves the counters at zero for the next launch
     __shared__ bool is_last;
-    __shared__ double iou[kConfThreads];
-    __shared__ int present[kConfThreads];
+    __shared__ double iou[kMiouClasses];
+    __shared__ int present[kMiouClasses];
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) is_last = atomicAdd(fin.ticket, 1u) == gridDim.x - 1;

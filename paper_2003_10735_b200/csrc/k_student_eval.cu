@@ -34,8 +34,8 @@ student_eval_kernel(StudentMaskArgs a, const __grid_constant__ CUtensorMap x_map
     unsigned int* hist = (unsigned int*)(zt + CB * TZ);                    // [C][C] (CONF), under the stages as well
     __shared__ fused::Shared fsh;
     __shared__ bool is_last;
-    __shared__ double iou[256];
-    __shared__ int present[256];
+    __shared__ double iou[kMiouClasses];
+    __shared__ int present[kMiouClasses];
     const int C = a.C, h = a.h, w = a.w, H = h * kUp, W = w * kUp;
     const int tid = threadIdx.x, wi = tid >> 5, l = tid & 31;
     const int x0 = blockIdx.x * kOwnCols, y0 = blockIdx.y * kOwnRows;

@@ -22,7 +22,6 @@ constexpr int SM_WARPS = 4;                                              // cell
 #endif
 constexpr int SM_SPLIT = ST_MASK_SPLIT, SM_RW = 4 / SM_SPLIT;           // warps per cell row, frame rows per warp
 constexpr int SM_THREADS = SM_WARPS * SM_SPLIT * 32;
-static_assert(SM_THREADS == 256, "the mean IoU is taken by blocks of 256 threads");
 constexpr int SM_TH = SM_WARPS + 1, SM_TW = 40, SM_T = SM_TH * SM_TW;   // tile: 5 node rows x 40 columns (34 used, start at a multiple of 4)
 constexpr int kMaxChunk = 32;                                            // classes held in shared memory at a time
 
@@ -42,8 +41,8 @@ student_mask_kernel(StudentMaskArgs a, int chunk)
     extern __shared__ __align__(16) float zs[];                   // [chunk][SM_TH][SM_TW]
     unsigned int* hist = reinterpret_cast<unsigned int*>(zs + chunk * SM_T);   // [C][C] (CONF)
     __shared__ bool is_last;
-    __shared__ double iou[SM_THREADS];
-    __shared__ int present[SM_THREADS];
+    __shared__ double iou[kMiouClasses];
+    __shared__ int present[kMiouClasses];
     const int C = a.C, h = a.h, w = a.w, H = h * kUp, W = w * kUp;
     const int64_t p = (int64_t)h * w;
     const int tid = threadIdx.x, wi = tid / (32 * SM_SPLIT), l = tid & 31;   // wi: cell row inside the block

@@ -20,6 +20,7 @@ bool pdl_enabled()
 }
 
 constexpr int kUpdThreads = 256;
+static_assert(kUpdThreads == kMiouFetchThreads, "the update fetches the confusion matrix with all of its threads");
 
 // bf16 copies of weight element e (internal order [tap][cout][cin]) of a layer: the one the forward and the weight
 // gradient read, and, for a 3x3 layer whose gradient is passed back, the mirrored and transposed one
@@ -397,8 +398,8 @@ void launch_step_tick(long long* step_base, int S, int add, cudaStream_t s)
 
 __global__ void __launch_bounds__(256) miou_kernel(const unsigned long long* __restrict__ conf, int C, double* out)
 {
-    __shared__ double iou[256];
-    __shared__ int present[256];
+    __shared__ double iou[kMiouClasses];
+    __shared__ int present[kMiouClasses];
     const double m = block_miou(conf, C, iou, present);
     if (threadIdx.x == 0) *out = m;
 }

@@ -7,32 +7,35 @@ namespace st {
 
 // Mean IoU (Section 3.2): IoU_c = conf[c][c] / (row_c + col_c - conf[c][c]), averaged over the
 // classes present in the label (row_c > 0).  Integer counts, double arithmetic, fixed order.
-// Called by all 256 threads of a block; the value is returned to thread 0 only.  The counts are read past the L1
+// Called by all threads of a block of any number of whole warps; the value is returned to thread 0 only.  `iou` and `present`
+// are the block's shared arrays, written for classes below C only.  The counts are read past the L1
 // cache: the caller may be the last block of a kernel whose other blocks have just added to them.  Matrices of up to kMiouStage classes
 // are first copied to shared memory in one coalesced pass (one memory latency instead of one per row element).
-constexpr int kMiouStage = 32;
+constexpr int kMiouStage = 32, kMiouClasses = 256;
 // The copy to shared memory in two halves, for a caller that has other loads to issue while these are on their way:
-// miou_fetch starts the thread's share (blocks of 256 threads, C <= kMiouStage), block_miou takes it over.
-struct MiouFetch { unsigned long long v[kMiouStage * kMiouStage / 256]; };
+// miou_fetch starts the thread's share (blocks of kMiouFetchThreads threads, C <= kMiouStage), block_miou takes it over.
+constexpr int kMiouFetchThreads = 256;
+struct MiouFetch { unsigned long long v[kMiouStage * kMiouStage / kMiouFetchThreads]; };
 __device__ __forceinline__ MiouFetch miou_fetch(const unsigned long long* conf_g, int C)
 {
     MiouFetch f;
 #pragma unroll
-    for (int k = 0; k < kMiouStage * kMiouStage / 256; ++k) {
-        const int e = threadIdx.x + 256 * k;
+    for (int k = 0; k < kMiouStage * kMiouStage / kMiouFetchThreads; ++k) {
+        const int e = threadIdx.x + kMiouFetchThreads * k;
         f.v[k] = e < C * C ? __ldcg(conf_g + e) : 0ull;
     }
     return f;
 }
-__device__ __forceinline__ double block_miou(const unsigned long long* conf_g, int C, double* iou, int* present, const MiouFetch* fetched = nullptr)
+__device__ __forceinline__ double block_miou(const unsigned long long* conf_g, int C, double (&iou)[kMiouClasses], int (&present)[kMiouClasses],
+                                           const MiouFetch* fetched = nullptr)
 {
     __shared__ unsigned long long staged[kMiouStage * kMiouStage];
     const unsigned long long* conf = conf_g;
     if (C <= kMiouStage) {                                 // block-uniform
         if (fetched) {
 #pragma unroll
-            for (int k = 0; k < kMiouStage * kMiouStage / 256; ++k) {
-                const int e = threadIdx.x + 256 * k;
+            for (int k = 0; k < kMiouStage * kMiouStage / kMiouFetchThreads; ++k) {
+                const int e = threadIdx.x + kMiouFetchThreads * k;
                 if (e < C * C) staged[e] = fetched->v[k];
             }
         } else {
@@ -42,14 +45,14 @@ __device__ __forceinline__ double block_miou(const unsigned long long* conf_g, i
         conf = staged;
     }
     if (conf == staged) {
-        const int c = threadIdx.x;
-        double v = 0.0; int pr = 0;
+        const int c = threadIdx.x;                         // a thread per class: a warp is enough
         if (c < C) {
             unsigned long long row = 0, col = 0;
             for (int q = 0; q < C; ++q) { row += conf[c * C + q]; col += conf[q * C + c]; }
-            if (row > 0) { const unsigned long long inter = conf[c * C + c]; v = (double)inter / (double)(row + col - inter); pr = 1; }
+            const unsigned long long inter = conf[c * C + c];
+            iou[c] = row > 0 ? (double)inter / (double)(row + col - inter) : 0.0;
+            present[c] = row > 0;
         }
-        iou[c] = v; present[c] = pr;
     } else {
         // larger matrices stay in global memory: a warp per class, its lanes along the row and the column (81 classes: 162
         // dependent-latency loads per thread otherwise)

@@ -12,7 +12,7 @@ namespace st {
 // or, where no backward follows the prediction, by every block of the update itself (same counts, same arithmetic,
 // same answer).  In three parts so that the loads overlap what else a kernel waits for: train_history reads what the
 // previous assessment left (it may run before the kernel's predecessors have finished), train_fetch starts the loads of
-// the prediction's confusion matrix (blocks of 256 threads), train_decision finishes.  Block-uniform; called by all
+// the prediction's confusion matrix (blocks of kMiouFetchThreads threads), train_decision finishes (blocks of any size).  Block-uniform; called by all
 // threads of the block.  `writer` (one block per stream) records the history.
 struct TrainHistory { bool ended; double prev_best; };
 __device__ __forceinline__ TrainHistory train_history(const TrainCtl& t, int s)
@@ -31,8 +31,8 @@ __device__ __forceinline__ MiouFetch train_fetch(const TrainCtl& t, int s, const
 __device__ __forceinline__ void train_decision(const TrainCtl& t, int s, bool writer, const TrainHistory& h, const MiouFetch* f,
                                                bool& skip, bool& better)
 {
-    __shared__ double iou[256];
-    __shared__ int present[256];
+    __shared__ double iou[kMiouClasses];
+    __shared__ int present[kMiouClasses];
     __shared__ double m_sh;
     const int i = t.iter;
     int* done = t.done + (int64_t)s * kCtlPitch;
