@@ -223,7 +223,7 @@ ST_API st_status st_train_key_frame(st_ctx *ctx, double threshold, int32_t max_u
  * st_pack_updated_params — UpdatedPart(student) (Algorithm 3; Table 4 sizes are fp32):
  * the current values of every trainable tensor of `stream`, fp32 little-endian, per layer in
  * forward order weight [Cout][Cin][kh][kw] then bias [Cout]; no header, no padding.
- *   dst           host or device.
+ *   dst           host or device, at any address; the call waits for the stream if it is host memory.
  *   dst_capacity  bytes available at dst; ST_ERR_BUFFER_TOO_SMALL if below the packed size.
  *   nbytes        host, may be NULL; receives the packed size (also on BUFFER_TOO_SMALL).
  * Momentum is not part of the buffer.  Feeding the buffer back to st_init_head reproduces
@@ -236,7 +236,7 @@ ST_API st_status st_pack_updated_params(st_ctx *ctx, int32_t stream, void *dst, 
  * st_pack_updated_params as the parameters of `stream`.  The updated part carries values, not differences, so the
  * trainable tensors are simply replaced; the momentum buffer is left as it is.  This is what the client does with
  * the server's reply, and what a server does to move a student between contexts.
- *   src     host or device; the packed buffer (layout of st_pack_updated_params).
+ *   src     host or device, at any address; the packed buffer (layout of st_pack_updated_params).
  *   nbytes  its size; must equal st_param_count * 4, else ST_ERR_INVALID_ARG.
  * pack -> apply -> pack reproduces the buffer bit for bit.
  */

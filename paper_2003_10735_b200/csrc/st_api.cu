@@ -179,24 +179,34 @@ st_status ensure_staging(st_ctx* ctx, size_t bytes)
     return ST_OK;
 }
 
+// Copy `bytes` of a caller's buffer, wherever it lies, into the staging buffer.
+st_status to_staging(st_ctx* ctx, const void* src, size_t bytes)
+{
+    st_status st = ensure_staging(ctx, bytes);
+    if (st != ST_OK) return st;
+    ST_CUDA(ctx, cudaMemcpyAsync(ctx->staging, src, bytes, cudaMemcpyDefault, ctx->stream));
+    return ST_OK;
+}
+
 // Bring `bytes` of a host-or-device source into device memory; *dev receives a device pointer
 // (the source itself if it already is one).
 st_status to_device(st_ctx* ctx, const void* src, size_t bytes, const void** dev)
 {
     if (is_device_ptr(src)) { *dev = src; return ST_OK; }
-    st_status st = ensure_staging(ctx, bytes);
-    if (st != ST_OK) return st;
-    ST_CUDA(ctx, cudaMemcpyAsync(ctx->staging, src, bytes, cudaMemcpyHostToDevice, ctx->stream));
-    *dev = ctx->staging;
-    return ST_OK;
+    *dev = nullptr;
+    st_status st = to_staging(ctx, src, bytes);
+    if (st == ST_OK) *dev = ctx->staging;
+    return st;
 }
 
-// The same for a buffer of a student's size: pinned host memory is read by the kernel itself (21 KB over the bus inside an
-// unpacking kernel: predict at 720p 46 -> 38 us; the copy engine's start and its hand-over to the kernel cost more than the bytes).
-st_status small_to_device(st_ctx* ctx, const void* src, size_t bytes, const void** dev)
+// Whether the kernels that pack and unpack can work on a caller's packed buffer itself (*dev: its device address): device
+// memory, or pinned host memory, which they read or write over the bus (21 KB inside an unpacking kernel: predict at 720p 46 ->
+// 38 us; the copy engine's start and its hand-over to the kernel cost more than the bytes).  They access floats, and the
+// buffer is one of bytes that may lie anywhere in a message: at other addresses it goes through the staging buffer.
+bool packed_in_place(const void* q, const void** dev, Where* where)
 {
-    if (locate(src, dev) != Where::host) return ST_OK;
-    return to_device(ctx, src, bytes, dev);
+    *where = locate(q, dev);
+    return *where != Where::host && ((uintptr_t)*dev & (sizeof(float) - 1)) == 0;
 }
 
 st_status check_stream_index(st_ctx* ctx, int32_t s)
@@ -1144,23 +1154,19 @@ st_status st_pack_updated_params(st_ctx* ctx, int32_t stream, void* dst, size_t 
     const float* src = ctx->theta + (int64_t)stream * ctx->n_params;
     const int first = ctx->bf16_mode ? ctx->first_trained : 0;
     const void* to = nullptr;
-    const Where where = locate(dst, &to);
-    if (where != Where::host) {             // device memory, or pinned host memory written by the kernel itself
-        launch_pack(src, (float*)const_cast<void*>(to), ctx->layout, first, 1, ctx->stream);
-        ctx->launches += 1;
-        st = check_launch(ctx, "pack");
-        if (st == ST_OK && where == Where::pinned) ST_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-        return st;
+    Where where;
+    const bool in_place = packed_in_place(dst, &to, &where);
+    if (!in_place) {                        // packed into the staging buffer, then copied out
+        st = ensure_staging(ctx, need);
+        if (st != ST_OK) return st;
+        to = ctx->staging;
     }
-    // other host memory: pack into the staging buffer, then copy out
-    st = ensure_staging(ctx, need);
-    if (st != ST_OK) return st;
-    launch_pack(src, (float*)ctx->staging, ctx->layout, first, 1, ctx->stream);
+    launch_pack(src, (float*)const_cast<void*>(to), ctx->layout, first, 1, ctx->stream);
     ctx->launches += 1;
     st = check_launch(ctx, "pack");
     if (st != ST_OK) return st;
-    ST_CUDA(ctx, cudaMemcpyAsync(dst, ctx->staging, need, cudaMemcpyDeviceToHost, ctx->stream));
-    ST_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (!in_place) ST_CUDA(ctx, cudaMemcpyAsync(dst, to, need, cudaMemcpyDefault, ctx->stream));
+    if (where != Where::device) ST_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return ST_OK;
 }
 
@@ -1172,8 +1178,12 @@ st_status st_apply_update(st_ctx* ctx, int32_t stream, const void* src, size_t n
     if (!src) return fail(ctx, ST_ERR_INVALID_ARG, "st_apply_update: NULL source");
     if (nbytes != need) return fail(ctx, ST_ERR_INVALID_ARG, "st_apply_update: %zu bytes given, the updated part has %zu", nbytes, need);
     const void* dev = nullptr;
-    st = small_to_device(ctx, src, need, &dev);
-    if (st != ST_OK) return st;
+    Where where;
+    if (!packed_in_place(src, &dev, &where)) {
+        st = to_staging(ctx, src, need);
+        if (st != ST_OK) return st;
+        dev = ctx->staging;
+    }
     ctx->z_current = false;
     UpdateArgs u = make_update_args(ctx, -1);
     if (!ctx->bf16_mode) u.n_layers = 0;

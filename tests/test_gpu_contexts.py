@@ -1,0 +1,59 @@
+"""What a context must not depend on: other contexts in the process, the number of streams beside a stream, the buffers that
+results are asked for in, and what it has been asked before."""
+import numpy as np
+import pytest
+
+import synth_inputs as si
+import paper_2003_10735_b200 as st
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(autouse=True)
+def side_stream():
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        yield s
+    s.synchronize()
+
+
+def make(c_in, ch, C, h, w, S=1, prec=0, seed=0, **kw):
+    """A context with inputs; stream s has the same student, features and labels whatever S is."""
+    thetas = [si.initial_head_params(c_in, ch, C, 100 + seed + s) for s in range(S)]
+    ctx = st.st_init_head(n_streams=S, c_in=c_in, c_hidden=ch, n_classes=C, feat_h=h, feat_w=w, gemm_precision=prec,
+                          lr=kw.pop("lr", 0.1), momentum=kw.pop("momentum", 0.9),
+                          cuda_stream=torch.cuda.current_stream().cuda_stream, init_params=np.concatenate(thetas), **kw)
+    for s in range(S):
+        rng = np.random.default_rng(seed + s)
+        st.st_set_frozen_features(ctx, s, np.maximum(rng.standard_normal((c_in, h, w)), 0).astype(np.float32))
+        st.st_set_labels(ctx, s, si.voronoi_map(4 * h, 4 * w, 9, C, 300 + seed + s))
+    return ctx
+
+
+def packed(ctx, s=0):
+    out = np.empty(ctx.n_params, np.float32)
+    st.st_pack_updated_params(ctx, s, out)
+    return out
+
+
+# ---- where packed buffers lie
+@pytest.mark.parametrize("where", ["pinned", "device", "ordinary"])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3, 4, 13])        # bytes of a message in front of the buffer
+@pytest.mark.parametrize("ch,prec", [(0, 1), (64, 1), (9, 0)])
+def test_packed_buffers_at_any_address(ch, prec, offset, where):
+    """Packed buffers are bytes: behind a header of any length they give and take the same parameters."""
+    server, client = make(64, ch, 5, 12, 20, prec=prec, seed=1), make(64, ch, 5, 12, 20, prec=prec, seed=2)
+    st.st_distill_step(server, 2)
+    want, n = packed(server).tobytes(), server.n_params * 4
+    message = torch.full((n + offset + 16,), 0x5a, dtype=torch.uint8)
+    message = message.pin_memory() if where == "pinned" else message.cuda() if where == "device" else message
+    lib = st.load_library()
+    st._check(lib.st_pack_updated_params(server.handle, 0, message.data_ptr() + offset, n, None), server)
+    got = message.cpu().numpy()
+    assert got[offset:offset + n].tobytes() == want
+    assert (got[:offset] == 0x5a).all() and (got[offset + n:] == 0x5a).all()
+    st._check(lib.st_apply_update(client.handle, 0, message.data_ptr() + offset, n), client)
+    assert packed(client).tobytes() == want
+    st.st_destroy(server)
+    st.st_destroy(client)
