@@ -349,10 +349,12 @@ conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
 namespace {
 
 // Thread groups per block, channel tiles and pixel ranges of a weight gradient: as many ranges as give every SM about
-// eight warps (a warp has enough independent sums to keep its scheduler busy with two), each range at least one chunk.
+// eight warps of one stream (a warp has enough independent sums to keep its scheduler busy with two), each range at least one
+// chunk.  The number of streams has no part in it: the ranges group a gradient's sums, and a stream's results must be the same
+// whatever it shares the launch with.
 struct WgradShape { int ng, ci_tiles, co_tiles, tiles_x, n_chunks, n_split; };
 template <int KS, int CO>
-WgradShape wgrad_shape(int Cin, int Cout, int h, int w, int S)
+WgradShape wgrad_shape(int Cin, int Cout, int h, int w)
 {
     WgradShape q;
     constexpr int RW = wg_rows<KS>(), kMost = wg_most_groups<KS>();
@@ -363,19 +365,19 @@ WgradShape wgrad_shape(int Cin, int Cout, int h, int w, int S)
     q.ci_tiles = (Cin + 31) / 32;
     q.tiles_x = (w + kTileX - 1) / kTileX;
     q.n_chunks = q.tiles_x * ((h + RW - 1) / RW);
-    const int64_t per_range = (int64_t)q.ci_tiles * q.co_tiles * S, warps = q.ng * RW;
-    int64_t n = 148 * (warps >= 5 ? 1 : 8 / warps) / per_range;
+    const int per_range = q.ci_tiles * q.co_tiles, warps = q.ng * RW;
+    int n = 148 * (warps >= 5 ? 1 : 8 / warps) / per_range;
     if (n > 128) n = 128;                              // the update adds the ranges' results one by one
     if (n > q.n_chunks) n = q.n_chunks;
-    q.n_split = (int)(n < 1 ? 1 : n);
+    q.n_split = n < 1 ? 1 : n;
     return q;
 }
 // 1x1 layers: 16 channels per warp keep the loads below the multiply-adds; a head with a handful of classes takes 4
 bool narrow(int Cout) { return Cout <= 4; }
-WgradShape wgrad_shape_of(int Cin, int Cout, int h, int w, int ks, int S)
+WgradShape wgrad_shape_of(int Cin, int Cout, int h, int w, int ks)
 {
-    if (ks == 3) return wgrad_shape<3, 8>(Cin, Cout, h, w, S);
-    return narrow(Cout) ? wgrad_shape<1, 4>(Cin, Cout, h, w, S) : wgrad_shape<1, 16>(Cin, Cout, h, w, S);
+    if (ks == 3) return wgrad_shape<3, 8>(Cin, Cout, h, w);
+    return narrow(Cout) ? wgrad_shape<1, 4>(Cin, Cout, h, w) : wgrad_shape<1, 16>(Cin, Cout, h, w);
 }
 
 template <int KS, int CO>
@@ -425,12 +427,12 @@ void launch_conv1x1_dgrad_relu_f32(const float* W2, const float* dz, const float
     launch_fwd_any(a, 1, S, early, s);
 }
 
-int conv_wgrad_f32_splits(int Cin, int Cout, int h, int w, int ks, int S) { return wgrad_shape_of(Cin, Cout, h, w, ks, S).n_split; }
+int conv_wgrad_f32_splits(int Cin, int Cout, int h, int w, int ks) { return wgrad_shape_of(Cin, Cout, h, w, ks).n_split; }
 
 void launch_conv_wgrad_f32(const float* in, const float* dout, int Cin, int Cout, int h, int w, int ks, float* partials,
                            float* b_partials, int S, bool early, cudaStream_t s)
 {
-    const WgradShape q = wgrad_shape_of(Cin, Cout, h, w, ks, S);
+    const WgradShape q = wgrad_shape_of(Cin, Cout, h, w, ks);
     const PadF32 pad(h, w);
     const WgradF32 a = {in, dout, partials, b_partials, Cin, Cout, h, w, q.n_split, Cin * pad.plane, Cout * pad.plane};
     if (ks == 3) launch_wgrad<3, 8>(a, q, S, early, s);

@@ -679,11 +679,11 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     } else {
         const int64_t plane = PadF32(c->h, c->w).plane;
         ALLOC(x_f32, S * c->Cin * plane);
-        c->n_split2 = conv_wgrad_f32_splits(c_last, c->C, c->h, c->w, 1, S);
+        c->n_split2 = conv_wgrad_f32_splits(c_last, c->C, c->h, c->w, 1);
         ALLOC(w2_partials, (size_t)S * c->n_split2 * c->C * c_last);
         if (c->Ch) {
             ALLOC(hid_f32, S * c->Ch * plane); ALLOC(dhid_f32, S * c->Ch * plane);
-            c->n_split1 = c->blk[0].n_bpart = conv_wgrad_f32_splits(c->Cin, c->Ch, c->h, c->w, 3, S);
+            c->n_split1 = c->blk[0].n_bpart = conv_wgrad_f32_splits(c->Cin, c->Ch, c->h, c->w, 3);
             ALLOC(blk[0].w_partials, (size_t)S * c->n_split1 * 9 * c->Ch * c->Cin);
             ALLOC(blk[0].b_partials, (size_t)S * c->n_split1 * c->Ch);
         }

@@ -185,7 +185,7 @@ void launch_conv_fwd_f32(const float* in, int Cin, int h, int w, const float* Wt
                          float* out, bool out_padded, int S, int64_t w_stride, bool early, cudaStream_t s);
 // Weight gradient as n_split = conv_wgrad_f32_splits(...) partial results [S][n_split][tap][Cout][Cin], which the parameter
 // update adds; with b_partials also the bias gradient's, [S][n_split][Cout]
-int conv_wgrad_f32_splits(int Cin, int Cout, int h, int w, int ks, int S);
+int conv_wgrad_f32_splits(int Cin, int Cout, int h, int w, int ks);
 void launch_conv_wgrad_f32(const float* in, const float* dout, int Cin, int Cout, int h, int w, int ks, float* partials,
                            float* b_partials, int S, bool early, cudaStream_t s);
 void launch_conv1x1_dgrad_relu_f32(const float* W2, const float* dz, const float* Hact, int C, int Ch, int h, int w, float* dH, int S,

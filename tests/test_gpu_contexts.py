@@ -57,3 +57,23 @@ def test_packed_buffers_at_any_address(ch, prec, offset, where):
     assert packed(client).tobytes() == want
     st.st_destroy(server)
     st.st_destroy(client)
+
+
+# ---- the number of streams
+@pytest.mark.parametrize("c_in,ch,C,h,w,prec", [
+    (33, 9, 5, 40, 70, 0), (96, 48, 40, 24, 40, 0), (5, 0, 4, 61, 90, 0), (64, 0, 21, 45, 80, 0),
+    (64, 64, 5, 24, 40, 1), (64, 64, 5, 90, 80, 1), (128, 0, 21, 45, 80, 1),       # the second: another form of the 1x1 forward for 16 streams
+])
+def test_results_of_a_stream_do_not_depend_on_its_neighbours(c_in, ch, C, h, w, prec):
+    K = 2
+    one = make(c_in, ch, C, h, w, 1, prec)
+    want = np.zeros((1, K), np.float32)
+    st.st_distill_step(one, K, want)
+    for S in (2, 5, 16):
+        many = make(c_in, ch, C, h, w, S, prec)
+        loss = np.zeros((S, K), np.float32)
+        st.st_distill_step(many, K, loss)
+        assert packed(many).tobytes() == packed(one).tobytes(), S
+        assert loss[0].tobytes() == want[0].tobytes(), S
+        st.st_destroy(many)
+    st.st_destroy(one)
