@@ -391,13 +391,12 @@ void launch_wgrad(const WgradF32& a, const WgradShape& q, int S, bool early, cud
 
 cudaError_t prepare_conv_f32()
 {
-    auto allow = [](const void* fn, size_t bytes) { return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); };
-    cudaError_t e = allow((const void*)conv_fwd_f32_kernel<3, 8>, fwd_smem<3, 8>(kFwdGroups));
-    if (e == cudaSuccess) e = allow((const void*)conv_fwd_f32_kernel<1, 8>, fwd_smem<1, 8>(kFwdGroups));
-    if (e == cudaSuccess) e = allow((const void*)conv_fwd_f32_kernel<1, 4>, fwd_smem<1, 4>(1));
-    if (e == cudaSuccess) e = allow((const void*)conv_wgrad_f32_kernel<3, 8>, wg_smem<3, 8>(wg_most_groups<3>()));
-    if (e == cudaSuccess) e = allow((const void*)conv_wgrad_f32_kernel<1, 16>, wg_smem<1, 16>(wg_most_groups<1>()));
-    if (e == cudaSuccess) e = allow((const void*)conv_wgrad_f32_kernel<1, 4>, wg_smem<1, 4>(1));
+    cudaError_t e = allow_shared_memory((const void*)conv_fwd_f32_kernel<3, 8>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_fwd_f32_kernel<1, 8>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_fwd_f32_kernel<1, 4>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<3, 8>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<1, 16>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<1, 4>);
     return e;
 }
 

@@ -1271,26 +1271,14 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         snprintf(err, err_len, "shared memory per block exceeds 227 KB for these channel counts");
         delete P; return nullptr;
     }
-    // Raise a kernel's shared-memory allowance to what this plan launches it with, never lower it: the attribute belongs
-    // to the function, not to a plan, and an earlier plan with larger layers may still be in use.
-    auto allow = [&](const void* fn, size_t need) -> cudaError_t {
-        cudaFuncAttributes at;
-        cudaError_t r = cudaFuncGetAttributes(&at, fn);
-        if (r != cudaSuccess) return r;
-        if (need <= (size_t)at.maxDynamicSharedSizeBytes) return cudaSuccess;
-        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    };
-    cudaError_t e = cudaSuccess;
-    if (!P->fwd1_persistent) e = allow((const void*)tc_fwd1x1_kernel, P->smem_fwd1);
-    if (e == cudaSuccess && P->fwd1_persistent) e = allow((const void*)tc_fwd1x1p_kernel, P->smem_fwd1p);
-    if (e == cudaSuccess) e = allow((const void*)tc_wgrad1x1_kernel<kWg1Stages>, P->smem_wg1);
+    cudaError_t e = allow_shared_memory(P->fwd1_persistent ? (const void*)tc_fwd1x1p_kernel : (const void*)tc_fwd1x1_kernel);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)tc_wgrad1x1_kernel<kWg1Stages>);
     for (int i = 0; i < nb; ++i) {
-        const TcBlockPlan& q = P->blk[i];
-        if (e == cudaSuccess) e = allow((const void*)fwd3_kernel<0>(b.blk[i].c_out), q.smem_fwd);
-        if (e == cudaSuccess && b.blk[i].pass_back) e = allow((const void*)fwd3_kernel<1>(b.blk[i].c_prev), q.smem_back);
-        if (e == cudaSuccess) e = allow((const void*)wgrad3_kernel(q.wg), q.wg.bytes);
+        if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd3_kernel<0>(b.blk[i].c_out));
+        if (e == cudaSuccess && b.blk[i].pass_back) e = allow_shared_memory((const void*)fwd3_kernel<1>(b.blk[i].c_prev));
+        if (e == cudaSuccess) e = allow_shared_memory((const void*)wgrad3_kernel(P->blk[i].wg));
     }
-    if (nb && e == cudaSuccess) e = allow((const void*)tc_back1x1_kernel, P->smem_back1);
+    if (nb && e == cudaSuccess) e = allow_shared_memory((const void*)tc_back1x1_kernel);
     if (e != cudaSuccess) { snprintf(err, err_len, "shared-memory attribute: %s", cudaGetErrorString(e)); delete P; return nullptr; }
     return P;
 }

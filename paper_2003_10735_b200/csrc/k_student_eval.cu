@@ -163,12 +163,11 @@ template <int CB>
 size_t eval_smem_bytes(int C) { return fused::smem_bytes(((size_t)CB * TZ + (size_t)C * C) * sizeof(float)); }
 
 template <int CB>
-cudaError_t prepare_cb(int C)
+cudaError_t prepare_cb()
 {
-    const int smem = (int)eval_smem_bytes<CB>(C);
-    cudaError_t e = cudaFuncSetAttribute(student_eval_kernel<CB, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(student_eval_kernel<CB, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(student_eval_kernel<CB, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_shared_memory((const void*)student_eval_kernel<CB, true, false>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)student_eval_kernel<CB, true, true>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)student_eval_kernel<CB, false, true>);
     return e;
 }
 
@@ -206,7 +205,7 @@ int bucket(int C)
 cudaError_t prepare_student_eval(int C)
 {
     if (C > kClassPad) return cudaSuccess;
-    ST_EVAL_DISPATCH(prepare_cb, C, C)
+    ST_EVAL_DISPATCH(prepare_cb, C)
 }
 
 cudaError_t launch_student_eval(const StudentMaskArgs& a, cudaStream_t s) { ST_EVAL_DISPATCH(launch_cb, a.C, a, s) }

@@ -185,15 +185,12 @@ bool student_mask_fused_supported(int C)
     return mask_smem(C, true, &chunk) <= 160 * 1024;
 }
 
-cudaError_t prepare_student_mask(int C)
+cudaError_t prepare_student_mask()
 {
-    int chunk;
-    cudaError_t e = cudaFuncSetAttribute(student_mask_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mask_smem(C, false, &chunk));
-    if (e != cudaSuccess || !student_mask_fused_supported(C)) return e;
-    const int smem = (int)mask_smem(C, true, &chunk);
-    e = cudaFuncSetAttribute(student_mask_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(student_mask_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_shared_memory((const void*)student_mask_kernel<true, false>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)student_mask_kernel<false, true>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)student_mask_kernel<true, true>);
+    return e;
 }
 
 void launch_student_mask(const StudentMaskArgs& a, cudaStream_t s)

@@ -384,9 +384,8 @@ upsample_ce_many_kernel(UpsampleCeArgs a)
 template <int NY, int G>
 cudaError_t allow_many()
 {
-    cudaError_t e = cudaFuncSetAttribute(upsample_ce_many_kernel<NY, G, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)many_smem<NY, G>(255, false));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(upsample_ce_many_kernel<NY, G, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)many_smem<NY, G>(255, true));
+    const cudaError_t e = allow_shared_memory((const void*)upsample_ce_many_kernel<NY, G, false>);
+    return e != cudaSuccess ? e : allow_shared_memory((const void*)upsample_ce_many_kernel<NY, G, true>);
 }
 
 template <int NY, int G>

@@ -643,12 +643,12 @@ size_t rows_smem_bytes(int C, bool conf)
 }
 
 template <int CB>
-cudaError_t prepare_cb(int C)
+cudaError_t prepare_cb()
 {
-    cudaError_t e = cudaFuncSetAttribute(upsample_ce_rows_kernel<CB, false, kTwLoad>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem_bytes<CB, kTwLoad>(C, false));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(upsample_ce_rows_kernel<CB, true, kTwLoad>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem_bytes<CB, kTwLoad>(C, true));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(upsample_ce_rows_kernel<CB, false, kTwFused>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem_bytes<CB, kTwFused>(C, false));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(upsample_ce_rows_kernel<CB, true, kTwFused>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem_bytes<CB, kTwFused>(C, true));
+    cudaError_t e = allow_shared_memory((const void*)upsample_ce_rows_kernel<CB, false, kTwLoad>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)upsample_ce_rows_kernel<CB, true, kTwLoad>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)upsample_ce_rows_kernel<CB, false, kTwFused>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)upsample_ce_rows_kernel<CB, true, kTwFused>);
     return e;
 }
 
@@ -692,7 +692,7 @@ int upsample_ce_rows_blocks(int h, int w) { return ((h + RN_Y - 1) / RN_Y) * ((w
         default: return FN<32>(__VA_ARGS__);         \
     }
 
-cudaError_t prepare_upsample_ce_rows(int C) { ST_ROWS_DISPATCH(prepare_cb, C, C) }
+cudaError_t prepare_upsample_ce_rows(int C) { ST_ROWS_DISPATCH(prepare_cb, C) }
 
 cudaError_t launch_rows_dispatch(const UpsampleCeArgs& a, const CUtensorMap& z_map, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
 {

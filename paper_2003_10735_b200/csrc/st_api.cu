@@ -691,7 +691,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
 #undef ALLOC
     if (e == cudaSuccess) e = prepare_upsample_ce(c->C);
     if (e == cudaSuccess) c->k3_has_map = make_logit_tile_map(&c->k3_map, c->z, S, c->C, c->h, c->w) ? 1 : 0;
-    if (e == cudaSuccess) e = prepare_student_mask(c->C);
+    if (e == cudaSuccess) e = prepare_student_mask();
     if (e == cudaSuccess && !c->bf16_mode) e = prepare_conv_f32();
     if (e != cudaSuccess) {
         st_status code = fail(nullptr, e == cudaErrorMemoryAllocation ? ST_ERR_OOM : ST_ERR_CUDA,

@@ -33,6 +33,19 @@ __device__ __forceinline__ void store_256(void* dst, const uint32_t* r)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Let launches of a kernel take all the shared memory that a block can have.  The limit belongs to the function and not to a
+// context: one set to what a context needs is taken from every other context that needs more.
+inline cudaError_t allow_shared_memory(const void* kernel)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes at;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
+}
+
 bool pdl_enabled();   // true unless the environment variable ST_PDL is set to 0
 
 // `early`: launch with the programmatic-serialization attribute, i.e. the kernel may start before its predecessor on
@@ -164,7 +177,7 @@ struct StudentMaskArgs {
 cudaError_t prepare_student_eval(int C);    // once per device and class count, outside any stream capture
 cudaError_t launch_student_eval(const StudentMaskArgs& a, cudaStream_t s);
 bool student_mask_fused_supported(int C);   // confusion counters fit shared memory
-cudaError_t prepare_student_mask(int C);    // once per device and class count, outside any stream capture
+cudaError_t prepare_student_mask();         // once per device, outside any stream capture
 void launch_student_mask(const StudentMaskArgs& a, cudaStream_t s);
 
 // ---- fp32 CUDA-core convolutions (gemm_precision 0) -------------------------------------------

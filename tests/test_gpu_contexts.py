@@ -77,3 +77,24 @@ def test_results_of_a_stream_do_not_depend_on_its_neighbours(c_in, ch, C, h, w, 
         assert loss[0].tobytes() == want[0].tobytes(), S
         st.st_destroy(many)
     st.st_destroy(one)
+
+
+# ---- other contexts
+@pytest.mark.parametrize("first,second,ch,prec", [(24, 22, 0, 1), (32, 29, 64, 1), (8, 5, 0, 0), (120, 60, 0, 0), (255, 33, 0, 0), (32, 9, 0, 0)])
+def test_a_later_context_of_fewer_classes_takes_nothing_from_an_earlier_one(first, second, ch, prec):
+    c_in, h, w = 64, 20, 40
+    want = {}
+    for C in (first, second):
+        ctx = make(c_in, ch, C, h, w, prec=prec)
+        conf = np.zeros((1, 2, C, C), np.int64)
+        st.st_distill_step(ctx, 2, None, conf)
+        want[C] = (packed(ctx).tobytes(), conf, st.st_agreement(ctx, 0))
+        st.st_destroy(ctx)
+    a, b = make(c_in, ch, first, h, w, prec=prec), make(c_in, ch, second, h, w, prec=prec)
+    for ctx, C in ((a, first), (b, second)):
+        conf = np.zeros((1, 2, C, C), np.int64)
+        st.st_distill_step(ctx, 2, None, conf)
+        np.testing.assert_array_equal(conf, want[C][1])
+        assert packed(ctx).tobytes() == want[C][0]
+        assert st.st_agreement(ctx, 0) == want[C][2]
+        st.st_destroy(ctx)
