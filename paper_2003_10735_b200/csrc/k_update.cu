@@ -329,9 +329,7 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (lane == 0) {
             if (a.loss_slot >= 0 && a.loss_slot < kMaxSteps) {
-                const float mean = (float)(t * a.inv_P);
-                a.loss_buf[(int64_t)s * kMaxSteps + a.loss_slot] = mean;
-                if (a.loss_out) a.loss_out[(int64_t)s * a.loss_pitch + a.loss_slot] = mean;
+                a.loss_buf[(int64_t)s * kMaxSteps + a.loss_slot] = (float)(t * a.inv_P);
             }
         }
     }
@@ -438,6 +436,19 @@ static unsigned copy_blocks(int64_t n_params)
 void launch_train_commit(const UpdateArgs& a, const float* best_theta, const int* n_updates, cudaStream_t s)
 {
     launch_early(pdl_enabled(), train_commit_kernel, dim3(copy_blocks(a.n_params - a.param_begin), (unsigned)a.S), dim3(256), 0, s, a, best_theta, n_updates);
+}
+
+__global__ void __launch_bounds__(256) train_begin_kernel(unsigned long long* __restrict__ conf, int64_t n, double* threshold, double value)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) conf[i] = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *threshold = value;
+}
+
+void launch_train_begin(unsigned long long* conf, int64_t n, double* threshold, double value, cudaStream_t s)
+{
+    launch_early(pdl_enabled(), train_begin_kernel, dim3(copy_blocks(n)), dim3(256), 0, s, conf, n, threshold, value);
 }
 
 __global__ void train_results_kernel(TrainCtl t, const float* __restrict__ loss_buf, TrainResults out)

@@ -20,14 +20,13 @@ using namespace st;
 namespace {
 thread_local std::string g_init_error;
 
-// A replayable graph: n_steps plain iterations (train = false), or Train with MAX_UPDATES = n_steps and the
-// threshold whose bit pattern is `thr` (train = true).
+// A replayable graph: n_steps plain iterations (train = false), or Train with MAX_UPDATES = n_steps (train = true).  Nothing that
+// may change from call to call is part of it: results are delivered by a kernel behind it, the threshold lies in device memory.
 struct GraphKey {
-    int n_steps; bool conf; bool train; uint64_t thr;
-    float* loss;       // nullptr, or the caller's device buffer that the updates write the losses to as well
-    bool operator<(const GraphKey& o) const { return std::tie(n_steps, conf, train, thr, loss) < std::tie(o.n_steps, o.conf, o.train, o.thr, o.loss); }
+    int n_steps; bool conf; bool train;
+    bool operator<(const GraphKey& o) const { return std::tie(n_steps, conf, train) < std::tie(o.n_steps, o.conf, o.train); }
 };
-constexpr size_t kMaxGraphs = 32;       // replayable graphs kept per context
+constexpr size_t kMaxGraphs = 32;       // replayable graphs kept per context (0.6 MB of device memory each with 64 predictions)
 }  // namespace
 
 struct st_ctx {
@@ -77,8 +76,6 @@ struct st_ctx {
     int fused_fwd = 0;          //   (one-layer head with bf16 GEMMs; ST_FUSED_FORWARD=0 switches it off)
     int test_stall_fused = 0;   // test of the give-up path inside that kernel (environment ST_TEST_STALL_FUSED=1 at context creation)
     float* loss_buf = nullptr;              // [S][kMaxSteps]
-    float* loss_seen = nullptr;             // the device buffer that the last st_distill_step delivered its losses to
-    float* loss_direct = nullptr; int loss_pitch = 0;   // during a call: where the updates write the losses as well
     unsigned long long* conf_buf = nullptr; // [S][kMaxSteps][C][C], allocated on first use
     // Train (Algorithm 1), allocated on first use
     float* best_theta = nullptr;            // [S][n_params] best_student
@@ -88,6 +85,7 @@ struct st_ctx {
     int* ctl_n_updates = nullptr;           // [S]
     int* ctl_best_iter = nullptr;           // [S]
     int* ctl_better = nullptr;              // [S][kCtlPitch]
+    double* ctl_threshold = nullptr;        // THRESHOLD of the call
     unsigned int* bad = nullptr;            // [3]: labels >= C met by a step / by st_agreement; [2] = first device wait that gave up
     uint8_t* mask_tmp = nullptr;            // [P]
     uint8_t* mask_tmp2 = nullptr;           // [P]
@@ -106,8 +104,9 @@ struct st_ctx {
     bool settled = false;                   // a step loop has run since the features and labels were last written: nothing in flight writes them
     bool z_unkept = false;                  // the last call multiplied its logits inside the loss kernel and kept none of them
     TcPlan* plan = nullptr;
-    struct StepGraph { cudaGraphExec_t exec; int64_t n_launches; };
+    struct StepGraph { cudaGraphExec_t exec; int64_t n_launches; int64_t used; };
     std::map<GraphKey, StepGraph> graphs;
+    int64_t replays = 0;                    // StepGraph::used: the replay that used it last
     bool use_graphs = true;
     bool chain_early = false;               // kernels of a step may start while their predecessor drains (one-layer heads)
     std::string err;
@@ -263,7 +262,6 @@ UpdateArgs make_update_args(st_ctx* c, int slot, const int* skip = nullptr, int6
     }
     u.loss_part = c->loss_part; u.n_loss_part = c->n_k3_blocks;
     u.loss_buf = c->loss_buf; u.loss_slot = slot;
-    u.loss_out = c->loss_direct; u.loss_pitch = c->loss_pitch;
     u.inv_P = 1.0 / (double)c->P;
     u.skip = skip; u.skip_stride = skip_stride;
     u.adam = c->adam ? 1 : 0; u.vel2 = c->vel2; u.step_base = c->step_base;
@@ -448,6 +446,55 @@ st_status report_bad_labels(st_ctx* c, int which, const char* what)
     return report_status(c, which == 1);
 }
 
+TrainCtl train_ctl(st_ctx* c, int iter, int max_updates)
+{
+    TrainCtl t;
+    t.conf = c->conf_buf + (int64_t)iter * c->C * c->C;
+    t.conf_stream_stride = (int64_t)kMaxSteps * c->C * c->C;
+    t.C = c->C; t.iter = iter; t.max_updates = max_updates; t.threshold = c->ctl_threshold;
+    t.done = c->ctl_done; t.best = c->ctl_best; t.metric = c->ctl_metric;
+    t.n_updates = c->ctl_n_updates; t.best_iter = c->ctl_best_iter; t.better = c->ctl_better;
+    t.theta = c->theta; t.best_theta = c->best_theta; t.n_params = c->n_params; t.S = c->S;
+    t.param_begin = c->trained_begin;
+    return t;
+}
+
+// Run what `enqueue` puts on the stream as a graph: captured the first time a key is asked for, replayed from then on.  A context
+// keeps the kMaxGraphs graphs used last.
+template <typename Enqueue>
+st_status run_as_graph(st_ctx* ctx, const GraphKey& key, const char* who, Enqueue enqueue)
+{
+    if (!ctx->use_graphs) return enqueue();
+    auto it = ctx->graphs.find(key);
+    if (it == ctx->graphs.end()) {
+        cudaGraph_t graph = nullptr;
+        const int64_t before = ctx->launches;
+        ST_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
+        const st_status st = enqueue();
+        cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
+        const int64_t n_launches = ctx->launches - before;
+        ctx->launches = before;
+        if (st != ST_OK) { if (graph) cudaGraphDestroy(graph); return st; }
+        if (e != cudaSuccess) return fail(ctx, ST_ERR_CUDA, "%s: graph capture: %s", who, cudaGetErrorString(e));
+        cudaGraphExec_t exec = nullptr;
+        e = cudaGraphInstantiate(&exec, graph, 0);
+        cudaGraphDestroy(graph);
+        if (e != cudaSuccess) return fail(ctx, ST_ERR_CUDA, "%s: graph instantiate: %s", who, cudaGetErrorString(e));
+        if (ctx->graphs.size() >= kMaxGraphs) {
+            auto oldest = ctx->graphs.begin();
+            for (auto g = ctx->graphs.begin(); g != ctx->graphs.end(); ++g)
+                if (g->second.used < oldest->second.used) oldest = g;
+            cudaStreamSynchronize(ctx->stream);               // it may be the one that is running
+            cudaGraphExecDestroy(oldest->second.exec);
+            ctx->graphs.erase(oldest);
+        }
+        it = ctx->graphs.emplace(key, st_ctx::StepGraph{exec, n_launches, 0}).first;
+    }
+    it->second.used = ++ctx->replays;
+    ctx->launches += it->second.n_launches;   // a replay launches the captured kernels again
+    ST_CUDA(ctx, cudaGraphLaunch(it->second.exec, ctx->stream));
+    return ST_OK;
+}
 }  // namespace
 
 extern "C" {
@@ -914,53 +961,27 @@ st_status st_distill_step(st_ctx* ctx, int32_t n_steps, float* loss_out, int64_t
         ST_CUDA(ctx, cudaMemsetAsync(ctx->conf_buf, 0, (size_t)ctx->S * kMaxSteps * cc * sizeof(unsigned long long), ctx->stream));
     }
 
-    st_status st = ST_OK;
-    // A caller that gives the same device buffer again gets its losses written by the updates themselves (one replayable graph
-    // per buffer); the first time, and for host memory, they are copied out behind the steps.
-    float* given = loss_out && ((uintptr_t)loss_out & 3u) == 0 && is_device_ptr(loss_out) ? loss_out : nullptr;
-    ctx->loss_direct = given && (given == ctx->loss_seen || !ctx->use_graphs) ? given : nullptr;
-    ctx->loss_pitch = n_steps;
-    ctx->loss_seen = given;
-    if (ctx->use_graphs) {
-        GraphKey key{n_steps, want_conf, false, 0, ctx->loss_direct};
-        if (ctx->graphs.size() >= kMaxGraphs && !ctx->graphs.count(key)) {
-            ST_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-            for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.second.exec);
-            ctx->graphs.clear();
-        }
-        auto it = ctx->graphs.find(key);
-        if (it == ctx->graphs.end()) {
-            cudaGraph_t graph = nullptr;
-            const int64_t before = ctx->launches;
-            ST_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-            for (int k = 0; k < n_steps && st == ST_OK; ++k) st = enqueue_step(ctx, k, want_conf, nullptr, k == n_steps - 1);
-            if (st == ST_OK && ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, n_steps, ctx->stream); ctx->launches += 1; }
-            cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
-            const int64_t n_launches = ctx->launches - before;
-            ctx->launches = before;
-            if (st != ST_OK) { if (graph) cudaGraphDestroy(graph); return st; }
-            if (e != cudaSuccess) return fail(ctx, ST_ERR_CUDA, "st_distill_step: graph capture: %s", cudaGetErrorString(e));
-            cudaGraphExec_t exec = nullptr;
-            e = cudaGraphInstantiate(&exec, graph, 0);
-            cudaGraphDestroy(graph);
-            if (e != cudaSuccess) return fail(ctx, ST_ERR_CUDA, "st_distill_step: graph instantiate: %s", cudaGetErrorString(e));
-            it = ctx->graphs.emplace(key, st_ctx::StepGraph{exec, n_launches}).first;
-        }
-        ctx->launches += it->second.n_launches;   // a replay launches the captured kernels again
-        ST_CUDA(ctx, cudaGraphLaunch(it->second.exec, ctx->stream));
-    } else {
-        for (int k = 0; k < n_steps; ++k) {
-            st = enqueue_step(ctx, k, want_conf, nullptr, k == n_steps - 1);
-            if (st != ST_OK) return st;
-        }
-        if (ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, n_steps, ctx->stream); ctx->launches += 1; }
-    }
+    const st_status st = run_as_graph(ctx, GraphKey{n_steps, want_conf, false}, "st_distill_step", [&] {
+        st_status r = ST_OK;
+        for (int k = 0; k < n_steps && r == ST_OK; ++k) r = enqueue_step(ctx, k, want_conf, nullptr, k == n_steps - 1);
+        if (r == ST_OK && ctx->adam) { launch_step_tick(ctx->step_base, ctx->S, n_steps, ctx->stream); ctx->launches += 1; }
+        return r;
+    });
+    if (st != ST_OK) return st;
     ctx->settled = true;
-    const bool delivered = ctx->loss_direct != nullptr;
-    ctx->loss_direct = nullptr;
-    if (loss_out && !delivered)
-        ST_CUDA(ctx, cudaMemcpy2DAsync(loss_out, (size_t)n_steps * sizeof(float), ctx->loss_buf, kMaxSteps * sizeof(float),
-                                       (size_t)n_steps * sizeof(float), ctx->S, cudaMemcpyDefault, ctx->stream));
+    if (loss_out) {
+        const void* dev = nullptr;
+        if (locate(loss_out, &dev) != Where::host && ((uintptr_t)dev & 3u) == 0) {
+            TrainResults out{};
+            out.loss = (float*)const_cast<void*>(dev);
+            launch_train_results(train_ctl(ctx, 0, n_steps - 1), ctx->loss_buf, out, ctx->stream);
+            ctx->launches += 1;
+            const st_status r = check_launch(ctx, "losses");
+            if (r != ST_OK) return r;
+        } else
+            ST_CUDA(ctx, cudaMemcpy2DAsync(loss_out, (size_t)n_steps * sizeof(float), ctx->loss_buf, kMaxSteps * sizeof(float),
+                                           (size_t)n_steps * sizeof(float), ctx->S, cudaMemcpyDefault, ctx->stream));
+    }
     if (conf_out)
         ST_CUDA(ctx, cudaMemcpy2DAsync(conf_out, (size_t)n_steps * cc * 8, ctx->conf_buf, (size_t)kMaxSteps * cc * 8,
                                        (size_t)n_steps * cc * 8, ctx->S, cudaMemcpyDefault, ctx->stream));
@@ -968,25 +989,12 @@ st_status st_distill_step(st_ctx* ctx, int32_t n_steps, float* loss_out, int64_t
 }
 
 namespace {
-TrainCtl train_ctl(st_ctx* c, int iter, int max_updates, double threshold)
-{
-    TrainCtl t;
-    t.conf = c->conf_buf + (int64_t)iter * c->C * c->C;
-    t.conf_stream_stride = (int64_t)kMaxSteps * c->C * c->C;
-    t.C = c->C; t.iter = iter; t.max_updates = max_updates; t.threshold = threshold;
-    t.done = c->ctl_done; t.best = c->ctl_best; t.metric = c->ctl_metric;
-    t.n_updates = c->ctl_n_updates; t.best_iter = c->ctl_best_iter; t.better = c->ctl_better;
-    t.theta = c->theta; t.best_theta = c->best_theta; t.n_params = c->n_params; t.S = c->S;
-    t.param_begin = c->trained_begin;
-    return t;
-}
-
 // Train of Algorithm 1 for all streams: one prediction per pass (forward, loss + gradient + confusion), the backward,
 // then the update kernel, which first assesses the prediction (metric, best_student, break) and takes the step only
 // where the loop goes on.  The backward of the pass in which a loop ends is therefore computed and not used; from the
 // next pass on the stream's blocks of the tensor-core GEMMs and of the loss kernel return at once (the fp32
 // convolutions still run: their results are simply not used).
-st_status enqueue_train(st_ctx* c, int max_updates, double threshold)
+st_status enqueue_train(st_ctx* c, int max_updates)
 {
     st_status st = ST_OK;
     for (int i = 0; i <= max_updates && st == ST_OK; ++i) {
@@ -996,7 +1004,7 @@ st_status enqueue_train(st_ctx* c, int max_updates, double threshold)
         // metric, best_student, break: assessed by an extra block of the backward's first tensor-core kernel while that
         // kernel works, or, where there is none (fp32 convolutions; the last prediction, after which every loop ends),
         // by the update itself, which in any case takes the step only where the loop goes on
-        const TrainCtl ctl = train_ctl(c, i, max_updates, threshold);
+        const TrainCtl ctl = train_ctl(c, i, max_updates);
         const bool side = c->bf16_mode && i < max_updates;
         if (st == ST_OK && i < max_updates) st = enqueue_backward(c, nullptr, ended_before, kCtlPitch, side ? &ctl : nullptr);
         if (st == ST_OK) st = enqueue_update(c, i, nullptr, 0, nullptr, &ctl, side ? 2 : 1);
@@ -1021,7 +1029,6 @@ st_status st_train_key_frame(st_ctx* ctx, double threshold, int32_t max_updates,
         if (ready != ST_OK) return ready;
     }
     const size_t cc = (size_t)ctx->C * ctx->C;
-    ctx->loss_direct = nullptr;
     ctx->z_current = false;
     ctx->z_unkept = ctx->fused_fwd != 0;    // the loop's logits never leave the loss kernel
     cudaError_t e = cudaSuccess;
@@ -1034,38 +1041,14 @@ st_status st_train_key_frame(st_ctx* ctx, double threshold, int32_t max_updates,
         if (e == cudaSuccess) e = dev_alloc(ctx, &ctx->ctl_n_updates, (size_t)ctx->S);
         if (e == cudaSuccess) e = dev_alloc(ctx, &ctx->ctl_best_iter, (size_t)ctx->S);
         if (e == cudaSuccess) e = dev_alloc(ctx, &ctx->ctl_better, (size_t)ctx->S * kCtlPitch);
+        if (e == cudaSuccess) e = dev_alloc(ctx, &ctx->ctl_threshold, 1);
     }
     if (e != cudaSuccess) return fail(ctx, ST_ERR_OOM, "st_train_key_frame: %s", cudaGetErrorString(e));
-    ST_CUDA(ctx, cudaMemsetAsync(ctx->conf_buf, 0, (size_t)ctx->S * kMaxSteps * cc * sizeof(unsigned long long), ctx->stream));
+    launch_train_begin(ctx->conf_buf, (int64_t)ctx->S * kMaxSteps * cc, ctx->ctl_threshold, threshold, ctx->stream);
+    ctx->launches += 1;
 
-    st_status st = ST_OK;
-    if (ctx->use_graphs) {
-        uint64_t thr_bits;
-        memcpy(&thr_bits, &threshold, sizeof thr_bits);
-        GraphKey key{max_updates, true, true, thr_bits, nullptr};
-        auto it = ctx->graphs.find(key);
-        if (it == ctx->graphs.end()) {
-            cudaGraph_t graph = nullptr;
-            const int64_t before = ctx->launches;
-            ST_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-            st = enqueue_train(ctx, max_updates, threshold);
-            e = cudaStreamEndCapture(ctx->stream, &graph);
-            const int64_t n_launches = ctx->launches - before;
-            ctx->launches = before;
-            if (st != ST_OK) { if (graph) cudaGraphDestroy(graph); return st; }
-            if (e != cudaSuccess) return fail(ctx, ST_ERR_CUDA, "st_train_key_frame: graph capture: %s", cudaGetErrorString(e));
-            cudaGraphExec_t exec = nullptr;
-            e = cudaGraphInstantiate(&exec, graph, 0);
-            cudaGraphDestroy(graph);
-            if (e != cudaSuccess) return fail(ctx, ST_ERR_CUDA, "st_train_key_frame: graph instantiate: %s", cudaGetErrorString(e));
-            it = ctx->graphs.emplace(key, st_ctx::StepGraph{exec, n_launches}).first;
-        }
-        ctx->launches += it->second.n_launches;
-        ST_CUDA(ctx, cudaGraphLaunch(it->second.exec, ctx->stream));
-    } else {
-        st = enqueue_train(ctx, max_updates, threshold);
-        if (st != ST_OK) return st;
-    }
+    const st_status st = run_as_graph(ctx, GraphKey{max_updates, true, true}, "st_train_key_frame", [&] { return enqueue_train(ctx, max_updates); });
+    if (st != ST_OK) return st;
     ctx->settled = true;
     const int n_pred = max_updates + 1;
     bool host_out = false;
@@ -1083,7 +1066,7 @@ st_status st_train_key_frame(st_ctx* ctx, double threshold, int32_t max_updates,
     const bool r_n = reach(n_updates_out, 4, &out.n_updates), r_best = reach(best_metric_out, 8, &out.best), r_metric = reach(metric_out, 8, &out.metric),
                r_loss = reach(loss_out, 4, &out.loss);
     if (out.n_updates || out.best || out.metric || out.loss) {
-        launch_train_results(train_ctl(ctx, 0, max_updates, threshold), ctx->loss_buf, out, ctx->stream);
+        launch_train_results(train_ctl(ctx, 0, max_updates), ctx->loss_buf, out, ctx->stream);
         ctx->launches += 1;
     }
     if (!r_n) ST_CUDA(ctx, cudaMemcpyAsync(n_updates_out, ctx->ctl_n_updates, (size_t)ctx->S * sizeof(int), cudaMemcpyDefault, ctx->stream));

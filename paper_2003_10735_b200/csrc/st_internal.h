@@ -217,7 +217,7 @@ struct TrainCtl {
     int C;
     int iter;                         // i: number of updates behind this prediction
     int max_updates;                  // MAX_UPDATES
-    double threshold;                 // THRESHOLD
+    const double* threshold;          // THRESHOLD of the call
     int* done;                        // [S][kCtlPitch]
     double* best;                     // [S][kCtlPitch]
     double* metric;                   // [S][kCtlPitch]  metric of prediction i; -1 where the loop had ended before
@@ -262,8 +262,6 @@ struct UpdateArgs {
     int n_loss_part;
     float* loss_buf;         // [S][kMaxSteps]
     int loss_slot;           // slot of loss_buf written by this step
-    float* loss_out;         // nullptr, or the caller's losses [S][loss_pitch], written as well
-    int loss_pitch;
     double inv_P;
     const int* skip;         // nullptr, or one flag per stream (skip[s * skip_stride]): non-zero = leave the stream's
     int64_t skip_stride;     //   parameters and momentum untouched (the loss is still finalised)
@@ -287,8 +285,11 @@ void launch_miou(const unsigned long long* conf, int C, double* out, cudaStream_
 // student <- best_student for the trained parameters (the layers of `a`) and their bf16 copies; Adam: step count += n_updates[s]
 void launch_train_commit(const UpdateArgs& a, const float* best_theta, const int* n_updates, cudaStream_t s);
 
-// Train's results to the caller (each optional, device or pinned host memory): updates taken [S], best metric [S], metrics and
-// losses [S][max_updates + 1]
+// Beginning of a Train call: clears its confusion counters and sets its threshold
+void launch_train_begin(unsigned long long* conf, int64_t n, double* threshold, double value, cudaStream_t s);
+
+// A call's results to the caller (each optional, device or pinned host memory): updates taken [S], best metric [S], metrics and
+// losses [S][max_updates + 1].  A plain loop of n steps delivers its losses the same way, as max_updates = n - 1.
 struct TrainResults { int* n_updates; double *best, *metric; float* loss; };
 void launch_train_results(const TrainCtl& t, const float* loss_buf, const TrainResults& out, cudaStream_t s);
 

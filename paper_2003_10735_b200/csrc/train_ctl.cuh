@@ -11,16 +11,17 @@ namespace st {
 // by one extra block of the first backward kernel, beside that kernel's own work (the update then reads the outcome),
 // or, where no backward follows the prediction, by every block of the update itself (same counts, same arithmetic,
 // same answer).  In three parts so that the loads overlap what else a kernel waits for: train_history reads what the
-// previous assessment left (it may run before the kernel's predecessors have finished), train_fetch starts the loads of
+// previous assessment and the call's beginning left (it may run before the kernel's predecessors have finished), train_fetch starts the loads of
 // the prediction's confusion matrix (blocks of kMiouFetchThreads threads), train_decision finishes (blocks of any size).  Block-uniform; called by all
 // threads of the block.  `writer` (one block per stream) records the history.
-struct TrainHistory { bool ended; double prev_best; };
+struct TrainHistory { bool ended; double prev_best, threshold; };
 __device__ __forceinline__ TrainHistory train_history(const TrainCtl& t, int s)
 {
     TrainHistory h;
     const int i = t.iter;
     h.ended = i > 0 && t.done[(int64_t)s * kCtlPitch + i] != 0;      // the loop had ended before this prediction
     h.prev_best = i > 0 ? t.best[(int64_t)s * kCtlPitch + i] : 0.0;
+    h.threshold = *t.threshold;
     return h;
 }
 __device__ __forceinline__ MiouFetch train_fetch(const TrainCtl& t, int s, const TrainHistory& h)
@@ -49,7 +50,7 @@ __device__ __forceinline__ void train_decision(const TrainCtl& t, int s, bool wr
     __syncthreads();
     const double m = m_sh;
     better = i == 0 || m > h.prev_best;
-    const bool stop = i == 0 ? !(m < t.threshold) : (m > t.threshold);
+    const bool stop = i == 0 ? !(m < h.threshold) : (m > h.threshold);
     skip = stop || i >= t.max_updates;
     if (writer && threadIdx.x == 0) {
         metric[i] = m;

@@ -98,3 +98,68 @@ def test_a_later_context_of_fewer_classes_takes_nothing_from_an_earlier_one(firs
         assert packed(ctx).tobytes() == want[C][0]
         assert st.st_agreement(ctx, 0) == want[C][2]
         st.st_destroy(ctx)
+
+
+# ---- the buffers that results are asked for in, and what a context has been asked before
+def test_losses_reach_any_buffer():
+    """The same steps with the losses asked for in one device buffer again and again, in two in turn, in a part of one, in pinned
+    and in ordinary memory, and not at all."""
+    K, S = 3, 2
+    ctx = make(64, 0, 5, 12, 20, S, prec=1, momentum=0.0)
+    start = [packed(ctx, s) for s in range(S)]
+    a, b = (torch.zeros((S, K), device="cuda") for _ in range(2))
+    part = torch.zeros(S * K + 3, device="cuda")
+    pinned, ordinary = torch.zeros((S, K)).pin_memory(), np.zeros((S, K), np.float32)
+    want = None
+    for buf in (None, a, a, b, a, b, part[3:], pinned, ordinary, a, None, pinned):
+        for s in range(S):
+            st.st_apply_update(ctx, s, start[s])
+        if buf is not None:
+            buf.fill(0) if buf is ordinary else buf.zero_()
+        st.st_distill_step(ctx, K, buf)
+        torch.cuda.current_stream().synchronize()
+        if buf is None:
+            continue
+        got = buf.copy() if buf is ordinary else buf.cpu().numpy().reshape(S, K)
+        want = got.copy() if want is None else want
+        assert got.tobytes() == want.tobytes()
+    assert (want > 0).all() and len(set(want.ravel())) == S * K and part[:3].sum() == 0
+    st.st_destroy(ctx)
+
+
+def test_a_threshold_that_changes_holds_no_memory():
+    """A server that adapts its threshold: the calls replay one graph (0.6 MB of device memory each would be 48 MB in all)."""
+    ctx = make(64, 0, 5, 12, 20, prec=1, momentum=0.0)
+    start, K = packed(ctx), 63
+
+    def train(threshold):
+        st.st_apply_update(ctx, 0, start)
+        n, metrics = np.zeros(1, np.int32), np.zeros((1, K + 1))
+        st.st_train_key_frame(ctx, threshold, K, n, None, metrics)
+        return n[0], metrics[0]
+
+    n, want = train(2.0)                                          # never met: every update is made
+    assert n == K
+    held = torch.cuda.mem_get_info()[0]
+    for i in range(80):
+        n, got = train(2.0 + i / 1024)
+        assert n == K and got.tobytes() == want.tobytes()
+    assert held - torch.cuda.mem_get_info()[0] < 8 << 20
+    for threshold in (0.0, 0.5 * (want[0] + want.max()), want.max()):      # each call goes by its own threshold
+        past = [i for i in range(K + 1) if (want[i] > threshold if i else not want[0] < threshold)]
+        n, got = train(threshold)
+        assert n == (past[0] if past else K)
+        np.testing.assert_array_equal(got[:n + 1], want[:n + 1])
+    st.st_destroy(ctx)
+
+
+def test_more_step_counts_than_graphs_are_kept():
+    ctx = make(64, 0, 5, 12, 20, prec=1, momentum=0.0)
+    start, want = packed(ctx), np.zeros((1, 40), np.float32)
+    st.st_distill_step(ctx, 40, want)
+    for n in [*range(1, 41), *range(1, 41), 40, 39, 1]:           # 32 graphs are kept: in the second round all have been given back
+        loss = np.zeros((1, n), np.float32)
+        st.st_apply_update(ctx, 0, start)
+        st.st_distill_step(ctx, n, loss)
+        assert loss.tobytes() == want[:, :n].tobytes(), n
+    st.st_destroy(ctx)
