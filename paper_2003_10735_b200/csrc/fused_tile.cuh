@@ -55,7 +55,7 @@ struct Shared {
 // for a node inside the frame.  ok = false: the block has to return at once (its stream is flagged, or a wait gave
 // up); the tensor memory is then already freed.
 struct Tile { bool ok; float m_loc; uint32_t tmem; };
-template <int CB, class AfterMma>
+template <class AfterMma>
 __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_map, const CUtensorMap* w_map, Shared& sh, float* zt,
                                            int s, int x0, int y0, AfterMma after_mma)
 {
@@ -145,10 +145,6 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
         return Tile{false, m_loc, 0u};
     }
     after_mma();                                        // the stages are dead
-    {
-        float4* zt4 = reinterpret_cast<float4*>(zt);    // classes the caller pads to: their exponentials are 0, they never win an arg-max
-        for (int e = tid; e < (CB - C) * (TZ / 4); e += kThreads) zt4[C * (TZ / 4) + e] = make_float4(-1e30f, -1e30f, -1e30f, -1e30f);
-    }
     // accumulator m holds tile rows 4m .. 4m+3 (one row of 32 nodes per 32 lanes of tensor memory, and a warp reaches
     // the lanes 32 (warp % 4) ..): warps 0-3 drain rows 0-3, warps 4-7 rows 4-7, warps 0 and 4 half of the classes of
     // row 8 each

@@ -14,8 +14,6 @@
 #include "fused_tile.cuh"
 #include "miou.cuh"
 
-#include <string.h>
-
 namespace st {
 
 namespace {
@@ -25,13 +23,13 @@ using fused::kOwnRows;
 using fused::kThreads;
 constexpr int TW = fused::kTileCols, TZ = fused::kTile;
 
-template <int CB, bool MASK, bool CONF>
+template <bool MASK, bool CONF>
 __global__ void __launch_bounds__(kThreads, 2)
 student_eval_kernel(StudentMaskArgs a, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map)
 {
     extern __shared__ __align__(128) float smem_e[];
-    float* zt = (float*)(((uintptr_t)smem_e + 1023) & ~(uintptr_t)1023);   // [CB][9][32] logits; the feature stages lie over it
-    unsigned int* hist = (unsigned int*)(zt + CB * TZ);                    // [C][C] (CONF), under the stages as well
+    float* zt = (float*)(((uintptr_t)smem_e + 1023) & ~(uintptr_t)1023);   // [C][9][32] logits; the feature stages lie over it
+    unsigned int* hist = (unsigned int*)(zt + a.C * TZ);                   // [C][C] (CONF), under the stages as well
     __shared__ fused::Shared fsh;
     __shared__ bool is_last;
     __shared__ double iou[kMiouClasses];
@@ -73,7 +71,7 @@ student_eval_kernel(StudentMaskArgs a, const __grid_constant__ CUtensorMap x_map
     auto after_mma = [&]() {
         if (CONF) for (int e = tid; e < C * C; e += kThreads) hist[e] = 0;
     };
-    const fused::Tile tile = fused::logit_tile<CB>(fa, &x_map, &w_map, fsh, zt, a.stream, x0, y0, after_mma);
+    const fused::Tile tile = fused::logit_tile(fa, &x_map, &w_map, fsh, zt, a.stream, x0, y0, after_mma);
     pdl_launch_dependents();
     if (!tile.ok) return;
     const uint32_t tmem = tile.tmem;
@@ -159,55 +157,30 @@ student_eval_kernel(StudentMaskArgs a, const __grid_constant__ CUtensorMap x_map
     }
 }
 
-template <int CB>
-size_t eval_smem_bytes(int C) { return fused::smem_bytes(((size_t)CB * TZ + (size_t)C * C) * sizeof(float)); }
-
-template <int CB>
-cudaError_t prepare_cb()
-{
-    cudaError_t e = allow_shared_memory((const void*)student_eval_kernel<CB, true, false>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)student_eval_kernel<CB, true, true>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)student_eval_kernel<CB, false, true>);
-    return e;
-}
-
-template <int CB>
-cudaError_t launch_cb(const StudentMaskArgs& a, cudaStream_t s)
+template <bool MASK, bool CONF>
+void launch_as(const StudentMaskArgs& a, cudaStream_t s)
 {
     const dim3 grid((unsigned)((a.w + kOwnCols - 1) / kOwnCols), (unsigned)((a.h + kOwnRows - 1) / kOwnRows));
-    const size_t smem = eval_smem_bytes<CB>(a.C);
-    const bool conf = a.labels != nullptr;
-    if (!conf) launch_early(pdl_enabled(), student_eval_kernel<CB, true, false>, grid, dim3(kThreads), smem, s, a, *a.x_map, *a.w_map);
-    else if (a.mask) launch_early(pdl_enabled(), student_eval_kernel<CB, true, true>, grid, dim3(kThreads), smem, s, a, *a.x_map, *a.w_map);
-    else launch_early(pdl_enabled(), student_eval_kernel<CB, false, true>, grid, dim3(kThreads), smem, s, a, *a.x_map, *a.w_map);
-    return cudaGetLastError();
-}
-
-// class-count buckets: the two workload sizes exactly, multiples of eight otherwise
-int bucket(int C)
-{
-    if (C == 19 || C == 21) return C;
-    return (C + 7) / 8 * 8;
+    const size_t smem = fused::smem_bytes(((size_t)a.C * TZ + (size_t)a.C * a.C) * sizeof(float));
+    launch_early(pdl_enabled(), student_eval_kernel<MASK, CONF>, grid, dim3(kThreads), smem, s, a, *a.x_map, *a.w_map);
 }
 
 }  // namespace
 
-#define ST_EVAL_DISPATCH(FN, C, ...)                 \
-    switch (bucket(C)) {                             \
-        case 8: return FN<8>(__VA_ARGS__);           \
-        case 16: return FN<16>(__VA_ARGS__);         \
-        case 19: return FN<19>(__VA_ARGS__);         \
-        case 21: return FN<21>(__VA_ARGS__);         \
-        case 24: return FN<24>(__VA_ARGS__);         \
-        default: return FN<32>(__VA_ARGS__);         \
-    }
-
-cudaError_t prepare_student_eval(int C)
+cudaError_t prepare_student_eval()
 {
-    if (C > kClassPad) return cudaSuccess;
-    ST_EVAL_DISPATCH(prepare_cb, C)
+    cudaError_t e = allow_shared_memory((const void*)student_eval_kernel<true, false>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)student_eval_kernel<true, true>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)student_eval_kernel<false, true>);
+    return e;
 }
 
-cudaError_t launch_student_eval(const StudentMaskArgs& a, cudaStream_t s) { ST_EVAL_DISPATCH(launch_cb, a.C, a, s) }
+cudaError_t launch_student_eval(const StudentMaskArgs& a, cudaStream_t s)
+{
+    if (!a.labels) launch_as<true, false>(a, s);
+    else if (a.mask) launch_as<true, true>(a, s);
+    else launch_as<false, true>(a, s);
+    return cudaGetLastError();
+}
 
 }  // namespace st

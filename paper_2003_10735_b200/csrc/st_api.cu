@@ -793,7 +793,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             c->fused_fwd = make_feature_tile_map(&c->fx_map, c->x_bf16, S, c->Cin, c->h, c->w) &&
                            encode_tensor_map(&c->fw_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, c->w2_shadow, 3,
                                              dims, str, box, msg, sizeof msg, "1x1 weight") &&
-                           prepare_student_eval(c->C) == cudaSuccess;
+                           prepare_student_eval() == cudaSuccess;
             if (const char* ts = getenv("ST_TEST_STALL_FUSED")) c->test_stall_fused = ts[0] == '1' ? 1 : 0;
         }
     }

@@ -174,7 +174,7 @@ struct StudentMaskArgs {
     const CUtensorMap* x_map;  // host copies of the tile maps of the features (make_feature_tile_map) and of the bf16 weights
     const CUtensorMap* w_map;
 };
-cudaError_t prepare_student_eval(int C);    // once per device and class count, outside any stream capture
+cudaError_t prepare_student_eval();         // once per device, outside any stream capture
 cudaError_t launch_student_eval(const StudentMaskArgs& a, cudaStream_t s);
 bool student_mask_fused_supported(int C);   // confusion counters fit shared memory
 cudaError_t prepare_student_mask();         // once per device, outside any stream capture
