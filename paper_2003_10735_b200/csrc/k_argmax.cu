@@ -10,7 +10,6 @@
 
 namespace st {
 
-template <int U>
 __global__ void __launch_bounds__(256)
 argmax_u8_vec4_kernel(const float4* __restrict__ T, int C, int64_t n_quads, uint32_t* __restrict__ out, uint32_t* __restrict__ copy)
 {
@@ -21,8 +20,8 @@ argmax_u8_vec4_kernel(const float4* __restrict__ T, int C, int64_t n_quads, uint
     const float4* p = T + q;
     float4 best = __ldcs(p);
     uint32_t ix = 0, iy = 0, iz = 0, iw = 0;
-    // U planes per iteration: each thread has U 16-byte loads in flight.
-#pragma unroll U
+    // Two planes per iteration: each thread has two 16-byte loads in flight.
+#pragma unroll 2
     for (int c = 1; c < C; ++c) {
         float4 v = __ldcs(p + (int64_t)c * n_quads);
         if (v.x > best.x) { best.x = v.x; ix = c; }
@@ -61,9 +60,10 @@ void launch_argmax_u8(const float* logits, int C, int64_t P, uint8_t* labels, ui
         int64_t nq = P / 4;
         unsigned blocks = (unsigned)((nq + 255) / 256);
         // Measured at 720p, C = 21 (78 MB): 16.1 us with one plane per iteration, 14.0 us with two, 17.6 us and more with
-        // three, four, seven or all (many concurrent streams spread the DRAM accesses too thin).  A frame that leaves
-        // the SMs half empty has too few bytes in flight with two: 360p, C = 21 (19 MB), 6.2 us with two, 5.1 us with eight.
-        launch_early(pdl_enabled(), nq <= 148 * 1024 ? argmax_u8_vec4_kernel<8> : argmax_u8_vec4_kernel<2>, dim3(blocks), dim3(256), 0, s,
+        // three, four, seven or all (many concurrent streams spread the DRAM accesses too thin).  Small frames want no more:
+        // at 360p two planes / eight take 7.3 / 9.5 us for 21 classes read from DRAM and 3.8 / 5.1 from L2, 4.9 / 6.3 and
+        // 3.5 / 3.5 for 13, 24.7 / 31.4 and 17.5 / 20.9 for 81 (the planes left over after whole groups of eight go one by one).
+        launch_early(pdl_enabled(), argmax_u8_vec4_kernel, dim3(blocks), dim3(256), 0, s,
                      (const float4*)logits, C, nq, (uint32_t*)labels, (uint32_t*)copy);
     } else {
         unsigned blocks = (unsigned)((P + 255) / 256);
