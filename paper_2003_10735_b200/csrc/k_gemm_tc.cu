@@ -1244,13 +1244,18 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
     P->smem_fwd1 = (size_t)(P->c_last / kBlockK) * (kTileM * 128 + kClassPad * 128) + kSmemAlign;
     P->smem_fwd1p = (size_t)kF1Stages * kF1StageBytes + (size_t)(P->c_last / kBlockK) * kClassPad * 128 + kSmemAlign;
     {
-        // The persistent form wins where every block has many tiles to stream (16 streams at 720p: 90 us against
-        // 110 us, 0.93 of the HBM copy bandwidth) or more than a ring of stages (one 720p stream of 256 channels, twelve
-        // stages per SM: 8.7 us against 10.6).  With three tiles of 64 channels per SM, or three of 128, its partly filled
-        // last round costs more than the one-tile blocks' second wave (8.6 us against 7.1).  ST_FWD1X1_PERSISTENT=0/1
-        // forces a choice.
+        // One tile per block, or persistent blocks?  us, one-tile / persistent:
+        // from 192 channels on the one-tile blocks are large (three an SM at 192, two at 256 and 320, one from 384 on) and the
+        // line is their first wave: 192 channels, 444 tiles 8.4 / 8.6, 508 tiles 9.6 / 8.6; 256, 254 tiles 6.5 / 6.5, 339 tiles
+        // 10.2 / 8.6, 7200 tiles 110 / 90 (0.93 of the HBM copy bandwidth); 320, 296 tiles 5.4 / 5.6, 450 tiles 9.3 / 7.7; 512, 148
+        // tiles 5.2 / 5.5, 226 tiles 8.7 / 6.7; 704, 148 tiles 5.7 / 6.1, 226 tiles 9.7 / 8.1.
+        // At 128 channels five blocks an SM have more bytes in flight than the ring and it pays late: 704 tiles 6.1 / 7.2, 1350
+        // tiles 10.2 / 10.7, 1808 tiles 13.2 / 13.1, 2112 tiles 15.5 / 14.9, 3600 tiles 32.0 / 29.7.  At 64 channels never: 1350
+        // tiles 8.7 / 10.2, 7200 tiles 36.7 / 40.8.
+        // ST_FWD1X1_PERSISTENT=0/1 forces a choice.
         const int64_t tiles = (int64_t)((P->p + kTileM - 1) / kTileM) * b.S;
-        bool use = tiles >= (int64_t)6 * 148 || tiles * (P->c_last / kBlockK) >= (int64_t)9 * 148;
+        const int slices = P->c_last / kBlockK, per_sm = (int)((size_t)227 * 1024 / P->smem_fwd1);
+        bool use = slices >= 3 ? tiles > (int64_t)148 * per_sm : slices == 2 && tiles >= (int64_t)148 * 13;
         if (const char* e = getenv("ST_FWD1X1_PERSISTENT")) { if (e[0] == '0') use = false; else if (e[0] == '1') use = true; }
         if (const char* e = getenv("ST_TEST_STALL_FWD1X1")) if (e[0] == '1') { P->test_stall = true; use = false; }
         // the one-tile form keeps the whole channel extent of its tile in shared memory: beyond 704 channels it no

@@ -62,7 +62,7 @@ def test_packed_buffers_at_any_address(ch, prec, offset, where):
 # ---- the number of streams
 @pytest.mark.parametrize("c_in,ch,C,h,w,prec", [
     (33, 9, 5, 40, 70, 0), (96, 48, 40, 24, 40, 0), (5, 0, 4, 61, 90, 0), (64, 0, 21, 45, 80, 0),
-    (64, 64, 5, 24, 40, 1), (64, 64, 5, 90, 80, 1), (128, 0, 21, 45, 80, 1),       # the second: another form of the 1x1 forward for 16 streams
+    (64, 64, 5, 24, 40, 1), (64, 192, 5, 45, 80, 1), (128, 0, 21, 45, 80, 1),      # the second: another form of the 1x1 forward for 16 streams
 ])
 def test_results_of_a_stream_do_not_depend_on_its_neighbours(c_in, ch, C, h, w, prec):
     K = 2
