@@ -24,7 +24,10 @@ constexpr int kChunk = 8;          // classes per group whose pulls are in share
 
 struct ManyShape { int own_y, groups; };
 // Fifteen or sixteen warps per block, one block per SM.  4 node rows and three warps per cell row where that fills the SMs once
-// at most (a frame of 90 x 160 nodes: 138 blocks); otherwise 7 rows and two warps, which computes fewer rows twice
+// at most; otherwise 7 rows and two warps, which computes fewer rows twice.  81 classes, us with 4 / with 7 rows: 96 x 160 nodes (144
+// blocks of 4) 38 / 55, 100 x 160 (150) 68 / 55, 180 x 320 (495) 139 / 106; 40 classes 24 / 32, 44 / 32, 88 / 61.  The line follows the map
+// alone, although a second round of 4-row blocks would do for one stream of 135 x 240 (72 / 103) and four streams of 61 x 90 would
+// rather have 7 rows (71 / 55): the shape groups the sums, and a stream's results must not depend on what shares its launch.
 ManyShape many_shape(int h, int w)
 {
     const int blocks4 = ((h + 3) / 4) * ((w + kOwnX - 1) / kOwnX);

@@ -654,8 +654,11 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     // before its predecessor's results are needed (label fetch, feature tiles) and the step is 2 us shorter.  Blocks of 3x3
     // layers with at most 128 output channels are many short kernels, whose starts (barriers, tensor memory) hide behind the one
     // before: 2 % of a call (two blocks of 64 channels, 720p: 1560 -> 1527 us; 128 channels, 101 x 187: 659 -> 645).  Kernels of
-    // 256 channels fill the SMs to the end and waiting blocks crowd those that finish first: 0.6 % slower; with fp32
-    // convolutions 10 us a step slower.  ST_PDL=0 / 1 force it.
+    // wider layers gain on small maps and lose on large ones and beside other streams, where they fill the SMs to the end and waiting
+    // blocks crowd those that finish first; the line is where nothing loses.  us per step launched late / early: 256 -> 256 channels
+    // 90 x 160 66 / 64, 180 x 320 138.6 / 137, three of 101 x 187 205 / 208, 270 x 480 277 / 284; 256 -> 192 56.5 / 52.9, 122.6 / 119.2,
+    // 179.5 / 178.1, 235 / 233, four of 135 x 240 321 / 325; blocks of 192 and 64 81.5 / 79, 175 / 172, 237 / 232, 318 / 325, 408 / 413.
+    // With fp32 convolutions 10 us a step slower.  ST_PDL=0 / 1 force it.
     int widest = 0;
     for (int i = 0; i < n_blocks; ++i) if (blk_out[i] > widest) widest = blk_out[i];
     c->chain_early = pdl_enabled() && (c->Ch == 0 || (c->bf16_mode && widest <= 128));
