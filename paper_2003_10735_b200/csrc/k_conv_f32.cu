@@ -188,12 +188,8 @@ void launch_fwd(const ConvF32& a, int S, bool early, cudaStream_t s)
         const int64_t busiest = ((int64_t)tiles * y * S + 147) / 148 * n;
         if (busiest < least) { least = busiest; ng = n; ny = y; }
     }
-    launch_chain(early, conv_fwd_f32_kernel<KS, CO>, dim3((unsigned)tiles, (unsigned)ny, (unsigned)S), dim3(32 * kCiSplit * ng), fwd_smem<KS, CO>(ng), s, a, tiles_x);
+    launch_early(early, conv_fwd_f32_kernel<KS, CO>, dim3((unsigned)tiles, (unsigned)ny, (unsigned)S), dim3(32 * kCiSplit * ng), fwd_smem<KS, CO>(ng), s, a, tiles_x);
 }
-
-}  // namespace
-
-namespace {
 
 // ------------------------------------------------------------------------------------------------
 // Weight gradients: dW[tap][co][ci] = sum_{y,x} dout[co][y][x] * in[ci][y+ky-r][x+kx-r].
@@ -344,10 +340,6 @@ conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
     }
 }
 
-}  // namespace
-
-namespace {
-
 // Thread groups per block, channel tiles and pixel ranges of a weight gradient: as many ranges as give every SM about
 // eight warps of one stream (a warp has enough independent sums to keep its scheduler busy with two), each range at least one
 // chunk.  The number of streams has no part in it: the ranges group a gradient's sums, and a stream's results must be the same
@@ -384,7 +376,7 @@ template <int KS, int CO>
 void launch_wgrad(const WgradF32& a, const WgradShape& q, int S, bool early, cudaStream_t s)
 {
     const dim3 grid((unsigned)q.n_split, (unsigned)(q.ci_tiles * q.co_tiles), (unsigned)S);
-    launch_chain(early, conv_wgrad_f32_kernel<KS, CO>, grid, dim3(32 * wg_rows<KS>() * q.ng), wg_smem<KS, CO>(q.ng), s, a, q.tiles_x, q.n_chunks, q.ci_tiles);
+    launch_early(early, conv_wgrad_f32_kernel<KS, CO>, grid, dim3(32 * wg_rows<KS>() * q.ng), wg_smem<KS, CO>(q.ng), s, a, q.tiles_x, q.n_chunks, q.ci_tiles);
 }
 
 }  // namespace

@@ -1323,7 +1323,7 @@ int tc_forward_blocks(const TcPlan* P, int first, int last, cudaStream_t s, Stag
         const TcBlockPlan& q = P->blk[i];
         int grid, tail_split;
         tile_walk(P, total, k.c_out, &grid, &tail_split);
-        ST_REPEAT(t) launch_chain(b.chain_early != 0, fwd3_kernel<0>(k.c_out), dim3(grid), dim3(kFwd3Threads), q.smem_fwd, s,
+        ST_REPEAT(t) launch_early(b.chain_early != 0, fwd3_kernel<0>(k.c_out), dim3(grid), dim3(kFwd3Threads), q.smem_fwd, s,
             q.in_fwd, q.skip_fwd, k.c_prev / kBlockK, k.c_skip / kBlockK, q.w_map, q.w_map_q, tail_split, b.theta, b.n_params, k.b_off,
             q.out_st, k.relu_bits, (float*)nullptr, k.c_out, b.h, b.w, total, pow2_cols(k.c_out), b.err, skip, skip_stride);
         if (t) t->mark(kFwd3Names[i], s, st_repeats(t));
@@ -1341,7 +1341,7 @@ int tc_forward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip, 
         int gx = P->n_sms / b.S;
         if (gx < 1) gx = 1;
         if (gx > tiles1) gx = tiles1;
-        ST_REPEAT(t) launch_chain(b.chain_early != 0, tc_fwd1x1p_kernel, dim3(gx, b.S), dim3(kF1Threads), P->smem_fwd1p, s,
+        ST_REPEAT(t) launch_early(b.chain_early != 0, tc_fwd1x1p_kernel, dim3(gx, b.S), dim3(kF1Threads), P->smem_fwd1p, s,
             P->act_fwd, P->w2_map, b.theta, b.n_params, b.b2_off, b.z, b.C, P->p, P->c_last / kBlockK, b.err, skip, skip_stride);
     } else {
         // one-layer head, no per-stream skip flags to wait for, not a timing run: the activations are the frozen
@@ -1365,7 +1365,7 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
     if (!nb || !b.blk[nb - 1].trained) {                  // nothing is passed back into a frozen block (Section 4.2)
         // one-layer head: the activations are the frozen features, which no kernel of the loop writes
         const int a_early = (!nb && !skip && !t && b.chain_early) ? 1 : 0;
-        ST_REPEAT(t) launch_chain(b.chain_early != 0, tc_wgrad1x1_kernel<kWg1Stages>, dim3(P->split2 * P->msplit2 + (ctl ? 1 : 0), b.S), dim3(kThreadsTc),
+        ST_REPEAT(t) launch_early(b.chain_early != 0, tc_wgrad1x1_kernel<kWg1Stages>, dim3(P->split2 * P->msplit2 + (ctl ? 1 : 0), b.S), dim3(kThreadsTc),
             P->smem_wg1, s, P->act_wg, P->dz_map, b.w2_partials, P->c_last, P->chunks2, P->per2, P->msplit2, P->cols2, b.err, skip, skip_stride,
             a_early, ctl ? 1 : 0, ctl ? *ctl : no_ctl);
         if (t) t->mark("tc_wgrad1x1", s, st_repeats(t));
@@ -1373,7 +1373,7 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
     }
     {
         const TcBlock& k = b.blk[nb - 1];
-        ST_REPEAT(t) launch_chain(b.chain_early != 0, tc_back1x1_kernel, dim3(P->split_b * P->groups_b + (ctl ? 1 : 0), b.S), dim3(kBackThreads),
+        ST_REPEAT(t) launch_early(b.chain_early != 0, tc_back1x1_kernel, dim3(P->split_b * P->groups_b + (ctl ? 1 : 0), b.S), dim3(kBackThreads),
             P->smem_back1, s, P->act_fwd, P->dz_map, P->w2_map, P->dout_map, k.relu_bits, k.b_partials, b.w2_partials, k.c_out, P->p, P->tiles_b,
             P->per_b, P->groups_b, b.err, skip, skip_stride, ctl ? 1 : 0, ctl ? *ctl : no_ctl);
         if (t) t->mark("tc_back1x1", s, st_repeats(t));
@@ -1383,7 +1383,7 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
     for (int i = nb - 1; i >= 0 && b.blk[i].trained; --i) {
         const TcBlock& k = b.blk[i];
         const TcBlockPlan& q = P->blk[i];
-        ST_REPEAT(t) launch_chain(b.chain_early != 0, wgrad3_kernel(q.wg), dim3(9 * P->split1, b.S), dim3(kThreadsTc), q.wg.bytes, s,
+        ST_REPEAT(t) launch_early(b.chain_early != 0, wgrad3_kernel(q.wg), dim3(9 * P->split1, b.S), dim3(kThreadsTc), q.wg.bytes, s,
             q.in_wg, q.skip_wg, k.c_prev / kBlockK, q.dout_wg, k.w_partials, k.c_prev + k.c_skip, k.c_out, b.h, b.w, P->chunks1, P->per1,
             P->split1, q.cols_wg, b.err, skip, skip_stride);
         if (t) t->mark(kWg3Names[i], s, st_repeats(t));
@@ -1394,7 +1394,7 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
             const TcBlock& r = b.blk[i - 1];
             int grid, tail_split;
             tile_walk(P, total, k.c_prev, &grid, &tail_split);
-            ST_REPEAT(t) launch_chain(b.chain_early != 0, fwd3_kernel<1>(k.c_prev), dim3(grid), dim3(kFwd3Threads), q.smem_back, s,
+            ST_REPEAT(t) launch_early(b.chain_early != 0, fwd3_kernel<1>(k.c_prev), dim3(grid), dim3(kFwd3Threads), q.smem_back, s,
                 q.dout_fwd, q.dout_fwd, k.c_out / kBlockK, 0, q.wt_map, q.wt_map_q, tail_split, (const float*)nullptr, (int64_t)0, (int64_t)0,
                 q.dprev_st, r.relu_bits, r.b_partials, k.c_prev, b.h, b.w, total, pow2_cols(k.c_prev), b.err, skip, skip_stride);
             if (t) t->mark("tc_dgrad3x3", s, st_repeats(t));

@@ -367,11 +367,11 @@ static int launch_sgd_update_t(const UpdateArgs& a, cudaStream_t s)
     const int n_grouped = n_param_blocks + n_red_blocks;
     const dim3 grid((unsigned)(n_grouped + stream_blocks), (unsigned)a.S);
     const dim3 blk(kUpdThreads);
-    if (G == 1 && E == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<1, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
-    else if (G == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<1, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
-    else if (G == 16) launch_chain(a.chain_early != 0, sgd_update_kernel<16, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
-    else if (E == 1) launch_chain(a.chain_early != 0, sgd_update_kernel<8, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
-    else launch_chain(a.chain_early != 0, sgd_update_kernel<8, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    if (G == 1 && E == 1) launch_early(a.chain_early != 0, sgd_update_kernel<1, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    else if (G == 1) launch_early(a.chain_early != 0, sgd_update_kernel<1, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    else if (G == 16) launch_early(a.chain_early != 0, sgd_update_kernel<16, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    else if (E == 1) launch_early(a.chain_early != 0, sgd_update_kernel<8, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    else launch_early(a.chain_early != 0, sgd_update_kernel<8, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
     return 1;
 }
 

@@ -396,8 +396,8 @@ void launch_many(const UpsampleCeArgs& a, cudaStream_t s)
 {
     const dim3 grid((unsigned)((a.w + kOwnX - 1) / kOwnX), (unsigned)((a.h + NY - 1) / NY), (unsigned)a.S), block((NY + 1) * G * 32);
     const bool early = a.chain_early != 0;
-    if (a.conf) launch_chain(early, upsample_ce_many_kernel<NY, G, true>, grid, block, many_smem<NY, G>(a.C, true), s, a);
-    else launch_chain(early, upsample_ce_many_kernel<NY, G, false>, grid, block, many_smem<NY, G>(a.C, false), s, a);
+    if (a.conf) launch_early(early, upsample_ce_many_kernel<NY, G, true>, grid, block, many_smem<NY, G>(a.C, true), s, a);
+    else launch_early(early, upsample_ce_many_kernel<NY, G, false>, grid, block, many_smem<NY, G>(a.C, false), s, a);
 }
 
 }  // namespace

@@ -17,8 +17,10 @@ typedef __nv_bfloat16 bf16;
 // The kernels of a step form a chain.  Launched with the programmatic-serialization attribute a kernel
 // may start while its predecessor is still draining; everything it does before pdl_wait() (barrier
 // set-up, tensor-memory allocation, index arithmetic) then overlaps the predecessor's tail.
-// pdl_wait() returns once the predecessor grid has completed and its writes are visible; no global
-// memory is read or written before it.  pdl_launch_dependents() lets the successor start launching.
+// pdl_wait() returns once the predecessor grid has completed and its writes are visible.  Before it a kernel reads only what no
+// kernel that may still be running writes: features, labels and parameters where their last writer lies at least two kernels back
+// on the stream (every kernel passes its own wait before it lets its successor start).  pdl_launch_dependents() lets the
+// successor start launching.
 #ifdef __CUDACC__
 // One 32-byte store (a whole sector) from eight 32-bit registers; the address must be 32-byte aligned.  Where the
 // lanes of a warp write to rows that lie far apart (pixel-major activations), a sector written as two 16-byte halves
@@ -49,7 +51,8 @@ inline cudaError_t allow_shared_memory(const void* kernel)
 bool pdl_enabled();   // true unless the environment variable ST_PDL is set to 0
 
 // `early`: launch with the programmatic-serialization attribute, i.e. the kernel may start before its predecessor on
-// the stream has completed and must call pdl_wait() before it touches anything the predecessor writes.
+// the stream has completed and must call pdl_wait() before it touches anything the predecessor writes.  Kernels of the step's
+// chain take the context's choice (the `chain_early` field of the argument structs).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_early(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args)
 {
@@ -60,13 +63,6 @@ inline cudaError_t launch_early(bool early, void (*kernel)(KArgs...), dim3 grid,
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
-// A kernel of the step's chain; `early` is the context's choice (the `chain_early` field of the argument structs).
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chain(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args)
-{
-    return launch_early(early, kernel, grid, block, smem, s, std::forward<Args>(args)...);
 }
 #endif
 
@@ -193,7 +189,7 @@ struct PadF32 {
 void launch_pad_planes(const float* plain, float* padded, int C, int h, int w, cudaStream_t s);
 void launch_unpad_planes(const float* padded, float* plain, int C, int h, int w, cudaStream_t s);
 // Inputs and gradients are padded planes of S streams back to back; the output is one too if out_padded, else [Cout][h][w].
-// Weight, bias and (w_stride floats per stream) parameters as in PackLayout.  `early`: see launch_chain.
+// Weight, bias and (w_stride floats per stream) parameters as in PackLayout.  `early`: see launch_early.
 void launch_conv_fwd_f32(const float* in, int Cin, int h, int w, const float* Wt, const float* b, int Cout, int ks, bool relu,
                          float* out, bool out_padded, int S, int64_t w_stride, bool early, cudaStream_t s);
 // Weight gradient as n_split = conv_wgrad_f32_splits(...) partial results [S][n_split][tap][Cout][Cin], which the parameter
