@@ -360,8 +360,8 @@ WgradShape wgrad_shape(int Cin, int Cout, int h, int w)
     const int per_range = q.ci_tiles * q.co_tiles, warps = q.ng * RW;
     int n = 148 * (warps >= 5 ? 1 : 8 / warps) / per_range;
     if (n > 128) n = 128;                              // the update adds the ranges' results one by one
-    if (n > q.n_chunks) n = q.n_chunks;
-    q.n_split = n < 1 ? 1 : n;
+    const int per = n < 1 ? q.n_chunks : (q.n_chunks + n - 1) / n;      // chunks of the longest range: no more ranges than it takes
+    q.n_split = (q.n_chunks + per - 1) / per;
     return q;
 }
 // 1x1 layers: 16 channels per warp keep the loads below the multiply-adds; a head with a handful of classes takes 4
