@@ -548,11 +548,12 @@ def run_ours(args, cfg):
                 os.environ[FUSED_SWITCH] = "0"
                 ctx_u = make_context(st, stream, cfg, theta0)
                 os.environ.pop(FUSED_SWITCH)
-                st.st_set_frozen_features(ctx_u, 0, feats_d[0][0])
-                st.st_teacher_labels(ctx_u, 0, logits_d[0][0])
+                for s in range(S):
+                    st.st_set_frozen_features(ctx_u, s, feats_d[0][s])
+                    st.st_teacher_labels(ctx_u, s, logits_d[0][s])
                 for _ in range(3):
-                    st.st_distill_step(ctx_u, K, loss_d[0:1])
-                ms_u = statistics.median(timed_blocks(torch, stream, barrier, 5, 50, lambda i: st.st_distill_step(ctx_u, K, loss_d[0:1]))) / 50
+                    st.st_distill_step(ctx_u, K, loss_d)
+                ms_u = statistics.median(timed_blocks(torch, stream, barrier, 5, 50, lambda i: st.st_distill_step(ctx_u, K, loss_d))) / 50
                 unfused = kernel_table(st, ctx_u, si.get_config(args.workload), peaks, arith, 20)
                 unfused["distill_loop_only_ms_per_step"] = ms_u / K
                 st.st_destroy(ctx_u)
