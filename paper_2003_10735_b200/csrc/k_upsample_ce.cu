@@ -2,7 +2,7 @@
 // fused: bilinear x4 upsample of the head's low-resolution logits z to frame resolution, per-pixel softmax cross-entropy
 // against the one-byte labels, and the gradient of the mean loss with respect to z (the transpose of the upsample applied
 // to softmax - onehot), without ever writing a frame-resolution tensor.  Same geometry and arithmetic as the kernel for
-// fewer classes (k_upsample_ce_rows.cu): warp = row of cells, lane = node column and the 4 x 4 frame pixels to its right,
+// fewer classes (k_upsample_ce_rows.cuh): warp = row of cells, lane = node column and the 4 x 4 frame pixels to its right,
 // 16 exponentials of a class as products of four (cell_softmax.cuh), exact per-pixel maxima for cells whose logits are
 // steep, integer sums for the one-hot part.
 //

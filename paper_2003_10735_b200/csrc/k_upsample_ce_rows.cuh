@@ -1,7 +1,7 @@
 // K3, row-walking form (n_classes <= 32) — ComputeLoss and the first half of PartialBackward
 // (Algorithm 1; loss of Section 5.2): bilinear x4 upsample of the low-resolution logits, per-pixel
 // softmax cross-entropy against the labels, and the gradient of the mean loss with respect to the
-// low-resolution logits.  Same result as the cell-per-thread kernel in k_upsample_ce.cu.
+// low-resolution logits.  For more classes: k_upsample_ce.cu.
 //
 // Geometry.  With half-pixel centres and factor 4 the frame pixels 4n+2 .. 4n+5 lie between node
 // columns n and n+1 ("cell" n) with weights 1/8, 3/8, 5/8, 7/8 toward n+1; rows alike.  Cells -1 and

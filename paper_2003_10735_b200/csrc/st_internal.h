@@ -143,7 +143,7 @@ void launch_upsample_ce(const UpsampleCeArgs& a, const CUtensorMap* z_map, cudaS
 bool fused_forward_supported(int C, int h, int w, int c_in);
 // Tile map of bf16 features [S][h][w][c_in] for the fused forward: {c_in, w, h, S}, one box = 64 channels of the block's tile
 bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w);
-// register-resident variant for C <= 32 (k_upsample_ce_rows.cu); launch_upsample_ce dispatches to it
+// variant for C <= 32 (k_upsample_ce_rows.cuh); launch_upsample_ce dispatches to it
 bool upsample_ce_rows_supported(int C);
 int upsample_ce_rows_blocks(int h, int w);
 cudaError_t prepare_upsample_ce_rows(int C);
