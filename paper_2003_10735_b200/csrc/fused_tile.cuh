@@ -1,6 +1,6 @@
 // Forward of a 1x1 classifier inside a block that needs the logits of a tile of feature-map nodes (Forward of
-// Algorithm 1 for the trainable back part of Section 4.2 when that part is one 1x1 layer): shared by the fused
-// upsample + cross-entropy kernel and by the student-mask kernel.
+// Algorithm 1 for the trainable back part of Section 4.2 when that part is one 1x1 layer): the student-mask kernel's.  The loss
+// kernel (k_fwd_ce.cuh) takes the same tiles and slices.
 //
 // z[pix][c] = b[c] + sum_k X[pix][k] W[c][k] for the kTileRows x kTileCols nodes of the tile (node rows y0-1 .. y0+7,
 // node columns x0-1 .. x0+30: the 7 x 30 nodes a block owns and the ring around them).  The feature tile arrives in
@@ -29,16 +29,9 @@ constexpr size_t kReachBytes = (size_t)(kStages - 1) * kStageBytes + 384 * 128;
 
 struct Args {
     int kblocks;             // 64-channel slices of the classifier's input
-    int x_early;             // the features are not written by the kernel just before this one: fetch them before waiting for it
-    const int* skip;         // nullptr, or the flag of this block's stream: non-zero = the block returns at once
     unsigned int* err;       // device word: first wait that gave up
     const float* bias;       // the classifier's bias of this block's stream (fp32 master parameters)
-    float* z_out;            // nullptr, or the stream's logits [C][h][w]: the block's own nodes are written there as well
     int C, h, w;
-    // tc::kSpinLimit and 0 in normal use.  A test of the give-up path lowers the limit and makes the first barrier expect
-    // stall_bytes more than its copy delivers, so that the wait on it runs out: every copy that was issued still lands,
-    // the block records where it gave up, writes nothing, frees its tensor memory and returns.
-    uint32_t spin_limit, stall_bytes;
 };
 
 // What the block keeps in static shared memory for this
@@ -51,20 +44,17 @@ struct Shared {
 // Called by all kFused threads of the block.  `zt` (1024-byte aligned) receives the tile; the ring and the weights lie
 // over it and the kRingBytes behind its start until the multiplication has finished, then `after_mma()` is called (the
 // caller gives the arrays under the ring their initial contents there) and the tile is written.  `tmem` is the block's
-// tensor memory, which the caller frees at its very end (free_tmem).  m_loc: the largest logit this thread has written
-// for a node inside the frame.  ok = false: the block has to return at once (its stream is flagged, or a wait gave
-// up); the tensor memory is then already freed.
-struct Tile { bool ok; float m_loc; uint32_t tmem; };
+// tensor memory, which the caller frees at its very end (free_tmem).  The features are fetched before the wait for the kernel
+// before this one.  ok = false: the block has to return at once (a wait gave up); the tensor memory is then already freed.
+struct Tile { bool ok; uint32_t tmem; };
 template <class AfterMma>
 __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_map, const CUtensorMap* w_map, Shared& sh, float* zt,
                                            int s, int x0, int y0, AfterMma after_mma)
 {
-    float m_loc = -INFINITY;
     uint32_t tmem;
-    constexpr int TW = kTileCols, TZ = kTile, RN_Y = kOwnRows, RN_X = kOwnCols;
+    constexpr int TW = kTileCols, TZ = kTile;
     const int tid = threadIdx.x, wi = __shfl_sync(0xffffffffu, tid >> 5, 0), l = tid & 31;
-    const int C = a.C, h = a.h, w = a.w;
-    const int64_t p = (int64_t)h * w;
+    const int C = a.C;
     const uint32_t ring = tc::smem_u32(zt), w_base = ring + kStages * kStageBytes;
     const uint32_t bar0 = tc::smem_u32(&sh.bar[0]);
     auto full_bar = [&](int st) { return bar0 + 8u * (uint32_t)st; };
@@ -81,21 +71,13 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
     tc::tc_fence_after_sync();
     tmem = sh.tmem_slot;
     const int kblocks = a.kblocks;
-    const int n_pre = a.x_early ? min(kStages, kblocks) : 0;
+    const int n_pre = min(kStages, kblocks);
     if (wi == 0 && tc::elect_one())
         for (int kb = 0; kb < n_pre; ++kb) {
-            tc::mbar_expect_tx(full_bar(kb), kStageBytes + (kb == 0 ? a.stall_bytes : 0u));
+            tc::mbar_expect_tx(full_bar(kb), kStageBytes);
             tc::tma_load_4d(ring + kb * kStageBytes, x_map, full_bar(kb), kb * 64, x0 - 1, y0 - 1, s);
         }
     pdl_wait();                                        // the weights come from the previous kernel of the stream
-    if (a.skip && *a.skip) {                           // this stream's training loop has ended (block-uniform)
-        if (wi == 0)                                    // copies already on their way land before shared memory is given back
-            for (int kb = 0; kb < n_pre; ++kb) tc::mbar_wait(full_bar(kb), 0, a.err, tc::kWaitFull);
-        tc::tc_fence_before_sync();
-        __syncthreads();
-        if (wi == 0) tc::tmem_dealloc(tmem, kTmemCols);
-        return Tile{false, m_loc, 0u};
-    }
     if (tid < kClassPad) sh.bias[tid] = tid < C ? a.bias[tid] : 0.f;
     bool ok = true;
     if (wi == 0) {               // producer and issuer walk their loops as whole warps, one lane issues
@@ -108,7 +90,7 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
             const int st = kb % kStages;
             if (kb >= kStages) ok = tc::mbar_wait(empty_bar(st), ((kb / kStages) - 1) & 1, a.err, tc::kWaitEmpty);
             if (ok && tc::elect_one()) {
-                tc::mbar_expect_tx(full_bar(st), kStageBytes + (kb == 0 ? a.stall_bytes : 0u));
+                tc::mbar_expect_tx(full_bar(st), kStageBytes);
                 tc::tma_load_4d(ring + st * kStageBytes, x_map, full_bar(st), kb * 64, x0 - 1, y0 - 1, s);
             }
             __syncwarp();
@@ -118,7 +100,7 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
         ok = tc::mbar_wait(w_bar, 0, a.err, tc::kWaitFull);
         for (int kb = 0; kb < kblocks && ok; ++kb) {
             const int st = kb % kStages;
-            ok = tc::mbar_wait(full_bar(st), (kb / kStages) & 1, a.err, tc::kWaitFull, a.spin_limit);
+            ok = tc::mbar_wait(full_bar(st), (kb / kStages) & 1, a.err, tc::kWaitFull);
             if (!ok) break;
             tc::tc_fence_after_sync();
             if (tc::elect_one()) {
@@ -142,27 +124,17 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
         tc::tc_fence_before_sync();
         __syncthreads();
         if (wi == 0) tc::tmem_dealloc(tmem, kTmemCols);
-        return Tile{false, m_loc, 0u};
+        return Tile{false, 0u};
     }
     after_mma();                                        // the stages are dead
     // accumulator m holds tile rows 4m .. 4m+3 (one row of 32 nodes per 32 lanes of tensor memory, and a warp reaches
     // the lanes 32 (warp % 4) ..): warps 0-3 drain rows 0-3, warps 4-7 rows 4-7, warps 0 and 4 half of the classes of
     // row 8 each
     auto put_row = [&](const float* v, int n_cols, int c0, int j) {     // v[i]: class c0 + i of node (row j, column l)
-        const int ny = y0 - 1 + j, nx = x0 - 1 + l;
-        const bool in_frame = ny >= 0 && ny < h && nx >= 0 && nx < w;
-        // the block's own nodes go to global memory as well where the caller wants the logits kept
-        const bool keep = a.z_out && in_frame && j >= 1 && j <= RN_Y && l >= 1 && l <= RN_X;
         float* dst = zt + c0 * TZ + j * TW + l;
-        float* zo = a.z_out + (int64_t)c0 * p + (int64_t)ny * w + nx;
 #pragma unroll
         for (int i = 0; i < 32; ++i)
-            if (i < n_cols && c0 + i < C) {
-                const float t = v[i] + sh.bias[c0 + i];
-                dst[i * TZ] = t;
-                if (in_frame) m_loc = fmaxf(m_loc, t);
-                if (keep) zo[(int64_t)i * p] = t;
-            }
+            if (i < n_cols && c0 + i < C) dst[i * TZ] = v[i] + sh.bias[c0 + i];
     };
     {
         float v[32];
@@ -177,7 +149,7 @@ __device__ __forceinline__ Tile logit_tile(const Args& a, const CUtensorMap* x_m
     }
     tc::tc_fence_before_sync();
     __syncthreads();                                   // the tile is complete
-    return Tile{true, m_loc, tmem};
+    return Tile{true, tmem};
 }
 
 // at the very end of the kernel, after a block-wide barrier that follows every warp's last read of tensor memory

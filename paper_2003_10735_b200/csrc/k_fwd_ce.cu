@@ -1,0 +1,37 @@
+// Host side of the forward + upsample + cross-entropy kernel (k_fwd_ce.cuh): which shapes it takes, which instantiation a launch
+// uses, and the tile map of its features.
+#include "k_fwd_ce.cuh"
+
+namespace st {
+
+static FwdCeKernels fwd_ce_kernels(int C)
+{
+    FwdCeKernels (*const file[])(int) = {fwd_ce_kernels_0, fwd_ce_kernels_1, fwd_ce_kernels_2, fwd_ce_kernels_3, fwd_ce_kernels_4};
+    int k = 0;
+    while (C > kFwdCeLast[k]) ++k;
+    return file[k](C);
+}
+
+// A classifier over at most 256 channels (a multiple of 64) and a feature map of at least one tile
+bool fused_forward_supported(int C, int h, int w, int c_in)
+{
+    return C <= kClassPad && c_in >= 64 && c_in % 64 == 0 && c_in / 64 <= fused::kMaxKBlocks && w >= F_COLS && h >= F_ROWS;
+}
+
+cudaError_t prepare_fwd_ce(int C) { return fwd_ce_kernels(C).prepare(); }
+
+void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s) { fwd_ce_kernels(a.C).launch(a, x_map, w_map, s); }
+
+bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w)
+{
+    if (c_in % 64 != 0 || w < F_COLS || h < F_ROWS || ((uintptr_t)x & 15u)) return false;
+    const uint64_t c = (uint64_t)c_in;
+    const uint64_t dims[4] = {c, (uint64_t)w, (uint64_t)h, (uint64_t)S};
+    const uint64_t strides[3] = {c * 2, (uint64_t)w * c * 2, (uint64_t)h * w * c * 2};
+    const uint32_t box[4] = {64, (uint32_t)F_COLS, (uint32_t)F_ROWS, 1};
+    char err[128];
+    return encode_tensor_map(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, x, 4, dims, strides, box, err,
+                             sizeof(err), "feature tile");
+}
+
+}  // namespace st

@@ -1,0 +1,720 @@
+// Forward of a 1x1 classifier, ComputeLoss and the first half of PartialBackward (Algorithm 1; loss of Section 5.2) in one
+// kernel, for at most 32 classes over at most 256 bf16 channels: logits of a tile of feature-map nodes (tcgen05), bilinear x4
+// upsample, per-pixel softmax cross-entropy against the labels, gradient of the mean loss with respect to the logits.
+//
+// Geometry.  With half-pixel centres and factor 4 the frame pixels 4n+2 .. 4n+5 lie between node columns n and n+1 ("cell" n)
+// with weights 1/8, 3/8, 5/8, 7/8 toward n+1; rows alike.  Cells -1 and w-1 are the clamped borders (their outer node is the
+// inner one).  A tile owns 7 rows x 30 columns of nodes.  Eight warps work on it: warp i owns cell row y0-1+i (the 4 x 4 frame
+// pixels between two node rows), lane l owns node column x0-1+l and the 16 pixels of the cell to its right.  Warp 0, lane 0 and
+// lane 31 are halo (recomputed by the neighbouring tile), so that a tile's nodes are finished in a fixed summation order,
+// without floating-point atomics.
+//
+// Logits.  A ninth warp feeds the tensor core: the features of the tile's 9 x 32 nodes arrive in 64-channel slices (one 4-d tile
+// copy each; nodes outside the map arrive as zeros), and four multiplications per 16 channels leave node row i of the tile and
+// node row i+1 of it in the same 32 tensor-memory lanes: the two rows that warp i's cells lie between.  A warp therefore takes
+// its logits out of tensor memory alone, without the other warps: bias added, shifted by the largest of them, in log2 units,
+// clamped at the frame's border, both rows of a class side by side in the warp's own slots of shared memory
+// [class][lane] (upper, lower).  The second class sweep leaves the cell's pull on the two node rows in the same slots.
+// Blocks are persistent where there are more tiles than blocks fit: once the eight warps have emptied the tensor memory, the
+// ninth multiplies the next tile, whose slices arrive while this one is worked on.
+//
+// Fast path (the usual case), class by class for all 16 pixels of a cell: inside a cell the interpolated logit is
+// u(r,k) = A + B k + G r + D k r, so its 16 exponentials are geometric progressions (cell_softmax.cuh).  Sweep 1 sums them per
+// pixel, sweep 2 forms their bases again (cheaper than keeping 16 x C registers) and reduces them to the pull on the nodes.
+// Slow path (a class that changes by more than kFastRange log2-units inside a cell, or a sum that underflows): the warp walks
+// its four frame rows one by one with exact per-pixel maxima.
+// The onehot part of the gradient is exact in units of 1/64: integer counts, two classes to a 32-bit word of shared memory (a
+// node receives at most 1024 times the largest pixel weight, 5), added by shared-memory atomics, one round per distinct label of
+// a cell.  Pixels tagged for the loss weighting (bit 7 of the label byte) count with an integer weight in the loss, in 1/Z and
+// in those counts.
+// The epilogue adds, per node row, the warp's upper pulls, the lower pulls of the warp above and the counts, writes the
+// gradient, and reduces the tile's share of the bias gradient.  With CONF the student's class of every pixel is taken from sweep
+// 1 and counted against the label.
+//
+// Bound by latency and issue slots at 16 working warps an SM (half of the slots, 0.47 of the multiply-add pipe, a third of the
+// shared-memory path go to the sweeps); in a single wave the forward's 2.5 us lie in front.  One launch, us, with each block
+// fetching, multiplying and exchanging its tile through shared memory before the sweeps / now: 720p, 256 channels, 21 classes
+// 24.4 / 23.3, 16 streams of it 316 / 227 (the fetch and the products, 13000 of 33400 cycles a tile, run beside the sweeps of the
+// tile before); 128 channels at 90 x 160 17.1 / 14.8; 32 classes, where one block fitted an SM, 39.8 / 29.6; 27 classes, 4 streams
+// 152 / 89.  Seven classes per iteration of sweep 1 instead of three: 232 -> 227.
+#pragma once
+
+#include "st_internal.h"
+#include "tc_common.cuh"
+#include "fused_tile.cuh"
+#include "cell_softmax.cuh"
+
+#include <utility>
+
+namespace st {
+
+namespace {
+
+constexpr int F_ROWS = fused::kTileRows, F_COLS = fused::kTileCols;         // nodes of a tile, halo included
+constexpr int FN_Y = fused::kOwnRows, FN_X = fused::kOwnCols;               // nodes a tile owns
+constexpr int F_WARPS = FN_Y + 1, F_WORKERS = F_WARPS * 32, F_THREADS = F_WORKERS + 32;
+constexpr int kNodes = F_ROWS * F_COLS;
+constexpr int kSweep1 = 7, kSweep2 = 3;                                     // classes per iteration of the two sweeps
+constexpr uint32_t kSliceBytes = fused::kStageBytes, kWBytes = fused::kWeightBytes;
+constexpr int kLogitCols = 4 * kClassPad;                                   // tensor memory: upper and lower rows of warps 0-3 and 4-7
+
+// Shared memory.  PREFETCH: slot A of the ring is its own, slot B lies over the warps' slots and serves the block's first tile
+// only (nobody has written there yet); the counts are cleared by the threads that read them.  Otherwise a block works on one tile
+// and both slots lie over its arrays.  The line is where two blocks no longer fit an SM with a slot to themselves (from 23
+// classes): 4 streams at 720p, 22 classes 68 us with the slot, 24 classes 83 us without.
+template <int C, bool CONF>
+struct FwdCeSmem {
+    static constexpr size_t kSlots = (size_t)F_WARPS * C * 32 * sizeof(float2), kCounts = (size_t)((C + 1) / 2) * kNodes * sizeof(uint32_t),
+                            kHist = CONF ? (size_t)C * C * sizeof(unsigned int) : 0, kWeights = (size_t)fused::kMaxKBlocks * kWBytes,
+                            kSlotsOrB = kSlots > kSliceBytes ? (kSlots + 1023) / 1024 * 1024 : kSliceBytes;
+    static constexpr size_t kHalfSm = 115712 - 2048;    // what two blocks on an SM leave each, less the static arrays
+    static constexpr bool kPrefetch = kSliceBytes + kSlotsOrB + kWeights + kCounts + kHist + 1024 <= kHalfSm;
+    static constexpr size_t kArrays = kSlots + kCounts + kHist;
+    static constexpr size_t kSlotsAt = kPrefetch ? kSliceBytes : 0, kSliceB = kSliceBytes,
+                            kWeightsAt = kPrefetch ? kSliceBytes + kSlotsOrB : (kArrays > 2 * kSliceBytes ? (kArrays + 1023) / 1024 * 1024 : 2 * kSliceBytes),
+                            kCountsAt = kPrefetch ? kWeightsAt + kWeights : kSlots, kHistAt = kCountsAt + kCounts,
+                            kEnd = kPrefetch ? kHistAt + kHist : kWeightsAt + kWeights, kBytes = kEnd + 1024;
+};
+
+__device__ __forceinline__ float lg2_approx(float x)
+{
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
+__device__ __forceinline__ void workers_sync() { asm volatile("barrier.cta.sync 1, %0;" ::"n"(F_WORKERS) : "memory"); }
+__device__ __forceinline__ bool workers_all(bool ok)
+{
+    int r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r) : "r"((int)ok), "n"(F_WORKERS) : "memory");
+    return r != 0;
+}
+
+// cell_bases of cell_softmax.cuh for values that are shifted and in log2 units already: L, R = (upper, lower) node row of the
+// left and the right node column
+__device__ __forceinline__ float cell_bases_log2(float2 L, float2 R, float2& x01, float2& x23, float2& q01, float2& q23)
+{
+    const float p = L.y - L.x, qq = R.y - R.x, e0 = R.x - L.x, qp = qq - p;
+    const float wv = fmaf(qp, 0.125f, e0), A = fmaf(wv, 0.125f, fmaf(p, 0.125f, L.x));
+    const float E00 = ex2_approx(A), QB = ex2_approx(0.25f * wv), TG = ex2_approx(fmaf(qp, 0.03125f, 0.25f * p)), SD = ex2_approx(0.0625f * qp);
+    const float TG2 = TG * TG, SD2 = SD * SD;
+    q01 = make_float2(QB, QB * SD);
+    q23 = __fmul2_rn(q01, make_float2(SD2, SD2));
+    x01 = make_float2(E00, E00 * TG);
+    x23 = __fmul2_rn(x01, make_float2(TG2, TG2));
+    return fmaxf(fabsf(p), fmaxf(fabsf(qq), fabsf(e0)));
+}
+
+// Slow path: values of the lane's four pixels of one frame row for a class
+__device__ __forceinline__ void row_values(float2 L, float2 R, float ly, float (&u)[4])
+{
+    const float vl = fmaf(ly, L.y - L.x, L.x), d = fmaf(ly, R.y - R.x, R.x) - vl;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) u[k] = fmaf((2 * k + 1) * 0.125f, d, vl);
+}
+
+// f(first, N) for C classes in groups of G: a rolled loop over the whole groups, then what is left
+template <int C, int G, class F>
+__device__ __forceinline__ void static_for_groups(F f)
+{
+#pragma unroll 1
+    for (int c = 0; c + G <= C; c += G) f(c, std::integral_constant<int, G>());
+    if constexpr (C % G != 0) f(C - C % G, std::integral_constant<int, C % G>());
+}
+
+// counts of one class (two classes to a word)
+__device__ __forceinline__ void add_counts(uint32_t* node, int cls, int right, int below, uint32_t tl, uint32_t tr, uint32_t bl, uint32_t br)
+{
+    uint32_t* w = node + (cls >> 1) * kNodes;
+    const int sh = (cls & 1) * 16;
+    atomicAdd(w, tl << sh);
+    atomicAdd(w + right, tr << sh);
+    atomicAdd(w + below, bl << sh);
+    atomicAdd(w + below + right, br << sh);
+}
+
+template <int C, bool CONF>
+__global__ void __launch_bounds__(F_THREADS, 2)
+fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map)
+{
+    using Smem = FwdCeSmem<C, CONF>;
+    extern __shared__ __align__(128) uint8_t smem_f[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_f + 1023) & ~(uintptr_t)1023);
+    float2* slots = (float2*)(smem + Smem::kSlotsAt);                      // [F_WARPS][C][32]
+    uint32_t* counts = (uint32_t*)(smem + Smem::kCountsAt);                // [(C + 1) / 2][F_ROWS][F_COLS]
+    unsigned int* hist = (unsigned int*)(smem + Smem::kHistAt);            // [C][C] (CONF)
+    __shared__ __align__(8) uint64_t bars[7];                              // full[2], free[2], weights, tile done, tile taken
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile uint32_t gave_up;
+    __shared__ float red[2][F_WARPS], wsum[F_WARPS][32];
+    __shared__ __align__(16) float bias[F_WARPS][32];
+    const uint32_t bar0 = tc::smem_u32(&bars[0]), w_bar = bar0 + 32, done_bar = bar0 + 40, taken_bar = bar0 + 48;
+    const int h = a.h, w = a.w, H = h * kUp, W = w * kUp;
+    const int64_t p = (int64_t)h * w;
+    const int tid = threadIdx.x, wi = __shfl_sync(0xffffffffu, tid >> 5, 0), l = tid & 31;
+    const int per_stream = tiles_x * tiles_y, n_tiles = per_stream * a.S;
+    // Tiles at the frame's border do extra work: the last tile row of a stream comes first, then rows 0, 1, ...
+    struct Tile { int s, x0, y0, blk; };
+    auto tile_at = [&](int t) {
+        Tile k;
+        k.s = t / per_stream;
+        const int q = t - k.s * per_stream, row = q / tiles_x, col = q - row * tiles_x, by = row == 0 ? tiles_y - 1 : row - 1;
+        k.x0 = col * FN_X; k.y0 = by * FN_Y; k.blk = by * tiles_x + col;
+        return k;
+    };
+
+    if (wi == F_WARPS) {
+        if (tc::elect_one()) { tc::prefetch_map(&x_map); tc::prefetch_map(&w_map); }
+        __syncwarp();
+        tc::tmem_alloc(tc::smem_u32(&tmem_slot), kLogitCols);
+    }
+    if (tid == 0) {
+        for (int k = 0; k < 6; ++k) tc::mbar_init(bar0 + 8u * (uint32_t)k, 1);
+        tc::mbar_init(taken_bar, F_WARPS);
+        gave_up = 0;
+        tc::fence_barrier_init();
+    }
+    if (Smem::kPrefetch && wi < F_WARPS) {
+        for (int e = tid; e < (int)(Smem::kCounts / 16); e += F_WORKERS) reinterpret_cast<uint4*>(counts)[e] = make_uint4(0, 0, 0, 0);
+        if (CONF) for (int e = tid; e < C * C; e += F_WORKERS) hist[e] = 0;
+    }
+    tc::tc_fence_before_sync();
+    __syncthreads();
+    tc::tc_fence_after_sync();
+    const uint32_t tmem = tmem_slot;
+
+    if (wi == F_WARPS) {
+        // ---------------------------------------------------------------- the ninth warp: copies and multiplications
+        const uint32_t ring = tc::smem_u32(smem), w_base = ring + (uint32_t)Smem::kWeightsAt;
+        constexpr uint32_t idesc = tc::instr_desc(128, kClassPad, 0, 0);
+        const int kblocks = a.kblocks;
+        bool ok = true, first = true;
+        uint32_t loads[2] = {0, 0}, mults[2] = {0, 0};    // per slot: copies / multiplications issued so far
+        int w_stream = -1, n_weights = 0, n_done = 0;
+        auto load = [&](int kb, int slot, const Tile& k, uint32_t stall) {
+            if (tc::elect_one()) {
+                tc::mbar_expect_tx(bar0 + 8u * slot, kSliceBytes + stall);
+                tc::tma_load_4d(ring + slot * (uint32_t)Smem::kSliceB, &x_map, bar0 + 8u * slot, kb * 64, k.x0 - 1, k.y0 - 1, k.s);
+            }
+            __syncwarp();
+            ++loads[slot];
+        };
+        const uint32_t limit = a.test_stall ? (1u << 12) : tc::kSpinLimit, stall = a.test_stall ? 16u : 0u;
+        // Inside the step loop the features are frozen: the first slices are fetched while the previous update still runs
+        int pre = 0;
+        if (a.x_early) {
+            const Tile k = tile_at(blockIdx.x);
+            for (; pre < 2 && pre < kblocks; ++pre) load(pre, pre, k, pre == 0 ? stall : 0u);
+        }
+        pdl_wait();                                        // the weights come from the previous kernel of the stream
+        for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+            const Tile k = tile_at(t);
+            if (a.skip && a.skip[(int64_t)k.s * a.skip_stride]) {          // this stream's training loop has ended
+                for (int kb = 0; kb < pre && ok; ++kb) ok = tc::mbar_wait(bar0 + 8u * kb, (loads[kb] - 1) & 1, a.err, tc::kWaitFull);
+                pre = 0;
+                continue;
+            }
+            const int n_slots = first ? 2 : 1;
+            if (w_stream != k.s) {
+                if (tc::elect_one()) {
+                    tc::mbar_expect_tx(w_bar, (uint32_t)kblocks * kWBytes);
+                    for (int kb = 0; kb < kblocks; ++kb) tc::tma_load_3d(w_base + kb * kWBytes, &w_map, w_bar, kb * 64, 0, k.s);
+                }
+                __syncwarp();
+                w_stream = k.s; ++n_weights;
+            }
+            for (int kb = pre; kb < n_slots && kb < kblocks; ++kb) load(kb, kb, k, first && kb == 0 ? stall : 0u);
+            pre = 0;
+            // as many slices as there are slots are multiplied back to back before their slots are filled again (a slice takes 1100
+            // cycles from its first multiplication to the signal that the last one has read it)
+            for (int k0 = 0; k0 < kblocks && ok; k0 += n_slots) {
+                for (int kb = k0; kb < k0 + n_slots && kb < kblocks; ++kb) {
+                    const int slot = kb - k0;
+                    ok = tc::mbar_wait(bar0 + 8u * slot, (loads[slot] - 1) & 1, a.err, tc::kWaitFull, limit);
+                    if (ok && kb == 0) {
+                        ok = tc::mbar_wait(w_bar, (n_weights - 1) & 1, a.err, tc::kWaitFull);
+                        if (ok && !first) ok = tc::mbar_wait(taken_bar, (n_done - 1) & 1, a.err, tc::kWaitEmpty);
+                    }
+                    if (!ok) break;
+                    tc::tc_fence_after_sync();
+                    if (tc::elect_one()) {
+                        const uint64_t dx = tc::smem_desc(ring + slot * (uint32_t)Smem::kSliceB, 16, 1024), dw = tc::smem_desc(w_base + kb * kWBytes, 16, 1024);
+#pragma unroll
+                        for (int m = 0; m < 4; ++m)        // node rows 0-3, 4-7 (upper), 1-4, 5-8 (lower); a node row is 32 x 128 bytes
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                tc::umma(tmem + m * kClassPad, dx + (((m & 1) * 4 + (m >> 1)) * (F_COLS * 128) >> 4) + 2 * j, dw + 2 * j, idesc, (kb | j) != 0);
+                        tc::umma_commit(bar0 + 16 + 8u * slot);
+                    }
+                    __syncwarp();
+                    ++mults[slot];
+                }
+                for (int kb = k0 + n_slots; kb < k0 + 2 * n_slots && kb < kblocks && ok; ++kb) {
+                    const int slot = kb - k0 - n_slots;
+                    ok = tc::mbar_wait(bar0 + 16 + 8u * slot, (mults[slot] - 1) & 1, a.err, tc::kWaitEmpty);
+                    if (ok) load(kb, slot, k, 0u);
+                }
+            }
+            if (!ok) break;
+            if (tc::elect_one()) tc::umma_commit(done_bar);
+            __syncwarp();
+            ok = tc::mbar_wait(done_bar, n_done & 1, a.err, tc::kWaitDone);
+            ++n_done;
+            first = false;
+        }
+        if (!ok) {                                         // nothing more is multiplied and nothing is written
+            gave_up = 1;
+            __syncwarp();
+            if (tc::elect_one()) arrive(done_bar);
+            tc::drain_after_error();
+        } else if (n_done) tc::mbar_wait(taken_bar, (n_done - 1) & 1, a.err, tc::kWaitEmpty);
+        pdl_launch_dependents();
+        __syncwarp();
+        tc::tc_fence_after_sync();
+        tc::tmem_dealloc(tmem, kLogitCols);
+        return;
+    }
+
+    // -------------------------------------------------------------------- the eight others
+    float2* my = slots + (size_t)wi * C * 32 + l;          // this lane's slot of class c: my[c * 32]
+    const int hw1 = a.heavy_w - 1;                         // what a weighted pixel counts on top of 1
+    const float invP = 1.0f / ((float)H * (float)W);
+    int n_done = 0;
+    bool waited = false;
+    // (neighbouring tiles at the same time on neighbouring blocks: what they share comes from L2.  16 streams of 256 channels at
+    // 720p: 227 us; with consecutive tiles per block, whose weights then stay, 240)
+    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const Tile k = tile_at(t);
+        const int x0 = k.x0, y0 = k.y0, s = k.s;
+        const int i = y0 - 1 + wi, n = x0 - 1 + l;         // cell row (frame rows 4i+2 .. 4i+5, node rows i, i+1), own node column
+        const bool cell_row = i <= h - 1, cell_valid = l <= 30 && n <= w - 1, node_owned = l >= 1 && l <= FN_X && n < w;
+        // the aligned 4-pixel words of the label rows: a cell's pixels are the upper half of its own column's word and the lower
+        // half of the next one's
+        uint32_t labw[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int Y = 4 * i + 2 + r;
+            labw[r] = cell_row && Y >= 0 && Y < H && n >= 0 && n < w
+                          ? __ldg(reinterpret_cast<const uint32_t*>(a.labels + (int64_t)s * H * W + (int64_t)Y * W + 4 * n)) : 0u;
+        }
+        if (!waited) { pdl_wait(); waited = true; }        // the parameters come from the previous kernel of the stream
+        if (a.skip && a.skip[(int64_t)s * a.skip_stride]) continue;
+        const float bias_l = l < C ? a.theta[(int64_t)s * a.n_params + a.b_off + l] : 0.f;
+        bool ok = tc::mbar_wait(done_bar, n_done & 1, a.err, tc::kWaitDone);
+        ++n_done;
+        tc::tc_fence_after_sync();
+        if (gave_up) ok = false;
+        if (!Smem::kPrefetch) {                            // the slices are dead: the arrays under them get their initial contents
+            if (!workers_all(ok)) return;                  // ... block-uniform
+            for (int e = tid; e < (int)(Smem::kCounts / 16); e += F_WORKERS) reinterpret_cast<uint4*>(counts)[e] = make_uint4(0, 0, 0, 0);
+            if (CONF) for (int e = tid; e < C * C; e += F_WORKERS) hist[e] = 0;
+            workers_sync();
+        }
+
+        float loss = 0.f;
+        unsigned n_bad = 0;
+        // where the cell's left and right node columns lie relative to the own slot (clamped at the frame's left and right border)
+        const int at_l = n == -1 ? 1 : 0, to_r = (l < 31 && n >= 0 && n < w - 1) ? 1 : 0;
+        const bool fold_l = n == -1, fold_r = n == w - 1;
+        const int t_row = min(i + 1, h - 1), t_col = min(n + 1, w - 1);    // the tile that owns this node counts the cell's loss
+        const bool own_cell = cell_row && cell_valid && t_row >= y0 && t_row < y0 + FN_Y && t_col >= x0 && t_col < x0 + FN_X;
+        if (cell_row && ok) {                              // warp-uniform
+            {
+                // ---- the warp's two node rows: tensor memory -> slots
+                bias[wi][l] = bias_l;
+                __syncwarp();
+                const uint32_t lanes = tmem + ((uint32_t)((wi & 3) * 32) << 16), upper = lanes + (wi >> 2) * kClassPad, lower = upper + 2 * kClassPad;
+                float up[32], lo[32];
+                if constexpr (C <= 16) {
+                    tc::tmem_ld_32x16(i == -1 ? lower : upper, reinterpret_cast<float(&)[16]>(up));
+                    tc::tmem_ld_32x16(i == h - 1 ? upper : lower, reinterpret_cast<float(&)[16]>(lo));
+                } else {
+                    tc::tmem_ld_32x32(i == -1 ? lower : upper, up);
+                    tc::tmem_ld_32x32(i == h - 1 ? upper : lower, lo);
+                }
+                tc::tc_fence_before_sync();
+                __syncwarp();
+                if (tc::elect_one()) arrive(taken_bar);
+                float m = -INFINITY;
+#pragma unroll
+                for (int c4 = 0; c4 < C; c4 += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4*>(&bias[wi][c4]);
+                    const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                    for (int c = c4; c < c4 + 4 && c < C; ++c) {
+                        up[c] += b[c - c4]; lo[c] += b[c - c4];
+                        m = fmaxf(m, fmaxf(up[c], lo[c]));
+                    }
+                }
+                const bool in_cols = n >= 0 && n < w;
+                if (!in_cols) m = -INFINITY;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                if (a.z_out && wi >= 1 && node_owned) {    // the own nodes, where the caller wants the logits kept
+                    float* zo = a.z_out + (int64_t)s * C * p + (int64_t)i * w + n;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) zo[(int64_t)c * p] = up[c];
+                }
+                // nodes outside the frame hold the bare bias: nobody's pixels, but they must not disturb the warp's vote
+                const float scale = in_cols ? kLog2e : 0.f, shift = in_cols ? -m * kLog2e : 0.f;
+#pragma unroll
+                for (int c = 0; c < C; ++c) my[c * 32] = make_float2(fmaf(up[c], scale, shift), fmaf(lo[c], scale, shift));
+                __syncwarp();
+            }
+            const float2* ps = my + at_l;
+            // ---- sweep 1: sums of the 16 pixels' exponentials
+            float2 Z01[4], Z23[4];                         // Z01[k] = (Z(0,k), Z(1,k)), Z23[k] = (Z(2,k), Z(3,k))
+#pragma unroll
+            for (int q = 0; q < 4; ++q) Z01[q] = Z23[q] = make_float2(0.f, 0.f);
+            float wmax = 0.f;
+            // CONF: the exponentials are positive and monotone in the logits, so the largest one marks the arg-max; its bit
+            // pattern with the low five bits replaced by 31 - c is compared as an integer (equal values: the lowest class
+            // wins).  Dropping five bits can only swap classes whose logits differ by less than 3e-6 relative.
+            uint32_t key[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) key[j] = 0;
+#pragma unroll kSweep1
+            for (int c = 0; c < C; ++c) {
+                float2 X01[4], X23[4], q01, q23;
+                wmax = fmaxf(wmax, cell_bases_log2(ps[c * 32], ps[c * 32 + to_r], X01[0], X23[0], q01, q23));
+#pragma unroll
+                for (int q = 1; q < 4; ++q) { X01[q] = __fmul2_rn(X01[q - 1], q01); X23[q] = __fmul2_rn(X23[q - 1], q23); }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) { Z01[q] = __fadd2_rn(Z01[q], X01[q]); Z23[q] = __fadd2_rn(Z23[q], X23[q]); }
+                if (CONF) {
+                    const uint32_t tag = 31u - (uint32_t)c;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        key[q] = max(key[q], (__float_as_uint(X01[q].x) & ~31u) | tag);
+                        key[4 + q] = max(key[4 + q], (__float_as_uint(X01[q].y) & ~31u) | tag);
+                        key[8 + q] = max(key[8 + q], (__float_as_uint(X23[q].x) & ~31u) | tag);
+                        key[12 + q] = max(key[12 + q], (__float_as_uint(X23[q].y) & ~31u) | tag);
+                    }
+                }
+            }
+            // ---- labels: the four rows' pixels of this cell, a byte each; 0x01 in the byte of a weighted pixel (hv), of a pixel
+            // inside the frame (vb) and of one that counts (rem: inside the frame, label below C)
+            uint32_t rem[4], hv[4], all = 0x01010101u;
+            {
+                const uint32_t cols = (cell_valid && n >= 0 ? 0x00000101u : 0u) | (cell_valid && n < w - 1 ? 0x01010000u : 0u);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int Y = 4 * i + 2 + r;
+                    labw[r] = __byte_perm(labw[r], __shfl_down_sync(0xffffffffu, labw[r], 1), 0x5432);
+                    const uint32_t vb = Y >= 0 && Y < H ? cols : 0u;
+                    hv[r] = 0;
+                    if (hw1 > 0) { hv[r] = (labw[r] >> 7) & 0x01010101u; labw[r] &= 0x7f7f7f7fu; }
+                    const uint32_t t8 = ((labw[r] & 0x7f7f7f7fu) + (uint32_t)(128 - C) * 0x01010101u) | labw[r];   // bit 7: label >= C
+                    rem[r] = (~t8 >> 7) & vb;
+                    all &= rem[r];
+                    if (own_cell) n_bad += __popc(rem[r] ^ vb);
+                }
+            }
+            float zmin = fminf(fminf(Z01[0].x, Z01[0].y), fminf(Z23[0].x, Z23[0].y));
+#pragma unroll
+            for (int q = 1; q < 4; ++q) zmin = fminf(zmin, fminf(fminf(Z01[q].x, Z01[q].y), fminf(Z23[q].x, Z23[q].y)));
+            bool off = !(wmax <= kFastRange) || (cell_valid && !(zmin > 1e-18f));
+            // a sum that is not a number passes fminf: all 16 are looked at through their total
+            {
+                float2 tot = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) tot = __fadd2_rn(tot, __fadd2_rn(Z01[q], Z23[q]));
+                off |= cell_valid && !(tot.x + tot.y < INFINITY);
+            }
+            uint32_t* node = counts + (min(max(i, 0), h - 1) - (y0 - 1)) * F_COLS + (min(max(n, 0), w - 1) - (x0 - 1));
+            const int right = min(max(n + 1, 0), w - 1) - min(max(n, 0), w - 1), below = (min(max(i + 1, 0), h - 1) - min(max(i, 0), h - 1)) * F_COLS;
+            if (!__any_sync(0xffffffffu, off)) {
+                float2 WL01[4], WL23[4], WR01[4], WR23[4];                 // a pixel's weight toward the left / right node column, over Z
+                float lz = 0.f;
+                if (__all_sync(0xffffffffu, hw1 == 0 && (all == 0x01010101u || !cell_valid))) {
+                    // every cell of the warp counts whole (nobody reads the pulls of lanes without a cell)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 r01 = make_float2(rcp_approx(Z01[q].x), rcp_approx(Z01[q].y)), r23 = make_float2(rcp_approx(Z23[q].x), rcp_approx(Z23[q].y));
+                        const float fr = (2 * q + 1) * 0.125f;
+                        const float2 f2 = make_float2(fr, fr), g2 = make_float2(1.0f - fr, 1.0f - fr);
+                        WL01[q] = __fmul2_rn(r01, g2); WL23[q] = __fmul2_rn(r23, g2);
+                        WR01[q] = __fmul2_rn(r01, f2); WR23[q] = __fmul2_rn(r23, f2);
+                        // sums lie between 1e-18 and C: products of two stay normal
+                        lz += lg2_approx(Z01[q].x * Z01[q].y) + lg2_approx(Z23[q].x * Z23[q].y);
+                    }
+                } else {
+                    float wl[16], wr[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const int r = j >> 2, q = j & 3;
+                        const float Z = r == 0 ? Z01[q].x : r == 1 ? Z01[q].y : r == 2 ? Z23[q].x : Z23[q].y;
+                        const bool counts_j = (rem[r] >> (8 * q)) & 1u;
+                        const float fr = (2 * q + 1) * 0.125f;
+                        const float wj = ((hv[r] >> (8 * q)) & 1u) ? (float)a.heavy_w : 1.0f;
+                        const float rz = counts_j ? rcp_approx(Z) * wj : 0.f;
+                        lz += counts_j ? wj * lg2_approx(Z) : 0.f;
+                        wl[j] = (fold_l ? 0.f : (fold_r ? 1.0f : 1.0f - fr)) * rz;
+                        wr[j] = (fold_r ? 0.f : (fold_l ? 1.0f : fr)) * rz;
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        WL01[q] = make_float2(wl[q], wl[4 + q]); WL23[q] = make_float2(wl[8 + q], wl[12 + q]);
+                        WR01[q] = make_float2(wr[q], wr[4 + q]); WR23[q] = make_float2(wr[8 + q], wr[12 + q]);
+                    }
+                }
+                if (CONF) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (own_cell && ((rem[j >> 2] >> (8 * (j & 3))) & 1u))
+                            atomicAdd(&hist[((labw[j >> 2] >> (8 * (j & 3))) & 0xffu) * C + (31u - (key[j] & 31u))], 1u);
+                }
+                // One round per distinct label of the cell (one round for most cells).  The pixels carrying the label pull
+                // the four corner nodes with integer weights (row eighths x column eighths, summed by byte-wise dot products);
+                // the same four sums weight the label's corner logits in the loss.
+                float lsum = 0.f;
+                while (rem[0] | rem[1] | rem[2] | rem[3]) {
+                    const uint32_t wsel = rem[0] ? labw[0] : rem[1] ? labw[1] : rem[2] ? labw[2] : labw[3];
+                    const uint32_t rsel = rem[0] ? rem[0] : rem[1] ? rem[1] : rem[2] ? rem[2] : rem[3];
+                    const uint32_t cur = (wsel >> (__ffs(rsel) - 1)) & 0xffu;
+                    const uint32_t cur4 = cur * 0x01010101u;
+                    uint32_t tl = 0, tr = 0, bl = 0, br = 0;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const uint32_t eq = ((0x80808080u - ((labw[r] ^ cur4) & 0x7f7f7f7fu)) >> 7) & rem[r];
+                        rem[r] ^= eq;
+                        const uint32_t ew = eq + (eq & hv[r]) * (uint32_t)hw1;          // each byte: the pixel's weight (1..5) or 0
+                        tl = __dp4a(ew, corner_weights(7 - 2 * r, false), tl);
+                        tr = __dp4a(ew, corner_weights(7 - 2 * r, true), tr);
+                        bl = __dp4a(ew, corner_weights(2 * r + 1, false), bl);
+                        br = __dp4a(ew, corner_weights(2 * r + 1, true), br);
+                    }
+                    add_counts(node, (int)cur, right, below, tl, tr, bl, br);
+                    const float2 L = ps[cur * 32], R = ps[cur * 32 + to_r];
+                    lsum = fmaf((float)tl, L.x, fmaf((float)tr, R.x, fmaf((float)bl, L.y, fmaf((float)br, R.y, lsum))));
+                }
+                if (own_cell) loss = (lz - lsum * (1.0f / 64.0f)) * kLn2;
+                // vertical weights of the rows toward the upper / lower node row (clamped borders fold into the inner row)
+                float tw[4], bw[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float ly = (2 * r + 1) * 0.125f;
+                    tw[r] = i == -1 ? 0.f : (i == h - 1 ? 1.0f : 1.0f - ly);
+                    bw[r] = i == h - 1 ? 0.f : (i == -1 ? 1.0f : ly);
+                }
+                const float2 tw01 = make_float2(tw[0], tw[1]), tw23 = make_float2(tw[2], tw[3]);
+                const float2 bw01 = make_float2(bw[0], bw[1]), bw23 = make_float2(bw[2], bw[3]);
+                __syncwarp();
+                // ---- sweep 2 (packed fp32x2: rows (0,1) and (2,3) side by side): the slots turn from logits into pulls.  The
+                // shuffles stand between every lane's reads of a class and its neighbours' writes.
+                auto pulls = [&](float2 L, float2 R) {
+                    float2 x01, x23, q01, q23, aL01, aL23, aR01, aR23;
+                    cell_bases_log2(L, R, x01, x23, q01, q23);
+                    cell_row_sums(x01, x23, q01, q23, WL01, WL23, aL01, aL23);
+                    cell_row_sums(x01, x23, q01, q23, WR01, WR23, aR01, aR23);
+                    // own cell's left part + left cell's right part, per row
+                    const float2 hs01 = __fadd2_rn(aL01, make_float2(__shfl_up_sync(0xffffffffu, aR01.x, 1), __shfl_up_sync(0xffffffffu, aR01.y, 1)));
+                    const float2 hs23 = __fadd2_rn(aL23, make_float2(__shfl_up_sync(0xffffffffu, aR23.x, 1), __shfl_up_sync(0xffffffffu, aR23.y, 1)));
+                    const float2 t2 = __ffma2_rn(hs23, tw23, __fmul2_rn(hs01, tw01));
+                    const float2 b2 = __ffma2_rn(hs23, bw23, __fmul2_rn(hs01, bw01));
+                    return make_float2(t2.x + t2.y, b2.x + b2.y);
+                };
+                constexpr int G = kSweep2;                 // classes in flight: all their reads come before the first write
+                static_for_groups<C, G>([&](int c0, auto count) {
+                    constexpr int N = decltype(count)::value;
+                    float2 L[N], R[N], o[N];
+#pragma unroll
+                    for (int g = 0; g < N; ++g) { L[g] = ps[(c0 + g) * 32]; R[g] = ps[(c0 + g) * 32 + to_r]; }
+#pragma unroll
+                    for (int g = 0; g < N; ++g) o[g] = pulls(L[g], R[g]);
+#pragma unroll
+                    for (int g = 0; g < N; ++g) my[(c0 + g) * 32] = o[g];
+                });
+            } else {
+                // ---- slow path: row by row, exact per-pixel maxima; the pulls stay in registers until the slots' logits are done with
+                float2 pull[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) pull[c] = make_float2(0.f, 0.f);
+                for (int r = 0; r < 4; ++r) {
+                    const int Y = 4 * i + 2 + r;
+                    if (!(Y >= 0 && Y < H)) continue;                      // warp-uniform
+                    const float ly = (2 * r + 1) * 0.125f;
+                    const uint32_t lab4 = r == 0 ? labw[0] : r == 1 ? labw[1] : r == 2 ? labw[2] : labw[3];
+                    const uint32_t rem4 = r == 0 ? rem[0] : r == 1 ? rem[1] : r == 2 ? rem[2] : rem[3];
+                    const uint32_t hv4 = r == 0 ? hv[0] : r == 1 ? hv[1] : r == 2 ? hv[2] : hv[3];
+                    float ex[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, Zs[4] = {0.f, 0.f, 0.f, 0.f};
+                    uint32_t arg[4] = {0, 0, 0, 0};
+#pragma unroll 3
+                    for (int c = 0; c < C; ++c) {
+                        float u[4];
+                        row_values(ps[c * 32], ps[c * 32 + to_r], ly, u);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (CONF) { if (u[q] > ex[q]) { ex[q] = u[q]; arg[q] = c; } }
+                            else ex[q] = fmaxf(ex[q], u[q]);
+                    }
+#pragma unroll 3
+                    for (int c = 0; c < C; ++c) {
+                        float u[4];
+                        row_values(ps[c * 32], ps[c * 32 + to_r], ly, u);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) Zs[q] += ex2_approx(u[q] - ex[q]);
+                    }
+                    float wl[4], wr[4];
+                    const int wy1 = 2 * r + 1, wy0 = 8 - wy1;              // eighths toward node rows i+1 / i
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int lab = (lab4 >> (8 * q)) & 0xff;
+                        float rz = 0.f;
+                        if ((rem4 >> (8 * q)) & 1u) {
+                            const int iw = ((hv4 >> (8 * q)) & 1u) ? a.heavy_w : 1;
+                            rz = rcp_approx(Zs[q]) * (float)iw;
+                            if (own_cell) {
+                                float u[4];
+                                row_values(ps[lab * 32], ps[lab * 32 + to_r], ly, u);
+                                loss += (float)iw * (lg2_approx(Zs[q]) - (u[q] - ex[q])) * kLn2;
+                                if (CONF) atomicAdd(&hist[lab * C + arg[q]], 1u);
+                            }
+                            const uint32_t wb = (2 * q + 1) * iw, wa = (7 - 2 * q) * iw;   // eighths toward node columns n+1 / n, times the weight
+                            add_counts(node, lab, right, below, wy0 * wa, wy0 * wb, wy1 * wa, wy1 * wb);
+                        }
+                        const float fr = (2 * q + 1) * 0.125f;
+                        wl[q] = (fold_l ? 0.f : (fold_r ? 1.0f : 1.0f - fr)) * rz;
+                        wr[q] = (fold_r ? 0.f : (fold_l ? 1.0f : fr)) * rz;
+                    }
+                    const float twr = i == -1 ? 0.f : (i == h - 1 ? 1.0f : 1.0f - ly), bwr = i == h - 1 ? 0.f : (i == -1 ? 1.0f : ly);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        float u[4], e[4];
+                        row_values(ps[c * 32], ps[c * 32 + to_r], ly, u);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) e[q] = ex2_approx(u[q] - ex[q]);
+                        const float aL = fmaf(wl[0], e[0], fmaf(wl[1], e[1], fmaf(wl[2], e[2], wl[3] * e[3])));
+                        const float aR = fmaf(wr[0], e[0], fmaf(wr[1], e[1], fmaf(wr[2], e[2], wr[3] * e[3])));
+                        const float hs = aL + __shfl_up_sync(0xffffffffu, aR, 1);
+                        pull[c] = make_float2(fmaf(twr, hs, pull[c].x), fmaf(bwr, hs, pull[c].y));
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < C; ++c) my[c * 32] = pull[c];
+            }
+        } else if (ok) {                                   // a warp below the frame has nothing to take, but says so
+            tc::tc_fence_before_sync();
+            __syncwarp();
+            if (tc::elect_one()) arrive(taken_bar);
+        }
+        // loss of the tile, fixed order
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        if (l == 0) red[n_done & 1][wi] = loss;            // (two of them: warps may be one tile ahead of the one that adds)
+        if (n_bad) atomicAdd(a.bad, n_bad);
+        if (!workers_all(ok)) return;                      // block-uniform: a wait ran out, nothing is written
+        if (t + (int)gridDim.x >= n_tiles) pdl_launch_dependents();        // only the epilogue is left
+        if (CONF) {                                        // one global update per non-empty counter of the tile
+            for (int e = tid; e < C * C; e += F_WORKERS) {
+                const unsigned int v = hist[e];
+                if (v) { atomicAdd(a.conf + (int64_t)s * a.conf_stream_stride + e, (unsigned long long)v); hist[e] = 0; }
+            }
+        }
+        // ---- node row y0-1+wi (warps 1..FN_Y): own upper pulls + lower pulls of the warp above - counts
+        const bool node_ok = wi >= 1 && i < h && node_owned;
+        float v[32];
+#pragma unroll
+        for (int c = 0; c < 32; ++c) v[c] = 0.f;
+        if (node_ok) {
+            const float2* above = my - C * 32;
+            uint32_t* mine = counts + wi * F_COLS + l;
+#pragma unroll
+            for (int c = 0; c < C; c += 2) {
+                const uint32_t ct = mine[(c >> 1) * kNodes];
+                mine[(c >> 1) * kNodes] = 0;               // ready for the next tile (words outside the owned nodes are never read)
+                v[c] = (my[c * 32].x + above[c * 32].y - (float)(ct & 0xffffu) * (1.0f / 64.0f)) * invP;
+                if (c + 1 < C) v[c + 1] = (my[(c + 1) * 32].x + above[(c + 1) * 32].y - (float)(ct >> 16) * (1.0f / 64.0f)) * invP;
+            }
+            if (a.dz) {
+                float* dzp = a.dz + (int64_t)s * C * a.dz_plane + (int64_t)i * a.dz_pitch + n;
+#pragma unroll
+                for (int c = 0; c < C; ++c) dzp[(int64_t)c * a.dz_plane] = v[c];
+            }
+            if (a.dz_bf16) {
+                bf16* dzb = a.dz_bf16 + (int64_t)s * kClassPad * a.dz_bf16_pitch + (int64_t)i * w + n;
+#pragma unroll
+                for (int c = 0; c < C; ++c) dzb[(int64_t)c * a.dz_bf16_pitch] = __float2bfloat16_rn(v[c]);
+            }
+        }
+        // bias-gradient partial of the tile.  Lane reduce-scatter inside each warp (31 exchanges: at distance o a lane keeps the
+        // half of its values whose class has bit o equal to its own lane bit and adds the partner's), after which lane c holds
+        // class c; then the warps' sums are added in warp order.  Fixed order throughout.
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const bool hi = l & o;
+#pragma unroll
+            for (int j = 0; j < o; ++j) {
+                const float send = hi ? v[j] : v[j + o];
+                const float keep = hi ? v[j + o] : v[j];
+                v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+        wsum[wi][l] = v[0];
+        workers_sync();
+        if (tid < C) {
+            float q = 0.f;
+#pragma unroll
+            for (int r = 1; r < F_WARPS; ++r) q += wsum[r][tid];
+            a.db_part[((int64_t)s * per_stream + k.blk) * C + tid] = q;
+        }
+        if (tid == 32) {
+            float q = 0.f;
+            for (int r = 0; r < F_WARPS; ++r) q += red[n_done & 1][r];
+            a.loss_part[(int64_t)s * per_stream + k.blk] = q;
+        }
+    }
+}
+
+template <int C>
+cudaError_t prepare_fwd_ce_as()
+{
+    cudaError_t e = allow_shared_memory((const void*)fwd_ce_kernel<C, false>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, true>);
+    return e;
+}
+
+template <int C, bool CONF>
+void launch_fwd_ce_as(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
+{
+    using Smem = FwdCeSmem<C, CONF>;
+    const int tx = (a.w + FN_X - 1) / FN_X, ty = (a.h + FN_Y - 1) / FN_Y, tiles = tx * ty * a.S;
+    const int grid = Smem::kPrefetch && tiles > 2 * a.n_sms ? 2 * a.n_sms : tiles;
+    launch_early(a.chain_early != 0 || a.x_early != 0, fwd_ce_kernel<C, CONF>, dim3(grid), dim3(F_THREADS), Smem::kBytes, s, a, tx, ty, x_map, w_map);
+}
+
+template <int C>
+void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
+{
+    if (a.conf) launch_fwd_ce_as<C, true>(a, x_map, w_map, s);
+    else launch_fwd_ce_as<C, false>(a, x_map, w_map, s);
+}
+
+}  // namespace
+
+// The kernels of one class count
+struct FwdCeKernels {
+    cudaError_t (*prepare)();
+    void (*launch)(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s);
+};
+
+// ... of class count `n`, one of FIRST + I...
+template <int FIRST, int... I>
+static FwdCeKernels fwd_ce_kernels_of(int n, std::integer_sequence<int, I...>)
+{
+    static const FwdCeKernels all[] = {{prepare_fwd_ce_as<FIRST + I>, launch_fwd_ce_of<FIRST + I>}...};
+    return all[n - FIRST];
+}
+
+// one file each, so that they compile side by side
+constexpr int kFwdCeLast[] = {12, 18, 23, 28, 32};      // the last class count of each file; the first one begins at 2
+FwdCeKernels fwd_ce_kernels_0(int n);
+FwdCeKernels fwd_ce_kernels_1(int n);
+FwdCeKernels fwd_ce_kernels_2(int n);
+FwdCeKernels fwd_ce_kernels_3(int n);
+FwdCeKernels fwd_ce_kernels_4(int n);
+
+}  // namespace st

@@ -1,0 +1,12 @@
+// Class counts 2 to 12 of the forward + upsample + cross-entropy kernel.
+#include "k_fwd_ce.cuh"
+
+namespace st {
+
+FwdCeKernels fwd_ce_kernels_0(int n)
+{
+    constexpr int first = 2;
+    return fwd_ce_kernels_of<first>(n, std::make_integer_sequence<int, kFwdCeLast[0] - first + 1>());
+}
+
+}  // namespace st

@@ -1,0 +1,12 @@
+// Class counts 13 to 18 of the forward + upsample + cross-entropy kernel.
+#include "k_fwd_ce.cuh"
+
+namespace st {
+
+FwdCeKernels fwd_ce_kernels_1(int n)
+{
+    constexpr int first = kFwdCeLast[0] + 1;
+    return fwd_ce_kernels_of<first>(n, std::make_integer_sequence<int, kFwdCeLast[1] - first + 1>());
+}
+
+}  // namespace st

@@ -1,0 +1,12 @@
+// Class counts 24 to 28 of the forward + upsample + cross-entropy kernel.
+#include "k_fwd_ce.cuh"
+
+namespace st {
+
+FwdCeKernels fwd_ce_kernels_3(int n)
+{
+    constexpr int first = kFwdCeLast[2] + 1;
+    return fwd_ce_kernels_of<first>(n, std::make_integer_sequence<int, kFwdCeLast[3] - first + 1>());
+}
+
+}  // namespace st

@@ -416,9 +416,9 @@ cudaError_t prepare_upsample_ce(int C)
     return e != cudaSuccess ? e : allow_many<4, 3>();
 }
 
-void launch_upsample_ce(const UpsampleCeArgs& a, const CUtensorMap* z_map, cudaStream_t s, const CUtensorMap* x_map, const CUtensorMap* w_map)
+void launch_upsample_ce(const UpsampleCeArgs& a, const CUtensorMap* z_map, cudaStream_t s)
 {
-    if (upsample_ce_rows_supported(a.C)) { launch_upsample_ce_rows(a, z_map, s, x_map, w_map); return; }
+    if (upsample_ce_rows_supported(a.C)) { launch_upsample_ce_rows(a, z_map, s); return; }
     if (many_shape(a.h, a.w).own_y == 7) launch_many<7, 2>(a, s);
     else launch_many<4, 3>(a, s);
 }

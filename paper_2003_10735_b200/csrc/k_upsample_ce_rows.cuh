@@ -43,7 +43,6 @@
 
 #include "st_internal.h"
 #include "tc_common.cuh"
-#include "fused_tile.cuh"
 #include "cell_softmax.cuh"
 
 #include <utility>
@@ -52,13 +51,11 @@ namespace st {
 
 namespace {
 
-constexpr int RN_Y = fused::kOwnRows, RN_X = fused::kOwnCols;      // nodes a block owns: 7 rows x 30 columns
+constexpr int RN_Y = 7, RN_X = 30;           // nodes a block owns
 constexpr int R_WARPS = RN_Y + 1, R_THREADS = R_WARPS * 32;
 constexpr int TZ_H = RN_Y + 2;
-// Columns of a tile row (template parameter TW of everything below): 36 when the logits are fetched from global memory
-// (32 used, starting at a multiple of 4 so that rows are whole 16-byte vectors), 32 when the block computes its logits
-// itself (kTwFused).
-constexpr int kTwLoad = 36, kTwFused = fused::kTileCols;
+// Columns of a tile row: 32 used, starting at a multiple of 4 so that rows are whole 16-byte vectors
+constexpr int TZ_W = 36, TZ = TZ_H * TZ_W;
 // Classes per iteration of the two fast-path class sweeps.  The sweeps are rolled loops: unrolled over all classes
 // they were ~70 KB of straight-line code that every warp ran through once, and instruction fetch was the main stall.
 #ifndef ST_K3_CLASS_UNROLL
@@ -76,10 +73,9 @@ struct RowCtx {
 };
 
 // interpolated, shifted logits of the lane's four pixels for class c
-template <bool SHIFT, int TW>
+template <bool SHIFT>
 __device__ __forceinline__ void pixel_logits(const RowCtx& rc, int c, const float (&sk)[4], float (&u)[4])
 {
-    constexpr int TZ = TZ_H * TW;
     const float a = rc.za[c * TZ], b = rc.za[c * TZ + rc.dq];
     const float vl = fmaf(fmaf(rc.ly, b - a, a), kLog2e, -rc.M);
     const float vr = __shfl_down_sync(0xffffffffu, vl, 1);
@@ -91,7 +87,7 @@ __device__ __forceinline__ void pixel_logits(const RowCtx& rc, int c, const floa
     }
 }
 
-template <int C, bool CONF, bool SHIFT, int TW>
+template <int C, bool CONF, bool SHIFT>
 __device__ __forceinline__ void pass1(const RowCtx& rc, const float (&sk)[4], float (&Zs)[4], uint32_t (&arg)[4])
 {
     float best[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -99,7 +95,7 @@ __device__ __forceinline__ void pass1(const RowCtx& rc, const float (&sk)[4], fl
 #pragma unroll
     for (int c = 0; c < C; ++c) {
         float u[4];
-        pixel_logits<SHIFT, TW>(rc, c, sk, u);
+        pixel_logits<SHIFT>(rc, c, sk, u);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             if (CONF && !SHIFT) { if (u[k] > best[k]) { best[k] = u[k]; arg[k] = c; } }
@@ -111,14 +107,14 @@ __device__ __forceinline__ void pass1(const RowCtx& rc, const float (&sk)[4], fl
 // pass 2 of one row on the slow path: the exponentials are formed again, multiplied by the adjoint interpolation
 // weights / Z, the right-hand part goes to the next lane, and the row is added into this thread's shared-memory
 // slots of the upper and the lower node row
-template <int C, int TW>
+template <int C>
 __device__ __forceinline__ void pass2_slow(const RowCtx& rc, const float (&sk)[4], const float (&wl)[4], const float (&wr)[4],
                                            float tw, float bw, float2* my_acc)
 {
 #pragma unroll
     for (int c = 0; c < C; ++c) {
         float u[4];
-        pixel_logits<true, TW>(rc, c, sk, u);
+        pixel_logits<true>(rc, c, sk, u);
         const float e0 = ex2_approx(u[0]), e1 = ex2_approx(u[1]), e2 = ex2_approx(u[2]), e3 = ex2_approx(u[3]);
         const float aL = fmaf(wl[0], e0, fmaf(wl[1], e1, fmaf(wl[2], e2, wl[3] * e3)));
         const float aR = fmaf(wr[0], e0, fmaf(wr[1], e1, fmaf(wr[2], e2, wr[3] * e3)));
@@ -128,24 +124,18 @@ __device__ __forceinline__ void pass2_slow(const RowCtx& rc, const float (&sk)[4
     }
 }
 
-template <int C, bool CONF, int TW>
+template <int C, bool CONF>
 __global__ void __launch_bounds__(R_THREADS, 2)
-upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_map, const __grid_constant__ CUtensorMap x_map,
-                        const __grid_constant__ CUtensorMap w_map)
+upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_map)
 {
-    constexpr bool FUSED = TW == kTwFused;      // the block multiplies its own logit tile (Forward of Algorithm 1 for a 1x1 classifier)
-    constexpr int TZ_W = TW, TZ = TZ_H * TW;
     extern __shared__ __align__(128) float smem_r[];
     const int h = a.h, w = a.w, H = h * kUp, W = w * kUp;
-    // [C][TZ_H][TW]  logits, borders replicated.  FUSED: the feature
-    // stages and the classifier weights lie over this and the next two arrays until the multiplication has finished.
-    float* zt = FUSED ? (float*)(((uintptr_t)smem_r + 1023) & ~(uintptr_t)1023) : smem_r;
-    int* corr = (int*)(zt + C * TZ);            // [C][TZ_H][TW]    -64 * (adjoint of onehot)
+    float* zt = smem_r;                         // [C][TZ_H][TZ_W]  logits, borders replicated
+    int* corr = (int*)(zt + C * TZ);            // [C][TZ_H][TZ_W]  -64 * (adjoint of onehot)
     float2* acc = (float2*)(corr + C * TZ);     // [R_WARPS][C][32] (x, y): the cell's pull on its upper / lower node row
     unsigned int* hist = (unsigned int*)(acc + R_WARPS * C * 32);   // [C][C] (CONF): the block's share of the confusion matrix
     __shared__ float red[R_WARPS], red_m[R_WARPS];
     __shared__ __align__(8) uint64_t tile_bar;
-    __shared__ fused::Shared fsh;               // FUSED: barriers, tensor-memory slot, bias of the block's own forward
 
     // Launch order: the last block row first, then rows 0, 1, ...  Blocks at the frame border do extra work, and the
     // blocks that reach an SM first finish earlier than their later companions, so the border rows go first.
@@ -160,7 +150,7 @@ upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_
     // ---- tile: node rows y0-1 .. y0+RN_Y, node columns xa .. xa+35 where xa = (x0-1) rounded down to a
     // multiple of 4 (so that rows are fetched as 16-byte vectors), clamped at the borders, scaled by
     // log2(e).  Fully unrolled: all of a thread's loads are in flight together.
-    const bool vec_ok = !FUSED && (w % 4 == 0) && ((uintptr_t)z % 16 == 0);
+    const bool vec_ok = (w % 4 == 0) && ((uintptr_t)z % 16 == 0);
     const int xa = vec_ok ? ((x0 - 1) & ~3) : x0 - 1;      // x0-1 >= -1; (-1 & ~3) = -4
     const int off = (x0 - 1) - xa;                         // column of node x0-1 inside the tile
     const int i = y0 - 1 + wi;                  // cell row: frame rows 4i+2 .. 4i+5, node rows (i, i+1)
@@ -199,7 +189,7 @@ upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_
         for (int r = 0; r < 4; ++r) { hv[r] = (labw[r] >> 7) & 0x01010101u; labw[r] &= 0x7f7f7f7fu; }
     }
     // Node rows above 0 / below h-1 and node columns left of 0 / right of w-1 repeat the border row / column (the tile
-    // holds something else there: zeros from the tile copy, or the bare bias from the block's own multiplication).
+    // copy has left zeros there).
     auto replicate_borders = [&]() {
         float4* zt4 = reinterpret_cast<float4*>(zt);
         const bool edge_rows = y0 == 0 || y0 + RN_Y > h - 1, edge_cols = xa < 0 || xa + TZ_W > w;
@@ -228,25 +218,6 @@ upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_
         }
     };
     float m_loc = -INFINITY;                               // largest logit of this thread's share of the tile
-    uint32_t tmem = 0;                                     // FUSED: the block's tensor memory (given back at the very end)
-    if constexpr (FUSED) {
-        // ---- Forward for a 1x1 classifier, inside the block (fused_tile.cuh)
-        fused::Args fa;
-        fa.kblocks = a.kblocks; fa.x_early = a.x_early;
-        fa.skip = a.skip ? a.skip + (int64_t)s * a.skip_stride : nullptr;
-        fa.err = a.err;
-        fa.bias = a.theta + (int64_t)s * a.n_params + a.b_off;
-        fa.z_out = a.z_out ? a.z_out + (int64_t)s * C * p : nullptr;
-        fa.C = C; fa.h = h; fa.w = w;
-        fa.spin_limit = a.test_stall ? (1u << 12) : tc::kSpinLimit; fa.stall_bytes = a.test_stall ? 16u : 0u;
-        auto after_mma = [&]() {                        // the arrays the stages lay over get their initial contents
-            for (int e = tid; e < C * TZ / 4; e += R_THREADS) reinterpret_cast<int4*>(corr)[e] = make_int4(0, 0, 0, 0);
-            if (CONF) for (int e = tid; e < C * C; e += R_THREADS) hist[e] = 0;
-        };
-        const fused::Tile tile = fused::logit_tile(fa, &x_map, &w_map, fsh, zt, s, x0, y0, after_mma);
-        if (!tile.ok) return;
-        m_loc = tile.m_loc; tmem = tile.tmem;
-    } else
     {
         // a thread keeps one 16-byte group of the tile plane (81 groups) and walks the classes three at a time
         constexpr int kQuads = TZ / 4, kPlanes = R_THREADS / kQuads;       // 81, 3
@@ -539,19 +510,19 @@ upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_
                 const float zero4[4] = {0.f, 0.f, 0.f, 0.f};
                 for (int c = 0; c < C; ++c) {
                     float u[4];
-                    pixel_logits<false, TW>(rc, c, zero4, u);
+                    pixel_logits<false>(rc, c, zero4, u);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) ex[k] = fmaxf(ex[k], u[k]);
                 }
                 float Zs[4];
                 uint32_t ar4[4] = {0, 0, 0, 0};
-                if (CONF) pass1<C, true, false, TW>(rc, zero4, Zs, ar4);    // arg-max of the interpolated logits
-                pass1<C, false, true, TW>(rc, ex, Zs, ar4);
+                if (CONF) pass1<C, true, false>(rc, zero4, Zs, ar4);    // arg-max of the interpolated logits
+                pass1<C, false, true>(rc, ex, Zs, ar4);
                 float wl4[4], wr4[4];
                 finish_row(r, Zs, ex, ar4, wl4, wr4);
                 const float twr = i == -1 ? 0.f : (i == h - 1 ? 1.0f : 1.0f - rc.ly);
                 const float bwr = i == h - 1 ? 0.f : (i == -1 ? 1.0f : rc.ly);
-                pass2_slow<C, TW>(rc, ex, wl4, wr4, twr, bwr, my_acc);
+                pass2_slow<C>(rc, ex, wl4, wr4, twr, bwr, my_acc);
             }
         }
     } else {
@@ -633,42 +604,28 @@ upsample_ce_rows_kernel(UpsampleCeArgs a, const __grid_constant__ CUtensorMap z_
         for (int k = 0; k < R_WARPS; ++k) t += red[k];
         a.loss_part[(int64_t)s * n_blk + blk] = t;
     }
-    if constexpr (FUSED) fused::free_tmem(tmem);     // every warp's reads of tensor memory ended before the barriers above
 }
 
-template <int C, int TW>
+template <int C>
 constexpr size_t rows_smem_bytes(bool conf)
 {
-    constexpr size_t TZ = (size_t)TZ_H * TW;
-    const size_t plain = (2 * C * TZ + (size_t)R_WARPS * C * 32 * 2 + (conf ? C * C : 0)) * sizeof(float) + 128;
-    return TW != kTwFused ? plain : fused::smem_bytes(plain);      // the feature stages and the weights lie over the kernel's arrays
+    return (2 * C * (size_t)TZ + (size_t)R_WARPS * C * 32 * 2 + (conf ? C * C : 0)) * sizeof(float) + 128;
 }
 
 template <int C>
 cudaError_t prepare_rows()
 {
-    cudaError_t e = allow_shared_memory((const void*)upsample_ce_rows_kernel<C, false, kTwLoad>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)upsample_ce_rows_kernel<C, true, kTwLoad>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)upsample_ce_rows_kernel<C, false, kTwFused>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)upsample_ce_rows_kernel<C, true, kTwFused>);
-    return e;
-}
-
-template <int C, bool CONF, int TW>
-void launch_rows_as(const UpsampleCeArgs& a, const CUtensorMap& z_map, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
-{
-    const dim3 grid((unsigned)((a.w + RN_X - 1) / RN_X), (unsigned)((a.h + RN_Y - 1) / RN_Y), (unsigned)a.S);
-    launch_early(a.chain_early != 0 || a.x_early != 0, upsample_ce_rows_kernel<C, CONF, TW>, grid, dim3(R_THREADS), rows_smem_bytes<C, TW>(CONF), s,
-                 a, z_map, x_map, w_map);
+    const cudaError_t e = allow_shared_memory((const void*)upsample_ce_rows_kernel<C, false>);
+    return e != cudaSuccess ? e : allow_shared_memory((const void*)upsample_ce_rows_kernel<C, true>);
 }
 
 template <int C>
-void launch_rows(const UpsampleCeArgs& a, const CUtensorMap& z_map, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
+void launch_rows(const UpsampleCeArgs& a, const CUtensorMap& z_map, cudaStream_t s)
 {
-    if (a.fused && a.conf) launch_rows_as<C, true, kTwFused>(a, z_map, x_map, w_map, s);
-    else if (a.fused) launch_rows_as<C, false, kTwFused>(a, z_map, x_map, w_map, s);
-    else if (a.conf) launch_rows_as<C, true, kTwLoad>(a, z_map, x_map, w_map, s);
-    else launch_rows_as<C, false, kTwLoad>(a, z_map, x_map, w_map, s);
+    const dim3 grid((unsigned)((a.w + RN_X - 1) / RN_X), (unsigned)((a.h + RN_Y - 1) / RN_Y), (unsigned)a.S);
+    const bool early = a.chain_early != 0;
+    if (a.conf) launch_early(early, upsample_ce_rows_kernel<C, true>, grid, dim3(R_THREADS), rows_smem_bytes<C>(true), s, a, z_map);
+    else launch_early(early, upsample_ce_rows_kernel<C, false>, grid, dim3(R_THREADS), rows_smem_bytes<C>(false), s, a, z_map);
 }
 
 }  // namespace
@@ -676,7 +633,7 @@ void launch_rows(const UpsampleCeArgs& a, const CUtensorMap& z_map, const CUtens
 // The kernels of one class count
 struct RowsKernels {
     cudaError_t (*prepare)();
-    void (*launch)(const UpsampleCeArgs& a, const CUtensorMap& z_map, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s);
+    void (*launch)(const UpsampleCeArgs& a, const CUtensorMap& z_map, cudaStream_t s);
 };
 
 // ... of class count `n`, one of FIRST + I...

@@ -73,6 +73,7 @@ struct st_ctx {
     CUtensorMap k3_map;        // tile map of z for the fused upsample + cross-entropy kernel
     int k3_has_map = 0;
     CUtensorMap fx_map, fw_map; // tile maps of the features and of the bf16 classifier weights: the loss kernel multiplies its own logits
+    int n_sms = 0;
     int fused_fwd = 0;          //   (one-layer head with bf16 GEMMs; ST_FUSED_FORWARD=0 switches it off)
     int test_stall_fused = 0;   // test of the give-up path inside that kernel (environment ST_TEST_STALL_FUSED=1 at context creation)
     float* loss_buf = nullptr;              // [S][kMaxSteps]
@@ -343,7 +344,7 @@ UpsampleCeArgs k3_args(st_ctx* c, bool fp32_grad, bool bf16_grad, unsigned long 
     k3.has_map = c->k3_has_map;
     k3.skip = skip; k3.skip_stride = skip_stride;
     k3.chain_early = c->chain_early ? 1 : 0;
-    k3.fused = 0; k3.x_early = 0; k3.kblocks = 0; k3.theta = nullptr; k3.n_params = 0; k3.b_off = 0; k3.z_out = nullptr; k3.test_stall = 0;
+    k3.n_sms = c->n_sms; k3.x_early = 0; k3.kblocks = 0; k3.theta = nullptr; k3.n_params = 0; k3.b_off = 0; k3.z_out = nullptr; k3.test_stall = 0;
     return k3;
 }
 
@@ -357,15 +358,18 @@ st_status enqueue_loss(st_ctx* c, unsigned long long* conf, StageTimer* t = null
     if (c->fused_fwd) {
         // Forward as well: the features are frozen, so after a parameter update (which writes weights only) their tiles
         // may be fetched while that update is still running
-        k3.fused = 1; k3.x_early = after_update && !t ? 1 : 0; k3.kblocks = c->Cin / 64;
+        k3.x_early = after_update && !t ? 1 : 0; k3.kblocks = c->Cin / 64;
         k3.theta = c->theta; k3.n_params = c->n_params; k3.b_off = c->layout.b_off[c->layout.n_layers - 1];
         k3.z_out = keep_logits ? c->z : nullptr;         // logits that the next iteration overwrites unread stay on the chip
         k3.test_stall = c->test_stall_fused;
         // the first iteration's predecessor may have written the labels and the features, which are fetched before the wait
         if (!after_update) k3.chain_early = 0;
     }
-    ST_REPEAT(t) launch_upsample_ce(k3, &c->k3_map, s, &c->fx_map, &c->fw_map);
-    if (t) t->mark(k3.fused ? "fwd1x1_upsample_ce" : "upsample_ce", s, st_repeats(t));
+    ST_REPEAT(t) {
+        if (c->fused_fwd) launch_fwd_ce(k3, c->fx_map, c->fw_map, s);
+        else launch_upsample_ce(k3, &c->k3_map, s);
+    }
+    if (t) t->mark(c->fused_fwd ? "fwd1x1_upsample_ce" : "upsample_ce", s, st_repeats(t));
     c->launches += st_repeats(t);
     return check_launch(c, "upsample + cross-entropy");
 }
@@ -638,6 +642,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     c->h = d.feat_h; c->w = d.feat_w; c->H = d.feat_h * kUp; c->W = d.feat_w * kUp;
     c->p = (int64_t)c->h * c->w; c->P = (int64_t)c->H * c->W;
     c->bf16_mode = d.gemm_precision == 1;
+    if (cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || c->n_sms < 1) { c->n_sms = 148; cudaGetLastError(); }
     c->n_blocks = n_blocks; c->first_trained = first_trained;
     for (int i = 0, prev = d.c_in; i < n_blocks; ++i) {
         c->blk[i].c_prev = prev; c->blk[i].c_skip = blk_skip[i]; c->blk[i].c_out = blk_out[i];
@@ -796,7 +801,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             c->fused_fwd = make_feature_tile_map(&c->fx_map, c->x_bf16, S, c->Cin, c->h, c->w) &&
                            encode_tensor_map(&c->fw_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, c->w2_shadow, 3,
                                              dims, str, box, msg, sizeof msg, "1x1 weight") &&
-                           prepare_student_eval() == cudaSuccess;
+                           prepare_student_eval() == cudaSuccess && prepare_fwd_ce(c->C) == cudaSuccess;
             if (const char* ts = getenv("ST_TEST_STALL_FUSED")) c->test_stall_fused = ts[0] == '1' ? 1 : 0;
         }
     }
