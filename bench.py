@@ -252,7 +252,7 @@ def kernel_table(st, ctx, cfg, peaks, arith, n_profile_steps):
                 # 9 x 32 nodes around its 7 x 30 from L2, so the launch streams 288/210 of the feature map
                 n_tiles = -(-cfg.feat_h // 7) * -(-cfg.feat_w // 30)
                 k.update(hbm_gbs=S * (p * c_last * 2 + P) / ms / 1e6,
-                         forward={"tensor_tflops": 2.0 * S * n_tiles * 384 * 32 * c_last / ms / 1e9,
+                         forward={"tensor_tflops": 2.0 * S * n_tiles * 512 * 32 * c_last / ms / 1e9,
                                   "feature_bytes_fetched_by_blocks": S * n_tiles * 288 * c_last * 2,
                                   "note": "replaces tc_fwd1x1 + upsample_ce (see kernels_unfused for those two)"})
         elif name == "tc_fwd1x1":

@@ -1,5 +1,5 @@
-// Host side of the forward + upsample + cross-entropy kernel (k_fwd_ce.cuh): which shapes it takes, which instantiation a launch
-// uses, and the tile map of its features.
+// Host side of the upsample + cross-entropy kernel for at most 32 classes (k_fwd_ce.cuh): which shapes its own forward takes, which
+// instantiation a launch uses, and the tile map of the features.
 #include "k_fwd_ce.cuh"
 
 namespace st {
@@ -18,9 +18,22 @@ bool fused_forward_supported(int C, int h, int w, int c_in)
     return C <= kClassPad && c_in >= 64 && c_in % 64 == 0 && c_in / 64 <= fused::kMaxKBlocks && w >= F_COLS && h >= F_ROWS;
 }
 
+bool upsample_ce_rows_supported(int C) { return C <= kClassPad; }
+
+int upsample_ce_rows_blocks(int h, int w) { return ((h + FN_Y - 1) / FN_Y) * ((w + FN_X - 1) / FN_X); }
+
 cudaError_t prepare_fwd_ce(int C) { return fwd_ce_kernels(C).prepare(); }
 
-void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s) { fwd_ce_kernels(a.C).launch(a, x_map, w_map, s); }
+void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s) { fwd_ce_kernels(a.C).launch[1](a, x_map, w_map, s); }
+
+void launch_upsample_ce_rows(const UpsampleCeArgs& a, cudaStream_t s)
+{
+    UpsampleCeArgs b = a;
+    b.x_early = 0;
+    CUtensorMap none;
+    memset(&none, 0, sizeof none);
+    fwd_ce_kernels(b.C).launch[0](b, none, none, s);
+}
 
 bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w)
 {

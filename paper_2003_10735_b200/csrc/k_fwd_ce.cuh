@@ -1,6 +1,7 @@
-// Forward of a 1x1 classifier, ComputeLoss and the first half of PartialBackward (Algorithm 1; loss of Section 5.2) in one
-// kernel, for at most 32 classes over at most 256 bf16 channels: logits of a tile of feature-map nodes (tcgen05), bilinear x4
-// upsample, per-pixel softmax cross-entropy against the labels, gradient of the mean loss with respect to the logits.
+// K3 for at most 32 classes — ComputeLoss and the first half of PartialBackward (Algorithm 1; loss of Section 5.2): bilinear x4
+// upsample of the low-resolution logits, per-pixel softmax cross-entropy against the labels, gradient of the mean loss with
+// respect to the logits.  With FORWARD the block multiplies its logits itself (1x1 classifier over at most 256 bf16 channels);
+// without it they are read from memory.  Both forms do the same with them, bit for bit.  For more classes: k_upsample_ce.cu.
 //
 // Geometry.  With half-pixel centres and factor 4 the frame pixels 4n+2 .. 4n+5 lie between node columns n and n+1 ("cell" n)
 // with weights 1/8, 3/8, 5/8, 7/8 toward n+1; rows alike.  Cells -1 and w-1 are the clamped borders (their outer node is the
@@ -9,14 +10,15 @@
 // lane 31 are halo (recomputed by the neighbouring tile), so that a tile's nodes are finished in a fixed summation order,
 // without floating-point atomics.
 //
-// Logits.  A ninth warp feeds the tensor core: the features of the tile's 9 x 32 nodes arrive in 64-channel slices (one 4-d tile
+// Logits with FORWARD.  A ninth warp feeds the tensor core: the features of the tile's 9 x 32 nodes arrive in 64-channel slices (one 4-d tile
 // copy each; nodes outside the map arrive as zeros), and four multiplications per 16 channels leave node row i of the tile and
 // node row i+1 of it in the same 32 tensor-memory lanes: the two rows that warp i's cells lie between.  A warp therefore takes
 // its logits out of tensor memory alone, without the other warps: bias added, shifted by the largest of them, in log2 units,
 // clamped at the frame's border, both rows of a class side by side in the warp's own slots of shared memory
 // [class][lane] (upper, lower).  The second class sweep leaves the cell's pull on the two node rows in the same slots.
 // Blocks are persistent where there are more tiles than blocks fit: once the eight warps have emptied the tensor memory, the
-// ninth multiplies the next tile, whose slices arrive while this one is worked on.
+// ninth multiplies the next tile, whose slices arrive while this one is worked on.  Without FORWARD a warp reads its two node rows
+// from memory (all classes' loads in flight together) and a block works on one tile.
 //
 // Fast path (the usual case), class by class for all 16 pixels of a cell: inside a cell the interpolated logit is
 // u(r,k) = A + B k + G r + D k r, so its 16 exponentials are geometric progressions (cell_softmax.cuh).  Sweep 1 sums them per
@@ -34,9 +36,11 @@
 // Bound by latency and issue slots at 16 working warps an SM (half of the slots, 0.47 of the multiply-add pipe, a third of the
 // shared-memory path go to the sweeps); in a single wave the forward's 2.5 us lie in front.  One launch, us, with each block
 // fetching, multiplying and exchanging its tile through shared memory before the sweeps / now: 720p, 256 channels, 21 classes
-// 24.4 / 23.3, 16 streams of it 316 / 227 (the fetch and the products, 13000 of 33400 cycles a tile, run beside the sweeps of the
+// 23.4 / 21.1, 16 streams of it 316 / 227 (the fetch and the products, 13000 of 33400 cycles a tile, run beside the sweeps of the
 // tile before); 128 channels at 90 x 160 17.1 / 14.8; 32 classes, where one block fitted an SM, 39.8 / 29.6; 27 classes, 4 streams
-// 152 / 89.  Seven classes per iteration of sweep 1 instead of three: 232 -> 227.
+// 152 / 89.  Behind a 3x3 layer (720p, 256 channels; a forward kernel of its own and a loss kernel that exchanged the logits through
+// shared memory / now) 26.1 / 21.2, 1080p 57 / 46.  Stored logits: 21 classes at 720p 15.4 / 14.8, 30 classes (fp32) 26.1 / 19.1.
+// Seven classes per iteration of sweep 1 instead of three: 232 -> 227.
 #pragma once
 
 #include "st_internal.h"
@@ -44,6 +48,7 @@
 #include "fused_tile.cuh"
 #include "cell_softmax.cuh"
 
+#include <string.h>
 #include <utility>
 
 namespace st {
@@ -62,18 +67,18 @@ constexpr int kLogitCols = 4 * kClassPad;                                   // t
 // only (nobody has written there yet); the counts are cleared by the threads that read them.  Otherwise a block works on one tile
 // and both slots lie over its arrays.  The line is where two blocks no longer fit an SM with a slot to themselves (from 23
 // classes): 4 streams at 720p, 22 classes 68 us with the slot, 24 classes 83 us without.
-template <int C, bool CONF>
+template <int C, bool CONF, bool FORWARD>
 struct FwdCeSmem {
     static constexpr size_t kSlots = (size_t)F_WARPS * C * 32 * sizeof(float2), kCounts = (size_t)((C + 1) / 2) * kNodes * sizeof(uint32_t),
                             kHist = CONF ? (size_t)C * C * sizeof(unsigned int) : 0, kWeights = (size_t)fused::kMaxKBlocks * kWBytes,
                             kSlotsOrB = kSlots > kSliceBytes ? (kSlots + 1023) / 1024 * 1024 : kSliceBytes;
     static constexpr size_t kHalfSm = 115712 - 2048;    // what two blocks on an SM leave each, less the static arrays
-    static constexpr bool kPrefetch = kSliceBytes + kSlotsOrB + kWeights + kCounts + kHist + 1024 <= kHalfSm;
+    static constexpr bool kPrefetch = FORWARD && kSliceBytes + kSlotsOrB + kWeights + kCounts + kHist + 1024 <= kHalfSm;
     static constexpr size_t kArrays = kSlots + kCounts + kHist;
     static constexpr size_t kSlotsAt = kPrefetch ? kSliceBytes : 0, kSliceB = kSliceBytes,
                             kWeightsAt = kPrefetch ? kSliceBytes + kSlotsOrB : (kArrays > 2 * kSliceBytes ? (kArrays + 1023) / 1024 * 1024 : 2 * kSliceBytes),
                             kCountsAt = kPrefetch ? kWeightsAt + kWeights : kSlots, kHistAt = kCountsAt + kCounts,
-                            kEnd = kPrefetch ? kHistAt + kHist : kWeightsAt + kWeights, kBytes = kEnd + 1024;
+                            kEnd = !FORWARD ? kArrays : kPrefetch ? kHistAt + kHist : kWeightsAt + kWeights, kBytes = kEnd + 1024;
 };
 
 __device__ __forceinline__ float lg2_approx(float x)
@@ -135,11 +140,11 @@ __device__ __forceinline__ void add_counts(uint32_t* node, int cls, int right, i
     atomicAdd(w + below + right, br << sh);
 }
 
-template <int C, bool CONF>
-__global__ void __launch_bounds__(F_THREADS, 2)
+template <int C, bool CONF, bool FORWARD>
+__global__ void __launch_bounds__(FORWARD ? F_THREADS : F_WORKERS, 2)
 fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map)
 {
-    using Smem = FwdCeSmem<C, CONF>;
+    using Smem = FwdCeSmem<C, CONF, FORWARD>;
     extern __shared__ __align__(128) uint8_t smem_f[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_f + 1023) & ~(uintptr_t)1023);
     float2* slots = (float2*)(smem + Smem::kSlotsAt);                      // [F_WARPS][C][32]
@@ -165,27 +170,27 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
         return k;
     };
 
-    if (wi == F_WARPS) {
+    if (FORWARD && wi == F_WARPS) {
         if (tc::elect_one()) { tc::prefetch_map(&x_map); tc::prefetch_map(&w_map); }
         __syncwarp();
         tc::tmem_alloc(tc::smem_u32(&tmem_slot), kLogitCols);
     }
-    if (tid == 0) {
+    if (FORWARD && tid == 0) {
         for (int k = 0; k < 6; ++k) tc::mbar_init(bar0 + 8u * (uint32_t)k, 1);
         tc::mbar_init(taken_bar, F_WARPS);
         gave_up = 0;
         tc::fence_barrier_init();
     }
-    if (Smem::kPrefetch && wi < F_WARPS) {
+    if ((Smem::kPrefetch || !FORWARD) && wi < F_WARPS) {
         for (int e = tid; e < (int)(Smem::kCounts / 16); e += F_WORKERS) reinterpret_cast<uint4*>(counts)[e] = make_uint4(0, 0, 0, 0);
         if (CONF) for (int e = tid; e < C * C; e += F_WORKERS) hist[e] = 0;
     }
     tc::tc_fence_before_sync();
     __syncthreads();
     tc::tc_fence_after_sync();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = FORWARD ? tmem_slot : 0;
 
-    if (wi == F_WARPS) {
+    if (FORWARD && wi == F_WARPS) {
         // ---------------------------------------------------------------- the ninth warp: copies and multiplications
         const uint32_t ring = tc::smem_u32(smem), w_base = ring + (uint32_t)Smem::kWeightsAt;
         constexpr uint32_t idesc = tc::instr_desc(128, kClassPad, 0, 0);
@@ -301,12 +306,16 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
         }
         if (!waited) { pdl_wait(); waited = true; }        // the parameters come from the previous kernel of the stream
         if (a.skip && a.skip[(int64_t)s * a.skip_stride]) continue;
-        const float bias_l = l < C ? a.theta[(int64_t)s * a.n_params + a.b_off + l] : 0.f;
-        bool ok = tc::mbar_wait(done_bar, n_done & 1, a.err, tc::kWaitDone);
+        float bias_l = 0.f;
+        bool ok = true;
         ++n_done;
-        tc::tc_fence_after_sync();
-        if (gave_up) ok = false;
-        if (!Smem::kPrefetch) {                            // the slices are dead: the arrays under them get their initial contents
+        if constexpr (FORWARD) {
+            if (l < C) bias_l = a.theta[(int64_t)s * a.n_params + a.b_off + l];
+            ok = tc::mbar_wait(done_bar, (n_done - 1) & 1, a.err, tc::kWaitDone);
+            tc::tc_fence_after_sync();
+            if (gave_up) ok = false;
+        }
+        if (FORWARD && !Smem::kPrefetch) {                            // the slices are dead: the arrays under them get their initial contents
             if (!workers_all(ok)) return;                  // ... block-uniform
             for (int e = tid; e < (int)(Smem::kCounts / 16); e += F_WORKERS) reinterpret_cast<uint4*>(counts)[e] = make_uint4(0, 0, 0, 0);
             if (CONF) for (int e = tid; e < C * C; e += F_WORKERS) hist[e] = 0;
@@ -322,37 +331,41 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
         const bool own_cell = cell_row && cell_valid && t_row >= y0 && t_row < y0 + FN_Y && t_col >= x0 && t_col < x0 + FN_X;
         if (cell_row && ok) {                              // warp-uniform
             {
-                // ---- the warp's two node rows: tensor memory -> slots
-                bias[wi][l] = bias_l;
-                __syncwarp();
-                const uint32_t lanes = tmem + ((uint32_t)((wi & 3) * 32) << 16), upper = lanes + (wi >> 2) * kClassPad, lower = upper + 2 * kClassPad;
-                float up[32], lo[32];
-                if constexpr (C <= 16) {
-                    tc::tmem_ld_32x16(i == -1 ? lower : upper, reinterpret_cast<float(&)[16]>(up));
-                    tc::tmem_ld_32x16(i == h - 1 ? upper : lower, reinterpret_cast<float(&)[16]>(lo));
-                } else {
-                    tc::tmem_ld_32x32(i == -1 ? lower : upper, up);
-                    tc::tmem_ld_32x32(i == h - 1 ? upper : lower, lo);
-                }
-                tc::tc_fence_before_sync();
-                __syncwarp();
-                if (tc::elect_one()) arrive(taken_bar);
-                float m = -INFINITY;
-#pragma unroll
-                for (int c4 = 0; c4 < C; c4 += 4) {
-                    const float4 b4 = *reinterpret_cast<const float4*>(&bias[wi][c4]);
-                    const float b[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-                    for (int c = c4; c < c4 + 4 && c < C; ++c) {
-                        up[c] += b[c - c4]; lo[c] += b[c - c4];
-                        m = fmaxf(m, fmaxf(up[c], lo[c]));
-                    }
-                }
+                // ---- the warp's two node rows, upper and lower, clamped at the frame's border -> slots
                 const bool in_cols = n >= 0 && n < w;
+                float up[32], lo[32], m = -INFINITY;
+                if constexpr (FORWARD) {
+                    bias[wi][l] = bias_l;
+                    __syncwarp();
+                    const uint32_t lanes = tmem + ((uint32_t)((wi & 3) * 32) << 16), upper = lanes + (wi >> 2) * kClassPad, lower = upper + 2 * kClassPad;
+                    if constexpr (C <= 16) {
+                        tc::tmem_ld_32x16(i == -1 ? lower : upper, reinterpret_cast<float(&)[16]>(up));
+                        tc::tmem_ld_32x16(i == h - 1 ? upper : lower, reinterpret_cast<float(&)[16]>(lo));
+                    } else {
+                        tc::tmem_ld_32x32(i == -1 ? lower : upper, up);
+                        tc::tmem_ld_32x32(i == h - 1 ? upper : lower, lo);
+                    }
+                    tc::tc_fence_before_sync();
+                    __syncwarp();
+                    if (tc::elect_one()) arrive(taken_bar);
+#pragma unroll
+                    for (int c4 = 0; c4 < C; c4 += 4) {
+                        const float4 b4 = *reinterpret_cast<const float4*>(&bias[wi][c4]);
+                        const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                        for (int c = c4; c < c4 + 4 && c < C; ++c) { up[c] += b[c - c4]; lo[c] += b[c - c4]; }
+                    }
+                } else {
+                    const float *zu = a.z + (int64_t)s * C * p + (int64_t)max(i, 0) * w + n, *zl = a.z + (int64_t)s * C * p + (int64_t)min(i + 1, h - 1) * w + n;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) { up[c] = in_cols ? zu[(int64_t)c * p] : 0.f; lo[c] = in_cols ? zl[(int64_t)c * p] : 0.f; }
+                }
+#pragma unroll
+                for (int c = 0; c < C; ++c) m = fmaxf(m, fmaxf(up[c], lo[c]));
                 if (!in_cols) m = -INFINITY;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                if (a.z_out && wi >= 1 && node_owned) {    // the own nodes, where the caller wants the logits kept
+                if (FORWARD && a.z_out && wi >= 1 && node_owned) {    // the own nodes, where the caller wants the logits kept
                     float* zo = a.z_out + (int64_t)s * C * p + (int64_t)i * w + n;
 #pragma unroll
                     for (int c = 0; c < C; ++c) zo[(int64_t)c * p] = up[c];
@@ -596,7 +609,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
 #pragma unroll
                 for (int c = 0; c < C; ++c) my[c * 32] = pull[c];
             }
-        } else if (ok) {                                   // a warp below the frame has nothing to take, but says so
+        } else if (FORWARD && ok) {                        // a warp below the frame has nothing to take, but says so
             tc::tc_fence_before_sync();
             __syncwarp();
             if (tc::elect_one()) arrive(taken_bar);
@@ -672,25 +685,29 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
 template <int C>
 cudaError_t prepare_fwd_ce_as()
 {
-    cudaError_t e = allow_shared_memory((const void*)fwd_ce_kernel<C, false>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, true>);
+    cudaError_t e = allow_shared_memory((const void*)fwd_ce_kernel<C, false, true>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, true, true>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, false, false>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, true, false>);
     return e;
 }
 
-template <int C, bool CONF>
+template <int C, bool CONF, bool FORWARD>
 void launch_fwd_ce_as(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
 {
-    using Smem = FwdCeSmem<C, CONF>;
+    using Smem = FwdCeSmem<C, CONF, FORWARD>;
     const int tx = (a.w + FN_X - 1) / FN_X, ty = (a.h + FN_Y - 1) / FN_Y, tiles = tx * ty * a.S;
     const int grid = Smem::kPrefetch && tiles > 2 * a.n_sms ? 2 * a.n_sms : tiles;
-    launch_early(a.chain_early != 0 || a.x_early != 0, fwd_ce_kernel<C, CONF>, dim3(grid), dim3(F_THREADS), Smem::kBytes, s, a, tx, ty, x_map, w_map);
+    // (78 tiles behind a 3x3 layer of 64 channels, whose 115 blocks leave 33 SMs free: 44.2 us a step, spread 39.7)
+    const size_t smem = one_per_sm(Smem::kBytes, tiles, a.n_sms);
+    launch_early(a.chain_early != 0 || a.x_early != 0, fwd_ce_kernel<C, CONF, FORWARD>, dim3(grid), dim3(FORWARD ? F_THREADS : F_WORKERS), smem, s, a, tx, ty, x_map, w_map);
 }
 
-template <int C>
+template <int C, bool FORWARD>
 void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
 {
-    if (a.conf) launch_fwd_ce_as<C, true>(a, x_map, w_map, s);
-    else launch_fwd_ce_as<C, false>(a, x_map, w_map, s);
+    if (a.conf) launch_fwd_ce_as<C, true, FORWARD>(a, x_map, w_map, s);
+    else launch_fwd_ce_as<C, false, FORWARD>(a, x_map, w_map, s);
 }
 
 }  // namespace
@@ -698,14 +715,14 @@ void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const C
 // The kernels of one class count
 struct FwdCeKernels {
     cudaError_t (*prepare)();
-    void (*launch)(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s);
+    void (*launch[2])(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s);   // stored logits, own forward
 };
 
 // ... of class count `n`, one of FIRST + I...
 template <int FIRST, int... I>
 static FwdCeKernels fwd_ce_kernels_of(int n, std::integer_sequence<int, I...>)
 {
-    static const FwdCeKernels all[] = {{prepare_fwd_ce_as<FIRST + I>, launch_fwd_ce_of<FIRST + I>}...};
+    static const FwdCeKernels all[] = {{prepare_fwd_ce_as<FIRST + I>, {launch_fwd_ce_of<FIRST + I, false>, launch_fwd_ce_of<FIRST + I, true>}}...};
     return all[n - FIRST];
 }
 

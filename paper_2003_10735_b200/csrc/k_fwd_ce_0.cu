@@ -1,4 +1,4 @@
-// Class counts 2 to 12 of the forward + upsample + cross-entropy kernel.
+// Class counts 2 to 12 of the upsample + cross-entropy kernel for at most 32.
 #include "k_fwd_ce.cuh"
 
 namespace st {

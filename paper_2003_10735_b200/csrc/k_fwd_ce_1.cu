@@ -1,4 +1,4 @@
-// Class counts 13 to 18 of the forward + upsample + cross-entropy kernel.
+// Class counts 13 to 18 of the upsample + cross-entropy kernel for at most 32.
 #include "k_fwd_ce.cuh"
 
 namespace st {

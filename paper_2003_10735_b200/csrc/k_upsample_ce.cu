@@ -2,7 +2,7 @@
 // fused: bilinear x4 upsample of the head's low-resolution logits z to frame resolution, per-pixel softmax cross-entropy
 // against the one-byte labels, and the gradient of the mean loss with respect to z (the transpose of the upsample applied
 // to softmax - onehot), without ever writing a frame-resolution tensor.  Same geometry and arithmetic as the kernel for
-// fewer classes (k_upsample_ce_rows.cuh): warp = row of cells, lane = node column and the 4 x 4 frame pixels to its right,
+// fewer classes (k_fwd_ce.cuh): warp = row of cells, lane = node column and the 4 x 4 frame pixels to its right,
 // 16 exponentials of a class as products of four (cell_softmax.cuh), exact per-pixel maxima for cells whose logits are
 // steep, integer sums for the one-hot part.
 //
@@ -411,14 +411,14 @@ int upsample_ce_blocks(int h, int w, int C)
 
 cudaError_t prepare_upsample_ce(int C)
 {
-    if (upsample_ce_rows_supported(C)) return prepare_upsample_ce_rows(C);
+    if (upsample_ce_rows_supported(C)) return prepare_fwd_ce(C);
     const cudaError_t e = allow_many<7, 2>();
     return e != cudaSuccess ? e : allow_many<4, 3>();
 }
 
-void launch_upsample_ce(const UpsampleCeArgs& a, const CUtensorMap* z_map, cudaStream_t s)
+void launch_upsample_ce(const UpsampleCeArgs& a, cudaStream_t s)
 {
-    if (upsample_ce_rows_supported(a.C)) { launch_upsample_ce_rows(a, z_map, s); return; }
+    if (upsample_ce_rows_supported(a.C)) { launch_upsample_ce_rows(a, s); return; }
     if (many_shape(a.h, a.w).own_y == 7) launch_many<7, 2>(a, s);
     else launch_many<4, 3>(a, s);
 }

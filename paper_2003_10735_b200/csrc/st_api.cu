@@ -70,11 +70,10 @@ struct st_ctx {
     int n_split1 = 0, n_split2 = 0;
     float *loss_part = nullptr, *db_part = nullptr;
     int n_k3_blocks = 0;
-    CUtensorMap k3_map;        // tile map of z for the fused upsample + cross-entropy kernel
-    int k3_has_map = 0;
-    CUtensorMap fx_map, fw_map; // tile maps of the features and of the bf16 classifier weights: the loss kernel multiplies its own logits
+    CUtensorMap fx_map, fw_map; // tile maps of the classifier's input and of its bf16 weights: the loss kernel multiplies its own logits
     int n_sms = 0;
-    int fused_fwd = 0;          //   (one-layer head with bf16 GEMMs; ST_FUSED_FORWARD=0 switches it off)
+    int fused_loss = 0;         //   (bf16 GEMMs, the classifier's input of a shape fused_forward_supported names; ST_FUSED_FORWARD=0
+    int fused_fwd = 0;          //   switches it off); with a one-layer head the student-mask kernel does so too
     int test_stall_fused = 0;   // test of the give-up path inside that kernel (environment ST_TEST_STALL_FUSED=1 at context creation)
     float* loss_buf = nullptr;              // [S][kMaxSteps]
     unsigned long long* conf_buf = nullptr; // [S][kMaxSteps][C][C], allocated on first use
@@ -292,8 +291,9 @@ st_status enqueue_forward(st_ctx* c, StageTimer* t = nullptr, const int* skip = 
                           bool after_update = false, bool loss_follows = false)
 {
     cudaStream_t s = c->stream;
-    if (c->fused_fwd && loss_follows) return ST_OK;      // the loss kernel multiplies the logits itself (and writes them)
-    if (c->bf16_mode) {
+    if (c->fused_loss && loss_follows) {                 // the loss kernel multiplies the logits itself (and writes them)
+        c->launches += tc_forward_blocks(c->plan, c->first_trained < c->n_blocks ? c->first_trained : c->n_blocks, c->n_blocks, s, t, skip, skip_stride);
+    } else if (c->bf16_mode) {
         c->launches += tc_forward(c->plan, s, t, skip, skip_stride, after_update, c->first_trained < c->n_blocks ? c->first_trained : c->n_blocks);
     } else if (c->Ch == 0) {
         ST_REPEAT(t) launch_conv_fwd_f32(c->x_f32, c->Cin, c->h, c->w, c->theta + c->layout.w_off[0], c->theta + c->layout.b_off[0],
@@ -341,7 +341,6 @@ UpsampleCeArgs k3_args(st_ctx* c, bool fp32_grad, bool bf16_grad, unsigned long 
     k3.conf_stream_stride = (int64_t)kMaxSteps * c->C * c->C;
     k3.bad = c->bad; k3.err = c->bad + 2;
     k3.S = c->S; k3.C = c->C; k3.h = c->h; k3.w = c->w;
-    k3.has_map = c->k3_has_map;
     k3.skip = skip; k3.skip_stride = skip_stride;
     k3.chain_early = c->chain_early ? 1 : 0;
     k3.n_sms = c->n_sms; k3.x_early = 0; k3.kblocks = 0; k3.theta = nullptr; k3.n_params = 0; k3.b_off = 0; k3.z_out = nullptr; k3.test_stall = 0;
@@ -355,21 +354,22 @@ st_status enqueue_loss(st_ctx* c, unsigned long long* conf, StageTimer* t = null
 {
     cudaStream_t s = c->stream;
     UpsampleCeArgs k3 = k3_args(c, !c->bf16_mode, c->bf16_mode, conf, skip, skip_stride);
-    if (c->fused_fwd) {
-        // Forward as well: the features are frozen, so after a parameter update (which writes weights only) their tiles
-        // may be fetched while that update is still running
-        k3.x_early = after_update && !t ? 1 : 0; k3.kblocks = c->Cin / 64;
+    if (c->fused_loss) {
+        // The classifier's forward as well.  Where its input is frozen, its tiles may be fetched after a parameter update (which
+        // writes weights only) while that update is still running.
+        const bool frozen_input = c->first_trained >= c->n_blocks;
+        k3.x_early = frozen_input && after_update && !t ? 1 : 0; k3.kblocks = (c->Ch ? c->Ch : c->Cin) / 64;
         k3.theta = c->theta; k3.n_params = c->n_params; k3.b_off = c->layout.b_off[c->layout.n_layers - 1];
         k3.z_out = keep_logits ? c->z : nullptr;         // logits that the next iteration overwrites unread stay on the chip
         k3.test_stall = c->test_stall_fused;
         // the first iteration's predecessor may have written the labels and the features, which are fetched before the wait
-        if (!after_update) k3.chain_early = 0;
+        if (frozen_input && !after_update) k3.chain_early = 0;
     }
     ST_REPEAT(t) {
-        if (c->fused_fwd) launch_fwd_ce(k3, c->fx_map, c->fw_map, s);
-        else launch_upsample_ce(k3, &c->k3_map, s);
+        if (c->fused_loss) launch_fwd_ce(k3, c->fx_map, c->fw_map, s);
+        else launch_upsample_ce(k3, s);
     }
-    if (t) t->mark(c->fused_fwd ? "fwd1x1_upsample_ce" : "upsample_ce", s, st_repeats(t));
+    if (t) t->mark(c->fused_loss ? "fwd1x1_upsample_ce" : "upsample_ce", s, st_repeats(t));
     c->launches += st_repeats(t);
     return check_launch(c, "upsample + cross-entropy");
 }
@@ -745,7 +745,6 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     }
 #undef ALLOC
     if (e == cudaSuccess) e = prepare_upsample_ce(c->C);
-    if (e == cudaSuccess) c->k3_has_map = make_logit_tile_map(&c->k3_map, c->z, S, c->C, c->h, c->w) ? 1 : 0;
     if (e == cudaSuccess) e = prepare_student_mask();
     if (e == cudaSuccess && !c->bf16_mode) e = prepare_conv_f32();
     if (e != cudaSuccess) {
@@ -794,14 +793,14 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             return code;
         }
         const char* off = getenv("ST_FUSED_FORWARD");
-        if (n_blocks == 0 && !(off && off[0] == '0') && fused_forward_supported(c->C, c->h, c->w, c->Cin)) {
-            const uint64_t ci = (uint64_t)c->Cin;
+        if (!(off && off[0] == '0') && fused_forward_supported(c->C, c->h, c->w, c_last)) {
+            const uint64_t ci = (uint64_t)c_last;
             const uint64_t dims[3] = {ci, (uint64_t)kClassPad, (uint64_t)S}, str[2] = {ci * 2, (uint64_t)kClassPad * ci * 2};
             const uint32_t box[3] = {64, (uint32_t)kClassPad, 1};
-            c->fused_fwd = make_feature_tile_map(&c->fx_map, c->x_bf16, S, c->Cin, c->h, c->w) &&
-                           encode_tensor_map(&c->fw_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, c->w2_shadow, 3,
-                                             dims, str, box, msg, sizeof msg, "1x1 weight") &&
-                           prepare_student_eval() == cudaSuccess && prepare_fwd_ce(c->C) == cudaSuccess;
+            c->fused_loss = make_feature_tile_map(&c->fx_map, n_blocks ? c->blk[n_blocks - 1].out : c->x_bf16, S, c_last, c->h, c->w) &&
+                            encode_tensor_map(&c->fw_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, c->w2_shadow, 3,
+                                              dims, str, box, msg, sizeof msg, "1x1 weight");
+            c->fused_fwd = c->fused_loss && n_blocks == 0 && prepare_student_eval() == cudaSuccess;
             if (const char* ts = getenv("ST_TEST_STALL_FUSED")) c->test_stall_fused = ts[0] == '1' ? 1 : 0;
         }
     }
@@ -1008,7 +1007,7 @@ st_status enqueue_train(st_ctx* c, int max_updates)
     for (int i = 0; i <= max_updates && st == ST_OK; ++i) {
         const int* ended_before = i > 0 ? c->ctl_done + i : nullptr;        // done[s][i]: no prediction i for stream s
         st = enqueue_forward(c, nullptr, ended_before, kCtlPitch, false, true);           // prediction <- Forward(student, frame)
-        if (st == ST_OK) st = enqueue_loss(c, c->conf_buf + (int64_t)i * c->C * c->C, nullptr, ended_before, kCtlPitch, i > 0, false);   // loss, gradient, confusion
+        if (st == ST_OK) st = enqueue_loss(c, c->conf_buf + (int64_t)i * c->C * c->C, nullptr, ended_before, kCtlPitch, i > 0, !c->fused_fwd);   // loss, gradient, confusion
         // metric, best_student, break: assessed by an extra block of the backward's first tensor-core kernel while that
         // kernel works, or, where there is none (fp32 convolutions; the last prediction, after which every loop ends),
         // by the update itself, which in any case takes the step only where the loop goes on
@@ -1347,7 +1346,7 @@ st_status st_read_tensor(st_ctx* ctx, int32_t stream, st_tensor which, float* ds
         case ST_TENSOR_LOGITS: src = ctx->z + s * ctx->C * ctx->p; break;
         case ST_TENSOR_LOGIT_GRAD:
             if (ctx->bf16_mode) {     // the step wrote the bf16 copy only: same logits, same labels, same arithmetic once more
-                launch_upsample_ce(k3_args(ctx, true, false, nullptr), &ctx->k3_map, ctx->stream);
+                launch_upsample_ce(k3_args(ctx, true, false, nullptr), ctx->stream);
                 ctx->launches += 1;
             }
             src = ctx->bf16_mode ? ctx->dz + s * ctx->C * ctx->p : unpad(ctx->dz, ctx->C);

@@ -64,6 +64,15 @@ inline cudaError_t launch_early(bool early, void (*kernel)(KArgs...), dim3 grid,
     cfg.attrs = at; cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
+
+// Dynamic shared memory to ask for where every block of a launch can have an SM of its own: more than half of what an SM has.
+// Blocks that are launched early would otherwise pile up on the few SMs that the kernel before leaves first, and work there side
+// by side while other SMs idle.
+inline size_t one_per_sm(size_t smem, int64_t blocks, int n_sms)
+{
+    constexpr size_t more_than_half = 116 * 1024;
+    return blocks <= n_sms && smem < more_than_half ? more_than_half : smem;
+}
 #endif
 
 constexpr int kUp = 4;            // bilinear upsample factor of the head (frame = feature map * 4)
@@ -111,7 +120,6 @@ struct UpsampleCeArgs {
     unsigned int* err;       // device word: first wait that gave up (0 = none)
     int S, C, h, w;
     int n_sms;               // of the context's device
-    int has_map;             // the launch carries a tile map of z (see make_logit_tile_map)
     const int* skip;         // nullptr, or one flag per stream (skip[s * skip_stride]): non-zero = the stream's blocks return at once
     int64_t skip_stride;
     int heavy_w;             // 1, or the integer weight (2..5) of the pixels whose label byte has bit 7 set
@@ -125,18 +133,13 @@ struct UpsampleCeArgs {
     float* z_out;            // nullptr, or [S][C][h][w]: the logits are written here as well
     int test_stall;          // test of the give-up path: the first wait of the block's forward runs out (see tc_fwd1x1_kernel)
 };
-// Tile map of the logits for the row-walking kernel: fp32 tensor {w, h, S*C}, one box = the block's tile of all
-// classes.  False if the shape does not allow it (w not a multiple of 4, C > 32) or the driver entry point is
-// missing; the kernel then fetches its tile with plain loads.
-bool make_logit_tile_map(CUtensorMap* m, const float* z, int S, int C, int h, int w);
-// general form: any element type and swizzle; dims innermost first, strides (bytes) for dimensions 1..rank-1
+// Tensor map of any element type and swizzle; dims innermost first, strides (bytes) for dimensions 1..rank-1
 bool encode_tensor_map(CUtensorMap* m, CUtensorMapDataType dtype, CUtensorMapSwizzle swizzle, const void* base, int rank,
                        const uint64_t* dims, const uint64_t* strides, const uint32_t* box, char* err, size_t err_len,
                        const char* what);
 int upsample_ce_blocks(int h, int w, int C);   // blocks per stream (sizes loss_part / db_part)
 cudaError_t prepare_upsample_ce(int C);   // once per device and class count, outside any stream capture
-// z_map: host copy, used if a.has_map
-void launch_upsample_ce(const UpsampleCeArgs& a, const CUtensorMap* z_map, cudaStream_t s);
+void launch_upsample_ce(const UpsampleCeArgs& a, cudaStream_t s);
 // The same with the forward of a 1x1 classifier over bf16 features in front, in one kernel (k_fwd_ce.cuh), for the shapes that
 // fused_forward_supported names; host copies of the tile maps of the features and of the bf16 weights
 bool fused_forward_supported(int C, int h, int w, int c_in);
@@ -144,11 +147,10 @@ cudaError_t prepare_fwd_ce(int C);
 void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s);
 // Tile map of bf16 features [S][h][w][c_in] for it: {c_in, w, h, S}, one box = 64 channels of a tile
 bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w);
-// variant for C <= 32 (k_upsample_ce_rows.cuh); launch_upsample_ce dispatches to it
+// the part of launch_upsample_ce for C <= 32 (k_fwd_ce.cuh)
 bool upsample_ce_rows_supported(int C);
 int upsample_ce_rows_blocks(int h, int w);
-cudaError_t prepare_upsample_ce_rows(int C);
-void launch_upsample_ce_rows(const UpsampleCeArgs& a, const CUtensorMap* z_map, cudaStream_t s);
+void launch_upsample_ce_rows(const UpsampleCeArgs& a, cudaStream_t s);
 // student mask: argmax_c of the upsampled logits, uint8 [H][W]; with `labels` also the confusion matrix of
 // (label, mask) added into `conf`, and with `miou` the mean IoU written by the last block (k_student_mask.cu)
 struct StudentMaskArgs {
