@@ -35,10 +35,9 @@ constexpr int kTileW = 32, kTileH = 4;   // 3x3 forward: 128 pixels = 4 rows x 3
 constexpr int kChunkW = 32, kChunkH = 2; // 3x3 wgrad: 64 pixels = 2 rows x 32 columns
 constexpr int kSmemAlign = 1024;
 constexpr int kMaxKBlocks = 16;
-#ifndef ST_WG1_STAGES
-#define ST_WG1_STAGES 3
-#endif
-constexpr int kWg1Stages = ST_WG1_STAGES;   // pipeline depth of the 1x1 weight gradient (20 KB per stage at 128 channels per block)
+// Pipeline depth of the 1x1 weight gradient (20 KB per stage): three, which lets three blocks work on an SM, or five where every
+// block has an SM of its own
+constexpr int kWg1Stages = 3, kWg1Deep = 5;
 
 __device__ __forceinline__ uint8_t* align_smem(uint8_t* p)
 {
@@ -1112,7 +1111,7 @@ struct TcPlan {
     int tiles_b, per_b, split_b, groups_b;   // backward of the 1x1 layer behind a trained block: pixel tiles, tiles per range, ranges, channel groups
     int split1, chunks1, per1;          // pixel chunks of the 3x3 weight gradients (the same for every block)
     size_t smem_fwd1, smem_fwd1p, smem_wg1, smem_back1;
-    bool fwd1_persistent;
+    bool fwd1_persistent, wg1_deep;
     int n_sms;
     bool test_stall;         // test of the give-up path (environment ST_TEST_STALL_FWD1X1=1 when the plan is made)
 };
@@ -1263,7 +1262,15 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         if (P->smem_fwd1 > (size_t)227 * 1024) use = true;
         P->fwd1_persistent = use && P->smem_fwd1p <= (size_t)227 * 1024;
     }
-    P->smem_wg1 = kWg1Stages * ((size_t)(m_last / P->msplit2) * 2 * kChunkPix * 128 + kClassPad * 128) + kSmemAlign;
+    // Launched early behind a loss kernel that fills the GPU, the weight gradient's blocks start as SMs are left: one block per SM
+    // then keeps them from piling up on the first ones, and the room goes into the ring.  Where that kernel leaves SMs free (its
+    // tiles are fewer), they start there at once, in pairs, and all features of a block's three stages are there when the gradient
+    // is.  (Train: one more block per stream assesses the prediction.)  us of a call of eight steps, three stages / one block per SM with three, five, seven, ten: 256 channels 180 x 320
+    // 283.7 / 278.5, 275.6, 276.2, 279.7; 128 channels 270 x 480 470 / 453, 442, 455, 460; 90 x 160 (78 tiles) 156.9 / 160.8, 161.8.
+    const int64_t wg1_blocks = (int64_t)P->split2 * P->msplit2 * b.S;
+    P->wg1_deep = b.chain_early && wg1_blocks + b.S <= P->n_sms && (int64_t)upsample_ce_blocks(b.h, b.w, b.C) * b.S > P->n_sms;
+    P->smem_wg1 = (P->wg1_deep ? kWg1Deep : kWg1Stages) * ((size_t)(m_last / P->msplit2) * 2 * kChunkPix * 128 + kClassPad * 128) + kSmemAlign;
+    if (P->wg1_deep) P->smem_wg1 = one_per_sm(P->smem_wg1, wg1_blocks, P->n_sms);
     if (nb) {
         P->chunks1 = ((b.w + kChunkW - 1) / kChunkW) * ((b.h + kChunkH - 1) / kChunkH);
         split_geometry(P->chunks1, 148 / 9, &P->per1, &P->split1);
@@ -1277,7 +1284,7 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         delete P; return nullptr;
     }
     cudaError_t e = allow_shared_memory(P->fwd1_persistent ? (const void*)tc_fwd1x1p_kernel : (const void*)tc_fwd1x1_kernel);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)tc_wgrad1x1_kernel<kWg1Stages>);
+    if (e == cudaSuccess) e = P->wg1_deep ? allow_shared_memory((const void*)tc_wgrad1x1_kernel<kWg1Deep>) : allow_shared_memory((const void*)tc_wgrad1x1_kernel<kWg1Stages>);
     for (int i = 0; i < nb; ++i) {
         if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd3_kernel<0>(b.blk[i].c_out));
         if (e == cudaSuccess && b.blk[i].pass_back) e = allow_shared_memory((const void*)fwd3_kernel<1>(b.blk[i].c_prev));
@@ -1365,8 +1372,8 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
     if (!nb || !b.blk[nb - 1].trained) {                  // nothing is passed back into a frozen block (Section 4.2)
         // one-layer head: the activations are the frozen features, which no kernel of the loop writes
         const int a_early = (!nb && !skip && !t && b.chain_early) ? 1 : 0;
-        ST_REPEAT(t) launch_early(b.chain_early != 0, tc_wgrad1x1_kernel<kWg1Stages>, dim3(P->split2 * P->msplit2 + (ctl ? 1 : 0), b.S), dim3(kThreadsTc),
-            P->smem_wg1, s, P->act_wg, P->dz_map, b.w2_partials, P->c_last, P->chunks2, P->per2, P->msplit2, P->cols2, b.err, skip, skip_stride,
+        ST_REPEAT(t) launch_early(b.chain_early != 0, P->wg1_deep ? tc_wgrad1x1_kernel<kWg1Deep> : tc_wgrad1x1_kernel<kWg1Stages>,
+            dim3(P->split2 * P->msplit2 + (ctl ? 1 : 0), b.S), dim3(kThreadsTc), P->smem_wg1, s, P->act_wg, P->dz_map, b.w2_partials, P->c_last, P->chunks2, P->per2, P->msplit2, P->cols2, b.err, skip, skip_stride,
             a_early, ctl ? 1 : 0, ctl ? *ctl : no_ctl);
         if (t) t->mark("tc_wgrad1x1", s, st_repeats(t));
         return n + st_repeats(t);
