@@ -12,8 +12,8 @@
 // Pixel-major activations [pix][channel] are K-major operands when the GEMM reduces over channels
 // (forward) and MN-major operands when it reduces over pixels (weight gradients); both forms are
 // read straight from the same TMA 128-byte-swizzled tiles, no transposing pass exists.
-// The zero padding of the 3x3 convolution is TMA's out-of-bounds fill: taps are plain box loads at
-// shifted (x, y) coordinates of a [channel][x][y][stream] tensor map.
+// The zero padding of the 3x3 convolution is TMA's out-of-bounds fill: boxes reach beyond the map of a [channel][x][y][stream]
+// tensor map.
 #include "st_internal.h"
 #include "tc_common.cuh"
 #include "train_ctl.cuh"
@@ -31,7 +31,7 @@ constexpr int kThreadsTc = 128;          // 4 warps: TMEM lanes 32w .. 32w+31 be
 constexpr int kBlockK = 64;              // bf16 elements per 128-byte swizzled row
 constexpr int kTileM = 128;              // UMMA M
 constexpr int kChunkPix = 64;            // pixels per pipeline stage of the weight-gradient GEMMs
-constexpr int kTileW = 32, kTileH = 4;   // 3x3 forward: 128 pixels = 4 rows x 32 columns
+constexpr int kTileW = 8, kTileH = 16;   // 3x3 forward: 128 pixels = 16 rows x 8 columns
 constexpr int kChunkW = 32, kChunkH = 2; // 3x3 wgrad: 64 pixels = 2 rows x 32 columns
 constexpr int kSmemAlign = 1024;
 constexpr int kMaxKBlocks = 16;
@@ -279,13 +279,16 @@ tc_wgrad1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}      
 }
 
 // ------------------------------------------------------------------------------------------------
-// fwd 3x3 (+bias, ReLU), persistent: one block per SM walks the tiles (4 rows x 32 columns of pixels,
-// N = Ch output channels; K loop = 9 taps x Cin/64 channel blocks).  Three roles: warp 0 feeds a ring of
-// shared-memory stages by TMA across tile boundaries (the pipeline never drains), warp 1 issues the
-// MMAs into one of two tensor-memory accumulators, warps 2-5 drain the other accumulator (bias, ReLU,
-// bf16, ReLU bit mask) while the next tile is being multiplied.
+// fwd 3x3 (+bias, ReLU), persistent: one block per SM walks items of one or two tiles (HALVES; a tile is 16 rows x 8 columns of
+// pixels) times N output channels.  All nine taps read one slab of pixels: for 64 channels the 18 rows x (8 HALVES + 2) columns
+// around the item, one copy.  A tap's operand of 128 pixels is the slab from another start: eight pixels of a row are eight
+// consecutive 128-byte rows of the slab (the swizzle follows the address, so they may begin anywhere) and the next image row
+// begins one slab row further, which is the descriptor's stride between groups of eight.  Four roles: warp 0 feeds a ring of weight
+// stages (one tap of 64 channels each) and the last warp two slabs, by TMA across item boundaries (the pipeline never drains), a
+// thread of warp 1 issues the MMAs into one of two sets of tensor-memory accumulators, two groups of four warps drain the other set (bias, ReLU,
+// bf16, ReLU bit mask) meanwhile: a tile each, or every other 64 channels where an item is one tile.
 // ------------------------------------------------------------------------------------------------
-constexpr int kFwd3Threads = 192;
+constexpr int kFwd3Threads = 352;
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
@@ -304,6 +307,9 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 #endif
 constexpr int kF1Threads = 192, kF1Stages = ST_F1_STAGES;
 constexpr uint32_t kOutPieceBytes = 32 * 128;     // 3x3 tile walk: 32 pixels x 64 channels of an epilogue warp on their way out
+constexpr int kMaxWStages = 16;                   // ... weight stages of its ring
+__host__ __device__ constexpr int slab_cols(int halves) { return kTileW * halves + 2; }
+__host__ __device__ constexpr uint32_t slab_bytes(int halves) { return ((uint32_t)slab_cols(halves) * (kTileH + 2) * 128 + 1023) / 1024 * 1024; }
 constexpr uint32_t kF1StageBytes = kTileM * 128;
 
 __global__ void __launch_bounds__(kF1Threads)
@@ -424,62 +430,77 @@ tc_fwd1x1p_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}  box {
 }
 
 // MODE 0: the layer's forward (bias, ReLU, bf16 output, one ReLU bit per output value).
-// MODE 1: the gradient passed back through the layer to the block before it: the same tile walk over the layer's output
-//         gradient with the weights transposed and their taps mirrored (prepared by the update kernel); the epilogue
-//         applies the ReLU mask of the receiving block, writes bf16 and emits per-tile channel sums of the unrounded
-//         values (the receiving block's bias gradient).
-// The K loop runs over 9 taps x (kblocks1 + kblocks2) channel blocks: the first kblocks1 come from tmA (the previous
-// block's output, or the frozen part's), the others from tmA2 (the block's skip input): the concatenation of
-// Section 5.2 is never materialised.
-// Bound by the tensor pipe at 256 channels inside a tile (512 cycles per stage), by start, tile changes and the issue of copies
-// and MMAs at 64 and 128.  720p: 256 channels 50.2 us, 192 -> 64 31.6, 128 -> 64 29.1, gradient 64 -> 64 passed back 18.7.  With
-// 32-byte stores of every lane's own pixel row instead of pieces laid down in shared memory and stored by TMA 53.8, 33.6, 31.0
-// and 21.0 (the epilogue of a tile took 16000 to 24000 cycles, its multiplications 18400); with the issuing lane picked by
-// number 57.5, 42.5, 39.7, 24.1.  Not kept: one slab of pixels per horizontal shift for the three taps above each other (39, 35
-// us in the narrow layers), two units per stage (34, 29, 23), the next tile's pixels prefetched into L2 (55 us).
-template <int STAGES, int MODE>
+// MODE 1: the gradient passed back through the layer to the block before it: the same walk over the layer's output gradient with
+//         the weights transposed and their taps mirrored (prepared by the update kernel); the epilogue applies the ReLU mask of
+//         the receiving block, writes bf16 and emits per-tile channel sums of the unrounded values (the receiving block's bias
+//         gradient).
+// The K loop runs over (kblocks1 + kblocks2) channel blocks x 9 taps: the first kblocks1 come from tmA (the previous block's
+// output, or the frozen part's), the others from tmA2 (the block's skip input): the concatenation of Section 5.2 is never
+// materialised.
+// Bound by the tensor pipe at 256 channels inside a tile (560 cycles per weight stage where its multiplications need 512, 58 bytes a
+// cycle of weights from L2), by the issue of MMAs at 64 (450 to 540 per stage of eight, which read operands for 384), and by start
+// and tile changes.  us a launch, 720p, with a copy of the shifted pixels for every tap, tiles of 4 rows x 32 columns and a warp that
+// waits, votes and elects per stage / now: 128 + 64 -> 64 channels 29.5 / 25.2, 64 + 64 -> 64 26.4 / 19.2, gradient 64 -> 64 passed
+// back 16.0 / 13.5, 256 -> 128 35.7 / 30.3; three of 101 x 187, 192 -> 128 29.0 / 25.0; 256 -> 256 50.0 / 50.2 (180 rows are 11.25
+// tiles; fewer copies, more tiles), at 1080p 110 / 109.  The slab alone, without the issuing thread, changed nothing: eight MMAs with a
+// wait between them took 780 cycles; the slabs' own warp 1 us at 1080p; small rings of pieces 52.4 -> 50.2.
+template <int HALVES, int MODE>
 __global__ void __launch_bounds__(kFwd3Threads)
-tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}     box {64, 32, 4, 1}
-                 const __grid_constant__ CUtensorMap tmA2,  // {C2, w, h, S}     box {64, 32, 4, 1} (unused if kblocks2 == 0)
+tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}     box {64, 8 HALVES + 2, 18, 1}
+                 const __grid_constant__ CUtensorMap tmA2,  // {C2, w, h, S}     same box (unused if kblocks2 == 0)
                  int kblocks1, int kblocks2,
                  const __grid_constant__ CUtensorMap tmB,   // {C1+C2, 9*Ch, S}  box {64, Ch, 1}
                  const __grid_constant__ CUtensorMap tmBq,  // same tensor, box {64, 64, 1}: one block of 64 output channels
-                 int tail_split,                             // the tiles of the last, partly filled round are cut into this many
-                                                             // ranges of output channels (1, 2 or 4), one work item each
+                 int w_stages,                               // weight stages of the ring
+                 int n_full, int n_items, int tail_split,    // items: n_full whole ones, then the others cut into tail_split (1, 2 or
+                                                             // 4) ranges of output channels
                  const float* __restrict__ theta, int64_t n_params, int64_t b_off,   // MODE 0: bias
-                 const __grid_constant__ CUtensorMap tmO,   // output {Ch, w, h, S} box {64, 32, 1, 1}
+                 const __grid_constant__ CUtensorMap tmO,   // output {Ch, w, h, S} box {64, 8, 4, 1}
                  uint32_t* __restrict__ relu_bits,           // [S][p][Ch/32]: bit k of word j = out[32j + k] > 0 (MODE 0: written;
                                                              //   MODE 1: the receiving block's bits, read)
                  float* __restrict__ b_partials,             // MODE 1: [S][tiles per stream][Ch] channel sums of each tile
-                 int Ch, int h, int w, int n_tiles_total, int acc_cols, unsigned int* err, const int* __restrict__ skip, int64_t skip_stride)
+                 int Ch, int h, int w, int acc_cols, unsigned int* err, const int* __restrict__ skip, int64_t skip_stride)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_smem(smem_raw);
     const uint32_t base = smem_u32(smem);
-    const uint32_t a_bytes = kTileM * 128, b_bytes = (uint32_t)Ch * 128, stage_bytes = a_bytes + b_bytes;
-    __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2];
+    constexpr int P = slab_cols(HALVES);
+    constexpr uint32_t kSlab = slab_bytes(HALVES);
+    const uint32_t w_base = base + 2 * kSlab, w_bytes = (uint32_t)Ch * 128;
+    // The ring of weight stages, and the one it becomes for items that are a range of the output channels: smaller stages, more of
+    // them (with four stages the copies' latency, not the tensor pipe, sets the pace of such items).
+    const int p_stages = min(kMaxWStages, w_stages * tail_split);
+    const uint32_t p_bytes = w_bytes / (uint32_t)tail_split;
+    __shared__ __align__(8) uint64_t s_full[2], s_empty[2], full[2 * kMaxWStages], empty[2 * kMaxWStages], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_slot;
-    __shared__ __align__(16) float part[4 * 256];               // per epilogue warp: MODE 0 the bias, MODE 1 channel sums of the tile
+    __shared__ __align__(16) float part_of[8 * 256];            // per epilogue warp: MODE 0 the bias, MODE 1 channel sums of the tile
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int tiles_x = (w + kTileW - 1) / kTileW, tiles_y = (h + kTileH - 1) / kTileH;
-    const int tiles_per_stream = tiles_x * tiles_y;
-    const int kblocks = kblocks1 + kblocks2, n_stages = 9 * kblocks;
-    // Work items: whole tiles while every block has one, then the remaining tiles in tail_split pieces each, so that
-    // the last round is short instead of leaving most blocks idle for a full tile's time.
-    const int n_full = tail_split > 1 ? (n_tiles_total / (int)gridDim.x) * (int)gridDim.x : n_tiles_total;
-    const int n_items = n_full + (n_tiles_total - n_full) * tail_split;
-    struct Item { int tile, ch0, chn; };
+    const int items_x = (tiles_x + HALVES - 1) / HALVES, items_per_stream = items_x * tiles_y;
+    const int kblocks = kblocks1 + kblocks2;
+    struct Item { int s, tx, ty, ch0, chn; };
     auto item_of = [&](int wi) {
         Item it;
-        if (wi < n_full) { it.tile = wi; it.ch0 = 0; it.chn = Ch; }
-        else { const int q = wi - n_full; it.tile = n_full + q / tail_split; it.chn = Ch / tail_split; it.ch0 = (q % tail_split) * it.chn; }
+        int k = wi;
+        it.ch0 = 0; it.chn = Ch;
+        if (wi >= n_full) { const int q = wi - n_full; k = n_full + q / tail_split; it.chn = Ch / tail_split; it.ch0 = (q % tail_split) * it.chn; }
+        it.s = k / items_per_stream;
+        const int r = k - it.s * items_per_stream;
+        it.ty = r / items_x; it.tx = (r - it.ty * items_x) * HALVES;
         return it;
     };
 
-    if (warp == 0) tmem_alloc(smem_u32(&tmem_slot), 2 * acc_cols);
+    if (warp == 0) {
+        if (elect_one()) { prefetch_map(&tmA); prefetch_map(&tmB); }
+        __syncwarp();
+        tmem_alloc(smem_u32(&tmem_slot), acc_cols);
+    }
     if (tid == 0) {
-        for (int i = 0; i < STAGES; ++i) { mbar_init(smem_u32(&full[i]), 1); mbar_init(smem_u32(&empty[i]), 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&acc_full[i]), 1); mbar_init(smem_u32(&acc_empty[i]), 4); }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_u32(&s_full[i]), 1); mbar_init(smem_u32(&s_empty[i]), 1);
+            mbar_init(smem_u32(&acc_full[i]), 1); mbar_init(smem_u32(&acc_empty[i]), 8);
+        }
+        for (int i = 0; i < 2 * kMaxWStages; ++i) { mbar_init(smem_u32(&full[i]), 1); mbar_init(smem_u32(&empty[i]), 1); }
         fence_barrier_init();
     }
     tc_fence_before_sync();
@@ -490,85 +511,125 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
     bool ok = true;
 
     if (warp == 0) {
-        // ---- producer (the whole warp walks the loop, its first lane issues): the ring runs on across tiles
-        int st = 0;
+        // ---- weights (the whole warp walks the loop, its first lane issues)
+        int st = 0, n_st = w_stages;
         uint32_t parity = 1;             // a barrier nobody has arrived at yet counts as one whose phase 1 has ended
+        uint32_t f0 = smem_u32(&full[0]), e0 = smem_u32(&empty[0]);
+        bool pieces = false;
         for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
             const Item im = item_of(wi);
-            const int s = im.tile / tiles_per_stream, tt = im.tile % tiles_per_stream;
-            if (skip && skip[(int64_t)s * skip_stride]) continue;     // all three roles leave out the same items
-            const int x0 = (tt % tiles_x) * kTileW, y0 = (tt / tiles_x) * kTileH;
-            const uint32_t item_bytes = a_bytes + (uint32_t)im.chn * 128;
-            // One stage: wait for its slot, then the activation block (from `src`, whose tensor map is fixed at each of
-            // the two places this is expanded: a map chosen at run time costs every copy a slow look-up) and the weights.
-#define ST_FWD3_STAGE(src, a_coord)                                                                                       \
-            {                                                                                                             \
-                ok = mbar_wait(smem_u32(&empty[st]), parity, err, kWaitEmpty);                                            \
-                if (!ok) break;                                                                                           \
-                if (elect_one()) {                                                                                        \
-                    const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;                               \
-                    mbar_expect_tx(bar, item_bytes);                                                                      \
-                    tma_load_4d(sa, &(src), bar, (a_coord), x, y, s);                                                     \
-                    if (im.chn == Ch) tma_load_3d(sa + a_bytes, &tmB, bar, kb * kBlockK, row, s);                         \
-                    else                                                                                                  \
-                        for (int j = 0; j < im.chn / 64; ++j)    /* 64 weight rows per copy, laid out like the single copy */ \
-                            tma_load_3d(sa + a_bytes + j * (64 * 128), &tmBq, bar, kb * kBlockK, row + im.ch0 + j * 64, s); \
-                }                                                                                                         \
-                __syncwarp();                                                                                             \
-                if (++st == STAGES) { st = 0; parity ^= 1; }                                                              \
-            }
-            int row = 0;
-            for (int y = y0 - 1; y <= y0 + 1 && ok; ++y)
-                for (int x = x0 - 1; x <= x0 + 1 && ok; ++x, row += Ch) {
-                    int kb = 0;
-                    for (; kb < kblocks1; ++kb) ST_FWD3_STAGE(tmA, kb * kBlockK)
-                    for (; kb < kblocks && ok; ++kb) ST_FWD3_STAGE(tmA2, (kb - kblocks1) * kBlockK)
+            if (skip && skip[(int64_t)im.s * skip_stride]) continue;     // all roles leave out the same items
+            const uint32_t item_w = (uint32_t)im.chn * 128;
+            if (!pieces && im.chn != Ch) {                               // the other ring begins when all of the first one has been read
+                for (int i = 0; i < w_stages && ok; ++i) {
+                    ok = mbar_wait(e0 + 8 * st, parity, err, kWaitEmpty);
+                    if (++st == w_stages) { st = 0; parity ^= 1; }
                 }
-#undef ST_FWD3_STAGE
+                pieces = true;
+                st = 0; n_st = p_stages; parity = 1;
+                f0 += 8 * kMaxWStages; e0 += 8 * kMaxWStages;
+            }
+            for (int kb = 0; kb < kblocks && ok; ++kb)
+                for (int row = 0; row < 9 * Ch; row += Ch) {
+                    ok = mbar_wait(e0 + 8 * st, parity, err, kWaitEmpty);
+                    if (!ok) break;
+                    if (elect_one()) {
+                        const uint32_t bar = f0 + 8 * st, sw = w_base + st * item_w;
+                        mbar_expect_tx(bar, item_w);
+                        if (im.chn == Ch) tma_load_3d(sw, &tmB, bar, kb * kBlockK, row, im.s);
+                        else
+                            for (int j = 0; j < im.chn / 64; ++j)    // 64 weight rows per copy, laid out like the single copy
+                                tma_load_3d(sw + j * (64 * 128), &tmBq, bar, kb * kBlockK, row + im.ch0 + j * 64, im.s);
+                    }
+                    __syncwarp();
+                    if (++st == n_st) { st = 0; parity ^= 1; }
+                }
         }
         pdl_launch_dependents();     // every load is issued: the next kernel of the step may set itself up
-    } else if (warp == 1) {
-        // ---- MMA issuer
-        int st = 0, j = 0;
-        uint32_t parity = 0;
+    } else if (warp == kFwd3Threads / 32 - 1) {
+        // ---- slabs
+        int sl = 0;
+        uint32_t parity = 1;
         for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
             const Item im = item_of(wi);
-            if (skip && skip[(int64_t)(im.tile / tiles_per_stream) * skip_stride]) continue;
-            const uint32_t idesc = instr_desc(kTileM, im.chn, 0, 0);
-            const int buf = j & 1;
-            if (j >= 2) ok = mbar_wait(smem_u32(&acc_empty[buf]), ((j >> 1) - 1) & 1, err, kWaitEmpty);
-            if (!ok) break;
-            tc_fence_after_sync();
-            const uint32_t acc = tmem + buf * acc_cols;
-            for (int it = 0; it < n_stages; ++it) {
-                ok = mbar_wait(smem_u32(&full[st]), parity, err, kWaitFull);
+            if (skip && skip[(int64_t)im.s * skip_stride]) continue;
+            const int x = im.tx * kTileW - 1, y = im.ty * kTileH - 1;
+            for (int kb = 0; kb < kblocks; ++kb) {
+                ok = mbar_wait(smem_u32(&s_empty[sl]), parity, err, kWaitEmpty);
                 if (!ok) break;
-                tc_fence_after_sync();
                 if (elect_one()) {
-                    const uint64_t da = smem_desc(base + st * stage_bytes, 16, 1024), db = da + (a_bytes >> 4);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) umma(acc, da + 2 * k, db + 2 * k, idesc, (it | k) != 0);
-                    umma_commit(smem_u32(&empty[st]));
+                    const uint32_t bar = smem_u32(&s_full[sl]);
+                    mbar_expect_tx(bar, P * (kTileH + 2) * 128);
+                    if (kb < kblocks1) tma_load_4d(base + sl * kSlab, &tmA, bar, kb * kBlockK, x, y, im.s);
+                    else tma_load_4d(base + sl * kSlab, &tmA2, bar, (kb - kblocks1) * kBlockK, x, y, im.s);
                 }
                 __syncwarp();
-                if (++st == STAGES) { st = 0; parity ^= 1; }
+                sl ^= 1; parity ^= sl == 0;
             }
-            if (ok && elect_one()) umma_commit(smem_u32(&acc_full[buf]));
-            __syncwarp();
-            ++j;                                                       // j counts the tiles this block works on
         }
+    } else if (warp == 1) {
+        // ---- MMA issuer: one thread
+        if (elect_one()) {
+            int st = 0, sl = 0, j = 0;
+            uint32_t parity = 0, sl_parity = 0;
+            uint32_t f0 = smem_u32(&full[0]), e0 = smem_u32(&empty[0]), w_step = w_bytes >> 4;
+            int n_st = w_stages;
+            bool pieces = false;
+            const uint64_t a0 = smem_desc(base, 16, P * 128), b0 = smem_desc(w_base, 16, 1024);
+            bool ready = false;                                        // what the look at stage `st` has said
+            for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
+                if (skip && skip[(int64_t)((wi < n_full ? wi : n_full + (wi - n_full) / tail_split) / items_per_stream) * skip_stride]) continue;
+                const uint32_t idesc = instr_desc(kTileM, wi < n_full ? Ch : Ch / tail_split, 0, 0);
+                if (!pieces && tail_split > 1 && wi >= n_full) {
+                    pieces = true;
+                    st = 0; n_st = p_stages; parity = 0; ready = false;
+                    f0 += 8 * kMaxWStages; e0 += 8 * kMaxWStages; w_step = p_bytes >> 4;
+                }
+                const int buf = j & 1;
+                if (j >= 2) ok = mbar_wait_from(false, smem_u32(&acc_empty[buf]), ((j >> 1) - 1) & 1, err, kWaitEmpty);
+                const uint32_t acc = tmem + buf * HALVES * Ch;
+                for (int kb = 0; kb < kblocks && ok; ++kb) {
+                    ok = mbar_wait_from(false, smem_u32(&s_full[sl]), sl_parity, err, kWaitFull);
+                    const uint64_t as = a0 + sl * (kSlab >> 4);
+#pragma unroll
+                    for (int tap = 0; tap < 9; ++tap) {
+                        if (ok) ok = mbar_wait_from(ready, f0 + 8 * st, parity, err, kWaitFull);
+                        const int now = st;
+                        if (++st == n_st) { st = 0; parity ^= 1; }
+                        ready = mbar_try_wait(f0 + 8 * st, parity);
+                        if (ok) {
+                            tc_fence_after_sync();
+                            const uint64_t da = as + ((tap / 3 * P + tap % 3) * 128 >> 4), db = b0 + now * w_step;
+#pragma unroll
+                            for (int hf = 0; hf < HALVES; ++hf)
+#pragma unroll
+                                for (int k = 0; k < 4; ++k)
+                                    umma(acc + hf * Ch, da + hf * (kTileW * 128 >> 4) + 2 * k, db + 2 * k, idesc, (kb | tap | k) != 0);
+                            umma_commit(e0 + 8 * now);
+                        }
+                    }
+                    if (ok) umma_commit(smem_u32(&s_empty[sl]));
+                    sl ^= 1; sl_parity ^= sl == 0;
+                }
+                if (ok) umma_commit(smem_u32(&acc_full[buf]));
+                ++j;                                                   // j counts the items this block works on
+            }
+        }
+        ok = __all_sync(0xffffffffu, ok);
     } else if (warp >= 2) {
-        // ---- epilogue warps: TMEM lanes 32*(warp % 4) .. +31 = pixel rows of the tile
-        // (a warp's 32 pixels are one row of the tile)
-        const int q = warp & 3, row = q * 32 + lane;
-        const uint32_t piece = base + STAGES * stage_bytes + q * kOutPieceBytes, orow = piece + lane * 128;
-        int j = 0;
+        // ---- epilogue warps: TMEM lanes 32*(warp % 4) .. +31 = four rows of eight pixels of a tile
+        const int q = warp & 3, set = (warp - 2) >> 2;
+        const uint32_t piece = w_base + w_stages * w_bytes + (warp - 2) * kOutPieceBytes, orow = piece + lane * 128;
+        float* part = part_of + set * 4 * 256;
+        int j = -1;
         for (int wi = blockIdx.x; wi < n_items && ok; wi += gridDim.x) {
             const Item im = item_of(wi);
-            const int s = im.tile / tiles_per_stream, tt = im.tile % tiles_per_stream;
+            const int s = im.s;
             if (skip && skip[(int64_t)s * skip_stride]) continue;
-            const int buf = j & 1;
-            const int x = (tt % tiles_x) * kTileW + row % kTileW, y = (tt / tiles_x) * kTileH + row / kTileW;
+            ++j;
+            const int hf = HALVES == 1 ? 0 : set, first = HALVES == 1 ? set * 64 : 0;
+            constexpr int kStep = HALVES == 1 ? 128 : 64;              // this group's channels: `first`, + kStep, ... 64 at a time
+            const int buf = j & 1, y = im.ty * kTileH + q * 4 + (lane >> 3);
             if (MODE == 0) {
                 const float* bias = theta + (int64_t)s * n_params + b_off + im.ch0;
                 for (int c = lane; c < im.chn; c += 32) part[q * 256 + c] = __ldg(bias + c);
@@ -577,94 +638,97 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
             ok = mbar_wait(smem_u32(&acc_full[buf]), (j >> 1) & 1, err, kWaitDone);
             if (MODE == 1) {                                           // the four epilogue warps stay together: they share `part`
                 int all_ok;
-                asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, 1, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-                             : "=r"(all_ok) : "r"((int)ok) : "memory");
+                asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, %2, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                             : "=r"(all_ok) : "r"((int)ok), "r"(1 + set) : "memory");
                 ok = all_ok != 0;
             }
             if (!ok) break;
             tc_fence_after_sync();
-            const bool in = y < h && x < w;
-            const int64_t pixel = (int64_t)s * h * w + (int64_t)y * w + x;
-            for (int n0 = 0; n0 < im.chn; n0 += 64) {
-                uint32_t words[2] = {0, 0};                            // ReLU bits
-                if (MODE == 1 && in) {
-                    const uint2 b = __ldg(reinterpret_cast<const uint2*>(relu_bits + pixel * (Ch / 32) + (im.ch0 + n0) / 32));
-                    words[0] = b.x; words[1] = b.y;                    // ... none where the tile reaches beyond the frame
-                }
-#pragma unroll
-                for (int g = 0; g < 2; ++g) {
-                    float v[32];
-                    tmem_ld_32x32(tmem + ((uint32_t)(q * 32) << 16) + buf * acc_cols + n0 + g * 32, v);
-                    uint32_t o[16];
-                    if (MODE == 0) {
-                        const float4* b4 = reinterpret_cast<const float4*>(part + q * 256 + n0 + g * 32);
-#pragma unroll
-                        for (int k = 0; k < 16; ++k) {
-                            const float4 b = b4[k >> 1];
-                            const float x0f = fmaxf(v[2 * k] + ((k & 1) ? b.z : b.x), 0.f), x1f = fmaxf(v[2 * k + 1] + ((k & 1) ? b.w : b.y), 0.f);
-                            const __nv_bfloat162 two = __floats2bfloat162_rn(x0f, x1f);
-                            o[k] = *reinterpret_cast<const uint32_t*>(&two);
-                            // the mask is taken on the stored (rounded) activation, the value the next layer sees
-                            words[g] |= (__low2float(two) > 0.f ? 1u : 0u) << (2 * k);
-                            words[g] |= (__high2float(two) > 0.f ? 1u : 0u) << (2 * k + 1);
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 16; ++k) {
-                            if (!((words[g] >> (2 * k)) & 1u)) v[2 * k] = 0.f;
-                            if (!((words[g] >> (2 * k + 1)) & 1u)) v[2 * k + 1] = 0.f;
-                            const __nv_bfloat162 two = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
-                            o[k] = *reinterpret_cast<const uint32_t*>(&two);
-                        }
-                    }
-                    if (g == 0) {
-                        if (lane == 0) tma_store_wait_read<0>();       // the piece that was here before has been read
-                        __syncwarp();
+            {
+                const int x = (im.tx + hf) * kTileW + (lane & 7);
+                const bool in = y < h && x < w;
+                const int64_t pixel = (int64_t)s * h * w + (int64_t)y * w + x;
+                for (int n0 = first; n0 < im.chn; n0 += kStep) {
+                    uint32_t words[2] = {0, 0};                        // ReLU bits
+                    if (MODE == 1 && in) {
+                        const uint2 b = __ldg(reinterpret_cast<const uint2*>(relu_bits + pixel * (Ch / 32) + (im.ch0 + n0) / 32));
+                        words[0] = b.x; words[1] = b.y;                // ... none where the tile reaches beyond the frame
                     }
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)                        // 128-byte swizzle: 16-byte chunks ^ (row % 8)
-                        st_shared_128(orow + (((g * 4 + k) ^ (lane & 7)) << 4), o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
-                    if (MODE == 1) {
-                        // sums over the warp's 32 pixels in a fixed order: a reduce-scatter over the lanes, after which lane c
-                        // holds the sum of channel c of the group
+                    for (int g = 0; g < 2; ++g) {
+                        float v[32];
+                        tmem_ld_32x32(tmem + ((uint32_t)(q * 32) << 16) + (buf * HALVES + hf) * Ch + n0 + g * 32, v);
+                        uint32_t o[16];
+                        if (MODE == 0) {
+                            const float4* b4 = reinterpret_cast<const float4*>(part + q * 256 + n0 + g * 32);
 #pragma unroll
-                        for (int half = 16; half >= 1; half >>= 1) {
-                            const bool up = (lane & half) != 0;
+                            for (int k = 0; k < 16; ++k) {
+                                const float4 b = b4[k >> 1];
+                                const float x0f = fmaxf(v[2 * k] + ((k & 1) ? b.z : b.x), 0.f), x1f = fmaxf(v[2 * k + 1] + ((k & 1) ? b.w : b.y), 0.f);
+                                const __nv_bfloat162 two = __floats2bfloat162_rn(x0f, x1f);
+                                o[k] = *reinterpret_cast<const uint32_t*>(&two);
+                                // the mask is taken on the stored (rounded) activation, the value the next layer sees
+                                words[g] |= (__low2float(two) > 0.f ? 1u : 0u) << (2 * k);
+                                words[g] |= (__high2float(two) > 0.f ? 1u : 0u) << (2 * k + 1);
+                            }
+                        } else {
 #pragma unroll
-                            for (int k = 0; k < half; ++k) {
-                                const float keep = up ? v[k + half] : v[k];
-                                const float send = up ? v[k] : v[k + half];
-                                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+                            for (int k = 0; k < 16; ++k) {
+                                if (!((words[g] >> (2 * k)) & 1u)) v[2 * k] = 0.f;
+                                if (!((words[g] >> (2 * k + 1)) & 1u)) v[2 * k + 1] = 0.f;
+                                const __nv_bfloat162 two = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+                                o[k] = *reinterpret_cast<const uint32_t*>(&two);
                             }
                         }
-                        part[q * 256 + n0 + g * 32 + lane] = v[0];
+                        if (g == 0) {
+                            if (lane == 0) tma_store_wait_read<0>();   // the piece that was here before has been read
+                            __syncwarp();
+                        }
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)                    // 128-byte swizzle: 16-byte chunks ^ (row % 8)
+                            st_shared_128(orow + (((g * 4 + k) ^ (lane & 7)) << 4), o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+                        if (MODE == 1) {
+                            // sums over the warp's 32 pixels in a fixed order: a reduce-scatter over the lanes, after which lane c
+                            // holds the sum of channel c of the group
+#pragma unroll
+                            for (int half = 16; half >= 1; half >>= 1) {
+                                const bool up = (lane & half) != 0;
+#pragma unroll
+                                for (int k = 0; k < half; ++k) {
+                                    const float keep = up ? v[k + half] : v[k];
+                                    const float send = up ? v[k] : v[k + half];
+                                    v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+                                }
+                            }
+                            part[q * 256 + n0 + g * 32 + lane] = v[0];
+                        }
                     }
+                    if (MODE == 0 && in)
+                        *reinterpret_cast<uint2*>(relu_bits + pixel * (Ch / 32) + (im.ch0 + n0) / 32) = make_uint2(words[0], words[1]);
+                    fence_async_shared();
+                    __syncwarp();
+                    if (lane == 0 && in) { tma_store_4d(&tmO, piece, im.ch0 + n0, x, y, s); tma_store_commit(); }
                 }
-                if (MODE == 0 && in)
-                    *reinterpret_cast<uint2*>(relu_bits + pixel * (Ch / 32) + (im.ch0 + n0) / 32) = make_uint2(words[0], words[1]);
-                fence_async_shared();
+                tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0 && y < h) { tma_store_4d(&tmO, piece, im.ch0 + n0, x, y, s); tma_store_commit(); }
+                if (lane == 0) mbar_arrive(smem_u32(&acc_empty[buf])); // this warp's quarter of the accumulator is free
+                if (MODE == 1) {
+                    asm volatile("barrier.cta.sync %0, 128;" ::"r"(1 + set) : "memory");
+                    const int e = ((warp - 2) & 3) * 32 + lane;        // 0..127 over the group's four warps
+                    if (im.tx + hf < tiles_x)
+                        for (int k = e; k < im.chn; k += 128)
+                            if (HALVES == 2 || ((k >> 6) & 1) == set) b_partials[((int64_t)s * tiles_x * tiles_y + im.ty * tiles_x + im.tx + hf) * Ch + im.ch0 + k] =
+                                (part[k] + part[256 + k]) + (part[512 + k] + part[768 + k]);
+                    asm volatile("barrier.cta.sync %0, 128;" ::"r"(1 + set) : "memory");
+                }
             }
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[buf]));     // this warp's quarter of the accumulator is free
-            if (MODE == 1) {
-                asm volatile("barrier.cta.sync 1, 128;" ::: "memory");
-                const int e = (warp - 2) * 32 + lane;                  // 0..127 over the four epilogue warps
-                for (int k = e; k < im.chn; k += 128)
-                    b_partials[((int64_t)s * tiles_per_stream + tt) * Ch + im.ch0 + k] =
-                        (part[k] + part[256 + k]) + (part[512 + k] + part[768 + k]);
-                asm volatile("barrier.cta.sync 1, 128;" ::: "memory");
-            }
-            ++j;
         }
         if (lane == 0) tma_store_wait();
     }
     if (!ok) drain_after_error();
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 2 * acc_cols);
+    if (warp == 0) tmem_dealloc(tmem, acc_cols);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1056,16 +1120,50 @@ bool encode_tensor_map(CUtensorMap* m, CUtensorMapDataType dtype, CUtensorMapSwi
     return true;
 }
 
-// Pipeline depth of the 3x3 tile walk: as many stages as fit beside the epilogue's pieces (a stage of a narrow layer is small,
-// and with only four of them in flight the copies' latency, not the tensor pipe, sets the pace).
-static int fwd3_stages(int n_out) { return n_out <= 64 ? 8 : (n_out <= 128 ? 6 : 4); }
-static size_t fwd3_bytes(int n_out) { return (size_t)fwd3_stages(n_out) * (kTileM + n_out) * 128 + 4 * kOutPieceBytes + kSmemAlign; }
-template <int MODE>
-static decltype(&tc_fwd3x3_kernel<4, MODE>) fwd3_kernel(int n_out)
+// Weight stages of the 3x3 tile walk: what fits beside two slabs and the epilogue's pieces
+static int fwd3_stages(int n_out, int halves)
 {
-    const int n = fwd3_stages(n_out);
-    return n == 8 ? tc_fwd3x3_kernel<8, MODE> : (n == 6 ? tc_fwd3x3_kernel<6, MODE> : tc_fwd3x3_kernel<4, MODE>);
+    const int n = (int)((218 * 1024 - 2 * (int)slab_bytes(halves) - 8 * (int)kOutPieceBytes - kSmemAlign) / (n_out * 128));
+    return n < kMaxWStages ? n : kMaxWStages;
 }
+static size_t fwd3_bytes(int n_out, int halves)
+{
+    return 2 * (size_t)slab_bytes(halves) + (size_t)fwd3_stages(n_out, halves) * n_out * 128 + 8 * kOutPieceBytes + kSmemAlign;
+}
+// How a launch walks the map: tiles per item, items, blocks, and into how many ranges of output channels (multiples of 64) the
+// items of a partly filled last round are cut, where that lets every piece have its own block.
+struct Fwd3Walk { int halves, n_full, n_items, tail_split, grid; };
+static Fwd3Walk fwd3_walk(int h, int w, int S, int n_out, int n_sms)
+{
+    const int tiles_x = (w + kTileW - 1) / kTileW, tiles_y = (h + kTileH - 1) / kTileH;
+    // Two tiles to an item share the weight stages.  What an item of 64 input channels costs, in cycles: its shared-memory bytes at
+    // 128 a cycle (36 MMAs per tile read 4 KB of pixels and 32 bytes per output channel each; slab and weights are written
+    // once), or its multiplications at N / 2 cycles an MMA.  The accumulators of two tiles fit twice up to 128 channels.
+    auto cost = [&](int halves) {
+        const int64_t items = (int64_t)((tiles_x + halves - 1) / halves) * tiles_y * S, rounds = (items + n_sms - 1) / n_sms;
+        const int64_t bytes = (int64_t)halves * 36 * (4096 + n_out * 32) + slab_bytes(halves) + 9 * n_out * 128, math = (int64_t)halves * 36 * n_out / 2;
+        return rounds * (bytes / 128 > math ? bytes / 128 : math);
+    };
+    Fwd3Walk q;
+    q.halves = n_out <= 128 && cost(2) < cost(1) ? 2 : 1;
+    const int items = (tiles_x + q.halves - 1) / q.halves * tiles_y * S;
+    q.grid = items < n_sms ? items : n_sms;
+    q.tail_split = 1;
+    const int tail = items % q.grid;
+    if (tail > 0) {
+        if (n_out % 256 == 0 && tail * 4 <= q.grid) q.tail_split = 4;
+        else if (n_out % 128 == 0 && tail * 2 <= q.grid) q.tail_split = 2;
+    } else if (items < n_sms) {                          // a small map: every item is cut
+        if (n_out % 256 == 0 && items * 4 <= n_sms) q.tail_split = 4;
+        else if (n_out % 128 == 0 && items * 2 <= n_sms) q.tail_split = 2;
+        q.grid = items * q.tail_split;
+    }
+    q.n_full = q.tail_split > 1 ? items / q.grid * q.grid : items;
+    q.n_items = q.n_full + (items - q.n_full) * q.tail_split;
+    return q;
+}
+template <int MODE>
+static decltype(&tc_fwd3x3_kernel<1, MODE>) fwd3_kernel(const Fwd3Walk& q) { return q.halves == 2 ? tc_fwd3x3_kernel<2, MODE> : tc_fwd3x3_kernel<1, MODE>; }
 // The stages of the weight gradient: two chunks of pixels each if three such stages fit (for the same reason), else one; as
 // many as fit in about 208 KB, five at most.
 struct Wg3Ring { int stages, chunks; size_t bytes; };
@@ -1086,15 +1184,16 @@ static decltype(&tc_wgrad3x3_kernel<3, 1>) wgrad3_kernel(const Wg3Ring& g)
 }
 
 struct TcBlockPlan {
-    CUtensorMap in_fwd, skip_fwd;    // the block's two inputs {C, w, h, S}, box {64, 32, 4, 1} (forward tiles)
+    CUtensorMap in_fwd, skip_fwd;    // the block's two inputs {C, w, h, S}, box {64, 8 halves + 2, 18, 1} (forward slabs)
     CUtensorMap in_wg, skip_wg;      // same tensors, box {64, 32, 2, 1} (weight-gradient chunks)
     CUtensorMap w_map, w_map_q;      // {c_tot, 9*c_out, S}, boxes {64, c_out, 1} and {64, 64, 1}
     CUtensorMap wt_map, wt_map_q;    // mirrored, transposed weights {c_out, 9*c_prev, S}, boxes {64, c_prev, 1} and {64, 64, 1}
-    CUtensorMap dout_fwd;            // the block's output gradient {c_out, w, h, S}, box {64, 32, 4, 1} (A operand when passed back)
-    CUtensorMap out_st, dprev_st;    // the block's output and its first input's gradient {C, w, h, S}, box {64, 32, 1, 1} (stores)
+    CUtensorMap dout_fwd;            // the block's output gradient {c_out, w, h, S}, the slab's box (A operand when passed back)
+    CUtensorMap out_st, dprev_st;    // the block's output and its first input's gradient {C, w, h, S}, box {64, 8, 4, 1} (stores)
     CUtensorMap dout_wg;             // same tensor, box {64, 32, 2, 1} (B operand of the weight gradient)
     int cols_wg;                     // tensor-memory columns of the weight gradient
     Wg3Ring wg;
+    Fwd3Walk walk_fwd, walk_back;
     size_t smem_fwd, smem_back;
 };
 
@@ -1185,8 +1284,10 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         TcBlockPlan& q = P->blk[i];
         const uint64_t w = (uint64_t)b.w, h = (uint64_t)b.h, c1 = (uint64_t)k.c_prev, c2 = (uint64_t)k.c_skip, co = (uint64_t)k.c_out,
                        ct = c1 + c2;
-        const uint32_t bf[4] = {64, (uint32_t)kTileW, (uint32_t)kTileH, 1};
-        auto act_maps = [&](const bf16* base, uint64_t c, CUtensorMap* fwd, CUtensorMap* wg, const char* what) {
+        q.walk_fwd = fwd3_walk(b.h, b.w, b.S, k.c_out, P->n_sms);
+        q.walk_back = fwd3_walk(b.h, b.w, b.S, k.c_prev, P->n_sms);
+        auto act_maps = [&](const bf16* base, uint64_t c, int halves, CUtensorMap* fwd, CUtensorMap* wg, const char* what) {
+            const uint32_t bf[4] = {64, (uint32_t)slab_cols(halves), (uint32_t)kTileH + 2, 1};
             uint64_t d[4] = {c, w, h, S}, st[3] = {c * 2, w * c * 2, h * w * c * 2};
             // all channels of a chunk in one copy: one block of 64 behind the other
             uint64_t d5[5] = {64, w, h, c / 64, S}, st5[4] = {c * 2, w * c * 2, 128, h * w * c * 2};
@@ -1196,10 +1297,10 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
             if (wg) r = r && make_map(wg, base, 5, d5, st5, bw, err, err_len, what);
             return r;
         };
-        ok = ok && act_maps(k.in_prev, c1, &q.in_fwd, &q.in_wg, "block input");
-        if (c2) ok = ok && act_maps(k.in_skip, c2, &q.skip_fwd, &q.skip_wg, "skip input");
+        ok = ok && act_maps(k.in_prev, c1, q.walk_fwd.halves, &q.in_fwd, &q.in_wg, "block input");
+        if (c2) ok = ok && act_maps(k.in_skip, c2, q.walk_fwd.halves, &q.skip_fwd, &q.skip_wg, "skip input");
         else { q.skip_fwd = q.in_fwd; q.skip_wg = q.in_wg; }
-        ok = ok && act_maps(k.dout, co, &q.dout_fwd, &q.dout_wg, "block output gradient");
+        ok = ok && act_maps(k.dout, co, q.walk_back.halves, &q.dout_fwd, &q.dout_wg, "block output gradient");
         {
             uint64_t dw[3] = {ct, 9 * co, S}, sw[2] = {ct * 2, 9 * co * ct * 2};
             uint32_t bwt[3] = {64, (uint32_t)co, 1}, bwq[3] = {64, 64, 1};
@@ -1208,7 +1309,7 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         }
         auto store_map = [&](const bf16* base, uint64_t c, CUtensorMap* m, const char* what) {
             uint64_t d[4] = {c, w, h, S}, st[3] = {c * 2, w * c * 2, h * w * c * 2};
-            uint32_t bo[4] = {64, (uint32_t)kTileW, 1, 1};
+            uint32_t bo[4] = {64, (uint32_t)kTileW, 4, 1};
             return make_map(m, base, 4, d, st, bo, err, err_len, what);
         };
         ok = ok && store_map(k.out, co, &q.out_st, "block output (stores)");
@@ -1222,8 +1323,8 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         const int m_in = ((int)ct + kTileM - 1) / kTileM;
         q.cols_wg = pow2_cols(m_in * k.c_out);
         q.wg = wg3_ring((int)ct, k.c_out);
-        q.smem_fwd = fwd3_bytes(k.c_out);
-        q.smem_back = fwd3_bytes(k.c_prev);
+        q.smem_fwd = fwd3_bytes(k.c_out, q.walk_fwd.halves);
+        q.smem_back = fwd3_bytes(k.c_prev, q.walk_back.halves);
         if (ok && q.cols_wg > 512) {
             snprintf(err, err_len, "a block with %d input and %d output channels needs %d TMEM columns (> 512)", (int)ct, k.c_out, q.cols_wg);
             ok = false;
@@ -1286,8 +1387,8 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
     cudaError_t e = allow_shared_memory(P->fwd1_persistent ? (const void*)tc_fwd1x1p_kernel : (const void*)tc_fwd1x1_kernel);
     if (e == cudaSuccess) e = P->wg1_deep ? allow_shared_memory((const void*)tc_wgrad1x1_kernel<kWg1Deep>) : allow_shared_memory((const void*)tc_wgrad1x1_kernel<kWg1Stages>);
     for (int i = 0; i < nb; ++i) {
-        if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd3_kernel<0>(b.blk[i].c_out));
-        if (e == cudaSuccess && b.blk[i].pass_back) e = allow_shared_memory((const void*)fwd3_kernel<1>(b.blk[i].c_prev));
+        if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd3_kernel<0>(P->blk[i].walk_fwd));
+        if (e == cudaSuccess && b.blk[i].pass_back) e = allow_shared_memory((const void*)fwd3_kernel<1>(P->blk[i].walk_back));
         if (e == cudaSuccess) e = allow_shared_memory((const void*)wgrad3_kernel(P->blk[i].wg));
     }
     if (nb && e == cudaSuccess) e = allow_shared_memory((const void*)tc_back1x1_kernel);
@@ -1306,33 +1407,18 @@ static bool fwd1_early_enabled()     // ST_FWD1_EARLY=0 switches the early activ
 static const char* const kFwd3Names[kMaxBlocks] = {"tc_fwd3x3", "tc_fwd3x3#2"};
 static const char* const kWg3Names[kMaxBlocks] = {"tc_wgrad3x3", "tc_wgrad3x3#2"};
 
-// the tile walk of a 3x3 layer over `total` tiles: grid size and how the tiles of a partly filled last round are cut
-static void tile_walk(const TcPlan* P, int total, int n_out, int* grid, int* tail_split)
-{
-    *grid = total < P->n_sms ? total : P->n_sms;
-    // the tiles of a partly filled last round are cut into 4 or 2 ranges of output channels if that lets every
-    // piece have its own block (pieces are multiples of 64 channels)
-    const int tail = total > *grid ? total % *grid : 0;
-    *tail_split = 1;
-    if (tail > 0) {
-        if (n_out % 256 == 0 && tail * 4 <= *grid) *tail_split = 4;
-        else if (n_out % 128 == 0 && tail * 2 <= *grid) *tail_split = 2;
-    }
-}
-
 int tc_forward_blocks(const TcPlan* P, int first, int last, cudaStream_t s, StageTimer* t, const int* skip, int64_t skip_stride)
 {
     const TcBuffers& b = P->b;
     int n = 0;
-    const int total = tc_tile3_count(b.h, b.w) * b.S;
     for (int i = first; i < last; ++i) {
         const TcBlock& k = b.blk[i];
         const TcBlockPlan& q = P->blk[i];
-        int grid, tail_split;
-        tile_walk(P, total, k.c_out, &grid, &tail_split);
-        ST_REPEAT(t) launch_early(b.chain_early != 0, fwd3_kernel<0>(k.c_out), dim3(grid), dim3(kFwd3Threads), q.smem_fwd, s,
-            q.in_fwd, q.skip_fwd, k.c_prev / kBlockK, k.c_skip / kBlockK, q.w_map, q.w_map_q, tail_split, b.theta, b.n_params, k.b_off,
-            q.out_st, k.relu_bits, (float*)nullptr, k.c_out, b.h, b.w, total, pow2_cols(k.c_out), b.err, skip, skip_stride);
+        const Fwd3Walk& wk = q.walk_fwd;
+        ST_REPEAT(t) launch_early(b.chain_early != 0, fwd3_kernel<0>(wk), dim3(wk.grid), dim3(kFwd3Threads), q.smem_fwd, s,
+            q.in_fwd, q.skip_fwd, k.c_prev / kBlockK, k.c_skip / kBlockK, q.w_map, q.w_map_q, fwd3_stages(k.c_out, wk.halves), wk.n_full, wk.n_items,
+            wk.tail_split, b.theta, b.n_params, k.b_off, q.out_st, k.relu_bits, (float*)nullptr, k.c_out, b.h, b.w, pow2_cols(2 * wk.halves * k.c_out),
+            b.err, skip, skip_stride);
         if (t) t->mark(kFwd3Names[i], s, st_repeats(t));
         n += st_repeats(t);
     }
@@ -1386,7 +1472,6 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
         if (t) t->mark("tc_back1x1", s, st_repeats(t));
         n += st_repeats(t);
     }
-    const int total = tc_tile3_count(b.h, b.w) * b.S;
     for (int i = nb - 1; i >= 0 && b.blk[i].trained; --i) {
         const TcBlock& k = b.blk[i];
         const TcBlockPlan& q = P->blk[i];
@@ -1399,11 +1484,11 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
             // gradient with respect to the previous block's output: the tile walk of the forward over this block's
             // output gradient, with the mirrored and transposed weights; masked by the previous block's ReLU bits
             const TcBlock& r = b.blk[i - 1];
-            int grid, tail_split;
-            tile_walk(P, total, k.c_prev, &grid, &tail_split);
-            ST_REPEAT(t) launch_early(b.chain_early != 0, fwd3_kernel<1>(k.c_prev), dim3(grid), dim3(kFwd3Threads), q.smem_back, s,
-                q.dout_fwd, q.dout_fwd, k.c_out / kBlockK, 0, q.wt_map, q.wt_map_q, tail_split, (const float*)nullptr, (int64_t)0, (int64_t)0,
-                q.dprev_st, r.relu_bits, r.b_partials, k.c_prev, b.h, b.w, total, pow2_cols(k.c_prev), b.err, skip, skip_stride);
+            const Fwd3Walk& wk = q.walk_back;
+            ST_REPEAT(t) launch_early(b.chain_early != 0, fwd3_kernel<1>(wk), dim3(wk.grid), dim3(kFwd3Threads), q.smem_back, s,
+                q.dout_fwd, q.dout_fwd, k.c_out / kBlockK, 0, q.wt_map, q.wt_map_q, fwd3_stages(k.c_prev, wk.halves), wk.n_full, wk.n_items, wk.tail_split,
+                (const float*)nullptr, (int64_t)0, (int64_t)0, q.dprev_st, r.relu_bits, r.b_partials, k.c_prev, b.h, b.w,
+                pow2_cols(2 * wk.halves * k.c_prev), b.err, skip, skip_stride);
             if (t) t->mark("tc_dgrad3x3", s, st_repeats(t));
             n += st_repeats(t);
         }

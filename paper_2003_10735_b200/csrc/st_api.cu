@@ -725,7 +725,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
                 ALLOC(blk[i].dout, S * c->p * k.c_out);
                 ALLOC(blk[i].w_partials, (size_t)S * c->n_split1 * 9 * k.c_out * tot);
                 // the block in front of the classifier gets its gradient from the 1x1 layer's backward kernel, the others from
-                // the 4 x 32 tiles of the 3x3 tile walk
+                // the 16 x 8 tiles of the 3x3 tile walk
                 k.n_bpart = i == n_blocks - 1 ? c->n_split2 : tc_tile3_count(c->h, c->w);
                 ALLOC(blk[i].b_partials, (size_t)S * k.n_bpart * k.c_out);
                 if (i > first_trained) ALLOC(blk[i].w_t, (size_t)S * 9 * k.c_prev * k.c_out);

@@ -49,3 +49,40 @@ def test_forward_and_weight_gradient_of_the_stored_operands(c_in, ch, h, w):
     assert (np.abs(hd - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-5 * np.abs(ref).max()).all()
     assert rel_l2(g, np.stack([dh @ X[t].T for t in range(9)], axis=2)) <= 1e-5
     st.st_destroy(ctx)
+
+
+@pytest.mark.parametrize("c_in,blocks,h,w", [
+    (64, ((64, 0), (64, 64)), 1, 1), (64, ((64, 64), (64, 0)), 17, 9), (128, ((128, 0), (64, 0)), 16, 8), (64, ((128, 64), (128, 0)), 33, 23),
+    (64, ((192, 0), (64, 0)), 18, 41), (64, ((256, 0), (64, 0)), 97, 150), (64, ((64, 0), (64, 0)), 180, 200),
+])
+def test_gradient_passed_back_at_the_edges_of_its_tiles(c_in, blocks, h, w):
+    """The first block's gradient, masked by its own ReLU, and its bias gradient, against sums over the second block's gradient as
+    stored: a lone pixel, one row and column beyond a tile of 16 x 8, whole tiles, items of one and of two tiles, items cut into
+    ranges of channels."""
+    C, rng = 5, np.random.default_rng(1)
+    shapes, prev = [], c_in
+    for co, cs in blocks:
+        shapes.append((co, prev + cs)); prev = co
+    theta = []
+    for co, ci in shapes:
+        theta += [rng.standard_normal(co * ci * 9) * np.sqrt(2 / (9 * ci)), np.linspace(-0.2, 0.3, co)]
+    theta += [rng.standard_normal(C * prev) * np.sqrt(2 / prev), np.zeros(C)]
+    ctx = st.st_init_head(c_in=c_in, n_classes=C, feat_h=h, feat_w=w, gemm_precision=1, lr=0.01, blocks=blocks,
+                          cuda_stream=torch.cuda.current_stream().cuda_stream, init_params=np.concatenate(theta).astype(np.float32))
+    feat, T = problem(3, c_in, C, h, w)
+    st.st_set_frozen_features(ctx, 0, dev(feat)); st.st_teacher_labels(ctx, 0, dev(T))
+    for b, (_, cs) in enumerate(blocks):
+        if cs:
+            st.st_set_skip_features(ctx, 0, b, dev(np.maximum(rng.standard_normal((cs, h, w)), 0).astype(np.float32)))
+    st.st_distill_step(ctx, 1)
+    read = lambda which, c: st.st_read_tensor(ctx, 0, which).reshape(c, h, w)
+    (c1, i1), (c2, i2) = shapes
+    out1, d1 = read(st.ST_TENSOR_HIDDEN_FIRST, c1), read(st.ST_TENSOR_HIDDEN_GRAD_FIRST, c1)
+    d2 = read(st.ST_TENSOR_HIDDEN_GRAD, c2).astype(np.float64)
+    W2 = oracle.round_bf16(np.asarray(theta[2], np.float32)).astype(np.float64).reshape(c2, i2, 9)[:, :c1]
+    back = taps(d2).reshape(9, c2, h * w)                       # under tap t: d2 at the pixel shifted by t; the transpose mirrors the taps
+    ref = sum(W2[:, :, 8 - t].T @ back[t] for t in range(9)).reshape(c1, h, w) * (out1 > 0)
+    assert (np.abs(d1 - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-5 * max(np.abs(ref).max(), 1e-30)).all()
+    g = st.st_read_tensor(ctx, 0, st.ST_TENSOR_PARAM_GRAD)[c1 * i1 * 9:][:c1]
+    assert rel_l2(g, ref.sum((1, 2))) <= 1e-5
+    st.st_destroy(ctx)
