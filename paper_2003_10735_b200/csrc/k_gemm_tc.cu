@@ -19,6 +19,7 @@
 #include "train_ctl.cuh"
 
 #include <cstdio>
+#include <algorithm>
 #include <cstring>
 
 namespace st {
@@ -32,7 +33,7 @@ constexpr int kBlockK = 64;              // bf16 elements per 128-byte swizzled 
 constexpr int kTileM = 128;              // UMMA M
 constexpr int kChunkPix = 64;            // pixels per pipeline stage of the weight-gradient GEMMs
 constexpr int kTileW = 8, kTileH = 16;   // 3x3 forward: 128 pixels = 16 rows x 8 columns
-constexpr int kChunkW = 32, kChunkH = 2; // 3x3 wgrad: 64 pixels = 2 rows x 32 columns
+constexpr int kChunkW = 32, kChunkH = 4; // 3x3 wgrad: 128 pixels = 4 rows x 32 columns
 constexpr int kSmemAlign = 1024;
 constexpr int kMaxKBlocks = 16;
 // Pipeline depth of the 1x1 weight gradient (20 KB per stage): three, which lets three blocks work on an SM, or five where every
@@ -307,6 +308,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 #endif
 constexpr int kF1Threads = 192, kF1Stages = ST_F1_STAGES;
 constexpr uint32_t kOutPieceBytes = 32 * 128;     // 3x3 tile walk: 32 pixels x 64 channels of an epilogue warp on their way out
+constexpr int kWg3LeastChunks = 5;                // chunks in a range of a 3x3 weight gradient
 constexpr int kMaxWStages = 16;                   // ... weight stages of its ring
 __host__ __device__ constexpr int slab_cols(int halves) { return kTileW * halves + 2; }
 __host__ __device__ constexpr uint32_t slab_bytes(int halves) { return ((uint32_t)slab_cols(halves) * (kTileH + 2) * 128 + 1023) / 1024 * 1024; }
@@ -732,42 +734,51 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
 }
 
 // ------------------------------------------------------------------------------------------------
-// wgrad 3x3: for one tap, D[ci][co] += sum over this block's pixel chunks of X[pix+tap][ci] * dHd[pix][co].
-// Both operands are MN-major (pixel-major activations, reduction over pixels).  A block keeps
-// ceil(Cin/128) accumulators of Ch columns (all input channels of one tap) so that the dHd tile of a
-// stage is shared by all of them.  Bound by the tensor pipe and
-// 37 MB of partial sums at 256 channels (47.5 us at 720p), by the issue of copies and MMAs in narrow layers.  With producer and
-// issuer as single threads 51.4 us, and 37 / 41 us in a stack of 64 and 128; as whole warps with elect_one 47.5, 30 and 33;
-// with one copy for all channels of a chunk (64 x w x h x blocks of 64) and two chunks per stage 47.4, 22.9 and 30.9.
+// wgrad 3x3: D[tap][ci][co] = sum over pixels q of X[q][ci] * dHd[q - tap][co].  A block takes 128 input channels, up to 128 output
+// channels (COB blocks of 64), one vertical shift and a range of pixel chunks, and forms the three horizontal taps at once: the
+// gradient arrives with one column more on either side, and the B operand of 192 columns is its 64 channels three times, each block
+// of 64 one pixel (128 bytes) behind the one before it, which is the descriptor's stride between blocks.  Both operands are
+// MN-major (pixel-major tensors, reduction over pixels).
+// Bound by the tensor pipe (96 cycles for 192 columns; a chunk of eight takes 810 to 850 with 64 output channels a block, whose copies
+// come at 60 bytes a cycle, and 1610 with 128) and by the partial sums at its end: 3 us for 14 MB at 256 channels.  A block per tap and
+// all input channels, N = the output channels, before / now, us at 720p: 192 -> 64 20.3 / 15.1, 64 -> 64 14.1 / 10.3, 192 -> 128 28.4 /
+// 24.9, 256 -> 128 28.3 / 25.2, 256 -> 256 47.0 / 46.5 (under the power cap; fewer partial sums for the update: 13 / 11.7); three of
+// 101 x 187, 192 -> 128 38.4 / 34.6.
 // ------------------------------------------------------------------------------------------------
-template <int STAGES, int G>
+constexpr uint32_t kWg3ABytes = kChunkW * kChunkH * 128, kWg3BCols = kChunkW + 2, kWg3BBytes = kWg3BCols * kChunkH * 128;   // 64 channels of a chunk
+static_assert(kWg3ABytes % 1024 == 0 && kWg3BBytes % 1024 == 0, "the operands begin where the swizzle pattern does");
+__host__ __device__ constexpr uint32_t wg3_stage_bytes(int cob) { return 2 * kWg3ABytes + cob * kWg3BBytes; }
+
+template <int STAGES, int COB>
 __global__ void __launch_bounds__(kThreadsTc)
-tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output {64, w, h, C1/64, S} box {64, 32, 2, C1/64, 1}
-                   const __grid_constant__ CUtensorMap tmA2,  // skip input      {64, w, h, C2/64, S} box {64, 32, 2, C2/64, 1} (unused if C2 == 0)
+tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output {C1, w, h, S} box {64, 32, 4, 1}
+                   const __grid_constant__ CUtensorMap tmA2,  // skip input      {C2, w, h, S} same box (unused if C2 == 0)
                    int blocks1,                                // C1 / 64: input-channel blocks that come from tmA
-                   const __grid_constant__ CUtensorMap tmB,   // dHd {64, w, h, Ch/64, S} box {64, 32, 2, Ch/64, 1}
+                   const __grid_constant__ CUtensorMap tmB,   // dHd {Ch, w, h, S} box {64, 34, 4, 1}
                    float* __restrict__ partials,              // [S][n_split][9][Ch][Cin]
-                   int Cin, int Ch, int h, int w, int n_chunks, int chunks_per_block, int n_split,
-                   int tmem_cols, unsigned int* err, const int* __restrict__ skip, int64_t skip_stride)
+                   int Cin, int Ch, int chunks_x, int n_chunks, int chunks_per_block, int n_split, unsigned int* err,
+                   const int* __restrict__ skip, int64_t skip_stride, int a_early)
 {
     // Cin = C1 + C2: the layer's input is the concatenation (previous output, skip input), read from its two sources
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_smem(smem_raw);
     const uint32_t base = smem_u32(smem);
-    const int m_tiles = (Cin + kTileM - 1) / kTileM;
-    const int a_blocks = Cin / kBlockK, b_blocks = Ch / kBlockK;
-    const uint32_t blk_bytes = kChunkPix * 128;
-    // G chunks of pixels per stage.  If the input channels end on an odd 64, the last accumulator's upper half multiplies what
-    // lies behind them in the stage; nobody looks at those rows.
-    const uint32_t a_bytes = a_blocks * blk_bytes, chunk_bytes = a_bytes + b_blocks * blk_bytes, stage_bytes = G * chunk_bytes;
+    constexpr uint32_t kStage = wg3_stage_bytes(COB), kCols = COB == 1 ? 256 : 512;
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const int tap = blockIdx.x % 9, dx = tap % 3 - 1, dy = tap / 3 - 1, split = blockIdx.x / 9, s = blockIdx.y;
-    const int chunks_x = (w + kChunkW - 1) / kChunkW;
-    const int c_begin = split * chunks_per_block, c_end = min(n_chunks, c_begin + chunks_per_block);
+    // the blocks of one pixel range are neighbours: what they share comes from L2
+    const int m_tiles = (Cin + kTileM - 1) / kTileM, units = 3 * m_tiles * (Ch / kBlockK / COB);
+    const int unit = blockIdx.x % units, split = blockIdx.x / units, s = blockIdx.y;
+    const int ky = unit % 3, m = unit / 3 % m_tiles, cg = unit / 3 / m_tiles;
+    const int a_blocks = min(2, Cin / kBlockK - 2 * m);
+    const int c_begin = min(n_chunks, split * chunks_per_block), c_end = min(n_chunks, c_begin + chunks_per_block);
 
-    if (warp == 0) tmem_alloc(smem_u32(&tmem_slot), tmem_cols);
+    if (warp == 0) {
+        if (elect_one()) { prefetch_map(&tmA); prefetch_map(&tmB); }
+        __syncwarp();
+        tmem_alloc(smem_u32(&tmem_slot), kCols);
+    }
     if (tid == 0) {
         for (int i = 0; i < STAGES; ++i) { mbar_init(smem_u32(&full[i]), 1); mbar_init(smem_u32(&empty[i]), 1); }
         mbar_init(smem_u32(&done), 1);
@@ -777,86 +788,99 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_slot;
+    bool ok = true;
+    // If a 128-channel tile ends on an odd 64, its upper half multiplies what lies in the stage; nobody looks at those rows.
+    auto load_a = [&](int i, int st) {                        // (one thread)
+        const int x0 = i % chunks_x * kChunkW, y0 = i / chunks_x * kChunkH;
+        const uint32_t bar = smem_u32(&full[st]), sa = base + st * kStage;
+        mbar_expect_tx(bar, a_blocks * kWg3ABytes + COB * kWg3BBytes);
+        for (int j = 0; j < a_blocks; ++j) {
+            const int cb = 2 * m + j;
+            if (cb < blocks1) tma_load_4d(sa + j * kWg3ABytes, &tmA, bar, cb * kBlockK, x0, y0, s);
+            else tma_load_4d(sa + j * kWg3ABytes, &tmA2, bar, (cb - blocks1) * kBlockK, x0, y0, s);
+        }
+    };
+    // a_early: the layer's input is frozen, so no kernel of the step writes it: the first stages' part of it is fetched before the
+    // wait for the kernel that produces the gradient
+    const int n_pre = a_early ? min(STAGES, c_end - c_begin) : 0;
+    if (warp == 0 && elect_one())
+        for (int it = 0; it < n_pre; ++it) load_a(c_begin + it, it);
     pdl_wait();                  // inputs come from the previous kernel of the step
     if (skip && skip[(int64_t)blockIdx.y * skip_stride]) {     // this stream's training loop has ended (block-uniform; the flag
         tc_fence_before_sync();                                 // comes from an earlier kernel, so it is read after the wait)
         __syncthreads();
-        if (warp == 0) tmem_dealloc(tmem, tmem_cols);
+        if (warp == 0) tmem_dealloc(tmem, kCols);
         return;
     }
-    bool ok = true;
 
-    if (warp == 0) {             // producer and issuer walk their loops as whole warps, one lane issues
+    if (warp == 0) {             // the producer walks its loop as a whole warp, one lane issues
         int st = 0;
         uint32_t parity = 1;
-        for (int i = c_begin; i < c_end && ok; i += G) {
-            ok = mbar_wait(smem_u32(&empty[st]), parity, err, kWaitEmpty);
+        for (int i = c_begin; i < c_end && ok; ++i) {
+            if (i - c_begin >= STAGES) ok = mbar_wait(smem_u32(&empty[st]), parity, err, kWaitEmpty);
             if (!ok) break;
             if (elect_one()) {
-                const uint32_t bar = smem_u32(&full[st]), sa = base + st * stage_bytes;
-                mbar_expect_tx(bar, min(G, c_end - i) * chunk_bytes);
-#pragma unroll
-                for (int n = 0; n < G; ++n)
-                    if (n == 0 || i + n < c_end) {
-                        const int x0 = (i + n) % chunks_x * kChunkW, y0 = (i + n) / chunks_x * kChunkH;
-                        const uint32_t to = sa + n * chunk_bytes;
-                        tma_load_5d(to, &tmA, bar, 0, x0 + dx, y0 + dy, 0, s);
-                        if (blocks1 < a_blocks) tma_load_5d(to + blocks1 * blk_bytes, &tmA2, bar, 0, x0 + dx, y0 + dy, 0, s);
-                        tma_load_5d(to + a_bytes, &tmB, bar, 0, x0, y0, 0, s);
-                    }
+                if (i - c_begin >= n_pre) load_a(i, st);
+                const int x0 = i % chunks_x * kChunkW, y0 = i / chunks_x * kChunkH;
+                for (int j = 0; j < COB; ++j)
+                    tma_load_4d(base + st * kStage + 2 * kWg3ABytes + j * kWg3BBytes, &tmB, smem_u32(&full[st]), (cg * COB + j) * kBlockK, x0 - 1, y0 + 1 - ky, s);
             }
             __syncwarp();
             if (++st == STAGES) { st = 0; parity ^= 1; }
         }
-    } else if (warp == 1) {
-        const uint32_t idesc = instr_desc(kTileM, Ch, 1, 1);
-        int st = 0;
-        uint32_t parity = 0;
-        for (int i = c_begin; i < c_end; i += G) {
-            ok = mbar_wait(smem_u32(&full[st]), parity, err, kWaitFull);
-            if (!ok) break;
-            tc_fence_after_sync();
-            if (elect_one()) {
-                const uint64_t d0 = smem_desc(base + st * stage_bytes, blk_bytes, 1024);
+    } else if (warp == 1) {      // one thread issues
+        if (elect_one()) {
+            constexpr uint32_t idesc = instr_desc(kTileM, 3 * kBlockK, 1, 1);
+            const uint64_t a0 = smem_desc(base, kWg3ABytes, 1024), b0 = smem_desc(base + 2 * kWg3ABytes, 128, 1024);
+            const uint32_t f0 = smem_u32(&full[0]);
+            int st = 0;
+            uint32_t parity = 0;
+            bool ready = false;
+            for (int i = c_begin; i < c_end && ok; ++i) {
+                ok = mbar_wait_from(ready, f0 + 8 * st, parity, err, kWaitFull);
+                if (!ok) break;
+                const int now = st;
+                if (++st == STAGES) { st = 0; parity ^= 1; }
+                ready = mbar_try_wait(f0 + 8 * st, parity);
+                tc_fence_after_sync();
+                const uint64_t da = a0 + now * (kStage >> 4), db = b0 + now * (kStage >> 4);
 #pragma unroll
-                for (int n = 0; n < G; ++n)
-                    if (n == 0 || i + n < c_end) {
-                        const uint64_t da = d0 + n * (chunk_bytes >> 4), db = da + (a_bytes >> 4);
-                        for (int m = 0; m < m_tiles; ++m)
+                for (int j = 0; j < kChunkW * kChunkH / 16; ++j)     // 16 pixels at a time, two to a row of the chunk
 #pragma unroll
-                            for (int j = 0; j < kChunkPix / 16; ++j)
-                                umma(tmem + m * Ch, da + ((2 * m * blk_bytes + j * (16 * 128)) >> 4), db + j * ((16 * 128) >> 4), idesc, i != c_begin || (n | j) != 0);
-                    }
-                umma_commit(smem_u32(&empty[st]));
+                    for (int c = 0; c < COB; ++c)
+                        umma(tmem + c * (3 * kBlockK), da + (j * (16 * 128) >> 4), db + ((c * kWg3BBytes + (j / 2 * kWg3BCols + j % 2 * 16) * 128) >> 4), idesc,
+                             i != c_begin || j != 0);
+                umma_commit(smem_u32(&empty[now]));
             }
-            __syncwarp();
-            if (++st == STAGES) { st = 0; parity ^= 1; }
+            umma_commit(smem_u32(&done));
         }
-        if (elect_one()) umma_commit(smem_u32(&done));
+        ok = __all_sync(0xffffffffu, ok);
     }
     __syncwarp();
-    ok = mbar_wait(smem_u32(&done), 0, err, kWaitDone);
+    if (!mbar_wait(smem_u32(&done), 0, err, kWaitDone)) ok = false;
     pdl_launch_dependents();     // only the epilogue is left
     tc_fence_after_sync();
+    ok = __syncthreads_and(ok);
     if (ok) {
-        float* dst = partials + (((int64_t)s * n_split + split) * 9 + tap) * Ch * Cin;
+        const int ci = m * kTileM + tid;
+        float* dst = partials + (((int64_t)s * n_split + split) * 9 + ky * 3) * Ch * Cin + (int64_t)cg * COB * kBlockK * Cin + ci;
         const bool any = c_end > c_begin;
-        for (int m = 0; m < m_tiles; ++m) {
-            const int ci = m * kTileM + tid;
-            for (int n0 = 0; n0 < Ch; n0 += 32) {
+        for (int c = 0; c < COB; ++c)
+            for (int n0 = 0; n0 < 3 * kBlockK; n0 += 32) {
                 float v[32];
-                tmem_ld_32x32(tmem + ((uint32_t)(warp * 32) << 16) + m * Ch + n0, v);
+                tmem_ld_32x32(tmem + ((uint32_t)(warp * 32) << 16) + c * (3 * kBlockK) + n0, v);
+                // the gradient's column x - 1 + k stands under input column x in block k of 64: horizontal tap 2 - k
+                float* row = dst + ((int64_t)(2 - n0 / kBlockK) * Ch + c * kBlockK + n0 % kBlockK) * Cin;
                 if (ci < Cin)
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) dst[(int64_t)(n0 + c) * Cin + ci] = any ? v[c] : 0.f;
+                    for (int k = 0; k < 32; ++k) row[(int64_t)k * Cin] = any ? v[k] : 0.f;
             }
-        }
     } else {
         drain_after_error();
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, tmem_cols);
+    if (warp == 0) tmem_dealloc(tmem, kCols);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1164,35 +1188,38 @@ static Fwd3Walk fwd3_walk(int h, int w, int S, int n_out, int n_sms)
 }
 template <int MODE>
 static decltype(&tc_fwd3x3_kernel<1, MODE>) fwd3_kernel(const Fwd3Walk& q) { return q.halves == 2 ? tc_fwd3x3_kernel<2, MODE> : tc_fwd3x3_kernel<1, MODE>; }
-// The stages of the weight gradient: two chunks of pixels each if three such stages fit (for the same reason), else one; as
-// many as fit in about 208 KB, five at most.
-struct Wg3Ring { int stages, chunks; size_t bytes; };
-static Wg3Ring wg3_ring(int c_in, int c_out)
+// The 3x3 weight gradient: output-channel blocks of 64 per block, its launch's units (input-channel tiles x output-channel groups x
+// vertical shifts), pixel chunks and ranges.  About one block per SM for one stream, no range shorter than five chunks (a block's
+// start and its partial sums cost as much; us of a call, four streams of 60 x 100, 128 channels: 693 with ranges of two
+// or three, 590 with five; 45 x 80, 282 and 276; one stream of 90 x 160, 320 and 324).  The number of streams has no part in it.
+// Blocks of 128 output channels fetch a third less per multiplication and leave twice the partial sums: they pay where ranges are
+// long (us of a call, 64 / 128: 256 channels, 85 chunks of a 1080p map a block 4301 / 4246; 38 chunks at 720p 1176 / 1191; 90 x 160
+// 538 / 562; three of 101 x 187, 128 channels 540 / 593).
+struct Wg3Shape { int cob, units, chunks_x, chunks, per, n_split; };
+static Wg3Shape wg3_shape(int c_in, int c_out, int h, int w)
 {
-    const size_t chunk = (size_t)((c_in + c_out) / kBlockK) * kChunkPix * 128;
-    const int fit = (int)((size_t)208 * 1024 / chunk);
-    Wg3Ring g;
-    g.chunks = fit >= 6 ? 2 : 1;
-    g.stages = g.chunks == 2 ? (fit >= 8 ? 4 : 3) : (fit >= 5 ? 5 : (fit >= 4 ? 4 : 3));
-    g.bytes = (size_t)g.stages * g.chunks * chunk + kSmemAlign;
-    return g;
+    Wg3Shape q;
+    q.chunks_x = (w + kChunkW - 1) / kChunkW;
+    q.chunks = q.chunks_x * ((h + kChunkH - 1) / kChunkH);
+    for (q.cob = c_out % 128 == 0 ? 2 : 1;; q.cob = 1) {
+        q.units = 3 * ((c_in + kTileM - 1) / kTileM) * (c_out / kBlockK / q.cob);
+        const int ranges = std::min(148 / q.units, q.chunks / kWg3LeastChunks);
+        split_geometry(q.chunks, std::max(ranges, 1), &q.per, &q.n_split);
+        if (q.cob == 1 || q.per >= 64) return q;
+    }
 }
-static decltype(&tc_wgrad3x3_kernel<3, 1>) wgrad3_kernel(const Wg3Ring& g)
-{
-    if (g.chunks == 2) return g.stages == 4 ? tc_wgrad3x3_kernel<4, 2> : tc_wgrad3x3_kernel<3, 2>;
-    return g.stages == 5 ? tc_wgrad3x3_kernel<5, 1> : (g.stages == 4 ? tc_wgrad3x3_kernel<4, 1> : tc_wgrad3x3_kernel<3, 1>);
-}
+static size_t wg3_bytes(const Wg3Shape& q) { return (size_t)(q.cob == 2 ? 3 : 4) * wg3_stage_bytes(q.cob) + kSmemAlign; }
+static decltype(&tc_wgrad3x3_kernel<3, 2>) wgrad3_kernel(const Wg3Shape& q) { return q.cob == 2 ? tc_wgrad3x3_kernel<3, 2> : tc_wgrad3x3_kernel<4, 1>; }
 
 struct TcBlockPlan {
     CUtensorMap in_fwd, skip_fwd;    // the block's two inputs {C, w, h, S}, box {64, 8 halves + 2, 18, 1} (forward slabs)
-    CUtensorMap in_wg, skip_wg;      // same tensors, box {64, 32, 2, 1} (weight-gradient chunks)
+    CUtensorMap in_wg, skip_wg;      // same tensors, box {64, 32, 4, 1} (weight-gradient chunks)
     CUtensorMap w_map, w_map_q;      // {c_tot, 9*c_out, S}, boxes {64, c_out, 1} and {64, 64, 1}
     CUtensorMap wt_map, wt_map_q;    // mirrored, transposed weights {c_out, 9*c_prev, S}, boxes {64, c_prev, 1} and {64, 64, 1}
     CUtensorMap dout_fwd;            // the block's output gradient {c_out, w, h, S}, the slab's box (A operand when passed back)
     CUtensorMap out_st, dprev_st;    // the block's output and its first input's gradient {C, w, h, S}, box {64, 8, 4, 1} (stores)
-    CUtensorMap dout_wg;             // same tensor, box {64, 32, 2, 1} (B operand of the weight gradient)
-    int cols_wg;                     // tensor-memory columns of the weight gradient
-    Wg3Ring wg;
+    CUtensorMap dout_wg;             // same tensor, box {64, 34, 4, 1} (B operand of the weight gradient)
+    Wg3Shape wg;
     Fwd3Walk walk_fwd, walk_back;
     size_t smem_fwd, smem_back;
 };
@@ -1208,7 +1235,6 @@ struct TcPlan {
     TcBlockPlan blk[kMaxBlocks];
     int split2, chunks2, per2, cols2, msplit2;
     int tiles_b, per_b, split_b, groups_b;   // backward of the 1x1 layer behind a trained block: pixel tiles, tiles per range, ranges, channel groups
-    int split1, chunks1, per1;          // pixel chunks of the 3x3 weight gradients (the same for every block)
     size_t smem_fwd1, smem_fwd1p, smem_wg1, smem_back1;
     bool fwd1_persistent, wg1_deep;
     int n_sms;
@@ -1218,18 +1244,14 @@ struct TcPlan {
 // blocks per pixel range of the 1x1 weight gradient: one per 128-channel accumulator
 static int wgrad1x1_m_split(int c_last) { const int m = (c_last + kTileM - 1) / kTileM; return m < 1 ? 1 : m; }
 
-int tc_wgrad_splits(int layer, int c_last, int h, int w)
+int tc_wgrad1x1_splits(int c_last, int h, int w)
 {
     int per, n;
-    if (layer == 2) {
-        const int64_t p = (int64_t)h * w;
-        split_geometry((int)((p + kChunkPix - 1) / kChunkPix), 148 / wgrad1x1_m_split(c_last), &per, &n);
-    } else {
-        const int chunks = ((w + kChunkW - 1) / kChunkW) * ((h + kChunkH - 1) / kChunkH);
-        split_geometry(chunks, 148 / 9, &per, &n);
-    }
+    const int64_t p = (int64_t)h * w;
+    split_geometry((int)((p + kChunkPix - 1) / kChunkPix), 148 / wgrad1x1_m_split(c_last), &per, &n);
     return n;
 }
+int tc_wgrad3x3_splits(int c_in, int c_out, int h, int w) { return wg3_shape(c_in, c_out, h, w).n_split; }
 
 // pixel ranges of the 1x1 layer's backward behind a trained hidden layer: with the groups of 128 channels about one block per SM
 int tc_back_splits(int c_last, int h, int w)
@@ -1286,21 +1308,15 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
                        ct = c1 + c2;
         q.walk_fwd = fwd3_walk(b.h, b.w, b.S, k.c_out, P->n_sms);
         q.walk_back = fwd3_walk(b.h, b.w, b.S, k.c_prev, P->n_sms);
-        auto act_maps = [&](const bf16* base, uint64_t c, int halves, CUtensorMap* fwd, CUtensorMap* wg, const char* what) {
-            const uint32_t bf[4] = {64, (uint32_t)slab_cols(halves), (uint32_t)kTileH + 2, 1};
+        auto act_maps = [&](const bf16* base, uint64_t c, int halves, CUtensorMap* fwd, CUtensorMap* wg, int wg_cols, const char* what) {
+            const uint32_t bf[4] = {64, (uint32_t)slab_cols(halves), (uint32_t)kTileH + 2, 1}, bw[4] = {64, (uint32_t)wg_cols, (uint32_t)kChunkH, 1};
             uint64_t d[4] = {c, w, h, S}, st[3] = {c * 2, w * c * 2, h * w * c * 2};
-            // all channels of a chunk in one copy: one block of 64 behind the other
-            uint64_t d5[5] = {64, w, h, c / 64, S}, st5[4] = {c * 2, w * c * 2, 128, h * w * c * 2};
-            uint32_t bw[5] = {64, (uint32_t)kChunkW, (uint32_t)kChunkH, (uint32_t)(c / 64), 1};
-            bool r = true;
-            if (fwd) r = r && make_map(fwd, base, 4, d, st, bf, err, err_len, what);
-            if (wg) r = r && make_map(wg, base, 5, d5, st5, bw, err, err_len, what);
-            return r;
+            return make_map(fwd, base, 4, d, st, bf, err, err_len, what) && make_map(wg, base, 4, d, st, bw, err, err_len, what);
         };
-        ok = ok && act_maps(k.in_prev, c1, q.walk_fwd.halves, &q.in_fwd, &q.in_wg, "block input");
-        if (c2) ok = ok && act_maps(k.in_skip, c2, q.walk_fwd.halves, &q.skip_fwd, &q.skip_wg, "skip input");
+        ok = ok && act_maps(k.in_prev, c1, q.walk_fwd.halves, &q.in_fwd, &q.in_wg, kChunkW, "block input");
+        if (c2) ok = ok && act_maps(k.in_skip, c2, q.walk_fwd.halves, &q.skip_fwd, &q.skip_wg, kChunkW, "skip input");
         else { q.skip_fwd = q.in_fwd; q.skip_wg = q.in_wg; }
-        ok = ok && act_maps(k.dout, co, q.walk_back.halves, &q.dout_fwd, &q.dout_wg, "block output gradient");
+        ok = ok && act_maps(k.dout, co, q.walk_back.halves, &q.dout_fwd, &q.dout_wg, kWg3BCols, "block output gradient");
         {
             uint64_t dw[3] = {ct, 9 * co, S}, sw[2] = {ct * 2, 9 * co * ct * 2};
             uint32_t bwt[3] = {64, (uint32_t)co, 1}, bwq[3] = {64, 64, 1};
@@ -1320,16 +1336,10 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
             ok = ok && make_map(&q.wt_map, k.w_t, 3, dw, sw, bwt, err, err_len, "3x3 weight, transposed");
             ok = ok && make_map(&q.wt_map_q, k.w_t, 3, dw, sw, bwq, err, err_len, "3x3 weight, transposed (64 rows)");
         }
-        const int m_in = ((int)ct + kTileM - 1) / kTileM;
-        q.cols_wg = pow2_cols(m_in * k.c_out);
-        q.wg = wg3_ring((int)ct, k.c_out);
+        q.wg = wg3_shape((int)ct, k.c_out, b.h, b.w);
         q.smem_fwd = fwd3_bytes(k.c_out, q.walk_fwd.halves);
         q.smem_back = fwd3_bytes(k.c_prev, q.walk_back.halves);
-        if (ok && q.cols_wg > 512) {
-            snprintf(err, err_len, "a block with %d input and %d output channels needs %d TMEM columns (> 512)", (int)ct, k.c_out, q.cols_wg);
-            ok = false;
-        }
-        if (ok && (q.smem_fwd > lim || q.wg.bytes > lim || (k.pass_back && (q.smem_back > lim || k.c_prev > 256)))) {
+        if (ok && (q.smem_fwd > lim || wg3_bytes(q.wg) > lim || (k.pass_back && (q.smem_back > lim || k.c_prev > 256)))) {
             snprintf(err, err_len, "shared memory per block exceeds 227 KB for these channel counts");
             ok = false;
         }
@@ -1373,8 +1383,6 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
     P->smem_wg1 = (P->wg1_deep ? kWg1Deep : kWg1Stages) * ((size_t)(m_last / P->msplit2) * 2 * kChunkPix * 128 + kClassPad * 128) + kSmemAlign;
     if (P->wg1_deep) P->smem_wg1 = one_per_sm(P->smem_wg1, wg1_blocks, P->n_sms);
     if (nb) {
-        P->chunks1 = ((b.w + kChunkW - 1) / kChunkW) * ((b.h + kChunkH - 1) / kChunkH);
-        split_geometry(P->chunks1, 148 / 9, &P->per1, &P->split1);
         P->tiles_b = (P->p + kTileM - 1) / kTileM;
         P->groups_b = (P->c_last + kBackCols - 1) / kBackCols;
         split_geometry(P->tiles_b, 148 / P->groups_b, &P->per_b, &P->split_b);
@@ -1475,9 +1483,9 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
     for (int i = nb - 1; i >= 0 && b.blk[i].trained; --i) {
         const TcBlock& k = b.blk[i];
         const TcBlockPlan& q = P->blk[i];
-        ST_REPEAT(t) launch_early(b.chain_early != 0, wgrad3_kernel(q.wg), dim3(9 * P->split1, b.S), dim3(kThreadsTc), q.wg.bytes, s,
-            q.in_wg, q.skip_wg, k.c_prev / kBlockK, q.dout_wg, k.w_partials, k.c_prev + k.c_skip, k.c_out, b.h, b.w, P->chunks1, P->per1,
-            P->split1, q.cols_wg, b.err, skip, skip_stride);
+        ST_REPEAT(t) launch_early(b.chain_early != 0, wgrad3_kernel(q.wg), dim3(q.wg.units * q.wg.n_split, b.S), dim3(kThreadsTc),
+            wg3_bytes(q.wg), s, q.in_wg, q.skip_wg, k.c_prev / kBlockK, q.dout_wg, k.w_partials, k.c_prev + k.c_skip, k.c_out, q.wg.chunks_x, q.wg.chunks,
+            q.wg.per, q.wg.n_split, b.err, skip, skip_stride, i == 0 && !skip && !t && b.chain_early ? 1 : 0);
         if (t) t->mark(kWg3Names[i], s, st_repeats(t));
         n += st_repeats(t);
         if (k.pass_back) {

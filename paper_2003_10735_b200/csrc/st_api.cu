@@ -60,14 +60,14 @@ struct st_ctx {
         bf16 *skip = nullptr, *out = nullptr, *dout = nullptr, *w = nullptr, *w_t = nullptr;
         uint32_t* relu_bits = nullptr;
         float *w_partials = nullptr, *b_partials = nullptr;
-        int n_bpart = 0;
+        int n_split = 0, n_bpart = 0;          // partial results of the weight gradient, of the bias gradient
         std::vector<char> has_skip;
     } blk[kMaxBlocks];
     bool prefix_current = false;            // the frozen blocks' outputs belong to the current features and skip inputs
     int64_t trained_begin = 0, n_trained = 0;   // where the trained layers start in one stream's parameters; how many values
     bf16* w2_shadow = nullptr;
     float* w2_partials = nullptr;
-    int n_split1 = 0, n_split2 = 0;
+    int n_split2 = 0;
     float *loss_part = nullptr, *db_part = nullptr;
     int n_k3_blocks = 0;
     CUtensorMap fx_map, fw_map; // tile maps of the classifier's input and of its bf16 weights: the loss kernel multiplies its own logits
@@ -245,9 +245,9 @@ UpdateArgs make_update_args(st_ctx* c, int slot, const int* skip = nullptr, int6
             ly.w_stream_stride = ly.w_split_stride * c->n_split2;
         } else {
             const st_ctx::Block& k = c->blk[L];
-            ly.w_partials = k.w_partials; ly.n_split = c->n_split1;
+            ly.w_partials = k.w_partials; ly.n_split = k.n_split;
             ly.w_split_stride = (int64_t)9 * ly.cout * ly.cin;
-            ly.w_stream_stride = ly.w_split_stride * c->n_split1;
+            ly.w_stream_stride = ly.w_split_stride * k.n_split;
             ly.b_partials = k.b_partials; ly.n_bpart = k.n_bpart;
         }
         if (c->bf16_mode) {
@@ -710,9 +710,8 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
         c->dz_pitch = tc_dz_pitch(c->h, c->w);
         ALLOC(dz_bf16, (size_t)S * kClassPad * c->dz_pitch);
         ALLOC(w2_shadow, (size_t)S * kClassPad * c_last);
-        c->n_split2 = n_blocks > first_trained ? tc_back_splits(c_last, c->h, c->w) : tc_wgrad_splits(2, c_last, c->h, c->w);
+        c->n_split2 = n_blocks > first_trained ? tc_back_splits(c_last, c->h, c->w) : tc_wgrad1x1_splits(c_last, c->h, c->w);
         ALLOC(w2_partials, (size_t)S * c->n_split2 * kClassPad * c_last);
-        c->n_split1 = n_blocks ? tc_wgrad_splits(1, 0, c->h, c->w) : 0;
         for (int i = 0; i < n_blocks; ++i) {
             st_ctx::Block& k = c->blk[i];
             const size_t tot = (size_t)k.c_prev + k.c_skip;
@@ -723,7 +722,8 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             ALLOC(blk[i].w, (size_t)S * 9 * k.c_out * tot);
             if (trained) {
                 ALLOC(blk[i].dout, S * c->p * k.c_out);
-                ALLOC(blk[i].w_partials, (size_t)S * c->n_split1 * 9 * k.c_out * tot);
+                k.n_split = tc_wgrad3x3_splits((int)tot, k.c_out, c->h, c->w);
+                ALLOC(blk[i].w_partials, (size_t)S * k.n_split * 9 * k.c_out * tot);
                 // the block in front of the classifier gets its gradient from the 1x1 layer's backward kernel, the others from
                 // the 16 x 8 tiles of the 3x3 tile walk
                 k.n_bpart = i == n_blocks - 1 ? c->n_split2 : tc_tile3_count(c->h, c->w);
@@ -738,9 +738,9 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
         ALLOC(w2_partials, (size_t)S * c->n_split2 * c->C * c_last);
         if (c->Ch) {
             ALLOC(hid_f32, S * c->Ch * plane); ALLOC(dhid_f32, S * c->Ch * plane);
-            c->n_split1 = c->blk[0].n_bpart = conv_wgrad_f32_splits(c->Cin, c->Ch, c->h, c->w, 3);
-            ALLOC(blk[0].w_partials, (size_t)S * c->n_split1 * 9 * c->Ch * c->Cin);
-            ALLOC(blk[0].b_partials, (size_t)S * c->n_split1 * c->Ch);
+            c->blk[0].n_split = c->blk[0].n_bpart = conv_wgrad_f32_splits(c->Cin, c->Ch, c->h, c->w, 3);
+            ALLOC(blk[0].w_partials, (size_t)S * c->blk[0].n_split * 9 * c->Ch * c->Cin);
+            ALLOC(blk[0].b_partials, (size_t)S * c->blk[0].n_split * c->Ch);
         }
     }
 #undef ALLOC

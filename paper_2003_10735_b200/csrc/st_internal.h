@@ -314,7 +314,7 @@ struct TcBlock {
     bf16* out;               // [S][p][c_out]
     uint32_t* relu_bits;     // [S][p][c_out/32]: one bit per output value, set where it is > 0
     bf16* dout;              // [S][p][c_out]     gradient with respect to the output, after the ReLU mask
-    float* w_partials;       // [S][n_split1][9][c_out][c_prev + c_skip]
+    float* w_partials;       // [S][tc_wgrad3x3_splits][9][c_out][c_prev + c_skip]
     float* b_partials;       // [S][n_bpart][c_out]: tc_back_splits for the last block, 16 x 8 tiles for the others
     int trained;             // the block lies behind the freeze boundary: its gradients are formed
     int pass_back;           // ... and so does the block before it: the gradient is passed on to it
@@ -335,7 +335,8 @@ struct TcBuffers {
     int chain_early;      // launch the kernels so that each may start while its predecessor on the stream drains
 };
 // Geometry is fixed by the shapes alone, so scratch can be sized before the plan exists.
-int tc_wgrad_splits(int layer /*1: 3x3, 2: 1x1*/, int c_last, int h, int w);
+int tc_wgrad1x1_splits(int c_last, int h, int w);
+int tc_wgrad3x3_splits(int c_in, int c_out, int h, int w);   // c_in: both inputs of the layer
 int tc_back_splits(int c_last, int h, int w);   // pixel ranges of tc_back1x1 (classifier behind a trained block: its weight-gradient and that block's bias-gradient partials)
 int tc_tile3_count(int h, int w);   // 16 x 8 pixel tiles of a 3x3 layer per stream (bias-gradient partials of earlier blocks)
 int tc_dz_pitch(int h, int w);      // row pitch (elements) of the bf16 logit gradient [S][kClassPad][pitch]
