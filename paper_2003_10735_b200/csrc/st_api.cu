@@ -655,18 +655,19 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     // The legacy default stream cannot be captured: steps are then enqueued kernel by kernel.
     c->use_graphs = c->stream != nullptr && c->stream != cudaStreamLegacy && c->stream != cudaStreamPerThread;
     if (const char* e = getenv("ST_NO_GRAPH")) if (e[0] == '1') c->use_graphs = false;
-    // Programmatic dependent launch along the step's chain: with the one-layer head every kernel has something to do
-    // before its predecessor's results are needed (label fetch, feature tiles) and the step is 2 us shorter.  Blocks of 3x3
-    // layers with at most 128 output channels are many short kernels, whose starts (barriers, tensor memory) hide behind the one
-    // before: 2 % of a call (two blocks of 64 channels, 720p: 1560 -> 1527 us; 128 channels, 101 x 187: 659 -> 645).  Kernels of
-    // wider layers gain on small maps and lose on large ones and beside other streams, where they fill the SMs to the end and waiting
-    // blocks crowd those that finish first; the line is where nothing loses.  us per step launched late / early: 256 -> 256 channels
-    // 90 x 160 66 / 64, 180 x 320 138.6 / 137, three of 101 x 187 205 / 208, 270 x 480 277 / 284; 256 -> 192 56.5 / 52.9, 122.6 / 119.2,
-    // 179.5 / 178.1, 235 / 233, four of 135 x 240 321 / 325; blocks of 192 and 64 81.5 / 79, 175 / 172, 237 / 232, 318 / 325, 408 / 413.
-    // With fp32 convolutions 10 us a step slower.  ST_PDL=0 / 1 force it.
+    // Programmatic dependent launch along the step's chain: with the one-layer head every kernel has something to do before its
+    // predecessor's results are needed (label fetch, feature tiles) and the step is 2 us shorter.  Blocks of 3x3 layers with at most
+    // 128 output channels are many short kernels, whose starts (barriers, tensor memory) hide behind the one before (two blocks of 64
+    // channels, 720p: 1560 -> 1527 us; 128 channels, 101 x 187: 659 -> 645).  Kernels of wider layers gain while a launch is a few
+    // rounds of tiles and lose where it is long, fills the SMs to its end and has waiting blocks crowd those that finish first: the
+    // line is three rounds.  us of a call launched late / early: 256 -> 256 channels, 120 tiles (90 x 160) 536 / 503, 270 (192 -> 192, 135 x
+    // 240) 663 / 633, 480 (720p) 1197 / 1161 now and then, 1273 / 1284 call after call (the power cap), 1020 (1080p) 4202..4244 /
+    // 4293..4383; three of 50 x 70 (105) 551 / 518; 256 -> 192, four at 720p (1920) 1986 / 2016.
+    // With fp32 convolutions behind a hidden layer some heads win 3 % and others lose 6: late.  ST_PDL=0 / 1 force it.
     int widest = 0;
     for (int i = 0; i < n_blocks; ++i) if (blk_out[i] > widest) widest = blk_out[i];
-    c->chain_early = pdl_enabled() && (c->Ch == 0 || (c->bf16_mode && widest <= 128));
+    const bool few_rounds = n_blocks > 0 && (int64_t)tc_tile3_count(c->h, c->w) * c->S <= 3 * (int64_t)c->n_sms;
+    c->chain_early = pdl_enabled() && (c->Ch == 0 || (c->bf16_mode && (widest <= 128 || few_rounds)));
     if (const char* e = getenv("ST_PDL")) if (e[0] == '1') c->chain_early = true;
 
     // layers in forward order: the 3x3 layers (blocks, or the fp32 path's hidden layer), then the classifier
