@@ -41,9 +41,8 @@ EX2_PER_CLASS_PIXEL = 1.0
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, ncu capture of (workload, kernel); see profiles/.
 # An entry is removed whenever its kernel changes and put back after the next capture.
 NCU_DRAM_BYTES = {
-    (2, "upsample_ce"): 5.84e6,      # profiles/upsample_ce_rows_720p.md
-    # profiles/fwd1x1_upsample_ce_rows_720p.md: a capture starts with cold caches, so the feature map (29.5 MB, L2 resident
-    # over the K iterations of the step loop) is read from DRAM once; labels 0.92 MB
+    # profiles/fwd_ce_720p.md: a capture starts with cold caches, so the feature map (29.5 MB, L2 resident over the K iterations of
+    # the step loop) is read from DRAM once; labels 0.92 MB
     (2, "fwd1x1_upsample_ce"): 30.51e6,
 }
 # st_init_head reads this when a context is made: "0" keeps the classifier's forward in a kernel of its own
