@@ -12,7 +12,7 @@
 // GPU sustains) and the issue slots beside them.  Both kernels therefore keep a register tile per thread whose operands
 // come from shared memory without bank conflicts at eight or more multiply-adds per load, multiply two output channels at
 // a time (packed fp32x2: half the instructions), and bring the next stage in with asynchronous copies while the current
-// one is multiplied.  That layer's forward / weight gradient: 50 / 39 us; one thread per pixel and eight channels, operands
+// one is multiplied.  That layer's forward / weight gradient: 50 / 37 us; one thread per pixel and eight channels, operands
 // from the L1 cache, took 378 / 115 us.
 #include "st_internal.h"
 
@@ -198,6 +198,12 @@ void launch_fwd(const ConvF32& a, int S, bool early, cudaStream_t s)
 // range and leaves its sums as one partial result; the parameter update adds the partial results in order.  The rows of a
 // chunk are divided among as many warps, whose sums are added in order at the end: one warp per channel group leaves the
 // schedulers idle while it waits (1.5 warps each for the layer above).
+// A 1x1 layer's warps hold CI = 1, 2 or 4 input channels per lane: a broadcast vector of gradients takes four cycles of the SM's
+// path from shared memory, so with one channel four of them feed eight packed multiply-adds that need four cycles, and the
+// path sets the time.  21 classes over 256 channels on 180 x 320 nodes, one channel / four: 78.4 / 40.6 us; 81 over 48 on
+// 90 x 160, one / two: 20.8 / 14.7; 40 over 128, one / four: 53.6 / 33.1; 12 over 40, one / two: 17.1 / 13.8.  A 3x3 layer's
+// inputs serve nine taps each already.  One barrier per chunk instead of two, and the bias sums divided among the rows' warps:
+// 3x3 96 -> 48 39.3 -> 37.3 us, 128 -> 128 503 -> 478.
 // ------------------------------------------------------------------------------------------------
 template <int KS> __host__ __device__ constexpr int wg_rows() { return KS == 1 ? 4 : 2; }      // pixel rows of a chunk = warps per channel group
 template <int KS> __host__ __device__ constexpr int wg_most_groups() { return KS == 1 ? 3 : 6; } // twelve warps per block at most
@@ -206,11 +212,11 @@ template <int KS> __host__ __device__ constexpr int wg_most_groups() { return KS
 template <int KS> __host__ __device__ constexpr int wg_ci_pitch() { return (wg_rows<KS>() + KS - 1) * row_floats<KS>() + 4; }
 // Gradient tile [pixel][co]: the pitch is a multiple of four floats for the broadcasts, odd in fours
 __host__ __device__ constexpr int wg_co_pitch(int COB) { return COB + (COB / 4 % 2 ? 0 : 4); }
-template <int KS, int CO>
+template <int KS, int CO, int CI>
 size_t wg_smem(int ng)
 {
-    const size_t stage = (size_t)32 * wg_ci_pitch<KS>() + (size_t)wg_rows<KS>() * kTileX * wg_co_pitch(CO * ng);
-    const size_t red = (size_t)(wg_rows<KS>() - 1) * ng * KS * KS * CO * 32;
+    const size_t stage = (size_t)32 * CI * wg_ci_pitch<KS>() + (size_t)wg_rows<KS>() * kTileX * wg_co_pitch(CO * ng);
+    const size_t red = (size_t)(wg_rows<KS>() - 1) * ng * KS * KS * CO * 32 * CI + (size_t)wg_rows<KS>() * ng * CO;
     return (2 * stage > red ? 2 * stage : red) * sizeof(float);
 }
 
@@ -220,17 +226,20 @@ struct WgradF32 {
     int64_t in_stride, dout_stride;
 };
 
-template <int KS, int CO>
+template <int KS, int CO, int CI>
 __global__ void __launch_bounds__(384)
 conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
 {
     constexpr int T = KS * KS, RW = wg_rows<KS>(), TH = RW + KS - 1, TW = row_floats<KS>(), VEC = TW / 4, CP = wg_ci_pitch<KS>();
+    // 1x1 with one channel per lane: the next copy before the wait and the bias by one warp per channel group are the faster form
+    // (21 classes over 32 channels on 180 x 320 nodes, three streams: 28.2 us, as the others 29.4)
+    constexpr bool kShort = KS == 1 && CI == 1;
     extern __shared__ __align__(16) float smem_w[];
     const int ng = blockDim.x / (32 * RW), COB = CO * ng, pitch = wg_co_pitch(COB);
-    const int stage = 32 * CP + RW * kTileX * pitch;
+    const int stage = 32 * CI * CP + RW * kTileX * pitch;
     const int s = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = (int)blockDim.x >> 5;
     const int g = warp / RW, rw = warp % RW;
-    const int split = blockIdx.x, ci0 = (blockIdx.y % ci_tiles) * 32, co0 = (blockIdx.y / ci_tiles) * COB;
+    const int split = blockIdx.x, ci0 = (blockIdx.y % ci_tiles) * 32 * CI, co0 = (blockIdx.y / ci_tiles) * COB;
     const PadF32 pad(a.h, a.w);
     pdl_wait();
     const float* in = a.in + s * a.in_stride + (KS == 3 ? 0 : kPadTop * pad.pitch + kPadLeft);
@@ -239,12 +248,12 @@ conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
 
     auto fetch = [&](int chunk, float* dst) {
         const int at = (chunk / tiles_x) * RW * pad.pitch + (chunk % tiles_x) * kTileX;
-        for (int e = tid; e < 32 * TH * VEC; e += blockDim.x) {
+        for (int e = tid; e < 32 * CI * TH * VEC; e += blockDim.x) {
             const int c = e / (TH * VEC), r = e / VEC % TH, q = e % VEC;
             const bool ok = ci0 + c < a.Cin;
             copy_async<16>(dst + c * CP + r * TW + 4 * q, ok ? in + (ci0 + c) * pad.plane + at + r * pad.pitch + 4 * q : in, ok);
         }
-        float* dd = dst + 32 * CP;
+        float* dd = dst + 32 * CI * CP;
         for (int row = warp; row < COB * RW; row += n_warps) {      // a warp copies one row of one channel at a time
             const int c = row / RW, r = row % RW;
             const bool ok = co0 + c < a.Cout;
@@ -253,20 +262,28 @@ conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
         copy_commit();
     };
 
-    float2 acc[CO / 2][T];                                  // two output channels side by side
+    float2 acc[CI][CO / 2][T];                              // two output channels side by side
     float bias = 0.f;
 #pragma unroll
-    for (int k = 0; k < CO / 2; ++k)
+    for (int j = 0; j < CI; ++j)
 #pragma unroll
-        for (int t = 0; t < T; ++t) acc[k][t] = make_float2(0.f, 0.f);
+        for (int k = 0; k < CO / 2; ++k)
+#pragma unroll
+            for (int t = 0; t < T; ++t) acc[j][k][t] = make_float2(0.f, 0.f);
     if (c_begin < c_end) fetch(c_begin, smem_w);
     int buf = 0;
     for (int chunk = c_begin; chunk < c_end; ++chunk, buf ^= 1) {
-        if (chunk + 1 < c_end) { fetch(chunk + 1, smem_w + (buf ^ 1) * stage); copy_wait<1>(); }
-        else copy_wait<0>();
-        __syncthreads();
+        if (kShort) {
+            if (chunk + 1 < c_end) { fetch(chunk + 1, smem_w + (buf ^ 1) * stage); copy_wait<1>(); }
+            else copy_wait<0>();
+            __syncthreads();
+        } else {
+            copy_wait<0>();
+            __syncthreads();        // and every thread has done with the chunk before, whose place the next copy takes
+            if (chunk + 1 < c_end) fetch(chunk + 1, smem_w + (buf ^ 1) * stage);
+        }
         const float4* xs = reinterpret_cast<const float4*>(smem_w + buf * stage + lane * CP);
-        const float* ds = smem_w + buf * stage + 32 * CP + g * CO;
+        const float* ds = smem_w + buf * stage + 32 * CI * CP + g * CO;
         {
             const int r = rw;
             // four pixels at a time; a 3x3 layer's window is the last column of the vector before, the vector, the first column after
@@ -277,66 +294,93 @@ conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
                 if (KS == 3) { before[ky] = xs[(r + ky) * VEC].w; now[ky] = xs[(r + ky) * VEC + 1]; }
 #pragma unroll 1
             for (int v = 0; v < kTileX / 4; ++v) {
-                float win[KS][KS + 3];
+                float win[CI][KS][KS + 3];
 #pragma unroll
-                for (int ky = 0; ky < KS; ++ky) {
-                    if (KS == 3) {
-                        const float4 next = xs[(r + ky) * VEC + v + 2];
-                        win[ky][0] = before[ky];
-                        win[ky][1] = now[ky].x; win[ky][KS / 2 + 1] = now[ky].y; win[ky][KS] = now[ky].z; win[ky][KS + 1] = now[ky].w;
-                        win[ky][KS + 2] = next.x;
-                        before[ky] = now[ky].w; now[ky] = next;
-                    } else {
-                        const float4 t = xs[r * VEC + v];
-                        win[0][0] = t.x; win[0][1] = t.y; win[0][2] = t.z; win[0][3] = t.w;
+                for (int j = 0; j < CI; ++j)
+#pragma unroll
+                    for (int ky = 0; ky < KS; ++ky) {
+                        if (KS == 3) {
+                            const float4 next = xs[(r + ky) * VEC + v + 2];
+                            win[j][ky][0] = before[ky];
+                            win[j][ky][1] = now[ky].x; win[j][ky][KS / 2 + 1] = now[ky].y; win[j][ky][KS] = now[ky].z; win[j][ky][KS + 1] = now[ky].w;
+                            win[j][ky][KS + 2] = next.x;
+                            before[ky] = now[ky].w; now[ky] = next;
+                        } else {
+                            const float4 t = xs[j * 8 * CP + r * VEC + v];      // 32 channels on, in vectors
+                            win[j][0][0] = t.x; win[j][0][1] = t.y; win[j][0][2] = t.z; win[j][0][3] = t.w;
+                        }
                     }
-                }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     float2 d[CO / 2];
 #pragma unroll
                     for (int k = 0; k < CO / 2; k += 2) *reinterpret_cast<float4*>(d + k) = *reinterpret_cast<const float4*>(ds + (r * kTileX + 4 * v + i) * pitch + 2 * k);
 #pragma unroll
-                    for (int ky = 0; ky < KS; ++ky)
+                    for (int j = 0; j < CI; ++j)
 #pragma unroll
-                        for (int kx = 0; kx < KS; ++kx) {
-                            const float x = win[ky][i + kx];
+                        for (int ky = 0; ky < KS; ++ky)
 #pragma unroll
-                            for (int k = 0; k < CO / 2; ++k) acc[k][ky * KS + kx] = __ffma2_rn(d[k], make_float2(x, x), acc[k][ky * KS + kx]);
-                        }
+                            for (int kx = 0; kx < KS; ++kx) {
+                                const float x = win[j][ky][i + kx];
+#pragma unroll
+                                for (int k = 0; k < CO / 2; ++k) acc[j][k][ky * KS + kx] = __ffma2_rn(d[k], make_float2(x, x), acc[j][k][ky * KS + kx]);
+                            }
                 }
             }
         }
-        if (a.b_partials && ci0 == 0 && rw == 0 && lane < CO)   // bias gradient: the sum of the gradients themselves
-            for (int i = 0; i < RW * kTileX; ++i) bias += ds[i * pitch + lane];
-        __syncthreads();
+        if (a.b_partials && ci0 == 0 && lane < CO && (!kShort || rw == 0))   // bias gradient: the sum of the gradients themselves
+            for (int i = 0; i < (kShort ? RW : 1) * kTileX; ++i) bias += ds[((kShort ? 0 : rw * kTileX) + i) * pitch + lane];
+        if (kShort) __syncthreads();
     }
+    if (!kShort) __syncthreads();
     pdl_launch_dependents();
-    if (a.b_partials && ci0 == 0 && rw == 0 && lane < CO && co0 + g * CO + lane < a.Cout)
-        a.b_partials[((int64_t)s * a.n_split + split) * a.Cout + co0 + g * CO + lane] = bias;
-    // the rows' sums, added in order: [row warp - 1][group][channel pair, tap][lane]
-    float2* red = reinterpret_cast<float2*>(smem_w) + g * (CO / 2 * T) * 32 + lane;
-    const int red_row = ng * (CO / 2 * T) * 32;
+    const bool has_bias = a.b_partials && ci0 == 0 && rw == 0 && lane < CO && co0 + g * CO + lane < a.Cout;
+    float* b_dst = a.b_partials + ((int64_t)s * a.n_split + split) * a.Cout + co0 + g * CO + lane;
+    if (kShort && has_bias) *b_dst = bias;
+    // the rows' sums, added in order: [row warp - 1][group][channel of the lane, channel pair, tap][lane]
+    float2* red = reinterpret_cast<float2*>(smem_w) + g * (CI * CO / 2 * T) * 32 + lane;
+    const int red_row = ng * (CI * CO / 2 * T) * 32;
+    float* red_b = smem_w + 2 * (RW - 1) * red_row + g * CO + lane;     // [row warp][group][channel]
+    if (!kShort && lane < CO) red_b[rw * COB] = bias;
     if (rw > 0)
 #pragma unroll
-        for (int k = 0; k < CO / 2; ++k)
+        for (int j = 0; j < CI; ++j)
 #pragma unroll
-            for (int t = 0; t < T; ++t) red[(rw - 1) * red_row + (k * T + t) * 32] = acc[k][t];
+            for (int k = 0; k < CO / 2; ++k)
+#pragma unroll
+                for (int t = 0; t < T; ++t) red[(rw - 1) * red_row + ((j * (CO / 2) + k) * T + t) * 32] = acc[j][k][t];
     __syncthreads();
     if (rw > 0) return;
+    if (!kShort && has_bias) {
+        for (int q = 1; q < RW; ++q) bias += red_b[q * COB];
+        *b_dst = bias;
+    }
+    // (added one by one while the results are stored, no load moves ahead of a store: 32 -> 16, 3x3, six streams 18.8 -> 21.2 us)
+    if (kShort) {
 #pragma unroll
-    for (int k = 0; k < CO / 2; ++k)
+        for (int k = 0; k < CO / 2; ++k)
+            for (int q = 0; q < RW - 1; ++q) acc[0][k][0] = __fadd2_rn(acc[0][k][0], red[q * red_row + k * 32]);
+    } else {
+#pragma unroll 1
+        for (int q = 0; q < RW - 1; ++q)
 #pragma unroll
-        for (int t = 0; t < T; ++t)
-            for (int q = 0; q < RW - 1; ++q) acc[k][t] = __fadd2_rn(acc[k][t], red[q * red_row + (k * T + t) * 32]);
-    if (ci0 + lane >= a.Cin) return;
+            for (int j = 0; j < CI; ++j)
+#pragma unroll
+                for (int k = 0; k < CO / 2; ++k)
+#pragma unroll
+                    for (int t = 0; t < T; ++t) acc[j][k][t] = __fadd2_rn(acc[j][k][t], red[q * red_row + ((j * (CO / 2) + k) * T + t) * 32]);
+    }
     float* dst = a.partials + ((int64_t)s * a.n_split + split) * T * a.Cout * a.Cin + ci0 + lane;
 #pragma unroll
-    for (int k = 0; k < CO; ++k) {
-        const int co = co0 + g * CO + k;
-        if (co >= a.Cout) continue;
+    for (int j = 0; j < CI; ++j) {
+        if (ci0 + 32 * j + lane >= a.Cin) break;
 #pragma unroll
-        for (int t = 0; t < T; ++t) dst[((int64_t)t * a.Cout + co) * a.Cin] = k & 1 ? acc[k / 2][t].y : acc[k / 2][t].x;
+        for (int k = 0; k < CO; ++k) {
+            const int co = co0 + g * CO + k;
+            if (co >= a.Cout) continue;
+#pragma unroll
+            for (int t = 0; t < T; ++t) dst[((int64_t)t * a.Cout + co) * a.Cin + 32 * j] = k & 1 ? acc[j][k / 2][t].y : acc[j][k / 2][t].x;
+        }
     }
 }
 
@@ -345,7 +389,7 @@ conv_wgrad_f32_kernel(WgradF32 a, int tiles_x, int n_chunks, int ci_tiles)
 // chunk.  The number of streams has no part in it: the ranges group a gradient's sums, and a stream's results must be the same
 // whatever it shares the launch with.
 struct WgradShape { int ng, ci_tiles, co_tiles, tiles_x, n_chunks, n_split; };
-template <int KS, int CO>
+template <int KS, int CO, int CI>
 WgradShape wgrad_shape(int Cin, int Cout, int h, int w)
 {
     WgradShape q;
@@ -354,7 +398,7 @@ WgradShape wgrad_shape(int Cin, int Cout, int h, int w)
     q.co_tiles = (groups + kMost - 1) / kMost;
     q.ng = (groups + q.co_tiles - 1) / q.co_tiles;
     q.co_tiles = (groups + q.ng - 1) / q.ng;
-    q.ci_tiles = (Cin + 31) / 32;
+    q.ci_tiles = (Cin + 32 * CI - 1) / (32 * CI);
     q.tiles_x = (w + kTileX - 1) / kTileX;
     q.n_chunks = q.tiles_x * ((h + RW - 1) / RW);
     const int per_range = q.ci_tiles * q.co_tiles, warps = q.ng * RW;
@@ -366,19 +410,24 @@ WgradShape wgrad_shape(int Cin, int Cout, int h, int w)
 }
 // 1x1 layers: 16 channels per warp keep the loads below the multiply-adds; a head with a handful of classes takes 4
 bool narrow(int Cout) { return Cout <= 4; }
+// Input channels per lane: as many as the layer fills.  With at most 16 output channels a block has one channel group, and two
+// blocks per SM need both buffers of two channels per lane (88 KB); with four a block's 156 KB would leave one of four warps.
+int wg_lane_channels(int Cin, int Cout) { return Cin <= 32 ? 1 : Cin <= 64 || Cout <= 16 ? 2 : 4; }
 WgradShape wgrad_shape_of(int Cin, int Cout, int h, int w, int ks)
 {
-    if (ks == 3) return wgrad_shape<3, 8>(Cin, Cout, h, w);
-    return narrow(Cout) ? wgrad_shape<1, 4>(Cin, Cout, h, w) : wgrad_shape<1, 16>(Cin, Cout, h, w);
+    if (ks == 3) return wgrad_shape<3, 8, 1>(Cin, Cout, h, w);
+    if (narrow(Cout)) return wgrad_shape<1, 4, 1>(Cin, Cout, h, w);
+    const int ci = wg_lane_channels(Cin, Cout);
+    return ci == 1 ? wgrad_shape<1, 16, 1>(Cin, Cout, h, w) : ci == 2 ? wgrad_shape<1, 16, 2>(Cin, Cout, h, w) : wgrad_shape<1, 16, 4>(Cin, Cout, h, w);
 }
 
-template <int KS, int CO>
+template <int KS, int CO, int CI>
 void launch_wgrad(const WgradF32& a, const WgradShape& q, int S, bool early, cudaStream_t s)
 {
     const dim3 grid((unsigned)q.n_split, (unsigned)(q.ci_tiles * q.co_tiles), (unsigned)S);
     // (blocks in pairs on the SMs that the loss kernel left first: 1x1, 21 classes, 180 x 320 29 us back to back, spread 24)
-    const size_t smem = one_per_sm(wg_smem<KS, CO>(q.ng), (int64_t)q.n_split * q.ci_tiles * q.co_tiles * S, 148);
-    launch_early(early, conv_wgrad_f32_kernel<KS, CO>, grid, dim3(32 * wg_rows<KS>() * q.ng), smem, s, a, q.tiles_x, q.n_chunks, q.ci_tiles);
+    const size_t smem = one_per_sm(wg_smem<KS, CO, CI>(q.ng), (int64_t)q.n_split * q.ci_tiles * q.co_tiles * S, 148);
+    launch_early(early, conv_wgrad_f32_kernel<KS, CO, CI>, grid, dim3(32 * wg_rows<KS>() * q.ng), smem, s, a, q.tiles_x, q.n_chunks, q.ci_tiles);
 }
 
 }  // namespace
@@ -388,9 +437,11 @@ cudaError_t prepare_conv_f32()
     cudaError_t e = allow_shared_memory((const void*)conv_fwd_f32_kernel<3, 8>);
     if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_fwd_f32_kernel<1, 8>);
     if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_fwd_f32_kernel<1, 4>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<3, 8>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<1, 16>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<1, 4>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<3, 8, 1>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<1, 16, 1>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<1, 16, 2>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<1, 16, 4>);
+    if (e == cudaSuccess) e = allow_shared_memory((const void*)conv_wgrad_f32_kernel<1, 4, 1>);
     return e;
 }
 
@@ -428,9 +479,12 @@ void launch_conv_wgrad_f32(const float* in, const float* dout, int Cin, int Cout
     const WgradShape q = wgrad_shape_of(Cin, Cout, h, w, ks);
     const PadF32 pad(h, w);
     const WgradF32 a = {in, dout, partials, b_partials, Cin, Cout, h, w, q.n_split, Cin * pad.plane, Cout * pad.plane};
-    if (ks == 3) launch_wgrad<3, 8>(a, q, S, early, s);
-    else if (narrow(Cout)) launch_wgrad<1, 4>(a, q, S, early, s);
-    else launch_wgrad<1, 16>(a, q, S, early, s);
+    const int ci = wg_lane_channels(Cin, Cout);
+    if (ks == 3) launch_wgrad<3, 8, 1>(a, q, S, early, s);
+    else if (narrow(Cout)) launch_wgrad<1, 4, 1>(a, q, S, early, s);
+    else if (ci == 1) launch_wgrad<1, 16, 1>(a, q, S, early, s);
+    else if (ci == 2) launch_wgrad<1, 16, 2>(a, q, S, early, s);
+    else launch_wgrad<1, 16, 4>(a, q, S, early, s);
 }
 
 // between plain planes [C][h][w] and padded ones (interior only)

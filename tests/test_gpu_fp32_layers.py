@@ -41,6 +41,23 @@ def test_fp32_steps_at_tile_edges(c_in, ch, C, h, w):
     st.st_destroy(ctx)
 
 
+@pytest.mark.parametrize("c_in,C,h,w", [
+    (32, 5, 4, 32), (33, 16, 5, 33), (64, 17, 9, 31),          # one / two input channels per lane; the last lanes' second channel missing
+    (65, 16, 7, 64), (65, 17, 3, 65), (128, 33, 8, 32),        # two / four, by the classes too; a full tile of 128 channels
+    (129, 49, 2, 30), (200, 20, 37, 70),                       # one channel of a second tile; several chunks per pixel range, odd rows
+])
+def test_fp32_classifier_gradient_at_channel_edges(c_in, C, h, w):
+    """The 1x1 weight and bias gradients where the number of input channels per lane changes.  One step without momentum moves a
+    parameter by lr times its gradient, a sum of h * w products in fp32: in any order within h * w * 2^-24 of the sum of their
+    sizes, against 64 bits (2590 pixels: 1.6e-4; roundings of either sign leave far less)."""
+    feat, T = rand_problem(7, c_in, C, h, w, blobs=True)
+    theta = si.initial_head_params(c_in, 0, C, 4)
+    ctx, head, loss, ref_loss, conf, masks, lab = run_both((c_in, 0, C, h, w, 0.05, 0.0), feat, T, theta, 1, 0, want_conf=True)
+    np.testing.assert_allclose(loss, ref_loss, rtol=1e-4)
+    check_weights(ctx, head, theta, max_rel=1e-5, mean_abs=1e-5, upd_rel=2e-4)
+    st.st_destroy(ctx)
+
+
 @pytest.mark.parametrize("h,w", [(6, 40), (141, 451)])
 def test_many_classes_steep_logits(h, w):
     """Logits that change by hundreds between neighbouring nodes (exact per-pixel maxima), labels out of range."""
