@@ -18,15 +18,15 @@ bool fused_forward_supported(int C, int h, int w, int c_in)
     return C <= kClassPad && c_in >= 64 && c_in % 64 == 0 && c_in / 64 <= fused::kMaxKBlocks && w >= F_COLS && h >= F_ROWS;
 }
 
-bool upsample_ce_rows_supported(int C) { return C <= kClassPad; }
+bool upsample_ce_few_supported(int C) { return C <= kClassPad; }
 
-int upsample_ce_rows_blocks(int h, int w) { return ((h + FN_Y - 1) / FN_Y) * ((w + FN_X - 1) / FN_X); }
+int upsample_ce_few_blocks(int h, int w) { return ((h + FN_Y - 1) / FN_Y) * ((w + FN_X - 1) / FN_X); }
 
 cudaError_t prepare_fwd_ce(int C) { return fwd_ce_kernels(C).prepare(); }
 
 void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s) { fwd_ce_kernels(a.C).launch[1](a, x_map, w_map, s); }
 
-void launch_upsample_ce_rows(const UpsampleCeArgs& a, cudaStream_t s)
+void launch_upsample_ce_few(const UpsampleCeArgs& a, cudaStream_t s)
 {
     UpsampleCeArgs b = a;
     b.x_early = 0;

@@ -66,13 +66,13 @@ constexpr int kLogitCols = 4 * kClassPad;                                   // t
 // Shared memory.  PREFETCH: slot A of the ring is its own, slot B lies over the warps' slots and serves the block's first tile
 // only (nobody has written there yet); the counts are cleared by the threads that read them.  Otherwise a block works on one tile
 // and both slots lie over its arrays.  The line is where two blocks no longer fit an SM with a slot to themselves (from 23
-// classes): 4 streams at 720p, 22 classes 68 us with the slot, 24 classes 83 us without.
+// classes, with the confusion matrix from 22): 4 streams at 720p, 22 classes 68 us with the slot, 24 classes 83 us without.
 template <int C, bool CONF, bool FORWARD>
 struct FwdCeSmem {
     static constexpr size_t kSlots = (size_t)F_WARPS * C * 32 * sizeof(float2), kCounts = (size_t)((C + 1) / 2) * kNodes * sizeof(uint32_t),
                             kHist = CONF ? (size_t)C * C * sizeof(unsigned int) : 0, kWeights = (size_t)fused::kMaxKBlocks * kWBytes,
                             kSlotsOrB = kSlots > kSliceBytes ? (kSlots + 1023) / 1024 * 1024 : kSliceBytes;
-    static constexpr size_t kHalfSm = 115712 - 2048;    // what two blocks on an SM leave each, less the static arrays
+    static constexpr size_t kHalfSm = 115712 - 2176;    // what two blocks on an SM leave each, less the static arrays
     static constexpr bool kPrefetch = FORWARD && kSliceBytes + kSlotsOrB + kWeights + kCounts + kHist + 1024 <= kHalfSm;
     static constexpr size_t kArrays = kSlots + kCounts + kHist;
     static constexpr size_t kSlotsAt = kPrefetch ? kSliceBytes : 0, kSliceB = kSliceBytes,
@@ -620,7 +620,8 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
         if (l == 0) red[n_done & 1][wi] = loss;            // (two of them: warps may be one tile ahead of the one that adds)
         if (n_bad) atomicAdd(a.bad, n_bad);
         if (!workers_all(ok)) return;                      // block-uniform: a wait ran out, nothing is written
-        if (t + (int)gridDim.x >= n_tiles) pdl_launch_dependents();        // only the epilogue is left
+        if (t + (int)gridDim.x >= n_tiles) pdl_launch_dependents();        // only the epilogue is left (with FORWARD the ninth warp has let
+                                                                           // the successor go when the last logits were taken)
         if (CONF) {                                        // one global update per non-empty counter of the tile
             for (int e = tid; e < C * C; e += F_WORKERS) {
                 const unsigned int v = hist[e];

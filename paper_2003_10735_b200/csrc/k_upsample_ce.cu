@@ -404,21 +404,21 @@ void launch_many(const UpsampleCeArgs& a, cudaStream_t s)
 
 int upsample_ce_blocks(int h, int w, int C)
 {
-    if (upsample_ce_rows_supported(C)) return upsample_ce_rows_blocks(h, w);
+    if (upsample_ce_few_supported(C)) return upsample_ce_few_blocks(h, w);
     const int ny = many_shape(h, w).own_y;
     return ((h + ny - 1) / ny) * ((w + kOwnX - 1) / kOwnX);
 }
 
 cudaError_t prepare_upsample_ce(int C)
 {
-    if (upsample_ce_rows_supported(C)) return prepare_fwd_ce(C);
+    if (upsample_ce_few_supported(C)) return prepare_fwd_ce(C);
     const cudaError_t e = allow_many<7, 2>();
     return e != cudaSuccess ? e : allow_many<4, 3>();
 }
 
 void launch_upsample_ce(const UpsampleCeArgs& a, cudaStream_t s)
 {
-    if (upsample_ce_rows_supported(a.C)) { launch_upsample_ce_rows(a, s); return; }
+    if (upsample_ce_few_supported(a.C)) { launch_upsample_ce_few(a, s); return; }
     if (many_shape(a.h, a.w).own_y == 7) launch_many<7, 2>(a, s);
     else launch_many<4, 3>(a, s);
 }

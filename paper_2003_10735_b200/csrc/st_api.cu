@@ -593,7 +593,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
     if (d.object_weight > 1) {
         if (d.object_radius < 0 || d.background_class < 0 || d.background_class >= d.n_classes)
             return fail(nullptr, ST_ERR_INVALID_ARG, "st_init_head: loss weighting needs object_radius >= 0 and a background class below n_classes");
-        if (d.object_weight > 5 || d.object_radius > 64 || !upsample_ce_rows_supported(d.n_classes))
+        if (d.object_weight > 5 || d.object_radius > 64 || !upsample_ce_few_supported(d.n_classes))
             return fail(nullptr, ST_ERR_UNSUPPORTED, "st_init_head: loss weighting covers weights 2..5, radii up to 64 and at most 32 classes");
     }
     if (d.gemm_precision != 0 && d.gemm_precision != 1)

@@ -148,9 +148,9 @@ void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUte
 // Tile map of bf16 features [S][h][w][c_in] for it: {c_in, w, h, S}, one box = 64 channels of a tile
 bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w);
 // the part of launch_upsample_ce for C <= 32 (k_fwd_ce.cuh)
-bool upsample_ce_rows_supported(int C);
-int upsample_ce_rows_blocks(int h, int w);
-void launch_upsample_ce_rows(const UpsampleCeArgs& a, cudaStream_t s);
+bool upsample_ce_few_supported(int C);
+int upsample_ce_few_blocks(int h, int w);
+void launch_upsample_ce_few(const UpsampleCeArgs& a, cudaStream_t s);
 // student mask: argmax_c of the upsampled logits, uint8 [H][W]; with `labels` also the confusion matrix of
 // (label, mask) added into `conf`, and with `miou` the mean IoU written by the last block (k_student_mask.cu)
 struct StudentMaskArgs {
