@@ -163,8 +163,11 @@ tc_wgrad1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}      
 {
     // Train: the block after the last one of the weight gradient assesses the prediction (metric, best so far, break)
     // while the others multiply; it takes no part in anything below
+    // The streams from the last to the first, as the loss kernel walks them from the first to the last: what it has left in L2 is read
+    // from there, and so is what this kernel leaves by the next loss kernel.  us of a call of eight steps, 256 channels 180 x 320, first to
+    // last / last to first: 4 streams 960 / 931, 8 1849 / 1799, 16 3513 / 3521; 128 channels, 6 streams 1146 / 1124.
+    const int s = (int)gridDim.y - 1 - (int)blockIdx.y;
     if (has_ctl && blockIdx.x == gridDim.x - 1) {
-        const int s = blockIdx.y;
         const TrainHistory hist = train_history(ctl, s);
         pdl_wait();
         bool stop, better;
@@ -187,7 +190,7 @@ tc_wgrad1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}      
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const int s = blockIdx.y, split = (int)blockIdx.x / m_split, n_split = n_blocks_x / m_split;
+    const int split = (int)blockIdx.x / m_split, n_split = n_blocks_x / m_split;
     const int c_begin = split * chunks_per_block;
     const int c_end = min(n_chunks, c_begin + chunks_per_block);
 
@@ -213,7 +216,7 @@ tc_wgrad1x1_kernel(const __grid_constant__ CUtensorMap tmA,   // {K, p, S}      
                 tma_load_3d(sa + cb * (kChunkPix * 128), &tmA, bar, (2 * m0 + cb) * kBlockK, (c_begin + it) * kChunkPix, s);
         }
     pdl_wait();                  // inputs come from the previous kernel of the step
-    if (skip && skip[(int64_t)blockIdx.y * skip_stride]) {     // this stream's training loop has ended (block-uniform; the flag
+    if (skip && skip[(int64_t)s * skip_stride]) {     // this stream's training loop has ended (block-uniform; the flag
         tc_fence_before_sync();                                 // comes from an earlier kernel, so it is read after the wait)
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, tmem_cols);
