@@ -174,13 +174,15 @@ __device__ __forceinline__ void update_stream(const UpdateArgs& a, const LayerUp
 // Parameter blocks: a block covers kUpdThreads / G consecutive parameters; the G thread groups of a
 // block each sum every G-th split-K partial of "their" parameter (coalesced along the parameters),
 // the group sums are added in group order through shared memory, and group 0 applies the update.
-template <int G, int E, bool ADAM>
-__global__ void __launch_bounds__(kUpdThreads)
+// `B` of its loads are in flight at a time.  With DECIDES (Train) a block has one warp more, which assesses the prediction meanwhile.
+template <int G, int E, int B, bool ADAM, bool DECIDES>
+__global__ void __launch_bounds__(kUpdThreads + (DECIDES ? 32 : 0))
 sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
 {
     constexpr int kRow = kUpdThreads / G;      // consecutive parameters covered by one thread group
     constexpr int kPer = kRow * E;             // parameters per block
     __shared__ float part[G][kPer];
+    __shared__ int verdict;
     const int s = blockIdx.y;
     const int64_t base = (int64_t)s * a.n_params;
     if ((int)blockIdx.x >= n_grouped) {                  // the streamed layers' blocks lie behind the grouped ones
@@ -227,20 +229,31 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
     if (a.has_ctl) hist = train_history(a.ctl, s);
     pdl_wait();
     pdl_launch_dependents();
+    if (DECIDES) {
+        if (hist.ended && blockIdx.x != 0 && param_block) return;
+        if (threadIdx.x >= kUpdThreads) {
+            bool stop, best;
+            train_decision_warp(a.ctl, s, blockIdx.x == 0, hist, stop, best);
+            if ((threadIdx.x & 31) == 0) verdict = (stop ? 1 : 0) | (best ? 2 : 0);
+            __syncthreads();
+            return;
+        }
+    }
     bool skip = a.skip && a.skip[(int64_t)s * a.skip_stride];   // block-uniform
     bool better = false;                                         // Train: this prediction is the best so far
     MiouFetch fetched{};
-    const bool decide_here = a.has_ctl == 1;                     // 2: the backward before this kernel has assessed the prediction
+    const bool decide_here = a.has_ctl == 1 && !DECIDES;                     // 2: the backward before this kernel has assessed the prediction
     if (decide_here) fetched = train_fetch(a.ctl, s, hist);      // on their way while the partial sums are fetched and added
     if (a.has_ctl == 2 && !hist.ended) train_outcome(a.ctl, s, skip, better);
     float* best_theta = a.has_ctl ? a.ctl.best_theta : nullptr;
     const AdamCorr corr = adam_corrections<ADAM>(a, s);
     if (param_block) {
         if (a.has_ctl && hist.ended) {                  // nothing to assess, nothing to update: the history goes on
+            if (DECIDES) __syncthreads();
             if (decide_here) train_decision(a.ctl, s, blockIdx.x == 0, hist, &fetched, skip, better);
             return;
         }
-        if (skip && !decide_here && !better) return;
+        if (skip && !decide_here && !DECIDES && !better) return;
         float sum[E];
         // E parameters per thread, all of their split-K loads issued before any is consumed
 #pragma unroll
@@ -249,17 +262,17 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
             if (layer[e] >= 0) {
                 const LayerUpdate& ly = a.layer[layer[e]];
                 const float* src = ly.w_partials + (int64_t)s * ly.w_stream_stride + (param[e] - ly.w_off);
-                // batches of 8 predicated loads: all in flight together, no one-at-a-time remainder loop
+                // batches of predicated loads: all in flight together, no one-at-a-time remainder loop
                 float t = 0.f;
-                for (int k0 = g; k0 < ly.n_split; k0 += 8 * G) {
-                    float v[8];
+                for (int k0 = g; k0 < ly.n_split; k0 += B * G) {
+                    float v[B];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
+                    for (int j = 0; j < B; ++j) {
                         const int k = k0 + j * G;
                         v[j] = k < ly.n_split ? __ldg(src + (int64_t)k * ly.w_split_stride) : 0.f;
                     }
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) t += v[j];
+                    for (int j = 0; j < B; ++j) t += v[j];
                 }
                 sum[e] = t;
             }
@@ -268,6 +281,7 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
         for (int e = 0; e < E; ++e) part[g][e * kRow + col] = sum[e];
         if (decide_here) train_decision(a.ctl, s, blockIdx.x == 0, hist, &fetched, skip, better);
         __syncthreads();
+        if (DECIDES) { skip = (verdict & 1) != 0; better = (verdict & 2) != 0; }
         if (g != 0 || (skip && !better)) return;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -287,31 +301,39 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
     else if (a.has_ctl && hist.ended) skip = true;
     const int warp = ((int)blockIdx.x - n_param_blocks) * (kUpdThreads / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    int item = warp;
-    for (int L = 0; L < a.n_layers; ++L) {
-        const LayerUpdate& ly = a.layer[L];
-        if (item < ly.cout) {
-            const float* src = ly.b_partials + (int64_t)s * ly.n_bpart * ly.cout + item;
-            float g = 0.f;
-            for (int k0 = lane; k0 < ly.n_bpart; k0 += 8 * 32) {
-                float v[8];
+    int item = warp, of = -1;                            // of: the layer whose bias element `item` is
+    for (int L = 0; L < a.n_layers && of < 0; ++L) {
+        if (item < a.layer[L].cout) of = L;
+        else item -= a.layer[L].cout;
+    }
+    float g_bias = 0.f;
+    if (of >= 0) {
+        const LayerUpdate& ly = a.layer[of];
+        const float* src = ly.b_partials + (int64_t)s * ly.n_bpart * ly.cout + item;
+        for (int k0 = lane; k0 < ly.n_bpart; k0 += 8 * 32) {
+            float v[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int k = k0 + j * 32;
-                    v[j] = k < ly.n_bpart ? __ldg(src + (int64_t)k * ly.cout) : 0.f;
-                }
-#pragma unroll
-                for (int j = 0; j < 8; ++j) g += v[j];
+            for (int j = 0; j < 8; ++j) {
+                const int k = k0 + j * 32;
+                v[j] = k < ly.n_bpart ? __ldg(src + (int64_t)k * ly.cout) : 0.f;
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-            if (lane == 0) {
-                if (better) best_theta[base + ly.b_off + item] = a.theta[base + ly.b_off + item];
-                if (!skip) apply_update<ADAM>(a, base + ly.b_off + item, g, corr);
-            }
-            return;
+            for (int j = 0; j < 8; ++j) g_bias += v[j];
         }
-        item -= ly.cout;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) g_bias += __shfl_xor_sync(0xffffffffu, g_bias, o);
+    }
+    if (DECIDES) {
+        __syncthreads();
+        skip = (verdict & 1) != 0; better = (verdict & 2) != 0;
+    }
+    if (of >= 0) {
+        const int64_t at = base + a.layer[of].b_off + item;
+        if (lane == 0) {
+            if (better) best_theta[at] = a.theta[at];
+            if (!skip) apply_update<ADAM>(a, at, g_bias, corr);
+        }
+        return;
     }
     if (item == 0 && a.loss_part) {
         double t = 0.0;
@@ -366,12 +388,16 @@ static int launch_sgd_update_t(const UpdateArgs& a, cudaStream_t s)
     const int n_param_blocks = (int)((n_rest + per - 1) / per);
     const int n_grouped = n_param_blocks + n_red_blocks;
     const dim3 grid((unsigned)(n_grouped + stream_blocks), (unsigned)a.S);
-    const dim3 blk(kUpdThreads);
-    if (G == 1 && E == 1) launch_early(a.chain_early != 0, sgd_update_kernel<1, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
-    else if (G == 1) launch_early(a.chain_early != 0, sgd_update_kernel<1, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
-    else if (G == 16) launch_early(a.chain_early != 0, sgd_update_kernel<16, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
-    else if (E == 1) launch_early(a.chain_early != 0, sgd_update_kernel<8, 1, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
-    else launch_early(a.chain_early != 0, sgd_update_kernel<8, 4, ADAM>, grid, blk, 0, s, g, n_param_blocks, n_grouped);
+    const bool early = a.chain_early != 0, decides = a.has_ctl == 1 && a.ctl.C <= kWarpClasses && stream_blocks == 0 && !big;
+    auto launch = [&](auto kernel) { launch_early(early, kernel, grid, dim3(kUpdThreads + (decides ? 32 : 0)), 0, s, g, n_param_blocks, n_grouped); };
+    // (a batch of loads is a round trip: 286 partial sums take one with twenty, three with eight)
+    const bool many = G == 16 && max_split > 16 * 8;
+    if (G == 1 && E == 4) launch(sgd_update_kernel<1, 4, 8, ADAM, false>);
+    else if (E == 4) launch(sgd_update_kernel<8, 4, 8, ADAM, false>);
+    else if (G == 1) launch(decides ? sgd_update_kernel<1, 1, 8, ADAM, true> : sgd_update_kernel<1, 1, 8, ADAM, false>);
+    else if (G == 8) launch(decides ? sgd_update_kernel<8, 1, 8, ADAM, true> : sgd_update_kernel<8, 1, 8, ADAM, false>);
+    else if (many) launch(decides ? sgd_update_kernel<16, 1, 20, ADAM, true> : sgd_update_kernel<16, 1, 20, ADAM, false>);
+    else launch(decides ? sgd_update_kernel<16, 1, 8, ADAM, true> : sgd_update_kernel<16, 1, 8, ADAM, false>);
     return 1;
 }
 
