@@ -5,20 +5,24 @@
 //
 // Geometry.  With half-pixel centres and factor 4 the frame pixels 4n+2 .. 4n+5 lie between node columns n and n+1 ("cell" n)
 // with weights 1/8, 3/8, 5/8, 7/8 toward n+1; rows alike.  Cells -1 and w-1 are the clamped borders (their outer node is the
-// inner one).  A tile owns 7 rows x 30 columns of nodes.  Eight warps work on it: warp i owns cell row y0-1+i (the 4 x 4 frame
+// inner one).  A tile owns 7 rows x 30 columns of nodes.  A group of eight warps works on it: warp i owns cell row y0-1+i (the 4 x 4 frame
 // pixels between two node rows), lane l owns node column x0-1+l and the 16 pixels of the cell to its right.  Warp 0, lane 0 and
 // lane 31 are halo (recomputed by the neighbouring tile), so that a tile's nodes are finished in a fixed summation order,
 // without floating-point atomics.
 //
-// Logits with FORWARD.  A ninth warp feeds the tensor core: the features of the tile's 9 x 32 nodes arrive in 64-channel slices (one 4-d tile
-// copy each; nodes outside the map arrive as zeros), and four multiplications per 16 channels leave node row i of the tile and
-// node row i+1 of it in the same 32 tensor-memory lanes: the two rows that warp i's cells lie between.  A warp therefore takes
-// its logits out of tensor memory alone, without the other warps: bias added, shifted by the largest of them, in log2 units,
-// clamped at the frame's border, both rows of a class side by side in the warp's own slots of shared memory
-// [class][lane] (upper, lower).  The second class sweep leaves the cell's pull on the two node rows in the same slots.
-// Blocks are persistent where there are more tiles than blocks fit: once the eight warps have emptied the tensor memory, the
-// ninth multiplies the next tile, whose slices arrive while this one is worked on.  Without FORWARD a warp reads its two node rows
-// from memory (all classes' loads in flight together) and a block works on one tile.
+// With FORWARD a block has an SM to itself and is persistent: two groups take its tiles in turn, a producer feeds a ring of chunks by
+// TMA, and two issuers (a thread each) feed the tensor core.
+//   Logits.  The features of the tile's 9 x 32 nodes arrive in chunks of 64 channels and five node rows (nodes outside the map arrive
+//   as zeros), and four multiplications per 16 channels leave node row i of the tile and node row i+1 of it in the same 32
+//   tensor-memory lanes: the two rows that warp i's cells lie between.  A warp therefore takes its logits out of tensor memory
+//   alone, without the other warps: bias added, shifted by the largest of them, in log2 units, clamped at the frame's border, both rows of
+//   a class side by side in the warp's own slots of shared memory [class][lane] (upper, lower).  The second class sweep leaves the
+//   cell's pull on the two node rows in the same slots.  A group's next tile is fetched and multiplied while it works on this one.
+//   Weight gradient of a one-layer head (w_part).  The epilogue leaves the bf16 gradient of the tile's own nodes in shared memory as an operand, the
+//   features come once more, from L2, and their product (reduction over the nodes) becomes one partial sum per tile, which the update adds in
+//   order.  A kernel of its own read the map again instead, from HBM where it is more than L2 holds, behind one more kernel boundary.
+// Without FORWARD a block is one group with one tile, and a warp reads its two node rows from memory (all classes' loads in flight
+// together).
 //
 // Fast path (the usual case), class by class for all 16 pixels of a cell: inside a cell the interpolated logit is
 // u(r,k) = A + B k + G r + D k r, so its 16 exponentials are geometric progressions (cell_softmax.cuh).  Sweep 1 sums them per
@@ -33,14 +37,15 @@
 // gradient, and reduces the tile's share of the bias gradient.  With CONF the student's class of every pixel is taken from sweep
 // 1 and counted against the label.
 //
-// Bound by latency and issue slots at 16 working warps an SM (half of the slots, 0.47 of the multiply-add pipe, a third of the
-// shared-memory path go to the sweeps); in a single wave the forward's 2.5 us lie in front.  One launch, us, with each block
-// fetching, multiplying and exchanging its tile through shared memory before the sweeps / now: 720p, 256 channels, 21 classes
-// 23.4 / 21.1, 16 streams of it 316 / 227 (the fetch and the products, 13000 of 33400 cycles a tile, run beside the sweeps of the
-// tile before); 128 channels at 90 x 160 17.1 / 14.8; 32 classes, where one block fitted an SM, 39.8 / 29.6; 27 classes, 4 streams
-// 152 / 89.  Behind a 3x3 layer (720p, 256 channels; a forward kernel of its own and a loss kernel that exchanged the logits through
-// shared memory / now) 26.1 / 21.2, 1080p 57 / 46.  Stored logits: 21 classes at 720p 15.4 / 14.8, 30 classes (fp32) 26.1 / 19.1.
-// Seven classes per iteration of sweep 1 instead of three: 232 -> 227.
+// Bound by latency and issue slots at 16 working warps an SM (half of the slots go to the sweeps), and at a launch's start by L2, from
+// which every block fetches two tiles (47 MB for one 720p frame of 256 channels): the first group has its logits after 8000 cycles, the
+// second after 12800.  us of a call of eight steps with two blocks of one group on an SM, a warp each to feed the tensor core and a kernel of its own for the
+// weight gradient / now, 256 channels on 180 x 320, 21 classes: 275.8 / 267.6, 4 streams 963 / 856, 16 streams 3535 / 3248; 30 classes (weight
+// gradient apart), 4 streams 1274 / 1137; 32 classes 351 / 330; 4 classes 201 / 184; 128 channels on 90 x 160 156.7 / 146.8.  Behind a 3x3 layer (no weight
+// gradient) it is the same within 1 %: 720p, 64 channels 16.9 / 16.7 us a launch, 1080p, 256 channels 43.9 / 45.8.
+// Tried: one group whose warps divide the classes (sums and labels are then worked out twice: 222 -> 370 us for 16 streams); places of the
+// ring over both groups' slots for a block's first tile (no change: L2 sets the pace); bias sums through shared memory (one more
+// barrier: 3250 -> 3280).
 #pragma once
 
 #include "st_internal.h"
@@ -57,28 +62,37 @@ namespace {
 
 constexpr int F_ROWS = fused::kTileRows, F_COLS = fused::kTileCols;         // nodes of a tile, halo included
 constexpr int FN_Y = fused::kOwnRows, FN_X = fused::kOwnCols;               // nodes a tile owns
-constexpr int F_WARPS = FN_Y + 1, F_WORKERS = F_WARPS * 32, F_THREADS = F_WORKERS + 32;
+constexpr int F_WARPS = FN_Y + 1, F_WORKERS = F_WARPS * 32;                 // of a group: the warps that work on one tile
+constexpr int kGroups = 2, kAllWarps = kGroups * F_WARPS, F_THREADS = kGroups * F_WORKERS + 128;   // with FORWARD; without, one group
 constexpr int kNodes = F_ROWS * F_COLS;
 constexpr int kSweep1 = 7, kSweep2 = 3;                                     // classes per iteration of the two sweeps
-constexpr uint32_t kSliceBytes = fused::kStageBytes, kWBytes = fused::kWeightBytes;
-constexpr int kLogitCols = 4 * kClassPad;                                   // tensor memory: upper and lower rows of warps 0-3 and 4-7
+constexpr uint32_t kWBytes = fused::kWeightBytes;
+constexpr uint32_t kRowBytes = F_COLS * 128;                                // a node row of 64 channels
+constexpr uint32_t kChunkBytes = 5 * kRowBytes;                             // a place of the ring
+constexpr int kLogitCols = 4 * kClassPad, kGradCols = 2 * kClassPad;        // tensor memory of a group: upper and lower rows of warps 0-3 and
+                                                                            // 4-7; the weight gradient of 256 channels
+constexpr int kMaxPlaces = 7, kIssuers = 2;
+// Registers with FORWARD.  Warps beyond sixteen put five on a scheduler, whose 16384 registers then give 96 a thread at launch; the
+// warpgroup of the producer and the issuer (its two others return at once) gives back what the sixteen take.
+constexpr int kLaunchRegs = 96, kWorkerRegs = 112, kFeederRegs = 32;
+static_assert(kGroups * F_WORKERS * kWorkerRegs + 128 * kFeederRegs <= F_THREADS * kLaunchRegs, "registers handed on are registers the block was launched with");
 
-// Shared memory.  PREFETCH: slot A of the ring is its own, slot B lies over the warps' slots and serves the block's first tile
-// only (nobody has written there yet); the counts are cleared by the threads that read them.  Otherwise a block works on one tile
-// and both slots lie over its arrays.  The line is where two blocks no longer fit an SM with a slot to themselves (from 23
-// classes, with the confusion matrix from 22): 4 streams at 720p, 22 classes 68 us with the slot, 24 classes 83 us without.
+// Shared memory.  With FORWARD a block has an SM to itself: the ring, then the two groups' arrays.  The ring's places go on over the
+// second group's slots, which are free until that group has its first logits (and for good where the block has one tile).
 template <int C, bool CONF, bool FORWARD>
 struct FwdCeSmem {
     static constexpr size_t kSlots = (size_t)F_WARPS * C * 32 * sizeof(float2), kCounts = (size_t)((C + 1) / 2) * kNodes * sizeof(uint32_t),
-                            kHist = CONF ? (size_t)C * C * sizeof(unsigned int) : 0, kWeights = (size_t)fused::kMaxKBlocks * kWBytes,
-                            kSlotsOrB = kSlots > kSliceBytes ? (kSlots + 1023) / 1024 * 1024 : kSliceBytes;
-    static constexpr size_t kHalfSm = 115712 - 2176;    // what two blocks on an SM leave each, less the static arrays
-    static constexpr bool kPrefetch = FORWARD && kSliceBytes + kSlotsOrB + kWeights + kCounts + kHist + 1024 <= kHalfSm;
-    static constexpr size_t kArrays = kSlots + kCounts + kHist;
-    static constexpr size_t kSlotsAt = kPrefetch ? kSliceBytes : 0, kSliceB = kSliceBytes,
-                            kWeightsAt = kPrefetch ? kSliceBytes + kSlotsOrB : (kArrays > 2 * kSliceBytes ? (kArrays + 1023) / 1024 * 1024 : 2 * kSliceBytes),
-                            kCountsAt = kPrefetch ? kWeightsAt + kWeights : kSlots, kHistAt = kCountsAt + kCounts,
-                            kEnd = !FORWARD ? kArrays : kPrefetch ? kHistAt + kHist : kWeightsAt + kWeights, kBytes = kEnd + 1024;
+                            kHist = CONF ? (size_t)C * C * sizeof(unsigned int) : 0, kWeights = FORWARD ? (size_t)fused::kMaxKBlocks * kWBytes : 0;
+    static constexpr int kN = FORWARD ? kGroups : 1;
+    static constexpr size_t kGrad = FORWARD && classifier_gradient_fits(C) ? (size_t)4 * kWBytes : 0;     // bf16 gradient of a tile's own nodes: [two node rows][32 classes][64 nodes]
+    static constexpr size_t kFixed = kN * (kSlots + kCounts + kHist + kGrad) + kWeights;
+    static constexpr size_t kMost = 227 * 1024 - 1024 - 4864;                // less the alignment and the static arrays
+    static constexpr int kSteady = !FORWARD ? 0 : (kMost - kFixed) / kChunkBytes > 4 ? 4 : (int)((kMost - kFixed) / kChunkBytes);
+    static constexpr int kExtra = !FORWARD ? 0 : kSteady + (int)(kSlots / kChunkBytes) > kMaxPlaces ? kMaxPlaces - kSteady : (int)(kSlots / kChunkBytes);
+    static_assert(!FORWARD || kSteady >= 1, "a block's shared memory");
+    // the second group's slots lie behind the ring, the first group's behind them
+    static constexpr size_t kSlotsAt = kSteady * (size_t)kChunkBytes, kWeightsAt = kSlotsAt + kN * kSlots, kGradAt = kWeightsAt + kWeights,
+                            kCountsAt = kGradAt + kN * kGrad, kHistAt = kCountsAt + kN * kCounts, kBytes = kHistAt + kN * kHist + 1024;
 };
 
 __device__ __forceinline__ float lg2_approx(float x)
@@ -88,12 +102,13 @@ __device__ __forceinline__ float lg2_approx(float x)
     return y;
 }
 __device__ __forceinline__ void arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
-__device__ __forceinline__ void workers_sync() { asm volatile("barrier.cta.sync 1, %0;" ::"n"(F_WORKERS) : "memory"); }
-__device__ __forceinline__ bool workers_all(bool ok)
+// the warps of a group
+__device__ __forceinline__ void workers_sync(int grp) { asm volatile("barrier.cta.sync %0, %1;" ::"r"(1 + grp), "n"(F_WORKERS) : "memory"); }
+__device__ __forceinline__ bool workers_all(int grp, bool ok)
 {
     int r;
-    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-                 : "=r"(r) : "r"((int)ok), "n"(F_WORKERS) : "memory");
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, %3, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r) : "r"((int)ok), "n"(F_WORKERS), "r"(1 + grp) : "memory");
     return r != 0;
 }
 
@@ -141,158 +156,257 @@ __device__ __forceinline__ void add_counts(uint32_t* node, int cls, int right, i
 }
 
 template <int C, bool CONF, bool FORWARD>
-__global__ void __launch_bounds__(FORWARD ? F_THREADS : F_WORKERS, 2)
-fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map)
+__global__ void __launch_bounds__(FORWARD ? F_THREADS : F_WORKERS, FORWARD ? 1 : 2)
+fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map,
+              const __grid_constant__ CUtensorMap row_map)
 {
     using Smem = FwdCeSmem<C, CONF, FORWARD>;
     extern __shared__ __align__(128) uint8_t smem_f[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_f + 1023) & ~(uintptr_t)1023);
-    float2* slots = (float2*)(smem + Smem::kSlotsAt);                      // [F_WARPS][C][32]
-    uint32_t* counts = (uint32_t*)(smem + Smem::kCountsAt);                // [(C + 1) / 2][F_ROWS][F_COLS]
-    unsigned int* hist = (unsigned int*)(smem + Smem::kHistAt);            // [C][C] (CONF)
-    __shared__ __align__(8) uint64_t bars[7];                              // full[2], free[2], weights, tile done, tile taken
+    __shared__ __align__(8) uint64_t bars[2 * kMaxPlaces + 1 + 5 * kGroups];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile uint32_t gave_up;
-    __shared__ float red[2][F_WARPS], wsum[F_WARPS][32];
-    __shared__ __align__(16) float bias[F_WARPS][32];
-    const uint32_t bar0 = tc::smem_u32(&bars[0]), w_bar = bar0 + 32, done_bar = bar0 + 40, taken_bar = bar0 + 48;
+    __shared__ float red[kGroups][2][F_WARPS], wsum[kAllWarps][32];
+    __shared__ __align__(16) float bias[kAllWarps][32];
+    // barriers: places of the ring filled / free, weights; per group: logits there / taken, gradient there, its product there / taken
+    const uint32_t full_bar = tc::smem_u32(&bars[0]), free_bar = full_bar + 8 * kMaxPlaces, w_bar = full_bar + 16 * kMaxPlaces, done_bars = w_bar + 8,
+                   taken_bars = done_bars + 8 * kGroups, dz_bars = taken_bars + 8 * kGroups, grad_bars = dz_bars + 8 * kGroups, grad_taken_bars = grad_bars + 8 * kGroups;
+    const bool with_grad = FORWARD && a.w_part != nullptr;                 // the classifier's weight gradient as well
     const int h = a.h, w = a.w, H = h * kUp, W = w * kUp;
     const int64_t p = (int64_t)h * w;
-    const int tid = threadIdx.x, wi = __shfl_sync(0xffffffffu, tid >> 5, 0), l = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), l = tid & 31;
+    const int grp = FORWARD ? warp / F_WARPS : 0, wi = warp % F_WARPS, gtid = tid % F_WORKERS;       // (of the workers)
+    float2* slots = (float2*)(smem + Smem::kSlotsAt + (FORWARD && grp == 0 ? Smem::kSlots : 0));      // [F_WARPS][C][32]
+    uint32_t* counts = (uint32_t*)(smem + Smem::kCountsAt + grp * Smem::kCounts);                    // [(C + 1) / 2][F_ROWS][F_COLS]
+    unsigned int* hist = (unsigned int*)(smem + Smem::kHistAt + grp * Smem::kHist);                  // [C][C] (CONF)
     const int per_stream = tiles_x * tiles_y, n_tiles = per_stream * a.S;
     // Tiles at the frame's border do extra work: the last tile row of a stream comes first, then rows 0, 1, ...
-    struct Tile { int s, x0, y0, blk; };
-    auto tile_at = [&](int t) {
-        Tile k;
-        k.s = t / per_stream;
-        const int q = t - k.s * per_stream, row = q / tiles_x, col = q - row * tiles_x, by = row == 0 ? tiles_y - 1 : row - 1;
-        k.x0 = col * FN_X; k.y0 = by * FN_Y; k.blk = by * tiles_x + col;
-        return k;
+    // A block walks its tiles by additions: a division takes the warp that feeds the tensor core 1500 cycles beside sixteen others.
+    struct Tile { int t, s, row, col; };                   // t: index in the order of the walk
+    const int d_s = (int)gridDim.x / per_stream, d_row = (int)gridDim.x % per_stream / tiles_x, d_col = (int)gridDim.x % per_stream % tiles_x;
+    auto step = [&](Tile& k) {
+        k.t += gridDim.x; k.s += d_s; k.row += d_row; k.col += d_col;
+        if (k.col >= tiles_x) { k.col -= tiles_x; ++k.row; }
+        if (k.row >= tiles_y) { k.row -= tiles_y; ++k.s; }
     };
+    // ... on to a tile whose stream still trains (the flags come from an earlier kernel: after the wait only)
+    auto settle = [&](Tile& k) { while (a.skip && k.t < n_tiles && a.skip[(int64_t)k.s * a.skip_stride]) step(k); };
+    auto next = [&](Tile& k) { step(k); settle(k); };
+    const Tile first{(int)blockIdx.x, (int)blockIdx.x / per_stream, (int)blockIdx.x % per_stream / tiles_x, (int)blockIdx.x % per_stream % tiles_x};
+    auto tile_row = [&](const Tile& k) { return k.row == 0 ? tiles_y - 1 : k.row - 1; };
+    auto node_x = [&](const Tile& k) { return k.col * FN_X; };             // the first node a tile owns
+    auto node_y = [&](const Tile& k) { return tile_row(k) * FN_Y; };
+    const int tmem_cols = (with_grad ? 4 : 2) * kLogitCols;
 
-    if (FORWARD && wi == F_WARPS) {
-        if (tc::elect_one()) { tc::prefetch_map(&x_map); tc::prefetch_map(&w_map); }
+    if (FORWARD && warp == kAllWarps + 1) {
+        if (tc::elect_one()) { tc::prefetch_map(&x_map); tc::prefetch_map(&w_map); if (with_grad) tc::prefetch_map(&row_map); }
         __syncwarp();
-        tc::tmem_alloc(tc::smem_u32(&tmem_slot), kLogitCols);
+        tc::tmem_alloc(tc::smem_u32(&tmem_slot), tmem_cols);
     }
     if (FORWARD && tid == 0) {
-        for (int k = 0; k < 6; ++k) tc::mbar_init(bar0 + 8u * (uint32_t)k, 1);
-        tc::mbar_init(taken_bar, F_WARPS);
+        for (int k = 0; k < kMaxPlaces; ++k) { tc::mbar_init(full_bar + 8u * (uint32_t)k, 1); tc::mbar_init(free_bar + 8u * (uint32_t)k, kIssuers); }
+        tc::mbar_init(w_bar, 1);
+        for (int g = 0; g < kGroups; ++g) {
+            tc::mbar_init(done_bars + 8 * g, kIssuers); tc::mbar_init(grad_bars + 8 * g, kIssuers);
+            tc::mbar_init(taken_bars + 8 * g, F_WARPS); tc::mbar_init(dz_bars + 8 * g, F_WARPS); tc::mbar_init(grad_taken_bars + 8 * g, F_WARPS);
+        }
         gave_up = 0;
         tc::fence_barrier_init();
     }
-    if ((Smem::kPrefetch || !FORWARD) && wi < F_WARPS) {
-        for (int e = tid; e < (int)(Smem::kCounts / 16); e += F_WORKERS) reinterpret_cast<uint4*>(counts)[e] = make_uint4(0, 0, 0, 0);
-        if (CONF) for (int e = tid; e < C * C; e += F_WORKERS) hist[e] = 0;
+    if (!FORWARD || warp < kAllWarps) {
+        for (int e = gtid; e < (int)(Smem::kCounts / 16); e += F_WORKERS) reinterpret_cast<uint4*>(counts)[e] = make_uint4(0, 0, 0, 0);
+        if (CONF) for (int e = gtid; e < C * C; e += F_WORKERS) hist[e] = 0;
     }
     tc::tc_fence_before_sync();
     __syncthreads();
     tc::tc_fence_after_sync();
     const uint32_t tmem = FORWARD ? tmem_slot : 0;
 
-    if (FORWARD && wi == F_WARPS) {
-        // ---------------------------------------------------------------- the ninth warp: copies and multiplications
+    if (FORWARD && warp >= kAllWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFeederRegs));
+        if (warp > kAllWarps + kIssuers) return;
+        // ---------------------------------------------------------------- the producer and the issuer
+        // Both walk the same list: for every tile F, its logits (per 64 channels two chunks, node rows 0-4 and 4-8), and three tiles later
+        // G, its weight gradient (per 128 channels four chunks of two own node rows).  A chunk takes the ring's next place.  One thread
+        // each: a whole warp's waits and elections between two chunks of eight multiplications take as long as the multiplications.
+        const bool producer = warp == kAllWarps;
+        const int me = warp - kAllWarps - 1;               // issuer: the first takes the upper node rows, the second the lower ones
         const uint32_t ring = tc::smem_u32(smem), w_base = ring + (uint32_t)Smem::kWeightsAt;
-        constexpr uint32_t idesc = tc::instr_desc(128, kClassPad, 0, 0);
-        const int kblocks = a.kblocks;
-        bool ok = true, first = true;
-        uint32_t loads[2] = {0, 0}, mults[2] = {0, 0};    // per slot: copies / multiplications issued so far
-        int w_stream = -1, n_weights = 0, n_done = 0;
-        auto load = [&](int kb, int slot, const Tile& k, uint32_t stall) {
-            if (tc::elect_one()) {
-                tc::mbar_expect_tx(bar0 + 8u * slot, kSliceBytes + stall);
-                tc::tma_load_4d(ring + slot * (uint32_t)Smem::kSliceB, &x_map, bar0 + 8u * slot, kb * 64, k.x0 - 1, k.y0 - 1, k.s);
-            }
-            __syncwarp();
-            ++loads[slot];
-        };
-        const uint32_t limit = a.test_stall ? (1u << 12) : tc::kSpinLimit, stall = a.test_stall ? 16u : 0u;
-        // Inside the step loop the features are frozen: the first slices are fetched while the previous update still runs
-        int pre = 0;
-        if (a.x_early) {
-            const Tile k = tile_at(blockIdx.x);
-            for (; pre < 2 && pre < kblocks; ++pre) load(pre, pre, k, pre == 0 ? stall : 0u);
-        }
-        pdl_wait();                                        // the weights come from the previous kernel of the stream
-        for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-            const Tile k = tile_at(t);
-            if (a.skip && a.skip[(int64_t)k.s * a.skip_stride]) {          // this stream's training loop has ended
-                for (int kb = 0; kb < pre && ok; ++kb) ok = tc::mbar_wait(bar0 + 8u * kb, (loads[kb] - 1) & 1, a.err, tc::kWaitFull);
-                pre = 0;
-                continue;
-            }
-            const int n_slots = first ? 2 : 1;
-            if (w_stream != k.s) {
-                if (tc::elect_one()) {
-                    tc::mbar_expect_tx(w_bar, (uint32_t)kblocks * kWBytes);
-                    for (int kb = 0; kb < kblocks; ++kb) tc::tma_load_3d(w_base + kb * kWBytes, &w_map, w_bar, kb * 64, 0, k.s);
+        const int kblocks = a.kblocks, mt = (kblocks + 1) / 2;
+        bool ok = true;
+        if (tc::elect_one()) {
+            int place = 0, n_places = Smem::kSteady + Smem::kExtra;
+            uint32_t used = 0, parity = 0;                 // per place: has been filled; parity of the wait that comes next
+            auto wait = [&](uint32_t bar, uint32_t par, unsigned code) { ok = ok && tc::mbar_wait_from(tc::mbar_try_wait(bar, par), bar, par, a.err, code); };
+            auto advance = [&]() { place = place + 1 == n_places ? 0 : place + 1; };
+            // (the producer) the place that is filled next, once what lay there has been multiplied
+            auto claim = [&](uint32_t bytes) {
+                const uint32_t bit = 1u << place;
+                if (used & bit) {
+                    wait(free_bar + 8 * place, (parity & bit) != 0, tc::kWaitEmpty);
+                    parity ^= bit;
                 }
-                __syncwarp();
-                w_stream = k.s; ++n_weights;
+                used |= bit;
+                if (ok) tc::mbar_expect_tx(full_bar + 8 * place, bytes);
+                return ok;
+            };
+            auto load_rows = [&](const Tile& k, int e, uint32_t stall) {   // chunk e of F
+                if (!claim(kChunkBytes + stall)) return;
+                tc::tma_load_4d(ring + place * kChunkBytes, &x_map, full_bar + 8 * place, (e >> 1) * 64, node_x(k) - 1, node_y(k) - 1 + 4 * (e & 1), k.s);
+                advance();
+            };
+            // Inside the step loop the features are frozen: the first chunks are fetched while the previous update still runs
+            int pre = a.x_early ? min(n_places, 2 * kblocks) : 0;
+            if (producer) {
+                for (int e = 0; e < pre && ok; ++e) load_rows(first, e, e == 0 && a.test_stall ? 16u : 0u);
             }
-            for (int kb = pre; kb < n_slots && kb < kblocks; ++kb) load(kb, kb, k, first && kb == 0 ? stall : 0u);
-            pre = 0;
-            // as many slices as there are slots are multiplied back to back before their slots are filled again (a slice takes 1100
-            // cycles from its first multiplication to the signal that the last one has read it)
-            for (int k0 = 0; k0 < kblocks && ok; k0 += n_slots) {
-                for (int kb = k0; kb < k0 + n_slots && kb < kblocks; ++kb) {
-                    const int slot = kb - k0;
-                    ok = tc::mbar_wait(bar0 + 8u * slot, (loads[slot] - 1) & 1, a.err, tc::kWaitFull, limit);
-                    if (ok && kb == 0) {
-                        ok = tc::mbar_wait(w_bar, (n_weights - 1) & 1, a.err, tc::kWaitFull);
-                        if (ok && !first) ok = tc::mbar_wait(taken_bar, (n_done - 1) & 1, a.err, tc::kWaitEmpty);
-                    }
-                    if (!ok) break;
-                    tc::tc_fence_after_sync();
-                    if (tc::elect_one()) {
-                        const uint64_t dx = tc::smem_desc(ring + slot * (uint32_t)Smem::kSliceB, 16, 1024), dw = tc::smem_desc(w_base + kb * kWBytes, 16, 1024);
+            pdl_wait();                                    // the weights come from the previous kernel of the stream
+            Tile k = first;
+            settle(k);
+            if (pre && k.t != first.t) {                   // the tile that was begun with is not worked on
+                if (producer) {
+                    for (int e = 0; e < pre; ++e) wait(full_bar + 8 * e, 0, tc::kWaitFull);
+                    used = 0;
+                } else parity = (1u << pre) - 1;
+                pre = 0; place = 0;
+            }
+            Tile back = k;                                 // the tile whose weight gradient comes next
+            int w_stream = -1, n_weights = 0, n_items = 0;
+            for (int q = 0; ok && (k.t < n_tiles || (with_grad && back.t < n_tiles)); ++q) {
+                if (q == 2 && n_items > 1) { n_places = Smem::kSteady; place = 0; }
+                if (k.t < n_tiles) {
+                    const int g = q & 1, j = q >> 1;
+                    if (producer) {
+                        for (int e = q == 0 ? pre : 0; e < 2 * kblocks && ok; ++e) load_rows(k, e, q == 0 && e == 0 && a.test_stall ? 16u : 0u);
+                    } else {
+                        constexpr uint32_t idesc = tc::instr_desc(128, kClassPad, 0, 0);
+                        if (w_stream != k.s) {             // the weights of the stream before are read until the last tile's logits are there
+                            if (q) wait(done_bars + 8 * ((q - 1) & 1), ((q - 1) >> 1) & 1, tc::kWaitDone);
+                            if (ok && me == 0) {
+                                tc::mbar_expect_tx(w_bar, (uint32_t)kblocks * kWBytes);
+                                for (int kb = 0; kb < kblocks; ++kb) tc::tma_load_3d(w_base + kb * kWBytes, &w_map, w_bar, kb * 64, 0, k.s);
+                            }
+                            w_stream = k.s;
+                            wait(w_bar, n_weights++ & 1, tc::kWaitFull);
+                        }
+                        if (j) wait(taken_bars + 8 * g, (j - 1) & 1, tc::kWaitEmpty);
+                        const uint32_t logits = tmem + g * kLogitCols + me * 2 * kClassPad;
+                        uint64_t dw = tc::smem_desc(w_base, 16, 1024);
+                        for (int e = 0; e < 2 * kblocks && ok; ++e) {
+                            const uint32_t bit = 1u << place, bar = full_bar + 8 * place;
+                            if (a.test_stall) {
+                                ok = false;
+                                for (int it = 0; it < (1 << 12) && !ok; ++it) ok = tc::mbar_try_wait(bar, (parity & bit) != 0);
+                                if (!ok) atomicCAS(a.err, 0u, (unsigned)tc::kWaitFull | (blockIdx.x << 8));
+                            } else wait(bar, (parity & bit) != 0, tc::kWaitFull);
+                            parity ^= bit;
+                            if (!ok) break;
+                            tc::tc_fence_after_sync();
+                            const uint64_t dx = tc::smem_desc(ring + place * kChunkBytes + me * kRowBytes, 16, 1024);
+                            const uint32_t to = logits + (e & 1) * kClassPad;  // (rows 0-3, 4-7 upper; 1-4, 5-8 lower)
 #pragma unroll
-                        for (int m = 0; m < 4; ++m)        // node rows 0-3, 4-7 (upper), 1-4, 5-8 (lower); a node row is 32 x 128 bytes
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                tc::umma(tmem + m * kClassPad, dx + (((m & 1) * 4 + (m >> 1)) * (F_COLS * 128) >> 4) + 2 * j, dw + 2 * j, idesc, (kb | j) != 0);
-                        tc::umma_commit(bar0 + 16 + 8u * slot);
+                            for (int u = 0; u < 4; ++u) tc::umma(to, dx + 2 * u, dw + 2 * u, idesc, (e >> 1 | u) != 0);
+                            tc::umma_commit(free_bar + 8 * place);
+                            if (e & 1) dw += kWBytes >> 4;
+                            advance();
+                        }
+                        if (ok) tc::umma_commit(done_bars + 8 * g);
                     }
-                    __syncwarp();
-                    ++mults[slot];
+                    ++n_items;
+                    next(k);
                 }
-                for (int kb = k0 + n_slots; kb < k0 + 2 * n_slots && kb < kblocks && ok; ++kb) {
-                    const int slot = kb - k0 - n_slots;
-                    ok = tc::mbar_wait(bar0 + 16 + 8u * slot, (mults[slot] - 1) & 1, a.err, tc::kWaitEmpty);
-                    if (ok) load(kb, slot, k, 0u);
+                if (with_grad && q >= 3 && back.t < n_tiles && ok) {
+                    // dW[channel][class] = sum of X[node][channel] dz[node][class] over the tile's own nodes: the group has left the bf16
+                    // gradient in shared memory (K-major, zeros at the halo), the features come again (MN-major)
+                    const int g = (q - 3) & 1, j = (q - 3) >> 1;
+                    if (producer) {
+                        for (int e = 0; e < 4 * mt && ok; ++e) {
+                            const int m = e >> 2, r0 = 2 * (e & 3), rows = r0 == 6 ? 1 : 2;
+                            if (!claim((uint32_t)(2 * rows) * kRowBytes)) break;
+                            for (int b = 0; b < 2; ++b)
+                                for (int r = 0; r < rows; ++r)
+                                    tc::tma_load_4d(ring + place * kChunkBytes + (uint32_t)(b * rows + r) * kRowBytes, &row_map, full_bar + 8 * place, (2 * m + b) * 64, node_x(back) - 1, node_y(back) + r0 + r, back.s);
+                            advance();
+                        }
+                    } else {
+                        constexpr uint32_t idesc = tc::instr_desc(128, kClassPad, 1, 0);
+                        wait(dz_bars + 8 * g, j & 1, tc::kWaitFull);
+                        if (j) wait(grad_taken_bars + 8 * g, (j - 1) & 1, tc::kWaitEmpty);
+                        const uint32_t to = tmem + kGroups * kLogitCols + g * kGradCols;
+                        const uint64_t dz = tc::smem_desc(ring + (uint32_t)Smem::kGradAt + g * (uint32_t)Smem::kGrad, 16, 1024);
+                        for (int e = 0; e < 4 * mt && ok; ++e) {
+                            const uint32_t bit = 1u << place;
+                            wait(full_bar + 8 * place, (parity & bit) != 0, tc::kWaitFull);
+                            parity ^= bit;
+                            if (!ok) break;
+                            if ((e >> 2) != me) { arrive(free_bar + 8 * place); advance(); continue; }     // the other issuer's channels
+                            tc::tc_fence_after_sync();
+                            const uint64_t dg = dz + (e & 3) * (kWBytes >> 4);
+                            const bool last = (e & 3) == 3;
+                            const uint64_t dx = tc::smem_desc(ring + place * kChunkBytes, last ? kRowBytes : 2 * kRowBytes, 1024);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)            // sixteen nodes at a time
+                                if (u < 2 || !last) tc::umma(to + (e >> 2) * kClassPad, dx + ((u * 16 * 128) >> 4), dg + 2 * u, idesc, ((e & 3) | u) != 0);
+                            tc::umma_commit(free_bar + 8 * place);
+                            advance();
+                        }
+                        if (ok) tc::umma_commit(grad_bars + 8 * g);
+                    }
+                    next(back);
                 }
             }
-            if (!ok) break;
-            if (tc::elect_one()) tc::umma_commit(done_bar);
-            __syncwarp();
-            ok = tc::mbar_wait(done_bar, n_done & 1, a.err, tc::kWaitDone);
-            ++n_done;
-            first = false;
+            if (!producer) {
+                for (int it = n_items > 2 ? n_items - 2 : 0; it < n_items && ok; ++it) {
+                    wait(taken_bars + 8 * (it & 1), (it >> 1) & 1, tc::kWaitEmpty);
+                    if (with_grad) wait(grad_taken_bars + 8 * (it & 1), (it >> 1) & 1, tc::kWaitEmpty);
+                }
+            }
+            if (!ok) {                                     // nothing more is multiplied and nothing is written
+                gave_up = 1;
+                if (!producer) for (int g = 0; g < kGroups; ++g) { arrive(done_bars + 8 * g); arrive(grad_bars + 8 * g); }
+                tc::drain_after_error();
+            }
         }
-        if (!ok) {                                         // nothing more is multiplied and nothing is written
-            gave_up = 1;
-            __syncwarp();
-            if (tc::elect_one()) arrive(done_bar);
-            tc::drain_after_error();
-        } else if (n_done) tc::mbar_wait(taken_bar, (n_done - 1) & 1, a.err, tc::kWaitEmpty);
-        pdl_launch_dependents();
         __syncwarp();
+        if (me != 0) return;
         tc::tc_fence_after_sync();
-        tc::tmem_dealloc(tmem, kLogitCols);
+        tc::tmem_dealloc(tmem, tmem_cols);
         return;
     }
 
-    // -------------------------------------------------------------------- the eight others
+    // -------------------------------------------------------------------- the workers
+    if (FORWARD) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWorkerRegs));
+    const uint32_t done_bar = done_bars + 8 * grp, taken_bar = taken_bars + 8 * grp, dz_bar = dz_bars + 8 * grp, grad_bar = grad_bars + 8 * grp,
+                   grad_taken = grad_taken_bars + 8 * grp, logits_at = tmem + grp * kLogitCols, grads_at = tmem + kGroups * kLogitCols + grp * kGradCols;
     float2* my = slots + (size_t)wi * C * 32 + l;          // this lane's slot of class c: my[c * 32]
     const int hw1 = a.heavy_w - 1;                         // what a weighted pixel counts on top of 1
     const float invP = 1.0f / ((float)H * (float)W);
     int n_done = 0;
     bool waited = false;
-    // (neighbouring tiles at the same time on neighbouring blocks: what they share comes from L2.  16 streams of 256 channels at
-    // 720p: 227 us; with consecutive tiles per block, whose weights then stay, 240)
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-        const Tile k = tile_at(t);
-        const int x0 = k.x0, y0 = k.y0, s = k.s;
+    // (neighbouring tiles at the same time on neighbouring blocks: what they share comes from L2)
+    // The weight gradient of the tile before this one, as the tensor core has left it -> its partial sum
+    auto store_gradient = [&](const Tile& k) {
+        const int m = wi >> 2, ch = m * 128 + (wi & 3) * 32 + l, K = a.kblocks * 64;
+        tc::tc_fence_after_sync();
+        if (2 * m < a.kblocks) {                           // warp-uniform
+            float g[32];
+            const uint32_t from = grads_at + ((uint32_t)((wi & 3) * 32) << 16) + m * kClassPad;
+            if constexpr (C <= 16) tc::tmem_ld_32x16(from, reinterpret_cast<float(&)[16]>(g));
+            else tc::tmem_ld_32x32(from, g);
+            float* dst = a.w_part + ((int64_t)k.s * per_stream + tile_row(k) * tiles_x + k.col) * C * K + ch;
+            if (ch < K)
+#pragma unroll
+                for (int c = 0; c < C; ++c) dst[c * K] = g[c];
+        }
+        tc::tc_fence_before_sync();
+        __syncwarp();
+        if (tc::elect_one()) arrive(grad_taken);
+    };
+    // the groups take the block's tiles in turn
+    Tile k = first, before = first;
+    if (grp) step(k);
+    while (k.t < n_tiles) {
+        const int x0 = node_x(k), y0 = node_y(k), s = k.s, blk = tile_row(k) * tiles_x + k.col;
         const int i = y0 - 1 + wi, n = x0 - 1 + l;         // cell row (frame rows 4i+2 .. 4i+5, node rows i, i+1), own node column
         const bool cell_row = i <= h - 1, cell_valid = l <= 30 && n <= w - 1, node_owned = l >= 1 && l <= FN_X && n < w;
         // the aligned 4-pixel words of the label rows: a cell's pixels are the upper half of its own column's word and the lower
@@ -304,8 +418,19 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
             labw[r] = cell_row && Y >= 0 && Y < H && n >= 0 && n < w
                           ? __ldg(reinterpret_cast<const uint32_t*>(a.labels + (int64_t)s * H * W + (int64_t)Y * W + 4 * n)) : 0u;
         }
-        if (!waited) { pdl_wait(); waited = true; }        // the parameters come from the previous kernel of the stream
-        if (a.skip && a.skip[(int64_t)s * a.skip_stride]) continue;
+        if (!waited) {                                     // the parameters come from the previous kernel of the stream
+            pdl_wait();
+            waited = true;
+            if (FORWARD && a.skip) {                       // ... and so does which tiles are worked on
+                Tile f = first;
+                settle(f);
+                if (grp) next(f);
+                if (f.t != k.t) { k = f; continue; }
+            }
+        }
+        if (!FORWARD && a.skip && a.skip[(int64_t)s * a.skip_stride]) return;
+        const Tile now = k;
+        next(k);
         float bias_l = 0.f;
         bool ok = true;
         ++n_done;
@@ -315,13 +440,6 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
             tc::tc_fence_after_sync();
             if (gave_up) ok = false;
         }
-        if (FORWARD && !Smem::kPrefetch) {                            // the slices are dead: the arrays under them get their initial contents
-            if (!workers_all(ok)) return;                  // ... block-uniform
-            for (int e = tid; e < (int)(Smem::kCounts / 16); e += F_WORKERS) reinterpret_cast<uint4*>(counts)[e] = make_uint4(0, 0, 0, 0);
-            if (CONF) for (int e = tid; e < C * C; e += F_WORKERS) hist[e] = 0;
-            workers_sync();
-        }
-
         float loss = 0.f;
         unsigned n_bad = 0;
         // where the cell's left and right node columns lie relative to the own slot (clamped at the frame's left and right border)
@@ -335,9 +453,9 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                 const bool in_cols = n >= 0 && n < w;
                 float up[32], lo[32], m = -INFINITY;
                 if constexpr (FORWARD) {
-                    bias[wi][l] = bias_l;
+                    bias[warp][l] = bias_l;
                     __syncwarp();
-                    const uint32_t lanes = tmem + ((uint32_t)((wi & 3) * 32) << 16), upper = lanes + (wi >> 2) * kClassPad, lower = upper + 2 * kClassPad;
+                    const uint32_t lanes = logits_at + ((uint32_t)((wi & 3) * 32) << 16), upper = lanes + (wi >> 2) * kClassPad, lower = upper + 2 * kClassPad;
                     if constexpr (C <= 16) {
                         tc::tmem_ld_32x16(i == -1 ? lower : upper, reinterpret_cast<float(&)[16]>(up));
                         tc::tmem_ld_32x16(i == h - 1 ? upper : lower, reinterpret_cast<float(&)[16]>(lo));
@@ -350,7 +468,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                     if (tc::elect_one()) arrive(taken_bar);
 #pragma unroll
                     for (int c4 = 0; c4 < C; c4 += 4) {
-                        const float4 b4 = *reinterpret_cast<const float4*>(&bias[wi][c4]);
+                        const float4 b4 = *reinterpret_cast<const float4*>(&bias[warp][c4]);
                         const float b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
                         for (int c = c4; c < c4 + 4 && c < C; ++c) { up[c] += b[c - c4]; lo[c] += b[c - c4]; }
@@ -617,17 +735,22 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
         // loss of the tile, fixed order
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-        if (l == 0) red[n_done & 1][wi] = loss;            // (two of them: warps may be one tile ahead of the one that adds)
+        if (l == 0) red[grp][n_done & 1][wi] = loss;       // (two of them: warps may be one tile ahead of the one that adds)
         if (n_bad) atomicAdd(a.bad, n_bad);
-        if (!workers_all(ok)) return;                      // block-uniform: a wait ran out, nothing is written
-        if (t + (int)gridDim.x >= n_tiles) pdl_launch_dependents();        // only the epilogue is left (with FORWARD the ninth warp has let
-                                                                           // the successor go when the last logits were taken)
+        if (FORWARD && with_grad && ok && n_done > 1) {    // the product of the group's tile before: its gradient has been read
+            ok = tc::mbar_wait(grad_bar, n_done & 1, a.err, tc::kWaitDone);
+            if (gave_up) ok = false;
+        }
+        if (!workers_all(grp, ok)) return;                 // uniform over the group: a wait ran out, nothing is written
+        if (!FORWARD || k.t >= n_tiles) pdl_launch_dependents();      // the block's last tile: only the epilogue is left
         if (CONF) {                                        // one global update per non-empty counter of the tile
-            for (int e = tid; e < C * C; e += F_WORKERS) {
+            for (int e = gtid; e < C * C; e += F_WORKERS) {
                 const unsigned int v = hist[e];
                 if (v) { atomicAdd(a.conf + (int64_t)s * a.conf_stream_stride + e, (unsigned long long)v); hist[e] = 0; }
             }
         }
+        if (FORWARD && with_grad && n_done > 1) store_gradient(before);
+        before = now;
         // ---- node row y0-1+wi (warps 1..FN_Y): own upper pulls + lower pulls of the warp above - counts
         const bool node_ok = wi >= 1 && i < h && node_owned;
         float v[32];
@@ -654,6 +777,18 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                 for (int c = 0; c < C; ++c) dzb[(int64_t)c * a.dz_bf16_pitch] = __float2bfloat16_rn(v[c]);
             }
         }
+        if (FORWARD && with_grad) {
+            // bf16, K-major with the 128-byte swizzle: [two node rows][class][64 nodes]
+            if (wi >= 1) {
+                uint8_t* to = smem + Smem::kGradAt + grp * Smem::kGrad + ((wi - 1) >> 1) * kWBytes + (l & 7) * 2;
+                const uint32_t chunk = (((wi - 1) & 1) * 4 + (l >> 3)) * 16;
+#pragma unroll
+                for (int c = 0; c < C; ++c) *reinterpret_cast<bf16*>(to + c * 128 + (chunk ^ ((c & 7) * 16))) = __float2bfloat16_rn(v[c]);
+            }
+            tc::fence_async_shared();                      // read by way of the async proxy
+            __syncwarp();
+            if (tc::elect_one()) arrive(dz_bar);
+        }
         // bias-gradient partial of the tile.  Lane reduce-scatter inside each warp (31 exchanges: at distance o a lane keeps the
         // half of its values whose class has bit o equal to its own lane bit and adds the partner's), after which lane c holds
         // class c; then the warps' sums are added in warp order.  Fixed order throughout.
@@ -667,20 +802,32 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                 v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
             }
         }
-        wsum[wi][l] = v[0];
-        workers_sync();
-        if (tid < C) {
+        wsum[warp][l] = v[0];
+        workers_sync(grp);
+        if (gtid < C) {
             float q = 0.f;
 #pragma unroll
-            for (int r = 1; r < F_WARPS; ++r) q += wsum[r][tid];
-            a.db_part[((int64_t)s * per_stream + k.blk) * C + tid] = q;
+            for (int r = 1; r < F_WARPS; ++r) q += wsum[grp * F_WARPS + r][gtid];
+            a.db_part[((int64_t)s * per_stream + blk) * C + gtid] = q;
         }
-        if (tid == 32) {
+        if (gtid == 32) {
             float q = 0.f;
-            for (int r = 0; r < F_WARPS; ++r) q += red[n_done & 1][r];
-            a.loss_part[(int64_t)s * per_stream + k.blk] = q;
+            for (int r = 0; r < F_WARPS; ++r) q += red[grp][n_done & 1][r];
+            a.loss_part[(int64_t)s * per_stream + blk] = q;
         }
+        if (FORWARD) next(k);                              // the other group's
     }
+    if (FORWARD && with_grad && n_done > 0) {
+        if (tc::mbar_wait(grad_bar, (n_done - 1) & 1, a.err, tc::kWaitDone) && !gave_up) store_gradient(before);
+    }
+}
+
+// A block that was launched with fewer registers than its warps ask for would wait for them forever
+inline cudaError_t check_launch_regs(const void* kernel)
+{
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+    return e != cudaSuccess ? e : at.numRegs < kLaunchRegs ? cudaErrorInvalidConfiguration : cudaSuccess;
 }
 
 template <int C>
@@ -690,25 +837,26 @@ cudaError_t prepare_fwd_ce_as()
     if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, true, true>);
     if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, false, false>);
     if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, true, false>);
+    if (e == cudaSuccess) e = check_launch_regs((const void*)fwd_ce_kernel<C, false, true>);
+    if (e == cudaSuccess) e = check_launch_regs((const void*)fwd_ce_kernel<C, true, true>);
     return e;
 }
 
 template <int C, bool CONF, bool FORWARD>
-void launch_fwd_ce_as(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
+void launch_fwd_ce_as(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s)
 {
     using Smem = FwdCeSmem<C, CONF, FORWARD>;
     const int tx = (a.w + FN_X - 1) / FN_X, ty = (a.h + FN_Y - 1) / FN_Y, tiles = tx * ty * a.S;
-    const int grid = Smem::kPrefetch && tiles > 2 * a.n_sms ? 2 * a.n_sms : tiles;
-    // (78 tiles behind a 3x3 layer of 64 channels, whose 115 blocks leave 33 SMs free: 44.2 us a step, spread 39.7)
+    const int grid = FORWARD && tiles > a.n_sms ? a.n_sms : tiles;
     const size_t smem = one_per_sm(Smem::kBytes, tiles, a.n_sms);
-    launch_early(a.chain_early != 0 || a.x_early != 0, fwd_ce_kernel<C, CONF, FORWARD>, dim3(grid), dim3(FORWARD ? F_THREADS : F_WORKERS), smem, s, a, tx, ty, x_map, w_map);
+    launch_early(a.chain_early != 0 || a.x_early != 0, fwd_ce_kernel<C, CONF, FORWARD>, dim3(grid), dim3(FORWARD ? F_THREADS : F_WORKERS), smem, s, a, tx, ty, x_map, w_map, row_map);
 }
 
 template <int C, bool FORWARD>
-void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s)
+void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s)
 {
-    if (a.conf) launch_fwd_ce_as<C, true, FORWARD>(a, x_map, w_map, s);
-    else launch_fwd_ce_as<C, false, FORWARD>(a, x_map, w_map, s);
+    if (a.conf) launch_fwd_ce_as<C, true, FORWARD>(a, x_map, w_map, row_map, s);
+    else launch_fwd_ce_as<C, false, FORWARD>(a, x_map, w_map, row_map, s);
 }
 
 }  // namespace
@@ -716,7 +864,7 @@ void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const C
 // The kernels of one class count
 struct FwdCeKernels {
     cudaError_t (*prepare)();
-    void (*launch[2])(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s);   // stored logits, own forward
+    void (*launch[2])(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s);   // stored logits, own forward
 };
 
 // ... of class count `n`, one of FIRST + I...

@@ -70,10 +70,11 @@ struct st_ctx {
     int n_split2 = 0;
     float *loss_part = nullptr, *db_part = nullptr;
     int n_k3_blocks = 0;
-    CUtensorMap fx_map, fw_map; // tile maps of the classifier's input and of its bf16 weights: the loss kernel multiplies its own logits
+    CUtensorMap fx_map, fc_map, fr_map, fw_map; // maps of the classifier's input (tiles, five rows, one row) and of its bf16 weights: the loss kernel multiplies its own logits
     int n_sms = 0;
     int fused_loss = 0;         //   (bf16 GEMMs, the classifier's input of a shape fused_forward_supported names; ST_FUSED_FORWARD=0
     int fused_fwd = 0;          //   switches it off); with a one-layer head the student-mask kernel does so too
+    int fused_grad = 0;         //   and the loss kernel forms the weight gradient (class counts that classifier_gradient_fits names)
     int test_stall_fused = 0;   // test of the give-up path inside that kernel (environment ST_TEST_STALL_FUSED=1 at context creation)
     float* loss_buf = nullptr;              // [S][kMaxSteps]
     unsigned long long* conf_buf = nullptr; // [S][kMaxSteps][C][C], allocated on first use
@@ -241,7 +242,7 @@ UpdateArgs make_update_args(st_ctx* c, int slot, const int* skip = nullptr, int6
         if (last) {
             ly.b_partials = c->db_part; ly.n_bpart = c->n_k3_blocks;
             ly.w_partials = c->w2_partials; ly.n_split = c->n_split2;
-            ly.w_split_stride = (int64_t)(c->bf16_mode ? kClassPad : ly.cout) * ly.cin;
+            ly.w_split_stride = (int64_t)(c->bf16_mode && !c->fused_grad ? kClassPad : ly.cout) * ly.cin;
             ly.w_stream_stride = ly.w_split_stride * c->n_split2;
         } else {
             const st_ctx::Block& k = c->blk[L];
@@ -343,7 +344,7 @@ UpsampleCeArgs k3_args(st_ctx* c, bool fp32_grad, bool bf16_grad, unsigned long 
     k3.S = c->S; k3.C = c->C; k3.h = c->h; k3.w = c->w;
     k3.skip = skip; k3.skip_stride = skip_stride;
     k3.chain_early = c->chain_early ? 1 : 0;
-    k3.n_sms = c->n_sms; k3.x_early = 0; k3.kblocks = 0; k3.theta = nullptr; k3.n_params = 0; k3.b_off = 0; k3.z_out = nullptr; k3.test_stall = 0;
+    k3.n_sms = c->n_sms; k3.x_early = 0; k3.kblocks = 0; k3.theta = nullptr; k3.n_params = 0; k3.b_off = 0; k3.z_out = nullptr; k3.w_part = nullptr; k3.test_stall = 0;
     return k3;
 }
 
@@ -360,13 +361,14 @@ st_status enqueue_loss(st_ctx* c, unsigned long long* conf, StageTimer* t = null
         const bool frozen_input = c->first_trained >= c->n_blocks;
         k3.x_early = frozen_input && after_update && !t ? 1 : 0; k3.kblocks = (c->Ch ? c->Ch : c->Cin) / 64;
         k3.theta = c->theta; k3.n_params = c->n_params; k3.b_off = c->layout.b_off[c->layout.n_layers - 1];
+        if (c->fused_grad) { k3.w_part = c->w2_partials; k3.dz_bf16 = nullptr; }      // and the weight gradient
         k3.z_out = keep_logits ? c->z : nullptr;         // logits that the next iteration overwrites unread stay on the chip
         k3.test_stall = c->test_stall_fused;
         // the first iteration's predecessor may have written the labels and the features, which are fetched before the wait
         if (frozen_input && !after_update) k3.chain_early = 0;
     }
     ST_REPEAT(t) {
-        if (c->fused_loss) launch_fwd_ce(k3, c->fx_map, c->fw_map, s);
+        if (c->fused_loss) launch_fwd_ce(k3, c->fc_map, c->fw_map, c->fr_map, s);
         else launch_upsample_ce(k3, s);
     }
     if (t) t->mark(c->fused_loss ? "fwd1x1_upsample_ce" : "upsample_ce", s, st_repeats(t));
@@ -378,6 +380,7 @@ st_status enqueue_loss(st_ctx* c, unsigned long long* conf, StageTimer* t = null
 st_status enqueue_backward(st_ctx* c, StageTimer* t = nullptr, const int* skip = nullptr, int64_t skip_stride = 0, const TrainCtl* ctl = nullptr)
 {
     cudaStream_t s = c->stream;
+    if (c->fused_grad) return ST_OK;                     // the loss kernel has formed the weight gradient too
     if (c->bf16_mode) {
         c->launches += tc_backward(c->plan, s, t, skip, skip_stride, ctl);
     } else if (c->Ch == 0) {
@@ -711,8 +714,12 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
         c->dz_pitch = tc_dz_pitch(c->h, c->w);
         ALLOC(dz_bf16, (size_t)S * kClassPad * c->dz_pitch);
         ALLOC(w2_shadow, (size_t)S * kClassPad * c_last);
-        c->n_split2 = n_blocks > first_trained ? tc_back_splits(c_last, c->h, c->w) : tc_wgrad1x1_splits(c_last, c->h, c->w);
-        ALLOC(w2_partials, (size_t)S * c->n_split2 * kClassPad * c_last);
+        // one-layer head: the loss kernel leaves a partial sum per tile
+        const char* off = getenv("ST_FUSED_FORWARD");
+        const bool fuse = !(off && off[0] == '0') && fused_forward_supported(c->C, c->h, c->w, c_last);
+        c->fused_loss = fuse ? 1 : 0; c->fused_fwd = fuse && n_blocks == 0 ? 1 : 0; c->fused_grad = c->fused_fwd && classifier_gradient_fits(c->C) ? 1 : 0;
+        c->n_split2 = c->fused_grad ? c->n_k3_blocks : n_blocks > first_trained ? tc_back_splits(c_last, c->h, c->w) : tc_wgrad1x1_splits(c_last, c->h, c->w);
+        ALLOC(w2_partials, (size_t)S * c->n_split2 * (c->fused_grad ? c->C : kClassPad) * c_last);
         for (int i = 0; i < n_blocks; ++i) {
             st_ctx::Block& k = c->blk[i];
             const size_t tot = (size_t)k.c_prev + k.c_skip;
@@ -793,15 +800,21 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             st_destroy(c);
             return code;
         }
-        const char* off = getenv("ST_FUSED_FORWARD");
-        if (!(off && off[0] == '0') && fused_forward_supported(c->C, c->h, c->w, c_last)) {
+        if (c->fused_loss) {
             const uint64_t ci = (uint64_t)c_last;
             const uint64_t dims[3] = {ci, (uint64_t)kClassPad, (uint64_t)S}, str[2] = {ci * 2, (uint64_t)kClassPad * ci * 2};
             const uint32_t box[3] = {64, (uint32_t)kClassPad, 1};
-            c->fused_loss = make_feature_tile_map(&c->fx_map, n_blocks ? c->blk[n_blocks - 1].out : c->x_bf16, S, c_last, c->h, c->w) &&
+            const bf16* x = n_blocks ? c->blk[n_blocks - 1].out : c->x_bf16;
+            bool made = make_feature_tile_map(&c->fx_map, x, S, c_last, c->h, c->w) && make_feature_chunk_map(&c->fc_map, x, S, c_last, c->h, c->w) &&
+                        make_feature_row_map(&c->fr_map, x, S, c_last, c->h, c->w) &&
                             encode_tensor_map(&c->fw_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, c->w2_shadow, 3,
                                               dims, str, box, msg, sizeof msg, "1x1 weight");
-            c->fused_fwd = c->fused_loss && n_blocks == 0 && prepare_student_eval() == cudaSuccess;
+            if (c->fused_fwd) made = made && prepare_student_eval() == cudaSuccess;
+            if (!made) {
+                st_status code = fail(nullptr, ST_ERR_CUDA, "st_init_head: maps of the loss kernel: %s", msg);
+                st_destroy(c);
+                return code;
+            }
             if (const char* ts = getenv("ST_TEST_STALL_FUSED")) c->test_stall_fused = ts[0] == '1' ? 1 : 0;
         }
     }
@@ -1013,7 +1026,7 @@ st_status enqueue_train(st_ctx* c, int max_updates)
         // kernel works, or, where there is none (fp32 convolutions; the last prediction, after which every loop ends),
         // by the update itself, which in any case takes the step only where the loop goes on
         const TrainCtl ctl = train_ctl(c, i, max_updates);
-        const bool side = c->bf16_mode && i < max_updates;
+        const bool side = c->bf16_mode && !c->fused_grad && i < max_updates;
         if (st == ST_OK && i < max_updates) st = enqueue_backward(c, nullptr, ended_before, kCtlPitch, side ? &ctl : nullptr);
         if (st == ST_OK) st = enqueue_update(c, i, nullptr, 0, nullptr, &ctl, side ? 2 : 1);
     }

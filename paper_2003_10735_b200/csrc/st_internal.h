@@ -131,6 +131,7 @@ struct UpsampleCeArgs {
     const float* theta;      // parameters (for the bias: theta[s * n_params + b_off + c])
     int64_t n_params, b_off;
     float* z_out;            // nullptr, or [S][C][h][w]: the logits are written here as well
+    float* w_part;           // nullptr, or [S][n_blocks][C][64 kblocks]: the classifier's weight gradient, a partial sum per tile
     int test_stall;          // test of the give-up path: the first wait of the block's forward runs out (see tc_fwd1x1_kernel)
 };
 // Tensor map of any element type and swizzle; dims innermost first, strides (bytes) for dimensions 1..rank-1
@@ -143,10 +144,15 @@ void launch_upsample_ce(const UpsampleCeArgs& a, cudaStream_t s);
 // The same with the forward of a 1x1 classifier over bf16 features in front, in one kernel (k_fwd_ce.cuh), for the shapes that
 // fused_forward_supported names; host copies of the tile maps of the features and of the bf16 weights
 bool fused_forward_supported(int C, int h, int w, int c_in);
+// Class counts with which the weight gradient of a one-layer head fits it too: two places of the ring at least beside the gradients of two
+// tiles (25 classes have one)
+constexpr bool classifier_gradient_fits(int C) { return C <= 24; }
 cudaError_t prepare_fwd_ce(int C);
-void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, cudaStream_t s);
+void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s);
 // Tile map of bf16 features [S][h][w][c_in] for it: {c_in, w, h, S}, one box = 64 channels of a tile
 bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w);
+bool make_feature_chunk_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w); // ... of five rows of a tile
+bool make_feature_row_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w);   // ... of one row
 // the part of launch_upsample_ce for C <= 32 (k_fwd_ce.cuh)
 bool upsample_ce_few_supported(int C);
 int upsample_ce_few_blocks(int h, int w);
