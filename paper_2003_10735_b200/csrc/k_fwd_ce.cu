@@ -35,21 +35,25 @@ void launch_upsample_ce_few(const UpsampleCeArgs& a, cudaStream_t s)
     fwd_ce_kernels(b.C).launch[0](b, none, none, none, s);
 }
 
-// one box: 64 channels of `rows` rows of a tile
-static bool make_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w, int rows)
+// one box: `channels` channels of `rows` rows of a tile
+static bool make_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w, int rows, int channels)
 {
     if (c_in % 64 != 0 || w < F_COLS || h < F_ROWS || ((uintptr_t)x & 15u)) return false;
     const uint64_t c = (uint64_t)c_in;
     const uint64_t dims[4] = {c, (uint64_t)w, (uint64_t)h, (uint64_t)S};
     const uint64_t strides[3] = {c * 2, (uint64_t)w * c * 2, (uint64_t)h * w * c * 2};
-    const uint32_t box[4] = {64, (uint32_t)F_COLS, (uint32_t)rows, 1};
+    const uint32_t box[4] = {(uint32_t)channels, (uint32_t)F_COLS, (uint32_t)rows, 1};
     char err[128];
-    return encode_tensor_map(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, x, 4, dims, strides, box, err,
+    return encode_tensor_map(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, channels == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, x, 4, dims, strides, box, err,
                              sizeof(err), "feature tile");
 }
 
-bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w) { return make_tile_map(m, x, S, c_in, h, w, F_ROWS); }
-bool make_feature_chunk_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w) { return make_tile_map(m, x, S, c_in, h, w, 5); }
-bool make_feature_row_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w) { return make_tile_map(m, x, S, c_in, h, w, 1); }
+bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w) { return make_tile_map(m, x, S, c_in, h, w, F_ROWS, 64); }
+bool make_feature_chunk_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w, bool two_groups)
+{
+    const bool half = half_rows(two_groups ? kTwoGroups : kOneGroup);
+    return make_tile_map(m, x, S, c_in, h, w, half ? F_ROWS : 5, half ? 32 : 64);
+}
+bool make_feature_row_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w) { return make_tile_map(m, x, S, c_in, h, w, 1, 64); }
 
 }  // namespace st

@@ -10,9 +10,10 @@
 // lane 31 are halo (recomputed by the neighbouring tile), so that a tile's nodes are finished in a fixed summation order,
 // without floating-point atomics.
 //
-// With FORWARD a block has an SM to itself and is persistent: two groups take its tiles in turn, a producer feeds a ring of chunks by
-// TMA, and two issuers (a thread each) feed the tensor core.
-//   Logits.  The features of the tile's 9 x 32 nodes arrive in chunks of 64 channels and five node rows (nodes outside the map arrive
+// With an own forward a block is persistent: a producer feeds a ring of chunks by TMA, and two issuers (a thread each) feed the tensor core.
+// Where the weight gradient is formed too (one-layer heads), and with more than 24 classes, it has an SM to itself and two groups take its
+// tiles in turn; otherwise it is one group, and two blocks fit an SM.
+//   Logits.  The features of the tile's 9 x 32 nodes arrive in chunks (nodes outside the map arrive
 //   as zeros), and four multiplications per 16 channels leave node row i of the tile and node row i+1 of it in the same 32
 //   tensor-memory lanes: the two rows that warp i's cells lie between.  A warp therefore takes its logits out of tensor memory
 //   alone, without the other warps: bias added, shifted by the largest of them, in log2 units, clamped at the frame's border, both rows of
@@ -42,7 +43,9 @@
 // second after 12800.  us of a call of eight steps with two blocks of one group on an SM, a warp each to feed the tensor core and a kernel of its own for the
 // weight gradient / now, 256 channels on 180 x 320, 21 classes: 275.8 / 267.6, 4 streams 963 / 856, 16 streams 3535 / 3248; 30 classes (weight
 // gradient apart), 4 streams 1274 / 1137; 32 classes 351 / 330; 4 classes 201 / 184; 128 channels on 90 x 160 156.7 / 146.8.  Behind a 3x3 layer (no weight
-// gradient) it is the same within 1 %: 720p, 64 channels 16.9 / 16.7 us a launch, 1080p, 256 channels 43.9 / 45.8.
+// gradient) two groups lose, since the kernels around theirs find no room beside a block that fills an SM; us a launch, a warp each to feed the
+// tensor core / two groups / one group as it is: three maps of 101 x 187, 128 channels 18.5 / 19.2 / 18.0, 720p, 64 channels 16.9 / 16.8 / 16.5,
+// 1080p, 256 channels 43.8 / 45.7 / 43.9; the stack's step 127.9 / 128.7 / 127.6.
 // Tried: one group whose warps divide the classes (sums and labels are then worked out twice: 222 -> 370 us for 16 streams); places of the
 // ring over both groups' slots for a block's first tile (no change: L2 sets the pace); bias sums through shared memory (one more
 // barrier: 3250 -> 3280).
@@ -63,34 +66,48 @@ namespace {
 constexpr int F_ROWS = fused::kTileRows, F_COLS = fused::kTileCols;         // nodes of a tile, halo included
 constexpr int FN_Y = fused::kOwnRows, FN_X = fused::kOwnCols;               // nodes a tile owns
 constexpr int F_WARPS = FN_Y + 1, F_WORKERS = F_WARPS * 32;                 // of a group: the warps that work on one tile
-constexpr int kGroups = 2, kAllWarps = kGroups * F_WARPS, F_THREADS = kGroups * F_WORKERS + 128;   // with FORWARD; without, one group
+// What a block is: one group that reads stored logits; one group with its own forward, two blocks to an SM; two groups with their own
+// forward, which have an SM to themselves
+enum Form { kStored = 0, kOneGroup = 1, kTwoGroups = 2 };
+__host__ __device__ constexpr int form_groups(int form) { return form == kTwoGroups ? 2 : 1; }
+__host__ __device__ constexpr int form_threads(int form) { return form_groups(form) * F_WORKERS + (form == kStored ? 0 : 128); }
 constexpr int kNodes = F_ROWS * F_COLS;
 constexpr int kSweep1 = 7, kSweep2 = 3;                                     // classes per iteration of the two sweeps
 constexpr uint32_t kWBytes = fused::kWeightBytes;
 constexpr uint32_t kRowBytes = F_COLS * 128;                                // a node row of 64 channels
-constexpr uint32_t kChunkBytes = 5 * kRowBytes;                             // a place of the ring
 constexpr int kLogitCols = 4 * kClassPad, kGradCols = 2 * kClassPad;        // tensor memory of a group: upper and lower rows of warps 0-3 and
                                                                             // 4-7; the weight gradient of 256 channels
 constexpr int kMaxPlaces = 7, kIssuers = 2;
-// Registers with FORWARD.  Warps beyond sixteen put five on a scheduler, whose 16384 registers then give 96 a thread at launch; the
-// warpgroup of the producer and the issuer (its two others return at once) gives back what the sixteen take.
-constexpr int kLaunchRegs = 96, kWorkerRegs = 112, kFeederRegs = 32;
-static_assert(kGroups * F_WORKERS * kWorkerRegs + 128 * kFeederRegs <= F_THREADS * kLaunchRegs, "registers handed on are registers the block was launched with");
+// A place of the ring.  Two groups: five node rows of 64 channels, so that a tile's channels are two chunks, rows 0-4 and 4-8.  One group,
+// whose shared memory holds one such place next to 21 classes: the tile's nine rows of 32 channels, of which there is room for two.  (Half rows
+// read from HBM are slower: with them in two groups 16 streams take 3312 us a call, 3260 with whole ones; one frame's 272 either way.)
+__host__ __device__ constexpr bool half_rows(int form) { return form == kOneGroup; }
+__host__ __device__ constexpr uint32_t chunk_bytes(int form) { return half_rows(form) ? F_ROWS * kRowBytes / 2 : 5 * kRowBytes; }
+// Registers with an own forward.  A scheduler's 16384 registers give 96 a thread at launch with five warps on it (two groups), 80 with six
+// (two blocks of one); the warpgroup of the producer and the issuers (its fourth warp returns at once) gives back what the workers take.
+constexpr int kFeederRegs = 32;
+__host__ __device__ constexpr int form_launch_regs(int form) { return form == kTwoGroups ? 96 : 80; }
+__host__ __device__ constexpr int form_worker_regs(int form) { return form == kTwoGroups ? 112 : 104; }
+constexpr bool regs_add_up(int form) { return form_groups(form) * F_WORKERS * form_worker_regs(form) + 128 * kFeederRegs <= form_threads(form) * form_launch_regs(form); }
+static_assert(regs_add_up(kOneGroup) && regs_add_up(kTwoGroups), "registers handed on are registers the block was launched with");
 
-// Shared memory.  With FORWARD a block has an SM to itself: the ring, then the two groups' arrays.  The ring's places go on over the
-// second group's slots, which are free until that group has its first logits (and for good where the block has one tile).
-template <int C, bool CONF, bool FORWARD>
+// Shared memory: the ring, then the groups' arrays.  The ring's places go on over the last group's slots, which are free until that
+// group has its first logits (and for good where it has no tile).
+template <int C, bool CONF, int FORM>
 struct FwdCeSmem {
+    static constexpr bool FORWARD = FORM != kStored;
+    static constexpr uint32_t kChunkBytes = chunk_bytes(FORM);
     static constexpr size_t kSlots = (size_t)F_WARPS * C * 32 * sizeof(float2), kCounts = (size_t)((C + 1) / 2) * kNodes * sizeof(uint32_t),
                             kHist = CONF ? (size_t)C * C * sizeof(unsigned int) : 0, kWeights = FORWARD ? (size_t)fused::kMaxKBlocks * kWBytes : 0;
-    static constexpr int kN = FORWARD ? kGroups : 1;
-    static constexpr size_t kGrad = FORWARD && classifier_gradient_fits(C) ? (size_t)4 * kWBytes : 0;     // bf16 gradient of a tile's own nodes: [two node rows][32 classes][64 nodes]
+    static constexpr int kN = form_groups(FORM);
+    static constexpr size_t kGrad = FORM == kTwoGroups && classifier_gradient_fits(C) ? (size_t)4 * kWBytes : 0;     // bf16 gradient of a tile's own nodes: [two node rows][32 classes][64 nodes]
     static constexpr size_t kFixed = kN * (kSlots + kCounts + kHist + kGrad) + kWeights;
-    static constexpr size_t kMost = 227 * 1024 - 1024 - 4864;                // less the alignment and the static arrays
-    static constexpr int kSteady = !FORWARD ? 0 : (kMost - kFixed) / kChunkBytes > 4 ? 4 : (int)((kMost - kFixed) / kChunkBytes);
+    // less what the system keeps of a block's share, the alignment and the static arrays
+    static constexpr size_t kStatic = kN * (F_WARPS * 256 + 64) + 512, kMost = (FORM == kTwoGroups ? 228 * 1024 : 114 * 1024) - 2048 - kStatic;
+    static constexpr int kSteady = !FORWARD ? 0 : kMost < kFixed ? 0 : (kMost - kFixed) / kChunkBytes > 4 ? 4 : (int)((kMost - kFixed) / kChunkBytes);
     static constexpr int kExtra = !FORWARD ? 0 : kSteady + (int)(kSlots / kChunkBytes) > kMaxPlaces ? kMaxPlaces - kSteady : (int)(kSlots / kChunkBytes);
-    static_assert(!FORWARD || kSteady >= 1, "a block's shared memory");
-    // the second group's slots lie behind the ring, the first group's behind them
+    static constexpr bool kFits = !FORWARD || (kMost >= kFixed && kSteady >= 1);
+    // the last group's slots lie behind the ring
     static constexpr size_t kSlotsAt = kSteady * (size_t)kChunkBytes, kWeightsAt = kSlotsAt + kN * kSlots, kGradAt = kWeightsAt + kWeights,
                             kCountsAt = kGradAt + kN * kGrad, kHistAt = kCountsAt + kN * kCounts, kBytes = kHistAt + kN * kHist + 1024;
 };
@@ -155,12 +172,16 @@ __device__ __forceinline__ void add_counts(uint32_t* node, int cls, int right, i
     atomicAdd(w + below + right, br << sh);
 }
 
-template <int C, bool CONF, bool FORWARD>
-__global__ void __launch_bounds__(FORWARD ? F_THREADS : F_WORKERS, FORWARD ? 1 : 2)
+template <int C, bool CONF, int FORM>
+__global__ void __launch_bounds__(form_threads(FORM), FORM == kTwoGroups ? 1 : 2)
 fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map,
               const __grid_constant__ CUtensorMap row_map)
 {
-    using Smem = FwdCeSmem<C, CONF, FORWARD>;
+    using Smem = FwdCeSmem<C, CONF, FORM>;
+    static_assert(Smem::kFits, "a block's shared memory");
+    constexpr bool FORWARD = FORM != kStored, with_grad = Smem::kGrad != 0;        // (with_grad: the classifier's weight gradient as well)
+    constexpr int kGroups = form_groups(FORM), kAllWarps = kGroups * F_WARPS;
+    constexpr uint32_t kChunkBytes = Smem::kChunkBytes;
     extern __shared__ __align__(128) uint8_t smem_f[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_f + 1023) & ~(uintptr_t)1023);
     __shared__ __align__(8) uint64_t bars[2 * kMaxPlaces + 1 + 5 * kGroups];
@@ -171,12 +192,11 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
     // barriers: places of the ring filled / free, weights; per group: logits there / taken, gradient there, its product there / taken
     const uint32_t full_bar = tc::smem_u32(&bars[0]), free_bar = full_bar + 8 * kMaxPlaces, w_bar = full_bar + 16 * kMaxPlaces, done_bars = w_bar + 8,
                    taken_bars = done_bars + 8 * kGroups, dz_bars = taken_bars + 8 * kGroups, grad_bars = dz_bars + 8 * kGroups, grad_taken_bars = grad_bars + 8 * kGroups;
-    const bool with_grad = FORWARD && a.w_part != nullptr;                 // the classifier's weight gradient as well
     const int h = a.h, w = a.w, H = h * kUp, W = w * kUp;
     const int64_t p = (int64_t)h * w;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), l = tid & 31;
     const int grp = FORWARD ? warp / F_WARPS : 0, wi = warp % F_WARPS, gtid = tid % F_WORKERS;       // (of the workers)
-    float2* slots = (float2*)(smem + Smem::kSlotsAt + (FORWARD && grp == 0 ? Smem::kSlots : 0));      // [F_WARPS][C][32]
+    float2* slots = (float2*)(smem + Smem::kSlotsAt + (grp + 1 < kGroups ? Smem::kSlots : 0));      // [F_WARPS][C][32]
     uint32_t* counts = (uint32_t*)(smem + Smem::kCountsAt + grp * Smem::kCounts);                    // [(C + 1) / 2][F_ROWS][F_COLS]
     unsigned int* hist = (unsigned int*)(smem + Smem::kHistAt + grp * Smem::kHist);                  // [C][C] (CONF)
     const int per_stream = tiles_x * tiles_y, n_tiles = per_stream * a.S;
@@ -196,7 +216,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
     auto tile_row = [&](const Tile& k) { return k.row == 0 ? tiles_y - 1 : k.row - 1; };
     auto node_x = [&](const Tile& k) { return k.col * FN_X; };             // the first node a tile owns
     auto node_y = [&](const Tile& k) { return tile_row(k) * FN_Y; };
-    const int tmem_cols = (with_grad ? 4 : 2) * kLogitCols;
+    constexpr int tmem_cols = (with_grad ? 2 : 1) * kGroups * kLogitCols;
 
     if (FORWARD && warp == kAllWarps + 1) {
         if (tc::elect_one()) { tc::prefetch_map(&x_map); tc::prefetch_map(&w_map); if (with_grad) tc::prefetch_map(&row_map); }
@@ -252,7 +272,8 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
             };
             auto load_rows = [&](const Tile& k, int e, uint32_t stall) {   // chunk e of F
                 if (!claim(kChunkBytes + stall)) return;
-                tc::tma_load_4d(ring + place * kChunkBytes, &x_map, full_bar + 8 * place, (e >> 1) * 64, node_x(k) - 1, node_y(k) - 1 + 4 * (e & 1), k.s);
+                tc::tma_load_4d(ring + place * kChunkBytes, &x_map, full_bar + 8 * place, half_rows(FORM) ? e * 32 : (e >> 1) * 64, node_x(k) - 1,
+                                node_y(k) - 1 + (half_rows(FORM) ? 0 : 4 * (e & 1)), k.s);
                 advance();
             };
             // Inside the step loop the features are frozen: the first chunks are fetched while the previous update still runs
@@ -273,15 +294,15 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
             Tile back = k;                                 // the tile whose weight gradient comes next
             int w_stream = -1, n_weights = 0, n_items = 0;
             for (int q = 0; ok && (k.t < n_tiles || (with_grad && back.t < n_tiles)); ++q) {
-                if (q == 2 && n_items > 1) { n_places = Smem::kSteady; place = 0; }
+                if (q == kGroups && n_items == kGroups) { n_places = Smem::kSteady; place = 0; }
                 if (k.t < n_tiles) {
-                    const int g = q & 1, j = q >> 1;
+                    const int g = q % kGroups, j = q / kGroups;
                     if (producer) {
                         for (int e = q == 0 ? pre : 0; e < 2 * kblocks && ok; ++e) load_rows(k, e, q == 0 && e == 0 && a.test_stall ? 16u : 0u);
                     } else {
                         constexpr uint32_t idesc = tc::instr_desc(128, kClassPad, 0, 0);
                         if (w_stream != k.s) {             // the weights of the stream before are read until the last tile's logits are there
-                            if (q) wait(done_bars + 8 * ((q - 1) & 1), ((q - 1) >> 1) & 1, tc::kWaitDone);
+                            if (q) wait(done_bars + 8 * ((q - 1) % kGroups), ((q - 1) / kGroups) & 1, tc::kWaitDone);
                             if (ok && me == 0) {
                                 tc::mbar_expect_tx(w_bar, (uint32_t)kblocks * kWBytes);
                                 for (int kb = 0; kb < kblocks; ++kb) tc::tma_load_3d(w_base + kb * kWBytes, &w_map, w_bar, kb * 64, 0, k.s);
@@ -302,12 +323,21 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                             parity ^= bit;
                             if (!ok) break;
                             tc::tc_fence_after_sync();
-                            const uint64_t dx = tc::smem_desc(ring + place * kChunkBytes + me * kRowBytes, 16, 1024);
-                            const uint32_t to = logits + (e & 1) * kClassPad;  // (rows 0-3, 4-7 upper; 1-4, 5-8 lower)
+                            const uint32_t at = ring + place * kChunkBytes;
+                            // (rows 0-3, 4-7 upper; 1-4, 5-8 lower)
+                            if constexpr (half_rows(FORM)) {
+                                const uint64_t dx = tc::smem_desc_64(at + me * (kRowBytes / 2), 512);
 #pragma unroll
-                            for (int u = 0; u < 4; ++u) tc::umma(to, dx + 2 * u, dw + 2 * u, idesc, (e >> 1 | u) != 0);
+                                for (int u = 0; u < 4; ++u)
+                                    tc::umma(logits + (u & 1) * kClassPad, dx + (u & 1) * (2 * kRowBytes >> 4) + (u & 2), dw + (u & 2), idesc, (e | u >> 1) != 0);
+                                dw += e & 1 ? (kWBytes >> 4) - 4 : 4;  // two chunks to the weights' 64 channels
+                            } else {
+                                const uint64_t dx = tc::smem_desc(at + me * kRowBytes, 16, 1024);
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) tc::umma(logits + (e & 1) * kClassPad, dx + 2 * u, dw + 2 * u, idesc, (e >> 1 | u) != 0);
+                                if (e & 1) dw += kWBytes >> 4;
+                            }
                             tc::umma_commit(free_bar + 8 * place);
-                            if (e & 1) dw += kWBytes >> 4;
                             advance();
                         }
                         if (ok) tc::umma_commit(done_bars + 8 * g);
@@ -356,9 +386,9 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                 }
             }
             if (!producer) {
-                for (int it = n_items > 2 ? n_items - 2 : 0; it < n_items && ok; ++it) {
-                    wait(taken_bars + 8 * (it & 1), (it >> 1) & 1, tc::kWaitEmpty);
-                    if (with_grad) wait(grad_taken_bars + 8 * (it & 1), (it >> 1) & 1, tc::kWaitEmpty);
+                for (int it = n_items > kGroups ? n_items - kGroups : 0; it < n_items && ok; ++it) {
+                    wait(taken_bars + 8 * (it % kGroups), (it / kGroups) & 1, tc::kWaitEmpty);
+                    if (with_grad) wait(grad_taken_bars + 8 * (it % kGroups), (it / kGroups) & 1, tc::kWaitEmpty);
                 }
             }
             if (!ok) {                                     // nothing more is multiplied and nothing is written
@@ -375,7 +405,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
     }
 
     // -------------------------------------------------------------------- the workers
-    if (FORWARD) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWorkerRegs));
+    if (FORWARD) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(form_worker_regs(FORM)));
     const uint32_t done_bar = done_bars + 8 * grp, taken_bar = taken_bars + 8 * grp, dz_bar = dz_bars + 8 * grp, grad_bar = grad_bars + 8 * grp,
                    grad_taken = grad_taken_bars + 8 * grp, logits_at = tmem + grp * kLogitCols, grads_at = tmem + kGroups * kLogitCols + grp * kGradCols;
     float2* my = slots + (size_t)wi * C * 32 + l;          // this lane's slot of class c: my[c * 32]
@@ -815,7 +845,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
             for (int r = 0; r < F_WARPS; ++r) q += red[grp][n_done & 1][r];
             a.loss_part[(int64_t)s * per_stream + blk] = q;
         }
-        if (FORWARD) next(k);                              // the other group's
+        if (kGroups > 1) next(k);                          // the other group's
     }
     if (FORWARD && with_grad && n_done > 0) {
         if (tc::mbar_wait(grad_bar, (n_done - 1) & 1, a.err, tc::kWaitDone) && !gave_up) store_gradient(before);
@@ -823,40 +853,54 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
 }
 
 // A block that was launched with fewer registers than its warps ask for would wait for them forever
-inline cudaError_t check_launch_regs(const void* kernel)
+template <int C, bool CONF, int FORM>
+cudaError_t prepare_fwd_ce_form()
 {
+    const void* kernel = (const void*)fwd_ce_kernel<C, CONF, FORM>;
+    cudaError_t e = allow_shared_memory(kernel);
     cudaFuncAttributes at;
-    const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
-    return e != cudaSuccess ? e : at.numRegs < kLaunchRegs ? cudaErrorInvalidConfiguration : cudaSuccess;
+    if (FORM != kStored && e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
+    return e != cudaSuccess ? e : FORM != kStored && at.numRegs < form_launch_regs(FORM) ? cudaErrorInvalidConfiguration : cudaSuccess;
 }
 
 template <int C>
 cudaError_t prepare_fwd_ce_as()
 {
-    cudaError_t e = allow_shared_memory((const void*)fwd_ce_kernel<C, false, true>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, true, true>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, false, false>);
-    if (e == cudaSuccess) e = allow_shared_memory((const void*)fwd_ce_kernel<C, true, false>);
-    if (e == cudaSuccess) e = check_launch_regs((const void*)fwd_ce_kernel<C, false, true>);
-    if (e == cudaSuccess) e = check_launch_regs((const void*)fwd_ce_kernel<C, true, true>);
+    cudaError_t e = prepare_fwd_ce_form<C, false, kStored>();
+    if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kStored>();
+    if (e == cudaSuccess) e = prepare_fwd_ce_form<C, false, kTwoGroups>();
+    if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kTwoGroups>();
+    if constexpr (!loss_kernel_two_groups(C, false)) {
+        if (e == cudaSuccess) e = prepare_fwd_ce_form<C, false, kOneGroup>();
+        if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kOneGroup>();
+    }
     return e;
 }
 
-template <int C, bool CONF, bool FORWARD>
+template <int C, bool CONF, int FORM>
 void launch_fwd_ce_as(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s)
 {
-    using Smem = FwdCeSmem<C, CONF, FORWARD>;
-    const int tx = (a.w + FN_X - 1) / FN_X, ty = (a.h + FN_Y - 1) / FN_Y, tiles = tx * ty * a.S;
-    const int grid = FORWARD && tiles > a.n_sms ? a.n_sms : tiles;
+    using Smem = FwdCeSmem<C, CONF, FORM>;
+    const int tx = (a.w + FN_X - 1) / FN_X, ty = (a.h + FN_Y - 1) / FN_Y, tiles = tx * ty * a.S, resident = FORM == kStored ? tiles : a.n_sms * (FORM == kOneGroup ? 2 : 1);
     const size_t smem = one_per_sm(Smem::kBytes, tiles, a.n_sms);
-    launch_early(a.chain_early != 0 || a.x_early != 0, fwd_ce_kernel<C, CONF, FORWARD>, dim3(grid), dim3(FORWARD ? F_THREADS : F_WORKERS), smem, s, a, tx, ty, x_map, w_map, row_map);
+    launch_early(a.chain_early != 0 || a.x_early != 0, fwd_ce_kernel<C, CONF, FORM>, dim3(tiles < resident ? tiles : resident), dim3(form_threads(FORM)), smem, s, a, tx, ty, x_map, w_map, row_map);
+}
+
+template <int C, int FORM>
+void launch_fwd_ce_form(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s)
+{
+    if (a.conf) launch_fwd_ce_as<C, true, FORM>(a, x_map, w_map, row_map, s);
+    else launch_fwd_ce_as<C, false, FORM>(a, x_map, w_map, row_map, s);
 }
 
 template <int C, bool FORWARD>
 void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s)
 {
-    if (a.conf) launch_fwd_ce_as<C, true, FORWARD>(a, x_map, w_map, row_map, s);
-    else launch_fwd_ce_as<C, false, FORWARD>(a, x_map, w_map, row_map, s);
+    if constexpr (!FORWARD) launch_fwd_ce_form<C, kStored>(a, x_map, w_map, row_map, s);
+    else {
+        if constexpr (!loss_kernel_two_groups(C, false)) if (!loss_kernel_two_groups(C, a.w_part != nullptr)) return launch_fwd_ce_form<C, kOneGroup>(a, x_map, w_map, row_map, s);
+        launch_fwd_ce_form<C, kTwoGroups>(a, x_map, w_map, row_map, s);
+    }
 }
 
 }  // namespace

@@ -70,7 +70,7 @@ struct st_ctx {
     int n_split2 = 0;
     float *loss_part = nullptr, *db_part = nullptr;
     int n_k3_blocks = 0;
-    CUtensorMap fx_map, fc_map, fr_map, fw_map; // maps of the classifier's input (tiles, five rows, one row) and of its bf16 weights: the loss kernel multiplies its own logits
+    CUtensorMap fx_map, fc_map, fr_map, fw_map; // maps of the classifier's input (tiles, what the loss kernel takes at a time, one row) and of its bf16 weights: the loss kernel multiplies its own logits
     int n_sms = 0;
     int fused_loss = 0;         //   (bf16 GEMMs, the classifier's input of a shape fused_forward_supported names; ST_FUSED_FORWARD=0
     int fused_fwd = 0;          //   switches it off); with a one-layer head the student-mask kernel does so too
@@ -805,7 +805,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
             const uint64_t dims[3] = {ci, (uint64_t)kClassPad, (uint64_t)S}, str[2] = {ci * 2, (uint64_t)kClassPad * ci * 2};
             const uint32_t box[3] = {64, (uint32_t)kClassPad, 1};
             const bf16* x = n_blocks ? c->blk[n_blocks - 1].out : c->x_bf16;
-            bool made = make_feature_tile_map(&c->fx_map, x, S, c_last, c->h, c->w) && make_feature_chunk_map(&c->fc_map, x, S, c_last, c->h, c->w) &&
+            bool made = make_feature_tile_map(&c->fx_map, x, S, c_last, c->h, c->w) && make_feature_chunk_map(&c->fc_map, x, S, c_last, c->h, c->w, loss_kernel_two_groups(c->C, c->fused_grad != 0)) &&
                         make_feature_row_map(&c->fr_map, x, S, c_last, c->h, c->w) &&
                             encode_tensor_map(&c->fw_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, c->w2_shadow, 3,
                                               dims, str, box, msg, sizeof msg, "1x1 weight");

@@ -147,11 +147,13 @@ bool fused_forward_supported(int C, int h, int w, int c_in);
 // Class counts with which the weight gradient of a one-layer head fits it too: two places of the ring at least beside the gradients of two
 // tiles (25 classes have one)
 constexpr bool classifier_gradient_fits(int C) { return C <= 24; }
+// ... and two groups of warps to a block where it is formed, or where two blocks of one group do not fit an SM (k_fwd_ce.cuh)
+constexpr bool loss_kernel_two_groups(int C, bool with_gradient) { return with_gradient || !classifier_gradient_fits(C); }
 cudaError_t prepare_fwd_ce(int C);
 void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s);
 // Tile map of bf16 features [S][h][w][c_in] for it: {c_in, w, h, S}, one box = 64 channels of a tile
 bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w);
-bool make_feature_chunk_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w); // ... of five rows of a tile
+bool make_feature_chunk_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w, bool two_groups); // ... what the loss kernel's ring takes at a time
 bool make_feature_row_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w);   // ... of one row
 // the part of launch_upsample_ce for C <= 32 (k_fwd_ce.cuh)
 bool upsample_ce_few_supported(int C);
