@@ -742,6 +742,10 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
 // gradient arrives with one column more on either side, and the B operand of 192 columns is its 64 channels three times, each block
 // of 64 one pixel (128 bytes) behind the one before it, which is the descriptor's stride between blocks.  Both operands are
 // MN-major (pixel-major tensors, reduction over pixels).
+// Where the input ends on an odd 64 channels, those stand twice in the A operand, an image row apart (five rows of pixels, the
+// descriptor's stride again), and a block forms two vertical taps of theirs; the third has an operand to itself, half of which nobody
+// looks at.  With such an operand for each of the three / so, us: 192 -> 128 at 720p 24.0 / 22.0, 192 -> 64 14.7 / 13.6, three of
+// 101 x 187, 192 -> 128 33.7 / 32.8 (longer ranges for the same number of blocks become more and shorter ones).
 // Bound by the tensor pipe (96 cycles for 192 columns; a chunk of eight takes 810 to 850 with 64 output channels a block, whose copies
 // come at 60 bytes a cycle, and 1610 with 128) and by the partial sums at its end: 3 us for 14 MB at 256 channels.  A block per tap and
 // all input channels, N = the output channels, before / now, us at 720p: 192 -> 64 20.3 / 15.1, 64 -> 64 14.1 / 10.3, 192 -> 128 28.4 /
@@ -750,6 +754,10 @@ tc_fwd3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // {C1, w, h, S}    
 // ------------------------------------------------------------------------------------------------
 constexpr uint32_t kWg3ABytes = kChunkW * kChunkH * 128, kWg3BCols = kChunkW + 2, kWg3BBytes = kWg3BCols * kChunkH * 128;   // 64 channels of a chunk
 static_assert(kWg3ABytes % 1024 == 0 && kWg3BBytes % 1024 == 0, "the operands begin where the swizzle pattern does");
+constexpr uint32_t kWg3OddBytes = kChunkW * (kChunkH + 1) * 128;
+static_assert(kWg3OddBytes <= 2 * kWg3ABytes, "five rows of 64 channels lie where four of 128 do");
+// blocks of one pixel range and output-channel group: three vertical taps per 128 input channels, two of an odd 64 in one
+__host__ __device__ constexpr int wg3_units(int c_in) { return 3 * (c_in / kTileM) + 2 * (c_in / kBlockK % 2); }
 __host__ __device__ constexpr uint32_t wg3_stage_bytes(int cob) { return 2 * kWg3ABytes + cob * kWg3BBytes; }
 
 template <int STAGES, int COB>
@@ -757,6 +765,8 @@ __global__ void __launch_bounds__(kThreadsTc)
 tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output {C1, w, h, S} box {64, 32, 4, 1}
                    const __grid_constant__ CUtensorMap tmA2,  // skip input      {C2, w, h, S} same box (unused if C2 == 0)
                    int blocks1,                                // C1 / 64: input-channel blocks that come from tmA
+                   const __grid_constant__ CUtensorMap tmO,   // where Cin ends on an odd 64: the source of those channels, box {64, 32, 5, 1}
+                   int odd_c0,                                 // ... and their place in it
                    const __grid_constant__ CUtensorMap tmB,   // dHd {Ch, w, h, S} box {64, 34, 4, 1}
                    float* __restrict__ partials,              // [S][n_split][9][Ch][Cin]
                    int Cin, int Ch, int chunks_x, int n_chunks, int chunks_per_block, int n_split, unsigned int* err,
@@ -771,10 +781,14 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     // the blocks of one pixel range are neighbours: what they share comes from L2
-    const int m_tiles = (Cin + kTileM - 1) / kTileM, units = 3 * m_tiles * (Ch / kBlockK / COB);
+    const int per_group = wg3_units(Cin), units = per_group * (Ch / kBlockK / COB);
     const int unit = blockIdx.x % units, split = blockIdx.x / units, s = blockIdx.y;
-    const int ky = unit % 3, m = unit / 3 % m_tiles, cg = unit / 3 / m_tiles;
+    const int cg = unit / per_group, u = unit % per_group, m = min(u / 3, Cin / kTileM);
     const int a_blocks = min(2, Cin / kBlockK - 2 * m);
+    const bool paired = a_blocks == 1 && u == 3 * m;            // vertical taps 0 and 1 of the odd 64 channels
+    const int ky = a_blocks == 1 ? 2 * (u - 3 * m) : u - 3 * m;
+    // a chunk's first rows: of the gradient y0 + 1 - ky, or y0 where two taps share it and the input begins a row above
+    const int dy_b = paired ? 0 : 1 - ky;
     const int c_begin = min(n_chunks, split * chunks_per_block), c_end = min(n_chunks, c_begin + chunks_per_block);
 
     if (warp == 0) {
@@ -792,11 +806,12 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     tc_fence_after_sync();
     const uint32_t tmem = tmem_slot;
     bool ok = true;
-    // If a 128-channel tile ends on an odd 64, its upper half multiplies what lies in the stage; nobody looks at those rows.
+    // The third vertical tap of an odd 64 channels: the operand's upper half is what lies in the stage; nobody looks at those rows.
     auto load_a = [&](int i, int st) {                        // (one thread)
         const int x0 = i % chunks_x * kChunkW, y0 = i / chunks_x * kChunkH;
         const uint32_t bar = smem_u32(&full[st]), sa = base + st * kStage;
-        mbar_expect_tx(bar, a_blocks * kWg3ABytes + COB * kWg3BBytes);
+        mbar_expect_tx(bar, (paired ? kWg3OddBytes : a_blocks * kWg3ABytes) + COB * kWg3BBytes);
+        if (paired) { tma_load_4d(sa, &tmO, bar, odd_c0, x0, y0 - 1, s); return; }
         for (int j = 0; j < a_blocks; ++j) {
             const int cb = 2 * m + j;
             if (cb < blocks1) tma_load_4d(sa + j * kWg3ABytes, &tmA, bar, cb * kBlockK, x0, y0, s);
@@ -826,7 +841,7 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
                 if (i - c_begin >= n_pre) load_a(i, st);
                 const int x0 = i % chunks_x * kChunkW, y0 = i / chunks_x * kChunkH;
                 for (int j = 0; j < COB; ++j)
-                    tma_load_4d(base + st * kStage + 2 * kWg3ABytes + j * kWg3BBytes, &tmB, smem_u32(&full[st]), (cg * COB + j) * kBlockK, x0 - 1, y0 + 1 - ky, s);
+                    tma_load_4d(base + st * kStage + 2 * kWg3ABytes + j * kWg3BBytes, &tmB, smem_u32(&full[st]), (cg * COB + j) * kBlockK, x0 - 1, y0 + dy_b, s);
             }
             __syncwarp();
             if (++st == STAGES) { st = 0; parity ^= 1; }
@@ -834,7 +849,7 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     } else if (warp == 1) {      // one thread issues
         if (elect_one()) {
             constexpr uint32_t idesc = instr_desc(kTileM, 3 * kBlockK, 1, 1);
-            const uint64_t a0 = smem_desc(base, kWg3ABytes, 1024), b0 = smem_desc(base + 2 * kWg3ABytes, 128, 1024);
+            const uint64_t a0 = smem_desc(base, paired ? kChunkW * 128 : kWg3ABytes, 1024), b0 = smem_desc(base + 2 * kWg3ABytes, 128, 1024);
             const uint32_t f0 = smem_u32(&full[0]);
             int st = 0;
             uint32_t parity = 0;
@@ -865,8 +880,8 @@ tc_wgrad3x3_kernel(const __grid_constant__ CUtensorMap tmA,   // previous output
     tc_fence_after_sync();
     ok = __syncthreads_and(ok);
     if (ok) {
-        const int ci = m * kTileM + tid;
-        float* dst = partials + (((int64_t)s * n_split + split) * 9 + ky * 3) * Ch * Cin + (int64_t)cg * COB * kBlockK * Cin + ci;
+        const int ci = m * kTileM + (paired ? tid % kBlockK : tid), tap = ky + (paired ? tid / kBlockK : 0);
+        float* dst = partials + (((int64_t)s * n_split + split) * 9 + tap * 3) * Ch * Cin + (int64_t)cg * COB * kBlockK * Cin + ci;
         const bool any = c_end > c_begin;
         for (int c = 0; c < COB; ++c)
             for (int n0 = 0; n0 < 3 * kBlockK; n0 += 32) {
@@ -1205,7 +1220,7 @@ static Wg3Shape wg3_shape(int c_in, int c_out, int h, int w)
     q.chunks_x = (w + kChunkW - 1) / kChunkW;
     q.chunks = q.chunks_x * ((h + kChunkH - 1) / kChunkH);
     for (q.cob = c_out % 128 == 0 ? 2 : 1;; q.cob = 1) {
-        q.units = 3 * ((c_in + kTileM - 1) / kTileM) * (c_out / kBlockK / q.cob);
+        q.units = wg3_units(c_in) * (c_out / kBlockK / q.cob);
         const int ranges = std::min(148 / q.units, q.chunks / kWg3LeastChunks);
         split_geometry(q.chunks, std::max(ranges, 1), &q.per, &q.n_split);
         if (q.cob == 1 || q.per >= 64) return q;
@@ -1217,6 +1232,7 @@ static decltype(&tc_wgrad3x3_kernel<3, 2>) wgrad3_kernel(const Wg3Shape& q) { re
 struct TcBlockPlan {
     CUtensorMap in_fwd, skip_fwd;    // the block's two inputs {C, w, h, S}, box {64, 8 halves + 2, 18, 1} (forward slabs)
     CUtensorMap in_wg, skip_wg;      // same tensors, box {64, 32, 4, 1} (weight-gradient chunks)
+    CUtensorMap odd_wg;              // the one that the last 64 of an odd number of channel blocks come from, box {64, 32, 5, 1}
     CUtensorMap w_map, w_map_q;      // {c_tot, 9*c_out, S}, boxes {64, c_out, 1} and {64, 64, 1}
     CUtensorMap wt_map, wt_map_q;    // mirrored, transposed weights {c_out, 9*c_prev, S}, boxes {64, c_prev, 1} and {64, 64, 1}
     CUtensorMap dout_fwd;            // the block's output gradient {c_out, w, h, S}, the slab's box (A operand when passed back)
@@ -1319,6 +1335,11 @@ TcPlan* tc_plan_create(const TcBuffers& b, char* err, size_t err_len)
         ok = ok && act_maps(k.in_prev, c1, q.walk_fwd.halves, &q.in_fwd, &q.in_wg, kChunkW, "block input");
         if (c2) ok = ok && act_maps(k.in_skip, c2, q.walk_fwd.halves, &q.skip_fwd, &q.skip_wg, kChunkW, "skip input");
         else { q.skip_fwd = q.in_fwd; q.skip_wg = q.in_wg; }
+        {
+            const uint64_t c = c2 ? c2 : c1, d[4] = {c, w, h, S}, st[3] = {c * 2, w * c * 2, h * w * c * 2};
+            const uint32_t bo[4] = {64, (uint32_t)kChunkW, (uint32_t)kChunkH + 1, 1};
+            ok = ok && make_map(&q.odd_wg, c2 ? k.in_skip : k.in_prev, 4, d, st, bo, err, err_len, "block input (odd 64 channels)");
+        }
         ok = ok && act_maps(k.dout, co, q.walk_back.halves, &q.dout_fwd, &q.dout_wg, kWg3BCols, "block output gradient");
         {
             uint64_t dw[3] = {ct, 9 * co, S}, sw[2] = {ct * 2, 9 * co * ct * 2};
@@ -1487,7 +1508,7 @@ int tc_backward(const TcPlan* P, cudaStream_t s, StageTimer* t, const int* skip,
         const TcBlock& k = b.blk[i];
         const TcBlockPlan& q = P->blk[i];
         ST_REPEAT(t) launch_early(b.chain_early != 0, wgrad3_kernel(q.wg), dim3(q.wg.units * q.wg.n_split, b.S), dim3(kThreadsTc),
-            wg3_bytes(q.wg), s, q.in_wg, q.skip_wg, k.c_prev / kBlockK, q.dout_wg, k.w_partials, k.c_prev + k.c_skip, k.c_out, q.wg.chunks_x, q.wg.chunks,
+            wg3_bytes(q.wg), s, q.in_wg, q.skip_wg, k.c_prev / kBlockK, q.odd_wg, (k.c_skip ? k.c_skip : k.c_prev) - kBlockK, q.dout_wg, k.w_partials, k.c_prev + k.c_skip, k.c_out, q.wg.chunks_x, q.wg.chunks,
             q.wg.per, q.wg.n_split, b.err, skip, skip_stride, i == 0 && !skip && !t && b.chain_early ? 1 : 0);
         if (t) t->mark(kWg3Names[i], s, st_repeats(t));
         n += st_repeats(t);
