@@ -20,6 +20,8 @@ bool pdl_enabled()
 }
 
 constexpr int kUpdThreads = 256;
+// how a layer is streamed (LayerUpdate::streamed): 1 or 4 weights to a thread, or the sums of its partials in vectors by 8, 16 or 64 lanes
+constexpr int kVec8 = 8, kVec16 = 16, kVec64 = 64;
 static_assert(kUpdThreads == kMiouFetchThreads, "the update fetches the confusion matrix with all of its threads");
 
 // bf16 copies of weight element e (internal order [tap][cout][cin]) of a layer: the one the forward and the weight
@@ -94,19 +96,81 @@ __device__ __forceinline__ float apply_update(const UpdateArgs& a, int64_t gi, f
     return apply_update<ADAM>(a, gi, g, k, load_state<ADAM>(a, gi));
 }
 
+// Train, for a block that streams: does this prediction go on to the step (skip), was it the best so far.  With DECIDES a warp of its own finds
+// out; `verdict` holds the answer behind the block's next barrier.  false: the thread has nothing more to do.  (The grouped part's
+// first block writes the history.)
+template <bool DECIDES>
+__device__ __forceinline__ bool stream_control(const UpdateArgs& a, int s, const TrainHistory& hist, int& verdict, bool& skip, bool& better)
+{
+    skip = a.skip && a.skip[(int64_t)s * a.skip_stride]; better = false;
+    if (DECIDES) {
+        if (hist.ended) return false;
+        if (threadIdx.x >= kUpdThreads) {
+            train_decision_warp(a.ctl, s, false, hist, skip, better);
+            if ((threadIdx.x & 31) == 0) verdict = (skip ? 1 : 0) | (better ? 2 : 0);
+            __syncthreads();
+            return false;
+        }
+        return true;
+    }
+    if (a.has_ctl == 1) { const MiouFetch f = train_fetch(a.ctl, s, hist); train_decision(a.ctl, s, false, hist, &f, skip, better); }
+    else if (a.has_ctl && hist.ended) skip = true;
+    else if (a.has_ctl) train_outcome(a.ctl, s, skip, better);
+    return !skip || better;
+}
+
+// A layer of fewer weights.  A block takes 4 LANES consecutive weights: its thread groups of LANES read every
+// G-th partial sum as vectors, `B` of them in flight, the group sums are added in group order, and then a thread takes the step for one weight.
+// A thread per weight and group with scalar loads (the grouped part below) read twelve streams of 23 times 36864 weights at 1 TB/s.
+template <int LANES, int B, bool ADAM, bool DECIDES>
+__device__ __forceinline__ void update_vectors(const UpdateArgs& a, const LayerUpdate& ly, int s, int block, const AdamCorr& corr, int& verdict, float4 (&part)[kUpdThreads])
+{
+    constexpr int G = kUpdThreads / LANES, W = 4 * LANES;
+    const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps, e = (int64_t)block * W + threadIdx.x, gi = (int64_t)s * a.n_params + ly.w_off + e;
+    const bool mine = threadIdx.x < W && e < nw;
+    ParamState state{};
+    if (mine) state = load_state<ADAM>(a, gi);
+    const TrainHistory hist = a.has_ctl ? train_history(a.ctl, s) : TrainHistory{};
+    pdl_wait();
+    pdl_launch_dependents();
+    bool skip, better;
+    if (!stream_control<DECIDES>(a, s, hist, verdict, skip, better)) return;
+    const int lane = threadIdx.x % LANES;
+    const int64_t v = (int64_t)block * W + 4 * lane;
+    const float* src = ly.w_partials + (int64_t)s * ly.w_stream_stride + v;
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = threadIdx.x / LANES; k0 < ly.n_split; k0 += B * G) {
+        float4 t[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            t[j] = k0 + j * G < ly.n_split && v < nw ? __ldg(reinterpret_cast<const float4*>(src + (int64_t)(k0 + j * G) * ly.w_split_stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < B; ++j) { sum.x += t[j].x; sum.y += t[j].y; sum.z += t[j].z; sum.w += t[j].w; }
+    }
+    part[threadIdx.x] = sum;
+    __syncthreads();
+    if (DECIDES) { skip = (verdict & 1) != 0; better = (verdict & 2) != 0; }
+    if (!mine || (skip && !better)) return;
+    const float* sums = reinterpret_cast<const float*>(part);
+    float g = 0.f;
+#pragma unroll
+    for (int k = 0; k < G; ++k) g += sums[k * W + threadIdx.x];
+    if (better) a.ctl.best_theta[gi] = state.theta;
+    if (!skip) write_shadows(ly, s, e, apply_update<ADAM>(a, gi, g, corr, state));
+}
+
+// weights of a block that streams a layer, by LayerUpdate::streamed
+__host__ __device__ constexpr int streamed_per_block(int code) { return code >= kVec8 ? 4 * code : kUpdThreads * code; }
+
 // A large weight tensor with a moderate number of split-K partials (a 3x3 layer): a pure stream.  Each thread owns VEC
 // consecutive weights and reads them from every partial with all loads in flight.
-template <int VEC, bool ADAM>
-__device__ __forceinline__ void update_stream(const UpdateArgs& a, const LayerUpdate& ly, int s, int block, const AdamCorr& corr)
+template <int VEC, bool ADAM, bool DECIDES>
+__device__ __forceinline__ void update_stream(const UpdateArgs& a, const LayerUpdate& ly, int s, int block, const AdamCorr& corr, int& verdict)
 {
-    bool skip = a.skip && a.skip[(int64_t)s * a.skip_stride], better = false;
-    if (a.has_ctl) {                                                   // the grouped part's first block writes the history
-        const TrainHistory hist = train_history(a.ctl, s);
-        if (a.has_ctl == 1) { const MiouFetch f = train_fetch(a.ctl, s, hist); train_decision(a.ctl, s, false, hist, &f, skip, better); }
-        else if (hist.ended) skip = true;
-        else train_outcome(a.ctl, s, skip, better);
-    }
-    if (skip && !better) return;
+    pdl_wait();
+    pdl_launch_dependents();
+    bool skip, better;
+    if (!stream_control<DECIDES>(a, s, a.has_ctl ? train_history(a.ctl, s) : TrainHistory{}, verdict, skip, better)) return;
     const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
     const int64_t mine = ((int64_t)block * kUpdThreads + threadIdx.x) * VEC, e = mine < nw ? mine : 0;    // (behind the end: loads for nothing)
     const float* src = ly.w_partials + (int64_t)s * ly.w_stream_stride + e;
@@ -143,8 +207,9 @@ __device__ __forceinline__ void update_stream(const UpdateArgs& a, const LayerUp
             for (int j = 0; j < 8; ++j) g[0] += t[j];
         }
     }
-    if (ADAM) __syncthreads();                                         // `corr` is there
-    if (mine >= nw) return;
+    if (ADAM || DECIDES) __syncthreads();                              // `corr` and `verdict` are there
+    if (DECIDES) { skip = (verdict & 1) != 0; better = (verdict & 2) != 0; }
+    if (mine >= nw || (skip && !better)) return;
     if (!vec || skip) {
 #pragma unroll
         for (int j = 0; j < VEC; ++j) {
@@ -175,7 +240,7 @@ __device__ __forceinline__ void update_stream(const UpdateArgs& a, const LayerUp
 // block each sum every G-th split-K partial of "their" parameter (coalesced along the parameters),
 // the group sums are added in group order through shared memory, and group 0 applies the update.
 // `B` of its loads are in flight at a time.  With DECIDES (Train) a block has one warp more, which assesses the prediction meanwhile.
-template <int G, int E, int B, bool ADAM, bool DECIDES>
+template <int G, int E, int B, bool ADAM, bool DECIDES, bool VECS>
 __global__ void __launch_bounds__(kUpdThreads + (DECIDES ? 32 : 0))
 sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
 {
@@ -188,17 +253,22 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
     const int64_t base = (int64_t)s * a.n_params;
     adam_corrections<ADAM>(a, s, corr);                  // (the step count was written by an earlier call's last kernel)
     if ((int)blockIdx.x >= n_grouped) {                  // the streamed layers' blocks lie behind the grouped ones
-        pdl_wait();
-        pdl_launch_dependents();
         int block = (int)blockIdx.x - n_grouped;
         for (int L = 0; L < a.n_layers; ++L) {
             const LayerUpdate& ly = a.layer[L];
             if (!ly.streamed) continue;
-            const int per = kUpdThreads * (ly.streamed == 4 ? 4 : 1);
+            const int per = streamed_per_block(ly.streamed);
             const int blocks = (int)(((int64_t)ly.cout * ly.cin * ly.taps + per - 1) / per);
             if (block >= blocks) { block -= blocks; continue; }
-            if (ly.streamed == 4) update_stream<4, ADAM>(a, ly, s, block, corr);
-            else update_stream<1, ADAM>(a, ly, s, block, corr);
+            if constexpr (VECS) {
+                __shared__ float4 vec_part[kUpdThreads];
+                if (ly.streamed == kVec8) update_vectors<8, 10, ADAM, DECIDES>(a, ly, s, block, corr, verdict, vec_part);
+                else if (ly.streamed == kVec16) update_vectors<16, 10, ADAM, DECIDES>(a, ly, s, block, corr, verdict, vec_part);
+                else update_vectors<64, 8, ADAM, DECIDES>(a, ly, s, block, corr, verdict, vec_part);
+            } else {
+                if (ly.streamed == 4) update_stream<4, ADAM, DECIDES>(a, ly, s, block, corr, verdict);
+                else update_stream<1, ADAM, DECIDES>(a, ly, s, block, corr, verdict);
+            }
             return;
         }
         return;
@@ -363,16 +433,24 @@ static int launch_sgd_update_t(const UpdateArgs& a, cudaStream_t s)
 {
     // Large layers are streamed, everything else (small layers, biases, loss) goes through the grouped part.  One launch: the
     // grouped part is all latency and hides behind the stream (256 -> 256 channels, 3x3: 19.9 us as two launches, 14.3 us as one, launch gap included).
+    // Heads of small layers only: the partial sums are read as vectors, shared among the thread groups of a block so that a thread's are one
+    // batch of loads: by 32 groups of 8 lanes, 16 of 16 or 4 of 64.  us a step, a thread per weight and group / so: 5376 weights and 286 partial
+    // sums 26.1 / 25.1, sixteen streams 286.5 / 278.5; 36864 weights and 23 partial sums 35.8 / 29.9, 65 partial sums 48.2 / 43.1, twelve streams of 7 79.4 / 53.2;
+    // 73728 and 23 33.7 / 32.5.  From 110592 weights on no gain over a thread's whole vectors, next to which the small layers hide.
     UpdateArgs g = a;
     int64_t stream_blocks = 0, n_rest = 0;
+    auto vectors = [&](const LayerUpdate& ly) {
+        return (int64_t)ly.cout * ly.cin * ly.taps % 4 == 0 && ly.w_split_stride % 4 == 0 && ly.w_stream_stride % 4 == 0 && ((uintptr_t)ly.w_partials % 16 == 0);
+    };
+    bool vecs = true;
+    for (int L = 0; L < a.n_layers; ++L) vecs = vecs && vectors(a.layer[L]) && a.layer[L].n_split > 1 && (int64_t)a.layer[L].cout * a.layer[L].cin * a.layer[L].taps < 98304;
     for (int L = 0; L < a.n_layers; ++L) {
         const LayerUpdate& ly = a.layer[L];
         const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
-        if (nw >= 65536) {
-            const bool vec = nw % 4 == 0 && ly.w_split_stride % 4 == 0 && ly.w_stream_stride % 4 == 0 &&
-                             ((uintptr_t)ly.w_partials % 16 == 0);
-            g.layer[L].streamed = vec ? 4 : 1;
-            const int per = kUpdThreads * (vec ? 4 : 1);
+        if (vecs) g.layer[L].streamed = ly.n_split > 160 ? kVec8 : ly.n_split > 32 || nw < 32768 ? kVec16 : kVec64;
+        else if (nw >= 65536) g.layer[L].streamed = vectors(ly) ? 4 : 1;
+        if (g.layer[L].streamed) {
+            const int per = streamed_per_block(g.layer[L].streamed);
             stream_blocks += (nw + per - 1) / per;
         } else n_rest += nw;
     }
@@ -389,16 +467,17 @@ static int launch_sgd_update_t(const UpdateArgs& a, cudaStream_t s)
     const int n_param_blocks = (int)((n_rest + per - 1) / per);
     const int n_grouped = n_param_blocks + n_red_blocks;
     const dim3 grid((unsigned)(n_grouped + stream_blocks), (unsigned)a.S);
-    const bool early = a.chain_early != 0, decides = a.has_ctl == 1 && a.ctl.C <= kWarpClasses && stream_blocks == 0 && !big;
+    const bool early = a.chain_early != 0, decides = a.has_ctl == 1 && a.ctl.C <= kWarpClasses && !big;
     auto launch = [&](auto kernel) { launch_early(early, kernel, grid, dim3(kUpdThreads + (decides ? 32 : 0)), 0, s, g, n_param_blocks, n_grouped); };
     // (a batch of loads is a round trip: 286 partial sums take one with twenty, three with eight)
     const bool many = G == 16 && max_split > 16 * 8;
-    if (G == 1 && E == 4) launch(sgd_update_kernel<1, 4, 8, ADAM, false>);
-    else if (E == 4) launch(sgd_update_kernel<8, 4, 8, ADAM, false>);
-    else if (G == 1) launch(decides ? sgd_update_kernel<1, 1, 8, ADAM, true> : sgd_update_kernel<1, 1, 8, ADAM, false>);
-    else if (G == 8) launch(decides ? sgd_update_kernel<8, 1, 8, ADAM, true> : sgd_update_kernel<8, 1, 8, ADAM, false>);
-    else if (many) launch(decides ? sgd_update_kernel<16, 1, 20, ADAM, true> : sgd_update_kernel<16, 1, 20, ADAM, false>);
-    else launch(decides ? sgd_update_kernel<16, 1, 8, ADAM, true> : sgd_update_kernel<16, 1, 8, ADAM, false>);
+    if (vecs) launch(decides ? sgd_update_kernel<1, 1, 8, ADAM, true, true> : sgd_update_kernel<1, 1, 8, ADAM, false, true>);
+    else if (G == 1 && E == 4) launch(sgd_update_kernel<1, 4, 8, ADAM, false, false>);
+    else if (E == 4) launch(sgd_update_kernel<8, 4, 8, ADAM, false, false>);
+    else if (G == 1) launch(decides ? sgd_update_kernel<1, 1, 8, ADAM, true, false> : sgd_update_kernel<1, 1, 8, ADAM, false, false>);
+    else if (G == 8) launch(decides ? sgd_update_kernel<8, 1, 8, ADAM, true, false> : sgd_update_kernel<8, 1, 8, ADAM, false, false>);
+    else if (many) launch(decides ? sgd_update_kernel<16, 1, 20, ADAM, true, false> : sgd_update_kernel<16, 1, 20, ADAM, false, false>);
+    else launch(decides ? sgd_update_kernel<16, 1, 8, ADAM, true, false> : sgd_update_kernel<16, 1, 8, ADAM, false, false>);
     return 1;
 }
 
