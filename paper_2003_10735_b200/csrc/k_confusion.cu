@@ -141,10 +141,14 @@ confusion_kernel(const uint8_t* __restrict__ label, const uint8_t* __restrict__ 
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    const double m = block_miou(conf, C, iou, present);
-    for (int i = threadIdx.x; i < CC; i += kConfThreads) {
-        fin.result[i] = __ldcg(conf + i);
-        conf[i] = 0;
+    double m;
+    if (MODE != 2) m = deliver_matrix<kConfThreads>(conf, C, fin.result, hist_all, iou, present);
+    else {                                                     // (no shared memory for the matrix)
+        m = block_miou(conf, C, iou, present);
+        for (int i = threadIdx.x; i < CC; i += kConfThreads) {
+            fin.result[i] = __ldcg(conf + i);
+            conf[i] = 0;
+        }
     }
     if (threadIdx.x == 0) { *fin.miou = m; *fin.ticket = 0; }
 }

@@ -143,13 +143,7 @@ student_eval_kernel(StudentMaskArgs a, const __grid_constant__ CUtensorMap x_map
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    const double m = block_miou(a.conf, C, iou, present);
-    if (a.conf_out) {
-        for (int e = tid; e < C * C; e += kThreads) {
-            a.conf_out[e] = __ldcg(&a.conf[e]);
-            a.conf[e] = 0;
-        }
-    }
+    const double m = deliver_matrix<kThreads>(a.conf, C, a.conf_out, hist, iou, present);
     if (tid == 0) {
         *a.miou = m;
         *a.ticket = 0;

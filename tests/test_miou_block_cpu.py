@@ -68,6 +68,27 @@ extern "C" int run(const unsigned long long* conf, int C, int threads, int prefe
     for (unsigned char b : m.after) stray += b != 0x5a;
     return stray;
 }
+// the same for a kernel's last block of 256 threads, which delivers the matrix as well
+extern "C" double deliver(unsigned long long* conf, int C, unsigned long long* result, unsigned int* stage)
+{
+    static double iou[256];
+    static int present[256];
+    double mean = 0;
+    blockDim = {256, 1, 1};
+    block_barrier = std::make_unique<std::barrier<>>(256);
+    warp_barrier.clear();
+    for (int k = 0; k < 8; ++k) warp_barrier.push_back(std::make_unique<std::barrier<>>(32));
+    lane_value.assign(256, 0);
+    std::vector<std::thread> block;
+    for (int t = 0; t < 256; ++t)
+        block.emplace_back([=, &mean] {
+            threadIdx = {(unsigned)t, 0, 0};
+            const double v = st::deliver_matrix<256>(conf, C, result, stage, iou, present);
+            if (t == 0) mean = v;
+        });
+    for (auto& t : block) t.join();
+    return mean;
+}
 """
 
 
@@ -87,6 +108,8 @@ def block_miou(tmp_path_factory):
         stray = run(flat.ctypes.data_as(ctypes.c_void_p), conf.shape[0], threads, int(prefetched), ctypes.byref(out))
         return out.value, stray
 
+    call.deliver = ctypes.CDLL(str(lib)).deliver
+    call.deliver.restype = ctypes.c_double
     return call
 
 
@@ -126,3 +149,14 @@ def test_block_miou_with_prefetched_counts(block_miou, C):
 
 def test_block_miou_of_an_empty_matrix(block_miou):
     assert block_miou(np.zeros((5, 5), np.int64), 320) == (0.0, 0)
+
+
+@pytest.mark.parametrize("C", [2, 21, 32, 33, 45, 46, 81, 255])    # 2025, 2116: a pass of eight counts per thread ends at 2048
+def test_last_block_delivers_the_matrix(block_miou, C):
+    conf = matrix(C, C).astype(np.uint64)
+    left, result, stage = np.append(conf, np.uint64(7)), np.full(C * C + 1, 5, np.uint64), np.full(C * C + 1, 3, np.uint32)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    assert block_miou.deliver(p(left), C, p(result), p(stage)) == expected(conf.astype(np.int64))
+    assert (result[:-1] == conf.ravel()).all() and not left[:-1].any()
+    assert (left[-1], result[-1], stage[-1]) == (7, 5, 3)
+    assert block_miou.deliver(p(result), C, None, p(stage)) == expected(conf.astype(np.int64)) and (result[:-1] == conf.ravel()).all()
