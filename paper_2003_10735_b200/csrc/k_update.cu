@@ -20,8 +20,8 @@ bool pdl_enabled()
 }
 
 constexpr int kUpdThreads = 256;
-// how a layer is streamed (LayerUpdate::streamed): 1 or 4 weights to a thread, or the sums of its partials in vectors by 8, 16 or 64 lanes
-constexpr int kVec8 = 8, kVec16 = 16, kVec64 = 64;
+// how a layer is streamed (LayerUpdate::streamed): 1 or 4 weights to a thread, or the sums of its partials in vectors by 8 to 64 lanes
+constexpr int kVec8 = 8, kVec16 = 16, kVec32 = 32, kVec64 = 64;
 static_assert(kUpdThreads == kMiouFetchThreads, "the update fetches the confusion matrix with all of its threads");
 
 // bf16 copies of weight element e (internal order [tap][cout][cin]) of a layer: the one the forward and the weight
@@ -264,6 +264,7 @@ sgd_update_kernel(UpdateArgs a, int n_param_blocks, int n_grouped)
                 __shared__ float4 vec_part[kUpdThreads];
                 if (ly.streamed == kVec8) update_vectors<8, 10, ADAM, DECIDES>(a, ly, s, block, corr, verdict, vec_part);
                 else if (ly.streamed == kVec16) update_vectors<16, 10, ADAM, DECIDES>(a, ly, s, block, corr, verdict, vec_part);
+                else if (ly.streamed == kVec32) update_vectors<32, 10, ADAM, DECIDES>(a, ly, s, block, corr, verdict, vec_part);
                 else update_vectors<64, 8, ADAM, DECIDES>(a, ly, s, block, corr, verdict, vec_part);
             } else {
                 if (ly.streamed == 4) update_stream<4, ADAM, DECIDES>(a, ly, s, block, corr, verdict);
@@ -434,7 +435,7 @@ static int launch_sgd_update_t(const UpdateArgs& a, cudaStream_t s)
     // Large layers are streamed, everything else (small layers, biases, loss) goes through the grouped part.  One launch: the
     // grouped part is all latency and hides behind the stream (256 -> 256 channels, 3x3: 19.9 us as two launches, 14.3 us as one, launch gap included).
     // Heads of small layers only: the partial sums are read as vectors, shared among the thread groups of a block so that a thread's are one
-    // batch of loads: by 32 groups of 8 lanes, 16 of 16 or 4 of 64.  us a step, a thread per weight and group / so: 5376 weights and 286 partial
+    // batch of loads: by 32 groups of 8 lanes, 16 of 16, 8 of 32 or 4 of 64.  us a step, a thread per weight and group / so: 5376 weights and 286 partial
     // sums 26.1 / 25.1, sixteen streams 286.5 / 278.5; 36864 weights and 23 partial sums 35.8 / 29.9, 65 partial sums 48.2 / 43.1, twelve streams of 7 79.4 / 53.2;
     // 73728 and 23 33.7 / 32.5.  From 110592 weights on no gain over a thread's whole vectors, next to which the small layers hide.
     UpdateArgs g = a;
@@ -447,7 +448,7 @@ static int launch_sgd_update_t(const UpdateArgs& a, cudaStream_t s)
     for (int L = 0; L < a.n_layers; ++L) {
         const LayerUpdate& ly = a.layer[L];
         const int64_t nw = (int64_t)ly.cout * ly.cin * ly.taps;
-        if (vecs) g.layer[L].streamed = ly.n_split > 160 ? kVec8 : ly.n_split > 32 || nw < 32768 ? kVec16 : kVec64;
+        if (vecs) g.layer[L].streamed = ly.n_split > 160 ? kVec8 : ly.n_split > 80 || nw < 32768 ? kVec16 : ly.n_split > 32 ? kVec32 : kVec64;
         else if (nw >= 65536) g.layer[L].streamed = vectors(ly) ? 4 : 1;
         if (g.layer[L].streamed) {
             const int per = streamed_per_block(g.layer[L].streamed);
