@@ -249,8 +249,10 @@ def test_bf16_steps_are_bit_reproducible():
 
 
 @pytest.mark.parametrize("c_in,ch,h,w", [
-    (64, 128, 72, 352),     # 198 tiles of 128 pixels: on 148 SMs the last 50 are cut into two channel ranges each
-    (64, 256, 56, 352),     # 154 tiles: the last 6 are cut into four channel ranges each
+    (64, 128, 72, 352),     # 110 items of two tiles of 16 x 8 pixels, one round on 148 SMs: none is cut
+    (64, 256, 56, 352),     # 176 items of one tile: the last 28 are cut into four channel ranges each
+    (64, 256, 56, 376),     # 188: the last 40 are cut into two
+    (64, 128, 104, 344),    # 301: the last 5 are cut into two
 ])
 def test_two_layer_forward_with_a_partly_filled_last_round(c_in, ch, h, w):
     C = 5
