@@ -12,7 +12,8 @@
 //
 // With an own forward a block is persistent: a producer feeds a ring of chunks by TMA, and two issuers (a thread each) feed the tensor core.
 // Where the weight gradient is formed too (one-layer heads), and with more than 24 classes, it has an SM to itself and two groups take its
-// tiles in turn; otherwise it is one group, and two blocks fit an SM.
+// tiles in turn; otherwise it is one group, and two blocks fit an SM.  A launch that forms the gradient of at most one tile per SM is one
+// group to a block too: half of the warps would have nothing to do, and its warps take their registers for more classes in flight.
 //   Logits.  The features of the tile's 9 x 32 nodes arrive in chunks (nodes outside the map arrive
 //   as zeros), and four multiplications per 16 channels leave node row i of the tile and node row i+1 of it in the same 32
 //   tensor-memory lanes: the two rows that warp i's cells lie between.  A warp therefore takes its logits out of tensor memory
@@ -67,17 +68,20 @@ constexpr int F_ROWS = fused::kTileRows, F_COLS = fused::kTileCols;         // n
 constexpr int FN_Y = fused::kOwnRows, FN_X = fused::kOwnCols;               // nodes a tile owns
 constexpr int F_WARPS = FN_Y + 1, F_WORKERS = F_WARPS * 32;                 // of a group: the warps that work on one tile
 // What a block is: one group that reads stored logits; one group with its own forward, two blocks to an SM; two groups with their own
-// forward, which have an SM to themselves
-enum Form { kStored = 0, kOneGroup = 1, kTwoGroups = 2 };
+// forward, which have an SM to themselves; one group alone on an SM, with the registers for more classes in flight
+enum Form { kStored = 0, kOneGroup = 1, kTwoGroups = 2, kLoneGroup = 3 };
+__host__ __device__ constexpr bool form_alone(int form) { return form == kTwoGroups || form == kLoneGroup; }
 __host__ __device__ constexpr int form_groups(int form) { return form == kTwoGroups ? 2 : 1; }
 __host__ __device__ constexpr int form_threads(int form) { return form_groups(form) * F_WORKERS + (form == kStored ? 0 : 128); }
 constexpr int kNodes = F_ROWS * F_COLS;
-constexpr int kSweep1 = 7, kSweep2 = 3;                                     // classes per iteration of the two sweeps
+constexpr int kSweep1 = 7;                                                  // classes per iteration of the first sweep, of the second
+__host__ __device__ constexpr int sweep2(int form) { return form == kLoneGroup ? 7 : 3; }
 constexpr uint32_t kWBytes = fused::kWeightBytes;
 constexpr uint32_t kRowBytes = F_COLS * 128;                                // a node row of 64 channels
 constexpr int kLogitCols = 4 * kClassPad, kGradCols = 2 * kClassPad;        // tensor memory of a group: upper and lower rows of warps 0-3 and
                                                                             // 4-7; the weight gradient of 256 channels
-constexpr int kMaxPlaces = 7, kIssuers = 2;
+constexpr int kIssuers = 2;
+__host__ __device__ constexpr int max_places(int form) { return form == kLoneGroup ? 8 : 7; }
 // A place of the ring.  Two groups: five node rows of 64 channels, so that a tile's channels are two chunks, rows 0-4 and 4-8.  One group,
 // whose shared memory holds one such place next to 21 classes: the tile's nine rows of 32 channels, of which there is room for two.  (Half rows
 // read from HBM are slower: with them in two groups 16 streams take 3312 us a call, 3260 with whole ones; one frame's 272 either way.)
@@ -86,10 +90,10 @@ __host__ __device__ constexpr uint32_t chunk_bytes(int form) { return half_rows(
 // Registers with an own forward.  A scheduler's 16384 registers give 96 a thread at launch with five warps on it (two groups), 80 with six
 // (two blocks of one); the warpgroup of the producer and the issuers (its fourth warp returns at once) gives back what the workers take.
 constexpr int kFeederRegs = 32;
-__host__ __device__ constexpr int form_launch_regs(int form) { return form == kTwoGroups ? 96 : 80; }
-__host__ __device__ constexpr int form_worker_regs(int form) { return form == kTwoGroups ? 112 : 104; }
+__host__ __device__ constexpr int form_launch_regs(int form) { return form == kTwoGroups ? 96 : form == kLoneGroup ? 168 : 80; }
+__host__ __device__ constexpr int form_worker_regs(int form) { return form == kTwoGroups ? 112 : form == kLoneGroup ? 232 : 104; }
 constexpr bool regs_add_up(int form) { return form_groups(form) * F_WORKERS * form_worker_regs(form) + 128 * kFeederRegs <= form_threads(form) * form_launch_regs(form); }
-static_assert(regs_add_up(kOneGroup) && regs_add_up(kTwoGroups), "registers handed on are registers the block was launched with");
+static_assert(regs_add_up(kOneGroup) && regs_add_up(kTwoGroups) && regs_add_up(kLoneGroup), "registers handed on are registers the block was launched with");
 
 // Shared memory: the ring, then the groups' arrays.  The ring's places go on over the last group's slots, which are free until that
 // group has its first logits (and for good where it has no tile).
@@ -100,11 +104,13 @@ struct FwdCeSmem {
     static constexpr size_t kSlots = (size_t)F_WARPS * C * 32 * sizeof(float2), kCounts = (size_t)((C + 1) / 2) * kNodes * sizeof(uint32_t),
                             kHist = CONF ? (size_t)C * C * sizeof(unsigned int) : 0, kWeights = FORWARD ? (size_t)fused::kMaxKBlocks * kWBytes : 0;
     static constexpr int kN = form_groups(FORM);
-    static constexpr size_t kGrad = FORM == kTwoGroups && classifier_gradient_fits(C) ? (size_t)4 * kWBytes : 0;     // bf16 gradient of a tile's own nodes: [two node rows][32 classes][64 nodes]
+    static constexpr size_t kGrad = form_alone(FORM) && classifier_gradient_fits(C) ? (size_t)4 * kWBytes : 0;     // bf16 gradient of a tile's own nodes: [two node rows][32 classes][64 nodes]
     static constexpr size_t kFixed = kN * (kSlots + kCounts + kHist + kGrad) + kWeights;
     // less what the system keeps of a block's share, the alignment and the static arrays
-    static constexpr size_t kStatic = kN * (F_WARPS * 256 + 64) + 512, kMost = (FORM == kTwoGroups ? 228 * 1024 : 114 * 1024) - 2048 - kStatic;
-    static constexpr int kSteady = !FORWARD ? 0 : kMost < kFixed ? 0 : (kMost - kFixed) / kChunkBytes > 4 ? 4 : (int)((kMost - kFixed) / kChunkBytes);
+    static constexpr size_t kStatic = kN * (F_WARPS * 256 + 64) + 512, kMost = (form_alone(FORM) ? 228 * 1024 : 114 * 1024) - 2048 - kStatic;
+    // (a lone group's one tile lies there whole, as far as there is room: all of it is fetched before the wait)
+    static constexpr int kMaxPlaces = max_places(FORM), kCap = FORM == kLoneGroup ? kMaxPlaces : 4;
+    static constexpr int kSteady = !FORWARD ? 0 : kMost < kFixed ? 0 : (kMost - kFixed) / kChunkBytes > kCap ? kCap : (int)((kMost - kFixed) / kChunkBytes);
     static constexpr int kExtra = !FORWARD ? 0 : kSteady + (int)(kSlots / kChunkBytes) > kMaxPlaces ? kMaxPlaces - kSteady : (int)(kSlots / kChunkBytes);
     static constexpr bool kFits = !FORWARD || (kMost >= kFixed && kSteady >= 1);
     // the last group's slots lie behind the ring
@@ -173,7 +179,7 @@ __device__ __forceinline__ void add_counts(uint32_t* node, int cls, int right, i
 }
 
 template <int C, bool CONF, int FORM>
-__global__ void __launch_bounds__(form_threads(FORM), FORM == kTwoGroups ? 1 : 2)
+__global__ void __launch_bounds__(form_threads(FORM), form_alone(FORM) ? 1 : 2)
 fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map,
               const __grid_constant__ CUtensorMap row_map)
 {
@@ -182,6 +188,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
     constexpr bool FORWARD = FORM != kStored, with_grad = Smem::kGrad != 0;        // (with_grad: the classifier's weight gradient as well)
     constexpr int kGroups = form_groups(FORM), kAllWarps = kGroups * F_WARPS;
     constexpr uint32_t kChunkBytes = Smem::kChunkBytes;
+    constexpr int kMaxPlaces = Smem::kMaxPlaces;
     extern __shared__ __align__(128) uint8_t smem_f[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_f + 1023) & ~(uintptr_t)1023);
     __shared__ __align__(8) uint64_t bars[2 * kMaxPlaces + 1 + 5 * kGroups];
@@ -216,7 +223,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
     auto tile_row = [&](const Tile& k) { return k.row == 0 ? tiles_y - 1 : k.row - 1; };
     auto node_x = [&](const Tile& k) { return k.col * FN_X; };             // the first node a tile owns
     auto node_y = [&](const Tile& k) { return tile_row(k) * FN_Y; };
-    constexpr int tmem_cols = (with_grad ? 2 : 1) * kGroups * kLogitCols;
+    constexpr int tmem_cols = (with_grad ? 2 : 1) * kGroups * kLogitCols;  // (a power of two)
 
     if (FORWARD && warp == kAllWarps + 1) {
         if (tc::elect_one()) { tc::prefetch_map(&x_map); tc::prefetch_map(&w_map); if (with_grad) tc::prefetch_map(&row_map); }
@@ -246,7 +253,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFeederRegs));
         if (warp > kAllWarps + kIssuers) return;
         // ---------------------------------------------------------------- the producer and the issuer
-        // Both walk the same list: for every tile F, its logits (per 64 channels two chunks, node rows 0-4 and 4-8), and three tiles later
+        // Both walk the same list: for every tile F, its logits (per 64 channels two chunks, node rows 0-4 and 4-8), and kLag tiles later
         // G, its weight gradient (per 128 channels four chunks of two own node rows).  A chunk takes the ring's next place.  One thread
         // each: a whole warp's waits and elections between two chunks of eight multiplications take as long as the multiplications.
         const bool producer = warp == kAllWarps;
@@ -291,6 +298,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                 } else parity = (1u << pre) - 1;
                 pre = 0; place = 0;
             }
+            constexpr int kLag = kGroups + 1;              // (a group takes its next tile's logits before it waits for this one's gradient)
             Tile back = k;                                 // the tile whose weight gradient comes next
             int w_stream = -1, n_weights = 0, n_items = 0;
             for (int q = 0; ok && (k.t < n_tiles || (with_grad && back.t < n_tiles)); ++q) {
@@ -345,10 +353,10 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                     ++n_items;
                     next(k);
                 }
-                if (with_grad && q >= 3 && back.t < n_tiles && ok) {
+                if (with_grad && q >= kLag && back.t < n_tiles && ok) {
                     // dW[channel][class] = sum of X[node][channel] dz[node][class] over the tile's own nodes: the group has left the bf16
                     // gradient in shared memory (K-major, zeros at the halo), the features come again (MN-major)
-                    const int g = (q - 3) & 1, j = (q - 3) >> 1;
+                    const int g = (q - kLag) % kGroups, j = (q - kLag) / kGroups;
                     if (producer) {
                         for (int e = 0; e < 4 * mt && ok; ++e) {
                             const int m = e >> 2, r0 = 2 * (e & 3), rows = r0 == 6 ? 1 : 2;
@@ -677,7 +685,7 @@ fwd_ce_kernel(UpsampleCeArgs a, int tiles_x, int tiles_y, const __grid_constant_
                     const float2 b2 = __ffma2_rn(hs23, bw23, __fmul2_rn(hs01, bw01));
                     return make_float2(t2.x + t2.y, b2.x + b2.y);
                 };
-                constexpr int G = kSweep2;                 // classes in flight: all their reads come before the first write
+                constexpr int G = sweep2(FORM);                 // classes in flight: all their reads come before the first write
                 static_for_groups<C, G>([&](int c0, auto count) {
                     constexpr int N = decltype(count)::value;
                     float2 L[N], R[N], o[N];
@@ -873,6 +881,8 @@ cudaError_t prepare_fwd_ce_as()
     if constexpr (!loss_kernel_two_groups(C, false)) {
         if (e == cudaSuccess) e = prepare_fwd_ce_form<C, false, kOneGroup>();
         if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kOneGroup>();
+        if (e == cudaSuccess) e = prepare_fwd_ce_form<C, false, kLoneGroup>();
+        if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kLoneGroup>();
     }
     return e;
 }
@@ -899,6 +909,10 @@ void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const C
     if constexpr (!FORWARD) launch_fwd_ce_form<C, kStored>(a, x_map, w_map, row_map, s);
     else {
         if constexpr (!loss_kernel_two_groups(C, false)) if (!loss_kernel_two_groups(C, a.w_part != nullptr)) return launch_fwd_ce_form<C, kOneGroup>(a, x_map, w_map, row_map, s);
+        // at most a tile per SM: us a step, two groups / a lone one, 128 channels on 90 x 160 (78 tiles) 14.8 / 14.6, 256 channels on 45 x 70
+        // (21 tiles) 16.8 / 16.4, with 4 classes 12.2 / 11.5.  With more tiles an SM has work for two groups.
+        if constexpr (classifier_gradient_fits(C))
+            if (upsample_ce_few_blocks(a.h, a.w) * a.S <= a.n_sms) return launch_fwd_ce_form<C, kLoneGroup>(a, x_map, w_map, row_map, s);
         launch_fwd_ce_form<C, kTwoGroups>(a, x_map, w_map, row_map, s);
     }
 }
