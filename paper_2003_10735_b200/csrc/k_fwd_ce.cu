@@ -22,7 +22,7 @@ bool upsample_ce_few_supported(int C) { return C <= kClassPad; }
 
 int upsample_ce_few_blocks(int h, int w) { return ((h + FN_Y - 1) / FN_Y) * ((w + FN_X - 1) / FN_X); }
 
-cudaError_t prepare_fwd_ce(int C) { return fwd_ce_kernels(C).prepare(); }
+cudaError_t prepare_fwd_ce(int C, bool own_forward, bool with_gradient, int tiles, int n_sms) { return fwd_ce_kernels(C).prepare(own_forward, with_gradient, tiles, n_sms); }
 
 void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s) { fwd_ce_kernels(a.C).launch[1](a, x_map, w_map, row_map, s); }
 

@@ -871,20 +871,23 @@ cudaError_t prepare_fwd_ce_form()
     return e != cudaSuccess ? e : FORM != kStored && at.numRegs < form_launch_regs(FORM) ? cudaErrorInvalidConfiguration : cudaSuccess;
 }
 
-template <int C>
-cudaError_t prepare_fwd_ce_as()
+template <int C, int FORM>
+cudaError_t prepare_fwd_ce_both()
 {
-    cudaError_t e = prepare_fwd_ce_form<C, false, kStored>();
-    if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kStored>();
-    if (e == cudaSuccess) e = prepare_fwd_ce_form<C, false, kTwoGroups>();
-    if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kTwoGroups>();
-    if constexpr (!loss_kernel_two_groups(C, false)) {
-        if (e == cudaSuccess) e = prepare_fwd_ce_form<C, false, kOneGroup>();
-        if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kOneGroup>();
-        if (e == cudaSuccess) e = prepare_fwd_ce_form<C, false, kLoneGroup>();
-        if (e == cudaSuccess) e = prepare_fwd_ce_form<C, true, kLoneGroup>();
+    const cudaError_t e = prepare_fwd_ce_form<C, false, FORM>();
+    return e != cudaSuccess ? e : prepare_fwd_ce_form<C, true, FORM>();
+}
+// The kernels that a context may launch: on stored logits, and its form with an own forward (each that is touched is loaded, 0.2 ms)
+template <int C>
+cudaError_t prepare_fwd_ce_as(bool own_forward, bool with_gradient, int tiles, int n_sms)
+{
+    const cudaError_t e = prepare_fwd_ce_both<C, kStored>();
+    if (e != cudaSuccess || !own_forward) return e;
+    if constexpr (classifier_gradient_fits(C)) {
+        if (!with_gradient) return prepare_fwd_ce_both<C, kOneGroup>();
+        if (tiles <= n_sms) return prepare_fwd_ce_both<C, kLoneGroup>();
     }
-    return e;
+    return prepare_fwd_ce_both<C, kTwoGroups>();
 }
 
 template <int C, bool CONF, int FORM>
@@ -921,7 +924,7 @@ void launch_fwd_ce_of(const UpsampleCeArgs& a, const CUtensorMap& x_map, const C
 
 // The kernels of one class count
 struct FwdCeKernels {
-    cudaError_t (*prepare)();
+    cudaError_t (*prepare)(bool own_forward, bool with_gradient, int tiles, int n_sms);
     void (*launch[2])(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s);   // stored logits, own forward
 };
 

@@ -409,9 +409,9 @@ int upsample_ce_blocks(int h, int w, int C)
     return ((h + ny - 1) / ny) * ((w + kOwnX - 1) / kOwnX);
 }
 
-cudaError_t prepare_upsample_ce(int C)
+cudaError_t prepare_upsample_ce(int C, bool own_forward, bool with_gradient, int tiles, int n_sms)
 {
-    if (upsample_ce_few_supported(C)) return prepare_fwd_ce(C);
+    if (upsample_ce_few_supported(C)) return prepare_fwd_ce(C, own_forward, with_gradient, tiles, n_sms);
     const cudaError_t e = allow_many<7, 2>();
     return e != cudaSuccess ? e : allow_many<4, 3>();
 }

@@ -752,7 +752,7 @@ st_status st_init_head(const st_head_desc* desc, const float* init_params, st_ct
         }
     }
 #undef ALLOC
-    if (e == cudaSuccess) e = prepare_upsample_ce(c->C);
+    if (e == cudaSuccess) e = prepare_upsample_ce(c->C, c->fused_loss != 0, c->fused_grad != 0, c->n_k3_blocks * S, c->n_sms);
     if (e == cudaSuccess) e = prepare_student_mask();
     if (e == cudaSuccess && !c->bf16_mode) e = prepare_conv_f32();
     if (e != cudaSuccess) {

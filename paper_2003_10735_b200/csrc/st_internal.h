@@ -139,7 +139,8 @@ bool encode_tensor_map(CUtensorMap* m, CUtensorMapDataType dtype, CUtensorMapSwi
                        const uint64_t* dims, const uint64_t* strides, const uint32_t* box, char* err, size_t err_len,
                        const char* what);
 int upsample_ce_blocks(int h, int w, int C);   // blocks per stream (sizes loss_part / db_part)
-cudaError_t prepare_upsample_ce(int C);   // once per device and class count, outside any stream capture
+// outside any stream capture; which kernels: of a context that multiplies its own logits, forms the gradient too, has so many tiles in a launch
+cudaError_t prepare_upsample_ce(int C, bool own_forward, bool with_gradient, int tiles, int n_sms);
 void launch_upsample_ce(const UpsampleCeArgs& a, cudaStream_t s);
 // The same with the forward of a 1x1 classifier over bf16 features in front, in one kernel (k_fwd_ce.cuh), for the shapes that
 // fused_forward_supported names; host copies of the tile maps of the features and of the bf16 weights
@@ -149,7 +150,7 @@ bool fused_forward_supported(int C, int h, int w, int c_in);
 constexpr bool classifier_gradient_fits(int C) { return C <= 24; }
 // ... and two groups of warps to a block where it is formed, or where two blocks of one group do not fit an SM (k_fwd_ce.cuh)
 constexpr bool loss_kernel_two_groups(int C, bool with_gradient) { return with_gradient || !classifier_gradient_fits(C); }
-cudaError_t prepare_fwd_ce(int C);
+cudaError_t prepare_fwd_ce(int C, bool own_forward, bool with_gradient, int tiles, int n_sms);   // tiles: of all streams
 void launch_fwd_ce(const UpsampleCeArgs& a, const CUtensorMap& x_map, const CUtensorMap& w_map, const CUtensorMap& row_map, cudaStream_t s);
 // Tile map of bf16 features [S][h][w][c_in] for it: {c_in, w, h, S}, one box = 64 channels of a tile
 bool make_feature_tile_map(CUtensorMap* m, const bf16* x, int S, int c_in, int h, int w);
